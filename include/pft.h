@@ -412,9 +412,10 @@ int pft_backward_last_launch_count(void);
  * counterpart; this is a calling convenience.)
  *  - Same arguments, result and options as pft3d_mesh, minus ws / ws_bytes.
  *    It allocates nothing and calls no allocating routine.
- *  - Scratch is a file-scope device array of 32 MiB, which every GPU that loads
+ *  - Scratch is a file-scope device array of 33 MiB, which every GPU that loads
  *    the library keeps until the process exits.  Problems whose
- *    pft3d_workspace_size() exceeds 32 MiB return PFT_ERR_SCRATCH_LIMIT at once.
+ *    pft3d_workspace_size() exceeds 32 MiB, not counting the up to 0.6 MiB that the
+ *    small-|Q| pass adds to it, return PFT_ERR_SCRATCH_LIMIT at once.
  *  - All calls on a device share that array and it keeps the last call's
  *    contents; calls whose GPU work overlaps (several streams or host threads)
  *    race on it, so serialise them.

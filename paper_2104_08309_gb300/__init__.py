@@ -318,7 +318,7 @@ def pft3d_polymesh(verts, face_idx, face_off, q, *, options=None, out=None, ws=N
 
 
 def pft3d_mesh_noalloc(verts, faces, q, out, *, options=None, stream=None):
-    """pft3d_mesh with the library's fixed 32 MiB device scratch instead of a workspace.
+    """pft3d_mesh with the library's fixed device scratch instead of a workspace.
 
     For callers that must not allocate at call time (stream capture, host
     applications that own all device memory): ``out`` ([n_q, 2] float64, CUDA)

@@ -6,7 +6,7 @@
 #include <unordered_map>
 #include <vector>
 
-#include "pft_kernels.cuh"
+#include "pft_small.cuh"
 
 namespace pft {
 namespace {
@@ -109,6 +109,7 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q) {
 
 struct FwdLayout {
   size_t mparts, items, partial, small, qperm, qscratch, total;
+  size_t grown;   // bytes that the small-|Q| pass adds to the total
   int nblk;
   bool tiled;   // the main kernel visits the Q points in the library's order (q_order option)
   FwdLaunch L;
@@ -122,6 +123,11 @@ FwdLayout layout_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_prep, in
   size_t off = align_up(sizeof(WsHeader));
   y.mparts = off;  off = align_up(off + sizeof(double) * (size_t)y.nblk);
   y.items = off;   off = align_up(off + item_bytes * (size_t)std::max<int64_t>(n_items, 1));
+  if (dim == 3) {   // the small-|Q| pass writes over the records once the pair sums are done
+    const size_t end = align_up(y.items + small3_bytes(n_items, device_sms()));
+    y.grown = end > off ? end - off : 0;
+    off += y.grown;
+  }
   y.partial = off; off = align_up(off + sizeof(double2) * (size_t)y.L.k_splits * (size_t)std::max<int64_t>(n_q, 1));
   y.small = off;   off = align_up(off + sizeof(int32_t) * (size_t)std::max<int64_t>(n_q, 1));
   y.tiled = o.q_order == PFT_Q_TILED && qorder_wanted(n_q, n_items, o.r, o.nt);
@@ -163,6 +169,13 @@ inline cudaError_t mark(cudaEvent_t ev, cudaStream_t st) { return ev ? cudaEvent
   } while (0)
 
 }  // namespace
+
+size_t small3_growth(int64_t n_faces, int64_t n_q, const pft_options* opts) {
+  Opts o;
+  if (resolve(opts, 3, o) != PFT_OK) return 0;
+  return layout_fwd(3, o, n_faces, n_faces, n_q).grown;
+}
+
 }  // namespace pft
 
 using namespace pft;
@@ -207,11 +220,11 @@ int pft2d_polygons(const float* verts, int64_t n_verts, const int64_t* loop_off,
   if (int e = fwd_qorder(2, y, q, n_q, ws, st, qperm)) return e;
   if (mark(o.ev_start, st) != cudaSuccess) return PFT_ERR_CUDA;
   PFT_LAUNCH(launch_fwd(2, o.fp64, y.L, at<void>(ws, y.items), n_verts, q, n_q, o.tau, at<double2>(ws, y.partial),
-                        &h->status, st, 0, qperm));
+                        h, at<int32_t>(ws, y.small), st, 0, qperm));
   if (mark(o.ev_stop, st) != cudaSuccess) return PFT_ERR_CUDA;
-  PFT_LAUNCH(launch_finalize(2, q, n_q, at<double2>(ws, y.partial), y.L.k_splits, o.fp64, h, mp, y.nblk,
-                             at<int32_t>(ws, y.small), out, st));
-  PFT_LAUNCH(launch_smallq2d(verts, n_verts, loop_off, n_loops, q, o.fp64, h, at<int32_t>(ws, y.small), out, st));
+  PFT_LAUNCH(launch_finalize2d(q, n_q, at<double2>(ws, y.partial), y.L.k_splits, h, mp, y.nblk,
+                               at<int32_t>(ws, y.small), out, st));
+  PFT_LAUNCH(launch_smallq2d(verts, n_verts, loop_off, n_loops, q, h, at<int32_t>(ws, y.small), out, st));
   return PFT_OK;
 }
 
@@ -243,11 +256,11 @@ int pft3d_mesh(const float* verts, int64_t n_verts, const int32_t* faces, int64_
   if (int e = fwd_qorder(3, y, q, n_q, ws, st, qperm)) return e;
   if (mark(o.ev_start, st) != cudaSuccess) return PFT_ERR_CUDA;
   PFT_LAUNCH(launch_fwd(3, o.fp64, y.L, at<void>(ws, y.items), n_faces, q, n_q, o.tau, at<double2>(ws, y.partial),
-                        &h->status, st, 2 * o.face_pairs, qperm));
+                        h, at<int32_t>(ws, y.small), st, 2 * o.face_pairs, qperm));
   if (mark(o.ev_stop, st) != cudaSuccess) return PFT_ERR_CUDA;
-  PFT_LAUNCH(launch_finalize(3, q, n_q, at<double2>(ws, y.partial), y.L.k_splits, o.fp64, h, mp, y.nblk,
-                             at<int32_t>(ws, y.small), out, st));
-  PFT_LAUNCH(launch_smallq3d(verts, n_verts, faces, n_faces, q, o.fp64, h, at<int32_t>(ws, y.small), out, st));
+  PFT_LAUNCH(launch_small3(verts, n_verts, faces, n_faces, q, h, mp, y.nblk, at<void>(ws, y.items), st));
+  PFT_LAUNCH(launch_finalize3d(q, n_q, n_faces, at<double2>(ws, y.partial), y.L.k_splits, h, at<int32_t>(ws, y.small),
+                               at<void>(ws, y.items), out, st));
   return PFT_OK;
 }
 
@@ -293,11 +306,11 @@ int pft3d_polymesh(const float* verts, int64_t n_verts, const int32_t* face_idx,
   if (int e = fwd_qorder(3, y, q, n_q, ws, st, qperm)) return e;
   if (mark(o.ev_start, st) != cudaSuccess) return PFT_ERR_CUDA;
   PFT_LAUNCH(launch_fwd(3, o.fp64, y.L, at<void>(ws, y.items), n_tris, q, n_q, o.tau, at<double2>(ws, y.partial),
-                        &h->status, st, 0, qperm));
+                        h, at<int32_t>(ws, y.small), st, 0, qperm));
   if (mark(o.ev_stop, st) != cudaSuccess) return PFT_ERR_CUDA;
-  PFT_LAUNCH(launch_finalize(3, q, n_q, at<double2>(ws, y.partial), y.L.k_splits, o.fp64, h, mp, y.nblk,
-                             at<int32_t>(ws, y.small), out, st));
-  PFT_LAUNCH(launch_smallq3d(verts, n_verts, tris, n_tris, q, o.fp64, h, at<int32_t>(ws, y.small), out, st));
+  PFT_LAUNCH(launch_small3(verts, n_verts, tris, n_tris, q, h, mp, y.nblk, at<void>(ws, y.items), st));
+  PFT_LAUNCH(launch_finalize3d(q, n_q, n_tris, at<double2>(ws, y.partial), y.L.k_splits, h, at<int32_t>(ws, y.small),
+                               at<void>(ws, y.items), out, st));
   return PFT_OK;
 }
 

@@ -31,15 +31,18 @@ constexpr uint32_t kWaitLimit = 1u << 22;
 // ---------------------------------------------------------------------------
 // Workspace header (256 bytes), filled by the prep kernels.
 // ---------------------------------------------------------------------------
+constexpr int kSmallDirect = 32;   // small Q points that a 3D forward call evaluates one by one (pft_small.cuh)
+
 struct WsHeader {
   uint32_t status;
   uint32_t small_q_count;   // number of Q points routed to the FP64 small-|Q| pass
   uint32_t bbox_enc[6];     // order-preserving encodings: min x,y,z then max x,y,z
   uint32_t rmax_bits;       // max |v - c| as float bits (non-negative floats order as ints)
-  uint32_t pad0;
+  uint32_t ticket;          // blocks of k_small3 that have written their part
   double center[3];         // bounding-box midpoint c (all coordinates are taken relative to c)
-  double measure;           // area (2D) or volume (3D), FP64, fixed-order sum
-  uint8_t pad[256 - 4 * 10 - 8 * 4];
+  double measure;           // volume (3D forward), FP64, fixed-order sum
+  int32_t small_list[kSmallDirect];   // the first listed small Q points (3D forward)
+  uint8_t pad[256 - 4 * 10 - 8 * 4 - 4 * kSmallDirect];
 };
 static_assert(sizeof(WsHeader) == 256, "header must stay 256 bytes");
 

@@ -30,8 +30,8 @@ namespace {
 template <class Pol, int R, int NT>
 __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typename Pol::Item* __restrict__ items, int64_t n_items,
                                             int64_t per_split, const double* __restrict__ q, int64_t n_q,
-                                            Thr th, double2* __restrict__ partial, uint32_t* status,
-                                            const int32_t* __restrict__ qperm) {
+                                            Thr th, double2* __restrict__ partial, WsHeader* h,
+                                            int32_t* __restrict__ small, const int32_t* __restrict__ qperm) {
   using Item = typename Pol::Item;
   using QT = typename Pol::QT;
   constexpr int TILE = Pol::kTile;
@@ -50,6 +50,8 @@ __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typena
   // slot qbase + r NT holds Q point qperm[slot] (the caller's index; without qperm the slot itself)
   QT qr[R][3];
   const int64_t qbase = (int64_t)blockIdx.x * (NT * R) + threadIdx.x;
+  bool live = D == 2;   // 3D: some point of this thread needs the pair sum (|Q| r_max >= 1/4)
+  const float rmax = D == 3 ? __uint_as_float(h->rmax_bits) : 0.f;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int64_t iq = qbase + (int64_t)r * NT;
@@ -59,8 +61,26 @@ __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typena
       const int64_t src = qperm ? (int64_t)qperm[iq] : iq;
 #pragma unroll
       for (int d = 0; d < D; ++d) qr[r][d] = (QT)q[src * D + d];
+      if constexpr (D == 3) {
+        // Points of the small-|Q| pass take no part in the pair sum (their place in a warp's largest
+        // P is immaterial: it is the smallest), and the first face chunk's blocks list them.  The
+        // FP32 test settles all but those near or below the bound.
+        const float fx = (float)qr[r][0] * rmax, fy = (float)qr[r][1] * rmax, fz = (float)qr[r][2] * rmax;
+        bool is_small = false;
+        if (!(fmaf(fx, fx, fmaf(fy, fy, fz * fz)) > 1.01f * (float)(kTauSmallQ * kTauSmallQ))) {
+          const double q2 = q_norm2(q[src * 3], q[src * 3 + 1], q[src * 3 + 2]);
+          is_small = q2 == 0.0 || small_q(q2, rmax);
+          if (is_small && q2 != 0.0 && blockIdx.y == 0) {
+            const uint32_t e = atomicAdd(&h->small_q_count, 1u);
+            small[src] = (int32_t)e;
+            if (e < (uint32_t)kSmallDirect) h->small_list[e] = (int32_t)src;
+          }
+        }
+        live = live || !is_small;
+      }
     }
   }
+  live = __any_sync(0xffffffffu, live);
   typename Pol::template Acc<R> acc;
   acc.init();
 
@@ -80,7 +100,7 @@ __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typena
     issued = 0;
     fence_mbar_init();
   }
-  __syncthreads();
+  if (!__syncthreads_or(live)) return;
   if (threadIdx.x == 0)
     for (int t = 0; t < min(kStages, ntiles); ++t) issue(t);
 
@@ -89,7 +109,7 @@ __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typena
     const int s = t % kStages;
     if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[s], (uint32_t)((t / kStages) & 1)))) { ok = false; break; }
     const int cnt = (int)min((int64_t)TILE, n - (int64_t)t * TILE);
-    Pol::template tile<R>(ring + s * TILE, cnt, qr, acc, th, i0 + (int64_t)t * TILE);
+    if (live) Pol::template tile<R>(ring + s * TILE, cnt, qr, acc, th, i0 + (int64_t)t * TILE);
     __syncwarp();
     if ((threadIdx.x & 31) == 0) {
       __threadfence_block();                       // this warp's reads of slot s come first
@@ -102,7 +122,7 @@ __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typena
       }
     }
   }
-  if (!ok) set_status(status, ST_TIMEOUT);
+  if (!ok) set_status(&h->status, ST_TIMEOUT);
   __syncthreads();   // reached by every thread: stop decisions above are per warp, never inside a warp
   if (threadIdx.x == 0) {   // no copy may still be writing into the ring when the block exits
     const int m = issued;
@@ -119,10 +139,11 @@ __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typena
 
 template <class Pol, int R, int NT>
 cudaError_t launch_one(const FwdLaunch& L, const void* items, int64_t n_items, const double* q, int64_t n_q,
-                       Thr th, double2* partial, uint32_t* status, cudaStream_t st, const int32_t* qperm) {
+                       Thr th, double2* partial, WsHeader* h, int32_t* small, cudaStream_t st,
+                       const int32_t* qperm) {
   dim3 grid((unsigned)L.q_tiles, (unsigned)L.k_splits);
   k_fwd<Pol, R, NT><<<grid, NT, 0, st>>>(static_cast<const typename Pol::Item*>(items), n_items, L.per_split, q,
-                                         n_q, th, partial, status, qperm);
+                                         n_q, th, partial, h, small, qperm);
   return cudaGetLastError();
 }
 
@@ -159,10 +180,10 @@ cudaError_t dispatch_pairs(int r, int nt, F&& f) {
 
 struct LaunchF {
   const FwdLaunch& L; const void* items; int64_t n_items; const double* q; int64_t n_q; Thr th;
-  double2* partial; uint32_t* status; cudaStream_t st; const int32_t* qperm;
+  double2* partial; WsHeader* h; int32_t* small; cudaStream_t st; const int32_t* qperm;
   template <class Pol, int R, int NT>
   cudaError_t operator()() const {
-    return launch_one<Pol, R, NT>(L, items, n_items, q, n_q, th, partial, status, st, qperm);
+    return launch_one<Pol, R, NT>(L, items, n_items, q, n_q, th, partial, h, small, st, qperm);
   }
 };
 
@@ -175,14 +196,14 @@ struct OccF {
 }  // namespace
 
 cudaError_t launch_fwd(int dim, bool fp64, const FwdLaunch& L, const void* items, int64_t n_items, const double* q,
-                       int64_t n_q, float tau, double2* partial, uint32_t* status, cudaStream_t st,
+                       int64_t n_q, float tau, double2* partial, WsHeader* h, int32_t* small, cudaStream_t st,
                        int64_t pair_faces, const int32_t* qperm) {
   // the FP64 path keeps its series (through k = 16) for P < 9/4, where it truncates below 1e-14
   if (fp64) tau = fminf(tau, 3.0f);
   const float tau_lo = fminf(tau, kTauLo);
   const Thr th{0.25f * tau * tau, 0.25f * tau_lo * tau_lo, tau > 1.0f ? 1 : 0, tau > 3.0f ? 1 : 0,
                dim == 3 && !fp64 ? pair_faces : 0};
-  LaunchF f{L, items, n_items, q, n_q, th, partial, status, st, qperm};
+  LaunchF f{L, items, n_items, q, n_q, th, partial, h, small, st, qperm};
   if (dim == 2) return fp64 ? dispatch<Pol2F64>(L.r, L.nt, f) : dispatch<Pol2F32>(L.r, L.nt, f);
   if (!fp64 && th.pair_end > 0) return dispatch_pairs(L.r, L.nt, f);
   return fp64 ? dispatch<Pol3F64>(L.r, L.nt, f) : dispatch<Pol3F32>(L.r, L.nt, f);

@@ -36,6 +36,14 @@ static_assert(sizeof(Face32) == 48 && sizeof(Face64) == 96, "face record sizes")
 // boundary sum (which cancels to O(|Q|^2 R^2) of its terms there).
 constexpr double kTauSmallQ = 0.25;
 
+// |Q|^2 in FP64 (one fixed rounding, whichever kernel asks), and the test for the small-|Q| pass.
+__device__ __forceinline__ double q_norm2(double x, double y, double z) {
+  return __fma_rn(x, x, __fma_rn(y, y, __dmul_rn(z, z)));
+}
+__device__ __forceinline__ bool small_q(double q2, float rmax) {
+  return __dmul_rn(__dsqrt_rn(q2), (double)rmax) < kTauSmallQ;
+}
+
 // sum_k i^k h_k(x) / (k + p)! for the n nodes x (FP64), K terms: the integral of exp(i Q.r)
 // over a simplex divided by p! times its volume, from its corner phases x (small-|Q| passes).
 template <int N, int P, int K>
@@ -81,19 +89,22 @@ cudaError_t launch_prep3d(const float* v, int64_t nv, const int32_t* f, int64_t 
                           void* faces, bool fp64, double* partials, int nblk, cudaStream_t st,
                           int64_t pair_faces = 0);
 // qperm: NULL, or the slot -> Q index map of launch_qorder (the kernel reads Q point qperm[slot]
-// and writes its partial sums at that index).
+// and writes its partial sums at that index).  In 3D the kernel also counts and lists the small-|Q|
+// points: small[i] is point i's place among them.
 cudaError_t launch_fwd(int dim, bool fp64, const FwdLaunch& L, const void* items, int64_t n_items,
-                       const double* q, int64_t n_q, float tau, double2* partial, uint32_t* status,
+                       const double* q, int64_t n_q, float tau, double2* partial, WsHeader* h, int32_t* small,
                        cudaStream_t st, int64_t pair_faces = 0, const int32_t* qperm = nullptr);
 cudaError_t launch_fan3d(const int32_t* idx, int64_t n_idx, const int64_t* off, int64_t n_faces, int32_t* tris,
                          int64_t n_tris, WsHeader* h, cudaStream_t st);
-cudaError_t launch_finalize(int dim, const double* q, int64_t n_q, const double2* partial, int k_splits,
-                            bool fp64, WsHeader* h, const double* measure_partials, int n_measure,
-                            int32_t* small_list, double* out, cudaStream_t st);
-cudaError_t launch_smallq2d(const float* v, int64_t nv, const int64_t* off, int64_t nl, const double* q, bool fp64,
+cudaError_t launch_finalize2d(const double* q, int64_t n_q, const double2* partial, int k_splits, WsHeader* h,
+                              const double* measure_partials, int n_measure, int32_t* small_list, double* out,
+                              cudaStream_t st);
+cudaError_t launch_smallq2d(const float* v, int64_t nv, const int64_t* off, int64_t nl, const double* q,
                             const WsHeader* h, const int32_t* small_list, double* out, cudaStream_t st);
-cudaError_t launch_smallq3d(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q, bool fp64,
-                            const WsHeader* h, const int32_t* small_list, double* out, cudaStream_t st);
+// scratch: what launch_small3 wrote.
+cudaError_t launch_finalize3d(const double* q, int64_t n_q, int64_t nf, const double2* partial, int k_splits,
+                              const WsHeader* h, const int32_t* small, const void* scratch, double* out,
+                              cudaStream_t st);
 
 // Prep blocks used for the per-block FP64 area/volume partial sums.
 constexpr int kPrepThreads = 256;

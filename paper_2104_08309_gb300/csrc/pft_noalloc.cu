@@ -23,12 +23,15 @@
 //    stale.
 #include <mutex>
 
-#include "pft_kernels.cuh"
+#include "pft_small.cuh"
 
 namespace pft {
 namespace {
 
-constexpr size_t kScratchBytes = size_t(32) << 20;   // 32 MiB per device
+// The limit on a problem's workspace, without what the small-|Q| pass adds to it (at most 0.6 MiB,
+// for which the array has room).
+constexpr size_t kScratchLimit = size_t(32) << 20;   // 32 MiB
+constexpr size_t kScratchBytes = size_t(33) << 20;   // 33 MiB per device
 constexpr int kMaxDevices = 64;
 
 // The scratch array.  In host code this name is only a stand-in for the device
@@ -69,7 +72,7 @@ extern "C" int pft3d_mesh_noalloc(const float* verts, int64_t n_verts, const int
   // Sizes or options that pft3d_workspace_size rejects: pft3d_mesh refuses them
   // before it looks at the workspace, with the code it would give any caller.
   if (need == 0) return pft3d_mesh(verts, n_verts, faces, n_faces, q, n_q, out, nullptr, 0, opts, stream);
-  if (need > pft::kScratchBytes) return PFT_ERR_SCRATCH_LIMIT;
+  if (need - pft::small3_growth(n_faces, n_q, opts) > pft::kScratchLimit || need > pft::kScratchBytes) return PFT_ERR_SCRATCH_LIMIT;
   void* scratch = nullptr;
   if (int e = pft::scratch_address(static_cast<cudaStream_t>(stream), &scratch)) return e;
   // The header at the start of the scratch (status word, counters, bounding box)

@@ -1,7 +1,9 @@
 // pft_prep.cu -- input validation, centring, segment/face records, the finalize
 // pass (fixed-order FP64 split sum, 1/|Q|^2, translation phase, Q = 0 limit) and
 // the FP64 small-|Q| pass.
-#include "pft_kernels.cuh"
+#include <algorithm>
+
+#include "pft_small.cuh"
 
 namespace pft {
 
@@ -250,21 +252,38 @@ __global__ void k_fan3d(const int32_t* __restrict__ idx, int64_t n_idx, const in
   tris[3 * t + 2] = i2;
 }
 
-// Finalize: out(Q) = exp(iQ.c) * scale / |Q|^2 * sum_splits partial (fixed order, FP64).
-__global__ void k_finalize(int dim, const double* __restrict__ q, int64_t n_q, const double2* __restrict__ partial,
-                           int ks, int fp64, WsHeader* h, const double* __restrict__ mparts, int nm,
-                           int32_t* small_list, double* __restrict__ out, double scale) {
+// Finalize: out(Q) = exp(iQ.c) * scale / |Q|^2 * sum_splits partial (fixed order, FP64), at the
+// caller's Q: the FP32 pair sums ran at Q rounded to float in coordinates centred on the bounding
+// box, where that moves them by ~1e-7 of |S|; in the phase Q.c the same rounding would move the
+// result by |c| times it, which for a shape far from the origin is not small.
+__device__ __forceinline__ void finish(const double (&Q)[3], double re, double im, const WsHeader* h,
+                                       double* __restrict__ out) {
+  const double ph = Q[0] * h->center[0] + Q[1] * h->center[1] + Q[2] * h->center[2];
+  double sp, cp;
+  sincos(ph, &sp, &cp);
+  out[0] = re * cp - im * sp;
+  out[1] = re * sp + im * cp;
+}
+__device__ __forceinline__ void split_sum(const double2* __restrict__ partial, int ks, int64_t n_q, int64_t i,
+                                          double k, double& re, double& im) {
+  re = 0.0;
+  im = 0.0;
+  for (int s = 0; s < ks; ++s) {
+    const double2 p = partial[(int64_t)s * n_q + i];
+    re += p.x;
+    im += p.y;
+  }
+  re *= k;
+  im *= k;
+}
+
+__global__ void k_finalize2d(const double* __restrict__ q, int64_t n_q, const double2* __restrict__ partial,
+                             int ks, WsHeader* h, const double* __restrict__ mparts, int nm, int32_t* small_list,
+                             double* __restrict__ out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n_q) return;
-  double Q[3] = {0, 0, 0};
-  for (int d = 0; d < dim; ++d) {
-    double x = q[dim * i + d];
-    // the caller's Q: the FP32 pair sums ran at Q rounded to float in coordinates centred on the
-    // bounding box, where that moves them by ~1e-7 of |S|; in the phase Q.c the same rounding would
-    // move the result by |c| times it, which for a shape far from the origin is not small
-    Q[d] = x;
-  }
-  const double q2 = Q[0] * Q[0] + Q[1] * Q[1] + Q[2] * Q[2];
+  const double Q[3] = {q[2 * i], q[2 * i + 1], 0.0};
+  const double q2 = q_norm2(Q[0], Q[1], Q[2]);
   if (q2 == 0.0) {
     double s = 0.0;
     for (int b = 0; b < nm; ++b) s += mparts[b];
@@ -272,78 +291,67 @@ __global__ void k_finalize(int dim, const double* __restrict__ q, int64_t n_q, c
     out[2 * i + 1] = 0.0;
     return;
   }
-  const double rmax = (double)__uint_as_float(h->rmax_bits);
-  if (sqrt(q2) * rmax < kTauSmallQ) {
-    uint32_t slot = atomicAdd(&h->small_q_count, 1u);
-    small_list[slot] = (int32_t)i;
+  if (small_q(q2, __uint_as_float(h->rmax_bits))) {
+    small_list[atomicAdd(&h->small_q_count, 1u)] = (int32_t)i;
     return;
   }
-  double re = 0.0, im = 0.0;
-  for (int s = 0; s < ks; ++s) {
-    double2 p = partial[(int64_t)s * n_q + i];
-    re += p.x;
-    im += p.y;
+  double re, im;
+  split_sum(partial, ks, n_q, i, 2.0 / q2, re, im);   // records hold half edge vectors
+  finish(Q, re, im, h, out + 2 * i);
+}
+
+// 3D: small-|Q| points (as k_fwd listed them) take their sum from k_small3's results.
+__global__ void k_finalize3d(const double* __restrict__ q, int64_t n_q, int64_t nf,
+                             const double2* __restrict__ partial, int ks, const WsHeader* __restrict__ h,
+                             const int32_t* __restrict__ small, const char* __restrict__ scratch,
+                             double* __restrict__ out) {
+  __shared__ double mom[kMomN];
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const float rmax = __uint_as_float(h->rmax_bits);
+  double Q[3] = {0.0, 0.0, 0.0}, q2 = 0.0;
+  bool is_small = false;
+  if (i < n_q) {
+    for (int d = 0; d < 3; ++d) Q[d] = q[3 * i + d];
+    q2 = q_norm2(Q[0], Q[1], Q[2]);
+    is_small = q2 != 0.0 && small_q(q2, rmax);
   }
-  const double k = scale / q2;
-  re *= k;
-  im *= k;
-  const double ph = Q[0] * h->center[0] + Q[1] * h->center[1] + Q[2] * h->center[2];
-  double sp, cp;
-  sincos(ph, &sp, &cp);
-  out[2 * i] = re * cp - im * sp;
-  out[2 * i + 1] = re * sp + im * cp;
+  const bool direct = h->small_q_count <= (uint32_t)kSmallDirect;
+  if (__syncthreads_or(is_small && !direct)) {
+    for (int t = threadIdx.x; t < kMomN; t += blockDim.x) mom[t] = reinterpret_cast<const double*>(scratch)[t];
+    __syncthreads();
+  }
+  if (i >= n_q) return;
+  if (q2 == 0.0) {
+    out[2 * i] = h->measure;
+    out[2 * i + 1] = 0.0;
+    return;
+  }
+  double re, im;
+  if (!is_small) {
+    split_sum(partial, ks, n_q, i, 1.0 / q2, re, im);
+  } else if (direct) {
+    const int64_t nch = small3_chunks(nf);
+    const double* p = reinterpret_cast<const double*>(scratch + kMomHead) + 2 * nch * small[i];
+    re = 0.0;
+    im = 0.0;
+    for (int64_t t = 0; t < nch; ++t) {
+      re += p[2 * t];
+      im += p[2 * t + 1];
+    }
+  } else {
+    double g[3][2];
+    mom_eval<false>(mom, Q[0] * (double)rmax, Q[1] * (double)rmax, Q[2] * (double)rmax, re, im, g);
+  }
+  finish(Q, re, im, h, out + 2 * i);
 }
 
 constexpr int kSmallThreads = 256;
 
-// Small |Q|: the integral of exp(iQ.(r - c)) over the signed tetrahedra (c, p0, p1, p2)
-// by the simplex series (|Q.(p - c)| < kTauSmallQ, so 16 terms reach FP64 rounding).
-__global__ void __launch_bounds__(kSmallThreads) k_smallq3d(const float* __restrict__ v, int64_t nv,
-                                                            const int32_t* __restrict__ f, int64_t nf,
-                                                            const double* __restrict__ q, int fp64,
-                                                            const WsHeader* h, const int32_t* list,
-                                                            double* __restrict__ out) {
-  __shared__ double sh[kSmallThreads / 32];
-  const uint32_t count = h->small_q_count;
-  const double c[3] = {h->center[0], h->center[1], h->center[2]};
-  for (uint32_t e = blockIdx.x; e < count; e += gridDim.x) {
-    const int64_t i = list[e];
-    double Q[3];
-    for (int d = 0; d < 3; ++d) Q[d] = q[3 * i + d];   // the caller's Q (FP64 series)
-    double re = 0.0, im = 0.0;
-    for (int64_t m = threadIdx.x; m < nf; m += kSmallThreads) {
-      const int32_t id[3] = {f[3 * m], f[3 * m + 1], f[3 * m + 2]};
-      if (id[0] < 0 || id[1] < 0 || id[2] < 0 || id[0] >= nv || id[1] >= nv || id[2] >= nv) continue;
-      double P[3][3], x[3];
-      for (int k = 0; k < 3; ++k) {
-        for (int d = 0; d < 3; ++d) P[k][d] = (double)v[3 * (int64_t)id[k] + d] - c[d];
-        x[k] = Q[0] * P[k][0] + Q[1] * P[k][1] + Q[2] * P[k][2];
-      }
-      const double det = P[0][0] * (P[1][1] * P[2][2] - P[1][2] * P[2][1]) +
-                         P[0][1] * (P[1][2] * P[2][0] - P[1][0] * P[2][2]) +
-                         P[0][2] * (P[1][0] * P[2][1] - P[1][1] * P[2][0]);
-      double sr, si;
-      simplex_series<3, 3, 16>(x, sr, si);
-      re += det * sr;
-      im += det * si;
-    }
-    re = block_sum<kSmallThreads>(re, sh);
-    im = block_sum<kSmallThreads>(im, sh);
-    if (threadIdx.x == 0) {
-      double sp, cp;
-      sincos(Q[0] * c[0] + Q[1] * c[1] + Q[2] * c[2], &sp, &cp);
-      out[2 * i] = re * cp - im * sp;
-      out[2 * i + 1] = re * sp + im * cp;
-    }
-  }
-}
-
 // Small |Q| in 2D: fan of signed triangles (c, p_j, p_{j+1}).
 __global__ void __launch_bounds__(kSmallThreads) k_smallq2d(const float* __restrict__ v, int64_t nv,
                                                             const int64_t* __restrict__ off, int64_t nl,
-                                                            const double* __restrict__ q, int fp64,
-                                                            const WsHeader* h, const int32_t* list,
-                                                            double* __restrict__ out) {
+                                                            const double* __restrict__ q, const WsHeader* h,
+                                                            const int32_t* list, double* __restrict__ out) {
   __shared__ double sh[kSmallThreads / 32];
   const uint32_t count = h->small_q_count;
   const double c[2] = {h->center[0], h->center[1]};
@@ -422,14 +430,24 @@ cudaError_t launch_fan3d(const int32_t* idx, int64_t n_idx, const int64_t* off, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(int dim, const double* q, int64_t n_q, const double2* partial, int k_splits, bool fp64,
-                            WsHeader* h, const double* mparts, int nm, int32_t* small_list, double* out,
-                            cudaStream_t st) {
-  const int nt = 256;
-  const int64_t blocks = (n_q + nt - 1) / nt;
-  const double scale = (dim == 2) ? 2.0 : 1.0;   // 2D records hold half edge vectors
-  k_finalize<<<(unsigned)blocks, nt, 0, st>>>(dim, q, n_q, partial, k_splits, fp64 ? 1 : 0, h, mparts, nm,
-                                               small_list, out, scale);
+// Block size of the finishing kernels: small enough that a small call's FP64 arithmetic (the phase's
+// sincos, the small-|Q| polynomial) spreads over all SMs.
+static int finish_threads(int64_t n_q) { return n_q >= 131072 ? 256 : (n_q >= 32768 ? 128 : (n_q >= 8192 ? 64 : 32)); }
+
+cudaError_t launch_finalize2d(const double* q, int64_t n_q, const double2* partial, int k_splits, WsHeader* h,
+                              const double* mparts, int nm, int32_t* small_list, double* out, cudaStream_t st) {
+  const int nt = finish_threads(n_q);
+  k_finalize2d<<<(unsigned)((n_q + nt - 1) / nt), nt, 0, st>>>(q, n_q, partial, k_splits, h, mparts, nm, small_list,
+                                                              out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_finalize3d(const double* q, int64_t n_q, int64_t nf, const double2* partial, int k_splits,
+                              const WsHeader* h, const int32_t* small, const void* scratch, double* out,
+                              cudaStream_t st) {
+  const int nt = finish_threads(n_q);
+  k_finalize3d<<<(unsigned)((n_q + nt - 1) / nt), nt, 0, st>>>(q, n_q, nf, partial, k_splits, h, small,
+                                                              static_cast<const char*>(scratch), out);
   return cudaGetLastError();
 }
 
@@ -440,15 +458,9 @@ static int small_grid() {
   return sms > 0 ? sms : 1;
 }
 
-cudaError_t launch_smallq2d(const float* v, int64_t nv, const int64_t* off, int64_t nl, const double* q, bool fp64,
+cudaError_t launch_smallq2d(const float* v, int64_t nv, const int64_t* off, int64_t nl, const double* q,
                             const WsHeader* h, const int32_t* list, double* out, cudaStream_t st) {
-  k_smallq2d<<<small_grid(), kSmallThreads, 0, st>>>(v, nv, off, nl, q, fp64 ? 1 : 0, h, list, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_smallq3d(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q, bool fp64,
-                            const WsHeader* h, const int32_t* list, double* out, cudaStream_t st) {
-  k_smallq3d<<<small_grid(), kSmallThreads, 0, st>>>(v, nv, f, nf, q, fp64 ? 1 : 0, h, list, out);
+  k_smallq2d<<<small_grid(), kSmallThreads, 0, st>>>(v, nv, off, nl, q, h, list, out);
   return cudaGetLastError();
 }
 
