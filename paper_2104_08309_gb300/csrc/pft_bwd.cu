@@ -18,6 +18,7 @@
 #include <cstring>
 
 #include "pft_pairs.cuh"
+#include "pft_small.cuh"
 
 namespace pft {
 namespace {
@@ -476,10 +477,9 @@ __global__ void k_bq(const double* __restrict__ q, const double* __restrict__ g,
     Q[d] = q[D * i + d];
     qf[d] = (float)Q[d];
   }
-  const double q2 = Q[0] * Q[0] + Q[1] * Q[1] + Q[2] * Q[2];
+  const double q2 = q_norm2(Q[0], Q[1], Q[2]);
   QRec r{qf[0], qf[1], qf[2], 0.f, 0.f, 0.f, 0.f, 0.f};
-  const double rmax = (double)__uint_as_float(h->rmax_bits);
-  if (q2 == 0.0 || sqrt(q2) * rmax < kTauSmallQ) {
+  if (q2 == 0.0 || small_q(q2, __uint_as_float(h->rmax_bits))) {
     small[atomicAdd(&h->small_q_count, 1u)] = (int32_t)i;
   } else {
     double sp, cp;
@@ -561,9 +561,8 @@ __global__ void k_qfinal(const double* __restrict__ q, const double* __restrict_
   if (i >= n_q) return;
   double Q[3];
   for (int d = 0; d < 3; ++d) Q[d] = q[3 * i + d];   // the caller's Q (factors and phase in FP64)
-  const double q2 = Q[0] * Q[0] + Q[1] * Q[1] + Q[2] * Q[2];
-  const double rmax = (double)__uint_as_float(h->rmax_bits);
-  if (q2 == 0.0 || sqrt(q2) * rmax < kTauSmallQ) return;   // k_qsmall's (same test as k_bq)
+  const double q2 = q_norm2(Q[0], Q[1], Q[2]);
+  if (q2 == 0.0 || small_q(q2, __uint_as_float(h->rmax_bits))) return;   // k_qsmall's (same test as k_bq)
   double v[kQG] = {0.0, 0.0, 0.0, 0.0, 0.0};
   for (int k = 0; k < ks; ++k)
     for (int f = 0; f < kQG; ++f) v[f] += partial[((int64_t)k * n_q + i) * kQG + f];
@@ -613,6 +612,7 @@ __global__ void __launch_bounds__(kAux) k_qsmall_part(const float* __restrict__ 
                                                       double* __restrict__ part) {
   __shared__ double sh[kAux / 32];
   const uint32_t count = h->small_q_count;   // <= n_q <= slots
+  if (count > (uint32_t)kSmallDirect) return;   // from the moments
   const int64_t nch = qsmall_chunks(count, nf, slots);
   const int64_t per = (nf + nch - 1) / nch;
   const double c[3] = {h->center[0], h->center[1], h->center[2]};
@@ -635,13 +635,13 @@ __global__ void __launch_bounds__(kAux) k_qsmall_part(const float* __restrict__ 
                          P[0][1] * (P[1][2] * P[2][0] - P[1][0] * P[2][2]) +
                          P[0][2] * (P[1][0] * P[2][1] - P[1][1] * P[2][0]);
       double sr, si;
-      simplex_series<3, 3, 16>(x, sr, si);
+      simplex_series<3, 3, kMomK>(x, sr, si);
       acc[0] += det * sr;
       acc[1] += det * si;
       for (int k = 0; k < 3; ++k) {
         x[3] = x[k];
         double tr, ti;
-        simplex_series<4, 4, 16>(x, tr, ti);
+        simplex_series<4, 4, kMomK>(x, tr, ti);
         for (int d = 0; d < 3; ++d) {   // i (tr + i ti) P_kd = (-ti + i tr) P_kd
           acc[2 + 2 * d] += -det * ti * P[k][d];
           acc[3 + 2 * d] += det * tr * P[k][d];
@@ -655,19 +655,37 @@ __global__ void __launch_bounds__(kAux) k_qsmall_part(const float* __restrict__ 
   }
 }
 
+// With more than kSmallDirect listed points, S0 and dS0/dQ are the polynomial of the shape's moments
+// (pft_small.cuh) and its gradient.
 __global__ void k_qsmall_fin(int64_t nf, const double* __restrict__ q, const double* __restrict__ g,
                              const WsHeader* h, const int32_t* list, int64_t slots, const double* __restrict__ part,
-                             double* __restrict__ out) {
+                             const double* __restrict__ moments, double* __restrict__ out) {
+  __shared__ double mom[kMomN];
   const uint32_t count = h->small_q_count;
+  if (blockIdx.x * (int64_t)blockDim.x >= count) return;
+  const bool direct = count <= (uint32_t)kSmallDirect;
+  if (!direct) {
+    for (int t = threadIdx.x; t < kMomN; t += blockDim.x) mom[t] = moments[t];
+    __syncthreads();
+  }
   const int64_t nch = qsmall_chunks(count, nf, slots);
-  const double c[3] = {h->center[0], h->center[1], h->center[2]};
+  const double c[3] = {h->center[0], h->center[1], h->center[2]}, rmax = (double)__uint_as_float(h->rmax_bits);
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = list[e];
-    double acc[kQsF] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int64_t ch = 0; ch < nch; ++ch)
-      for (int k = 0; k < kQsF; ++k) acc[k] += part[(e * nch + ch) * kQsF + k];
     double Q[3];
     for (int d = 0; d < 3; ++d) Q[d] = q[3 * i + d];
+    double acc[kQsF] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (direct) {
+      for (int64_t ch = 0; ch < nch; ++ch)
+        for (int k = 0; k < kQsF; ++k) acc[k] += part[(e * nch + ch) * kQsF + k];
+    } else {
+      double gr3[3][2];
+      mom_eval<true>(mom, Q[0] * rmax, Q[1] * rmax, Q[2] * rmax, acc[0], acc[1], gr3);
+      for (int d = 0; d < 3; ++d) {
+        acc[2 + 2 * d] = rmax * gr3[d][0];
+        acc[3 + 2 * d] = rmax * gr3[d][1];
+      }
+    }
     double sp, cp;
     sincos(Q[0] * c[0] + Q[1] * c[1] + Q[2] * c[2], &sp, &cp);
     const double gr = g[2 * i], gi = g[2 * i + 1];
@@ -758,9 +776,8 @@ __global__ void k_qfinal2d(const double* __restrict__ q, const double* __restric
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n_q) return;
   const double Q[2] = {q[2 * i], q[2 * i + 1]};   // the caller's Q (factors and phase in FP64)
-  const double q2 = Q[0] * Q[0] + Q[1] * Q[1];
-  const double rmax = (double)__uint_as_float(h->rmax_bits);
-  if (q2 == 0.0 || sqrt(q2) * rmax < kTauSmallQ) return;   // k_qsmall2d's (same test as k_bq)
+  const double q2 = q_norm2(Q[0], Q[1], 0.0);
+  if (q2 == 0.0 || small_q(q2, __uint_as_float(h->rmax_bits))) return;   // k_qsmall2d's (same test as k_bq)
   double v[kQG2] = {0.0, 0.0, 0.0, 0.0};
   for (int k = 0; k < ks; ++k)
     for (int f = 0; f < kQG2; ++f) v[f] += partial[((int64_t)k * n_q + i) * kQG2 + f];
@@ -1397,7 +1414,8 @@ __global__ void __launch_bounds__(kBwdNT) k_bbwd3(const Face32* __restrict__ rec
 __device__ void corner_adj(int64_t m, const float* __restrict__ v, int64_t nv, const int32_t* __restrict__ f,
                            int64_t nf, const double* __restrict__ partial, int ks, const double* c,
                            const int32_t* __restrict__ small, uint32_t ns, int64_t q_base, int64_t g_base,
-                           const double* __restrict__ q, const double* __restrict__ g, double* __restrict__ out);
+                           const double* __restrict__ q, const double* __restrict__ g,
+                           const double* __restrict__ face_phi, double* __restrict__ out);
 
 // Per face: its mesh (bisection over the offsets), then the corner adjoints with that mesh's
 // centre and small-|Q| rows.
@@ -1419,8 +1437,15 @@ __global__ void k_bbcorner3(const float* __restrict__ v, int64_t nv, const int32
   const PolyC C = mc[lo];
   const double c[3] = {C.cx, C.cy, C.cz};
   const uint32_t ns = (uint32_t)max(0, min(small_cnt[lo], (int32_t)nqi));
-  corner_adj(m, v, nv, f, nf, partial, ks, c, small + gb, ns, qb, gb, q, g, corner + 9 * m);
+  corner_adj(m, v, nv, f, nf, partial, ks, c, small + gb, ns, qb, gb, q, g, nullptr, corner + 9 * m);
 }
+
+// (-1)^(j/2) / (j + 3)!
+__constant__ double kInvFact3[16] = {
+    1.0 / 6,           1.0 / 24,           -1.0 / 120,           -1.0 / 720,
+    1.0 / 5040,        1.0 / 40320,        -1.0 / 362880,        -1.0 / 3628800,
+    1.0 / 39916800,    1.0 / 479001600,    -1.0 / 6227020800.0,  -1.0 / 87178291200.0,
+    1.0 / 1307674368000.0, 1.0 / 20922789888000.0, -1.0 / 355687428096000.0, -1.0 / 6402373705728000.0};
 
 // 3D: per face, chunk sums of the record adjoints -> corner adjoints (FP64), plus
 // small-|Q| corner terms dF/dp_k = exp(iQ.c) N sum_j i^j h_j(a, a_k)/(j+3)!.
@@ -1430,7 +1455,8 @@ __global__ void k_bbcorner3(const float* __restrict__ v, int64_t nv, const int32
 __device__ void corner_adj(int64_t m, const float* __restrict__ v, int64_t nv, const int32_t* __restrict__ f,
                            int64_t nf, const double* __restrict__ partial, int ks, const double* c,
                            const int32_t* __restrict__ small, uint32_t ns, int64_t q_base, int64_t g_base,
-                           const double* __restrict__ q, const double* __restrict__ g, double* __restrict__ out) {
+                           const double* __restrict__ q, const double* __restrict__ g,
+                           const double* __restrict__ face_phi, double* __restrict__ out) {
   const int32_t id[3] = {f[3 * m], f[3 * m + 1], f[3 * m + 2]};
   if (id[0] < 0 || id[1] < 0 || id[2] < 0 || id[0] >= nv || id[1] >= nv || id[2] >= nv) {
     for (int k = 0; k < 9; ++k) out[k] = 0.0;
@@ -1464,34 +1490,47 @@ __device__ void corner_adj(int64_t m, const float* __restrict__ v, int64_t nv, c
   }
   if (ns) {
     const double N[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2], e1[0] * e2[1] - e1[1] * e2[0]};
+    double cf[3] = {0, 0, 0};   // sum over the listed Q of Re(conj(g) * H_k)
+    if (face_phi != nullptr && ns > (uint32_t)kSmallAdjoint) {
+      for (int k = 0; k < 3; ++k) cf[k] = face_phi[3 * m + k];
+      ns = 0;
+    }
     for (uint32_t e = 0; e < ns; ++e) {
       const int64_t iq = q_base + small[e], ig = g_base + small[e];
       const double Q[3] = {q[3 * iq], q[3 * iq + 1], q[3 * iq + 2]};
       const double al[3] = {Q[0] * P[0][0] + Q[1] * P[0][1] + Q[2] * P[0][2],
                             Q[0] * P[1][0] + Q[1] * P[1][1] + Q[2] * P[1][2],
                             Q[0] * P[2][0] + Q[1] * P[2][1] + Q[2] * P[2][2]};
-      const double mu = (al[0] + al[1] + al[2]) / 3.0;
+      const double mu = (al[0] + al[1] + al[2]) * (1.0 / 3.0);
+      // H_k = sum_j i^j h_j(x, x_k) / (j+3)!, x the phases centred at mu (their sum is 0, so
+      // h_j(x) = P h_{j-2} + T h_{j-3}), h_j(x, x_k) = h_j(x) + x_k h_{j-1}(x, x_k).  |x| < 1/3 here; the
+      // terms left out are below 1e-18 of the first.
+      const double x[3] = {al[0] - mu, al[1] - mu, al[2] - mu};
+      const double Pq = fma(x[0], x[0] + x[1], x[1] * x[1]), T = x[0] * x[1] * x[2];
+      const double big = fmax(fabs(x[0]), fmax(fabs(x[1]), fabs(x[2])));
+      const int top = big == 0.0 ? 0 : (big < 1e-3 ? 5 : (big < 1e-2 ? 7 : (big < 6e-2 ? 9 : 15)));
+      double h0 = 1.0, h1 = 0.0, h2 = 0.0;   // h_j, h_{j-1}, h_{j-2}
+      double hh[3] = {1.0, 1.0, 1.0}, sr[3], si[3] = {0, 0, 0};
+      for (int k = 0; k < 3; ++k) sr[k] = kInvFact3[0];
+      for (int j = 1; j <= top; ++j) {
+        const double hn = fma(Pq, h1, T * h2), w = kInvFact3[j];
+        h2 = h1;
+        h1 = h0;
+        h0 = hn;
+        for (int k = 0; k < 3; ++k) {
+          hh[k] = fma(x[k], hh[k], hn);
+          if (j & 1) si[k] = fma(w, hh[k], si[k]);
+          else sr[k] = fma(w, hh[k], sr[k]);
+        }
+      }
       double se, ce;
       sincos(mu + Q[0] * c[0] + Q[1] * c[1] + Q[2] * c[2], &se, &ce);
-      for (int k = 0; k < 3; ++k) {
-        // sum_j i^j h_j(x) / (j+3)!, x = (a0, a1, a2, a_k) centred at mu, 18 terms
-        const double x[4] = {al[0] - mu, al[1] - mu, al[2] - mu, al[k] - mu};
-        double hh[19];
-        hh[0] = 1.0;
-        for (int j = 1; j <= 18; ++j) hh[j] = 0.0;
-        for (int t = 0; t < 4; ++t)
-          for (int j = 1; j <= 18; ++j) hh[j] = fma(x[t], hh[j - 1], hh[j]);
-        double sr = 0.0, si = 0.0, inv = 1.0 / 6.0;
-        for (int j = 0; j <= 18; ++j) {
-          const double t = hh[j] * inv;
-          switch (j & 3) { case 0: sr += t; break; case 1: si += t; break; case 2: sr -= t; break; default: si -= t; }
-          inv /= (double)(j + 4);
-        }
-        const double hr = ce * sr - se * si, hi = ce * si + se * sr;
-        const double cf = g[2 * ig] * hr + g[2 * ig + 1] * hi;   // Re(conj(g) * H)
-        for (int d = 0; d < 3; ++d) pb[k][d] += cf * N[d];
-      }
+      // conj(g) e^{i(mu + Q.c)} = wr + i wi
+      const double gr = g[2 * ig], gi = g[2 * ig + 1], wr = gr * ce + gi * se, wi = gr * se - gi * ce;
+      for (int k = 0; k < 3; ++k) cf[k] += wr * sr[k] - wi * si[k];
     }
+    for (int k = 0; k < 3; ++k)
+      for (int d = 0; d < 3; ++d) pb[k][d] = fma(cf[k], N[d], pb[k][d]);
   }
   for (int k = 0; k < 3; ++k)
     for (int d = 0; d < 3; ++d) out[3 * k + d] = pb[k][d];
@@ -1500,11 +1539,12 @@ __device__ void corner_adj(int64_t m, const float* __restrict__ v, int64_t nv, c
 __global__ void k_bcorner3d(const float* __restrict__ v, int64_t nv, const int32_t* __restrict__ f, int64_t nf,
                             const double* __restrict__ partial, int ks, const WsHeader* h,
                             const int32_t* __restrict__ small, const double* __restrict__ q,
-                            const double* __restrict__ g, double* __restrict__ corner) {
+                            const double* __restrict__ g, const double* __restrict__ face_phi,
+                            double* __restrict__ corner) {
   const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (m >= nf) return;
   const double c[3] = {h->center[0], h->center[1], h->center[2]};
-  corner_adj(m, v, nv, f, nf, partial, ks, c, small, h->small_q_count, 0, 0, q, g, corner + 9 * m);
+  corner_adj(m, v, nv, f, nf, partial, ks, c, small, h->small_q_count, 0, 0, q, g, face_phi, corner + 9 * m);
 }
 
 // Vertex -> face-corner CSR: degrees, exclusive scan, fill, per-vertex sort.
@@ -1627,7 +1667,7 @@ int more_chunks(int k, int64_t q_blocks, int64_t slots, int64_t tiles) {
 }
 
 struct BwdLayout {
-  size_t mparts, items, qrec, small, partial, corner, deg, cursor, start, btot, list, total;
+  size_t mparts, items, qrec, small, partial, corner, deg, cursor, start, btot, list, phi, total;
   int nblk, ks;
   int64_t per_split;
 };
@@ -1653,6 +1693,7 @@ BwdLayout bwd_layout(int dim, int64_t n_verts, int64_t n_items, int64_t n_prep, 
     y.start = o;  o = al(o + sizeof(int64_t) * (size_t)std::max<int64_t>(n_verts, 1));
     y.btot = o;   o = al(o + sizeof(int64_t) * (size_t)blocks(n_verts, kAux));
     y.list = o;   o = al(o + sizeof(int32_t) * 3 * (size_t)std::max<int64_t>(n_items, 1));
+    y.phi = o;    o = al(o + small_adjoint_bytes(n_items));
   }
   y.total = o;
   return y;
@@ -1661,7 +1702,7 @@ BwdLayout bwd_layout(int dim, int64_t n_verts, int64_t n_items, int64_t n_prep, 
 // Q-gradient workspace: header, volume partials (written by the prep kernel), face
 // records, Q records, small-|Q| list, kQG FP64 partials per (face chunk, Q).
 struct QgLayout {
-  size_t mparts, items, qrec, small, partial, spart, qperm, qscratch, total;
+  size_t mparts, items, qrec, small, partial, spart, mom, qperm, qscratch, total;
   bool tiled;   // the pair kernel visits the Q points in the library's order (q_order option)
   int nblk, ks;
   int64_t per_split, slots;
@@ -1706,6 +1747,7 @@ QgLayout qg_layout(int64_t n_faces, int64_t n_q, bool tiled) {
   y.partial = o; o = al(o + sizeof(double) * kQG * (size_t)y.ks * (size_t)std::max<int64_t>(n_q, 1));
   y.slots = std::max<int64_t>(kQsUnits, n_q);
   y.spart = o;   o = al(o + sizeof(double) * kQsF * (size_t)y.slots);
+  y.mom = o;     o = al(o + small3_bytes(n_faces, sm_count()));
   qg_order_regions(y, o, n_q, n_faces, tiled);
   y.total = o;
   return y;
@@ -1894,9 +1936,14 @@ int mesh3d_backward_body(const float* verts, int64_t n_verts, const int32_t* fac
                                         at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
-  k_bcorner3d<<<blocks(n_faces, kAux), kAux, 0, st>>>(verts, n_verts, faces, n_faces, at<double>(ws, y.partial),
-                                                      y.ks, h, at<int32_t>(ws, y.small), q, grad_out,
-                                                      at<double>(ws, y.corner));
+  if (launch_small_adjoint3(verts, n_verts, faces, n_faces, q, grad_out, n_q, h, at<void>(ws, y.phi), st) !=
+      cudaSuccess)
+    return PFT_ERR_CUDA;
+  g_bwd_launches += 2;
+  const int nt = n_faces >= 65536 ? kAux : 64;   // few faces: smaller blocks, so that all SMs take part
+  k_bcorner3d<<<blocks(n_faces, nt), nt, 0, st>>>(verts, n_verts, faces, n_faces, at<double>(ws, y.partial), y.ks, h,
+                                                  at<int32_t>(ws, y.small), q, grad_out,
+                                                  small_adjoint_faces(at<void>(ws, y.phi)), at<double>(ws, y.corner));
   PFT_BWD_LAUNCH();
   int32_t* deg = at<int32_t>(ws, y.deg);
   int32_t* cursor = at<int32_t>(ws, y.cursor);
@@ -2096,8 +2143,11 @@ int pft3d_mesh_qgrad(const float* verts, int64_t n_verts, const int32_t* faces, 
                                                              at<int32_t>(ws, y.small), y.slots,
                                                              at<double>(ws, y.spart));
   PFT_BWD_LAUNCH();
-  k_qsmall_fin<<<blocks(n_q, kAux), kAux, 0, st>>>(n_faces, q, grad_out, h, at<int32_t>(ws, y.small), y.slots,
-                                                   at<double>(ws, y.spart), grad_q);
+  if (launch_small3(verts, n_verts, faces, n_faces, nullptr, h, nullptr, 0, at<void>(ws, y.mom), st) != cudaSuccess)
+    return PFT_ERR_CUDA;
+  ++g_bwd_launches;
+  k_qsmall_fin<<<blocks(n_q, 32), 32, 0, st>>>(n_faces, q, grad_out, h, at<int32_t>(ws, y.small), y.slots,
+                                               at<double>(ws, y.spart), at<double>(ws, y.mom), grad_q);
   PFT_BWD_LAUNCH();
   return PFT_OK;
 }

@@ -120,8 +120,33 @@ __device__ __forceinline__ void mom_eval(const double* m, double x, double y, do
 // Bytes by which the scratch exceeds the records of a pft3d_mesh call (part of its workspace size).
 size_t small3_growth(int64_t n_faces, int64_t n_q, const pft_options* opts);
 
-// pft_small.cu
+// pft_small.cu.  q = NULL: only the moments (nothing for h->small_q_count <= kSmallDirect).
 cudaError_t launch_small3(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q, WsHeader* h,
                           const double* mparts, int n_measure, void* scratch, cudaStream_t st);
+
+// The vertex adjoint.  The small-|Q| points' share of dL/dv is the shape derivative of the integral of
+// Phi(r) = Re sum_Q conj(g_Q) e^{iQ.r}, for corner k of a face N times the face average of lambda_k Phi.
+// With few points each is evaluated in turn (corner_adj); with more than kSmallAdjoint of them Phi is
+// summed once into a polynomial in r - c (degree <= 12: the terms past it are below 1e-17), and every
+// face integrates that by Gauss quadrature of the order its size needs.
+constexpr int kSmallAdjoint = 24;
+constexpr int kPhiLo = 8;                  // degrees 0 .. 8 in FP64; 9 .. 12, below 1.1e-11, in FP32
+constexpr int kPhiBlocks = 64;             // blocks that sum Phi's coefficients
+struct PhiPoly {
+  double c64[mom_count(kPhiLo)];
+  float c32[kMomN - mom_count(kPhiLo)];    // in units of scale
+  double scale;                            // the largest coefficient (0: Phi vanishes)
+};
+constexpr size_t kPhiHead = 4096;
+static_assert(sizeof(PhiPoly) <= kPhiHead, "Phi's coefficients");
+inline size_t small_adjoint_bytes(int64_t nf) {
+  return kPhiHead + sizeof(double) * (kMomN * (size_t)kPhiBlocks + 3 * (size_t)std::max<int64_t>(nf, 1));
+}
+inline const double* small_adjoint_faces(const void* scratch) {   // [nf][3]: face averages of lambda_k Phi
+  return reinterpret_cast<const double*>(static_cast<const char*>(scratch) + kPhiHead) + kMomN * (size_t)kPhiBlocks;
+}
+// Two launches; they do nothing for h->small_q_count <= kSmallAdjoint.
+cudaError_t launch_small_adjoint3(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q,
+                                  const double* g, int64_t n_q, WsHeader* h, void* scratch, cudaStream_t st);
 
 }  // namespace pft

@@ -64,3 +64,31 @@ def test_small_q_against_the_oracle(torch_dev, n_small, level, keep, shift, scal
         assert np.abs(got - ref)[small].max() <= 1e-12 * scale_f
         if keep is None:
             assert np.abs(got - ref).max() <= (1e-5 if precision == "fp32" else 1e-12) * scale_f
+
+
+@pytest.mark.parametrize("n_small", [1, 24, 25, 33, 400])
+@pytest.mark.parametrize("level,shift,scale", [(0, 0.0, 1.0), (2, 2.0, 1e5), (4, 0.5, 1e-5)])
+def test_small_q_gradients_against_the_oracle(torch_dev, n_small, level, shift, scale):
+    """Vertex gradient (up to 24 small points one by one, more through the polynomial of their sum) and
+    Q-gradient (up to 32 one by one, more through the moments), small points only.  The vertex gradient
+    is rounded to float32 once: 6e-8 of a value, held to 2e-7 of the largest; the Q-gradient to 1e-9
+    of max|g| V max|r|."""
+    torch, dev = torch_dev
+    import paper_2104_08309_gb300 as pft
+    v, f = synth.perturbed_icosphere(level, seed=4)
+    v = ((v + np.float32(shift)) * np.float32(scale)).astype(np.float32)
+    c = 0.5 * (v.min(0).astype(np.float64) + v.max(0))
+    radius = np.linalg.norm(v - c, axis=1).max()
+    rng = np.random.default_rng(n_small)
+    d = rng.normal(size=(n_small, 3))
+    q = d / np.linalg.norm(d, axis=1, keepdims=True) * (10 ** rng.uniform(-3, np.log10(0.2499), (n_small, 1))) / radius
+    q[0] = 0.0
+    g = rng.normal(size=(n_small, 2))
+    vd, fd, qd, gd = (torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (v, f, q, g))
+    got = pft.pft3d_mesh_backward(vd, fd, qd, gd, check_status=True).cpu().numpy().astype(np.float64)
+    ref = oracle.grad3d(v, f, q, g[:, 0] + 1j * g[:, 1])
+    assert np.abs(got - ref).max() <= 2e-7 * np.abs(ref).max()
+    got = pft.pft3d_mesh_qgrad(vd, fd, qd, gd, check_status=True).cpu().numpy()
+    ref = oracle.qgrad3d(v, f, q, g[:, 0] + 1j * g[:, 1])
+    bar = np.abs(g).max() * abs(oracle.ft3d(v, f, np.zeros((1, 3)))[0]) * np.abs(v).max()
+    assert np.abs(got - ref).max() <= 1e-9 * bar
