@@ -63,7 +63,8 @@ int device_sms() {
 // waves (the last wave >= 97 % as full as the others), each chunk at least two
 // tiles long; then, for launches of fewer than 40 waves with chunks to spare,
 // more chunks (below).
-FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q) {
+// fine: more chunks than that where it pays (see layout_fwd for when it is not asked for).
+FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, bool fine) {
   FwdLaunch L{};
   L.r = o.r;
   L.nt = o.nt;
@@ -99,6 +100,18 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q) {
         if (waves >= 40.0) break;
       }
     }
+    // FP64: a launch of two waves left the SMs' FP64 pipes idle for a quarter of it (5,120 faces x
+    // 13,824 Q: 14 chunks, 1.99 waves, 15.4 ms; 60 chunks, 8.5 waves, 13.4 ms), so chunks down to two
+    // tiles, up to 10 waves.
+    if (fine && o.fp64 && (double)(L.q_tiles * k) / (double)slots < 10.0) {
+      const int kf = (int)std::min<int64_t>(64, item_tiles / 2);
+      for (int c = k + 1; c <= kf; ++c) {
+        const double waves = (double)(L.q_tiles * c) / (double)slots;
+        if (waves < 1.0 || waves / std::ceil(waves) < 0.85) continue;
+        k = c;
+        if (waves >= 10.0) break;
+      }
+    }
   }
   k = (int)std::min<int64_t>(k, item_tiles);
   const int64_t tiles_per = (item_tiles + k - 1) / k;
@@ -115,9 +128,9 @@ struct FwdLayout {
   FwdLaunch L;
 };
 
-FwdLayout layout_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_prep, int64_t n_q) {
+FwdLayout layout_plan(int dim, const Opts& o, int64_t n_items, int64_t n_prep, int64_t n_q, bool fine) {
   FwdLayout y{};
-  y.L = plan_fwd(dim, o, n_items, n_q);
+  y.L = plan_fwd(dim, o, n_items, n_q, fine);
   y.nblk = std::max(1, prep_blocks(n_prep));
   const size_t item_bytes = dim == 2 ? (o.fp64 ? sizeof(Seg64) : sizeof(Seg32)) : (o.fp64 ? sizeof(Face64) : sizeof(Face32));
   size_t off = align_up(sizeof(WsHeader));
@@ -139,6 +152,14 @@ FwdLayout layout_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_prep, in
   return y;
 }
 
+// A finer plan's partial sums must not push a problem out of the allocation-free call's scratch: one
+// that fits it with the coarser plan keeps that.
+FwdLayout layout_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_prep, int64_t n_q) {
+  const FwdLayout y = layout_plan(dim, o, n_items, n_prep, n_q, true);
+  if (y.total - y.grown <= kScratchLimit) return y;
+  const FwdLayout z = layout_plan(dim, o, n_items, n_prep, n_q, false);
+  return z.total - z.grown <= kScratchLimit ? z : y;
+}
 
 template <typename T>
 T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws) + off); }

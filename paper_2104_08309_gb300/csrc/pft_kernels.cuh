@@ -69,6 +69,9 @@ __device__ __forceinline__ void simplex_series(const double* x, double& re, doub
   }
 }
 
+// Largest workspace, without what the small-|Q| pass adds to it, that pft3d_mesh_noalloc takes.
+constexpr size_t kScratchLimit = size_t(32) << 20;   // 32 MiB
+
 // Launch description computed on the host.
 struct FwdLaunch {
   int r;              // Q points per thread

@@ -28,10 +28,9 @@
 namespace pft {
 namespace {
 
-// The limit on a problem's workspace, without what the small-|Q| pass adds to it (at most 0.6 MiB,
-// for which the array has room).
-constexpr size_t kScratchLimit = size_t(32) << 20;   // 32 MiB
-constexpr size_t kScratchBytes = size_t(33) << 20;   // 33 MiB per device
+// 33 MiB per device: the limit on a problem's workspace without what the small-|Q| pass adds to it,
+// and room for that (at most 0.6 MiB).
+constexpr size_t kScratchBytes = kScratchLimit + (size_t(1) << 20);
 constexpr int kMaxDevices = 64;
 
 // The scratch array.  In host code this name is only a stand-in for the device

@@ -5,7 +5,7 @@
 
 #include <type_traits>
 
-#include "pft_kernels.cuh"
+#include "pft_f64.cuh"
 
 namespace pft {
 
@@ -43,29 +43,6 @@ constexpr int kMinBlocks = sizeof(typename Pol::QT) == 8 ? 1
 // Records hold m and D/2, so w below is half the cross product; the factor 2
 // and 1/|Q|^2 are applied in FP64 by the finalize kernel.  The term itself is
 // evaluated in Pol2F32::tile (the sinc of |Q.D/2| > pi is a warp-uniform branch).
-
-__device__ __forceinline__ double sinc_f64(double u) {
-  const double u2 = u * u;
-  if (u2 < 1e-2) {   // Taylor through u^10: truncation < 1e-18 at |u| = 0.1
-    double p = fma(u2, -1.0 / 39916800.0, 1.0 / 362880.0);
-    p = fma(u2, p, -1.0 / 5040.0);
-    p = fma(u2, p, 1.0 / 120.0);
-    p = fma(u2, p, -1.0 / 6.0);
-    return fma(u2, p, 1.0);
-  }
-  return sin(u) / u;
-}
-
-__device__ __forceinline__ void seg_pair_f64(double qx, double qy, const Seg64& s, double& re, double& im) {
-  const double ph = fma(qx, s.mx, qy * s.my);
-  const double u = fma(qx, s.hx, qy * s.hy);
-  const double w = fma(qx, s.hy, -qy * s.hx);
-  double sn, cs;
-  sincos(ph, &sn, &cs);
-  const double ws = w * sinc_f64(u);
-  re = ws * sn;
-  im = -ws * cs;
-}
 
 // 3D, Eq. 14 with the sign fixed (Sec. 3).  With X = N x Q, s = Q.N and the
 // corner phases a_k = Q.(p_k - centroid) (a_0 + a_1 + a_2 = 0), a face gives
@@ -323,61 +300,6 @@ __device__ __forceinline__ void face_finish(V mu, V s, V zr, V zi, V& tre, V& ti
   tim = vfma(c, zi, vfma(d, zr, tim));
 }
 
-// Same face term in FP64 (comparison path): library sincos, series through k = 16.
-__device__ __forceinline__ void face_pair_f64(double qx, double qy, double qz, const Face64& f, double p_hi, double p_lo,
-                                              double& re, double& im) {
-  const double mu = fma(qx, f.gx, fma(qy, f.gy, qz * f.gz));
-  const double a0 = fma(qx, f.q0x, fma(qy, f.q0y, qz * f.q0z));
-  const double a1 = fma(qx, f.q1x, fma(qy, f.q1y, qz * f.q1z));
-  const double s = fma(qx, f.nx, fma(qy, f.ny, qz * f.nz));
-  const double a2 = -(a0 + a1);
-  const double P = fma(a0, a0 + a1, a1 * a1);
-  double zr, zi;
-  const bool series = __all_sync(0xffffffffu, P < p_hi) || (P < p_lo);
-  if (series) {
-    const double T = a0 * a1 * a2;
-    constexpr int K = 16;
-    double h[K + 1];
-    h[0] = 1.0; h[1] = 0.0; h[2] = P;
-#pragma unroll
-    for (int k = 3; k <= K; ++k) h[k] = fma(P, h[k - 2], T * h[k - 3]);
-    double gre = 0.0, gim = 0.0, inv = 0.5;   // 1/(k+2)!
-#pragma unroll
-    for (int k = 0; k <= K; ++k) {
-      const double t = h[k] * inv;
-      switch (k & 3) { case 0: gre += t; break; case 1: gim += t; break; case 2: gre -= t; break; default: gim -= t; }
-      inv /= (double)(k + 3);
-    }
-    zr = -gim;
-    zi = gre;
-  } else {
-    const double Xx = fma(f.ny, qz, -f.nz * qy), Xy = fma(f.nz, qx, -f.nx * qz), Xz = fma(f.nx, qy, -f.ny * qx);
-    const double x2 = fma(Xx, Xx, fma(Xy, Xy, Xz * Xz));
-    const double b0 = fma(f.q0x, Xx, fma(f.q0y, Xy, f.q0z * Xz));
-    const double b1 = fma(f.q1x, Xx, fma(f.q1y, Xy, f.q1z * Xz));
-    const double b2 = -(b0 + b1);
-    const double w[3] = {b1 - b0, b2 - b1, b0 - b2};
-    const double psi[3] = {-0.5 * a2, -0.5 * a0, -0.5 * a1};
-    const double u[3] = {0.5 * (a1 - a0), 0.5 * (a2 - a1), 0.5 * (a0 - a2)};
-    double sr = 0.0, si = 0.0;
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      double sp, cp;
-      sincos(psi[l], &sp, &cp);
-      const double ws = w[l] * sinc_f64(u[l]);
-      sr = fma(ws, cp, sr);
-      si = fma(ws, sp, si);
-    }
-    const double inv = (x2 > 0.0) ? 1.0 / x2 : 0.0;
-    zr = sr * inv;
-    zi = si * inv;
-  }
-  double sm, cm;
-  sincos(mu, &sm, &cm);
-  re = -s * fma(cm, zr, -sm * zi);
-  im = -s * fma(cm, zi, sm * zr);
-}
-
 // ---------------------------------------------------------------------------
 // Policies: record type, Q registers, accumulators and the per-tile loop.
 // ---------------------------------------------------------------------------
@@ -487,10 +409,7 @@ struct Pol2F64 {
       const Seg64 s = t[i];
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        double re, im;
-        seg_pair_f64(q[r][0], q[r][1], s, re, im);
-        acc.re[r] += re;
-        acc.im[r] += im;
+        seg_pair64(q[r][0], q[r][1], s, acc.re[r], acc.im[r]);
       }
     }
   }
@@ -625,10 +544,7 @@ struct Pol3F64 {
       const Face64 f = t[i];
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        double re, im;
-        face_pair_f64(q[r][0], q[r][1], q[r][2], f, (double)th.hi, (double)th.lo, re, im);
-        acc.re[r] += re;
-        acc.im[r] += im;
+        face_pair64(q[r][0], q[r][1], q[r][2], f, (double)th.hi, (double)th.lo, acc.re[r], acc.im[r]);
       }
     }
   }
