@@ -564,6 +564,7 @@ __global__ void k_qfinal(const double* __restrict__ q, const double* __restrict_
   const double q2 = q_norm2(Q[0], Q[1], Q[2]);
   if (q2 == 0.0 || small_q(q2, __uint_as_float(h->rmax_bits))) return;   // k_qsmall's (same test as k_bq)
   double v[kQG] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
   for (int k = 0; k < ks; ++k)
     for (int f = 0; f < kQG; ++f) v[f] += partial[((int64_t)k * n_q + i) * kQG + f];
   const double c[3] = {h->center[0], h->center[1], h->center[2]};
@@ -657,12 +658,14 @@ __global__ void __launch_bounds__(kAux) k_qsmall_part(const float* __restrict__ 
 
 // With more than kSmallDirect listed points, S0 and dS0/dQ are the polynomial of the shape's moments
 // (pft_small.cuh) and its gradient.
+// One warp per listed point (lane 0 finishes it).
 __global__ void k_qsmall_fin(int64_t nf, const double* __restrict__ q, const double* __restrict__ g,
                              const WsHeader* h, const int32_t* list, int64_t slots, const double* __restrict__ part,
                              const double* __restrict__ moments, double* __restrict__ out) {
   __shared__ double mom[kMomN];
   const uint32_t count = h->small_q_count;
-  if (blockIdx.x * (int64_t)blockDim.x >= count) return;
+  const int64_t per = blockDim.x / 32;
+  if (blockIdx.x * per >= count) return;
   const bool direct = count <= (uint32_t)kSmallDirect;
   if (!direct) {
     for (int t = threadIdx.x; t < kMomN; t += blockDim.x) mom[t] = moments[t];
@@ -670,15 +673,12 @@ __global__ void k_qsmall_fin(int64_t nf, const double* __restrict__ q, const dou
   }
   const int64_t nch = qsmall_chunks(count, nf, slots);
   const double c[3] = {h->center[0], h->center[1], h->center[2]}, rmax = (double)__uint_as_float(h->rmax_bits);
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t e = blockIdx.x * per + threadIdx.x / 32; e < count; e += gridDim.x * per) {   // uniform over a warp
     const int64_t i = list[e];
     double Q[3];
     for (int d = 0; d < 3; ++d) Q[d] = q[3 * i + d];
     double acc[kQsF] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (direct) {
-      for (int64_t ch = 0; ch < nch; ++ch)
-        for (int k = 0; k < kQsF; ++k) acc[k] += part[(e * nch + ch) * kQsF + k];
-    } else {
+    if (!direct) {
       double gr3[3][2];
       mom_eval<true>(mom, Q[0] * rmax, Q[1] * rmax, Q[2] * rmax, acc[0], acc[1], gr3);
       for (int d = 0; d < 3; ++d) {
@@ -686,6 +686,10 @@ __global__ void k_qsmall_fin(int64_t nf, const double* __restrict__ q, const dou
         acc[3 + 2 * d] = rmax * gr3[d][1];
       }
     }
+    if (threadIdx.x & 31) continue;
+    if (direct)
+      for (int64_t ch = 0; ch < nch; ++ch)
+        for (int k = 0; k < kQsF; ++k) acc[k] += part[(e * nch + ch) * kQsF + k];
     double sp, cp;
     sincos(Q[0] * c[0] + Q[1] * c[1] + Q[2] * c[2], &sp, &cp);
     const double gr = g[2 * i], gi = g[2 * i + 1];
@@ -2137,7 +2141,8 @@ int pft3d_mesh_qgrad(const float* verts, int64_t n_verts, const int32_t* faces, 
                                    at<double>(ws, y.partial), &h->status, perm);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
-  k_qfinal<<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, at<double>(ws, y.partial), y.ks, h, grad_q);
+  const int nt = n_q >= 65536 ? kAux : 32;
+  k_qfinal<<<blocks(n_q, nt), nt, 0, st>>>(q, grad_out, n_q, at<double>(ws, y.partial), y.ks, h, grad_q);
   PFT_BWD_LAUNCH();
   k_qsmall_part<<<(unsigned)(4 * sm_count()), kAux, 0, st>>>(verts, n_verts, faces, n_faces, q, h,
                                                              at<int32_t>(ws, y.small), y.slots,
@@ -2146,7 +2151,7 @@ int pft3d_mesh_qgrad(const float* verts, int64_t n_verts, const int32_t* faces, 
   if (launch_small3(verts, n_verts, faces, n_faces, nullptr, h, nullptr, 0, at<void>(ws, y.mom), st) != cudaSuccess)
     return PFT_ERR_CUDA;
   ++g_bwd_launches;
-  k_qsmall_fin<<<blocks(n_q, 32), 32, 0, st>>>(n_faces, q, grad_out, h, at<int32_t>(ws, y.small), y.slots,
+  k_qsmall_fin<<<std::min(blocks(n_q, 2), 4096u), 64, 0, st>>>(n_faces, q, grad_out, h, at<int32_t>(ws, y.small), y.slots,
                                                at<double>(ws, y.spart), at<double>(ws, y.mom), grad_q);
   PFT_BWD_LAUNCH();
   return PFT_OK;

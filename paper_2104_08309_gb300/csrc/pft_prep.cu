@@ -268,6 +268,7 @@ __device__ __forceinline__ void split_sum(const double2* __restrict__ partial, i
                                           double k, double& re, double& im) {
   re = 0.0;
   im = 0.0;
+#pragma unroll 8
   for (int s = 0; s < ks; ++s) {
     const double2 p = partial[(int64_t)s * n_q + i];
     re += p.x;
@@ -300,47 +301,72 @@ __global__ void k_finalize2d(const double* __restrict__ q, int64_t n_q, const do
   finish(Q, re, im, h, out + 2 * i);
 }
 
-// 3D: small-|Q| points (as k_fwd listed them) take their sum from k_small3's results.
-__global__ void k_finalize3d(const double* __restrict__ q, int64_t n_q, int64_t nf,
-                             const double2* __restrict__ partial, int ks, const WsHeader* __restrict__ h,
-                             const int32_t* __restrict__ small, const char* __restrict__ scratch,
-                             double* __restrict__ out) {
+// 3D: small-|Q| points (as k_fwd listed them) take their sum from k_small3's results.  A block finishes
+// per_block <= 256 points, one per thread; those that need the moments' polynomial are dealt to its warps.
+constexpr int kFinT = 256;
+__global__ void __launch_bounds__(kFinT) k_finalize3d(const double* __restrict__ q, int64_t n_q, int64_t nf,
+                                                      const double2* __restrict__ partial, int ks,
+                                                      const WsHeader* __restrict__ h,
+                                                      const int32_t* __restrict__ small,
+                                                      const char* __restrict__ scratch, double* __restrict__ out,
+                                                      int per_block) {
   __shared__ double mom[kMomN];
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  __shared__ double at[kFinT][3];   // a point's scaled Q, then its result
+  __shared__ int list[kFinT];
+  __shared__ int n_list;
+  const int t = threadIdx.x;
+  const int64_t i = blockIdx.x * (int64_t)per_block + t;
+  const bool mine = t < per_block && i < n_q;
   const float rmax = __uint_as_float(h->rmax_bits);
+  const bool direct = h->small_q_count <= (uint32_t)kSmallDirect;
   double Q[3] = {0.0, 0.0, 0.0}, q2 = 0.0;
   bool is_small = false;
-  if (i < n_q) {
+  if (mine) {
     for (int d = 0; d < 3; ++d) Q[d] = q[3 * i + d];
     q2 = q_norm2(Q[0], Q[1], Q[2]);
     is_small = q2 != 0.0 && small_q(q2, rmax);
   }
-  const bool direct = h->small_q_count <= (uint32_t)kSmallDirect;
-  if (__syncthreads_or(is_small && !direct)) {
-    for (int t = threadIdx.x; t < kMomN; t += blockDim.x) mom[t] = reinterpret_cast<const double*>(scratch)[t];
-    __syncthreads();
+  if (!direct) {   // uniform
+    if (t == 0) n_list = 0;
+    if (__syncthreads_or(is_small)) {
+      if (is_small) {
+        for (int d = 0; d < 3; ++d) at[t][d] = Q[d] * (double)rmax;
+        list[atomicAdd(&n_list, 1)] = t;   // their order is immaterial
+      }
+      for (int j = t; j < kMomN; j += kFinT) mom[j] = reinterpret_cast<const double*>(scratch)[j];
+      __syncthreads();
+      for (int e = t >> 5; e < n_list; e += kFinT / 32) {
+        const int l = list[e];
+        double re, im, g[3][2];
+        mom_eval<false>(mom, at[l][0], at[l][1], at[l][2], re, im, g);
+        __syncwarp();
+        if ((t & 31) == 0) {
+          at[l][0] = re;
+          at[l][1] = im;
+        }
+      }
+      __syncthreads();
+    }
   }
-  if (i >= n_q) return;
+  if (!mine) return;
   if (q2 == 0.0) {
     out[2 * i] = h->measure;
     out[2 * i + 1] = 0.0;
     return;
   }
-  double re, im;
+  double re = 0.0, im = 0.0;
   if (!is_small) {
     split_sum(partial, ks, n_q, i, 1.0 / q2, re, im);
   } else if (direct) {
     const int64_t nch = small3_chunks(nf);
     const double* p = reinterpret_cast<const double*>(scratch + kMomHead) + 2 * nch * small[i];
-    re = 0.0;
-    im = 0.0;
-    for (int64_t t = 0; t < nch; ++t) {
-      re += p[2 * t];
-      im += p[2 * t + 1];
+    for (int64_t c = 0; c < nch; ++c) {
+      re += p[2 * c];
+      im += p[2 * c + 1];
     }
   } else {
-    double g[3][2];
-    mom_eval<false>(mom, Q[0] * (double)rmax, Q[1] * (double)rmax, Q[2] * (double)rmax, re, im, g);
+    re = at[t][0];
+    im = at[t][1];
   }
   finish(Q, re, im, h, out + 2 * i);
 }
@@ -430,13 +456,17 @@ cudaError_t launch_fan3d(const int32_t* idx, int64_t n_idx, const int64_t* off, 
   return cudaGetLastError();
 }
 
-// Block size of the finishing kernels: small enough that a small call's FP64 arithmetic (the phase's
+// Points per block of the finishing kernels: few enough that a small call's FP64 arithmetic (the phase's
 // sincos, the small-|Q| polynomial) spreads over all SMs.
-static int finish_threads(int64_t n_q) { return n_q >= 131072 ? 256 : (n_q >= 32768 ? 128 : (n_q >= 8192 ? 64 : 32)); }
+static int finish_points(int64_t n_q) {
+  int n = 256;
+  while (n > 8 && n_q < (int64_t)n * 512) n /= 2;
+  return n;
+}
 
 cudaError_t launch_finalize2d(const double* q, int64_t n_q, const double2* partial, int k_splits, WsHeader* h,
                               const double* mparts, int nm, int32_t* small_list, double* out, cudaStream_t st) {
-  const int nt = finish_threads(n_q);
+  const int nt = std::max(32, finish_points(n_q));
   k_finalize2d<<<(unsigned)((n_q + nt - 1) / nt), nt, 0, st>>>(q, n_q, partial, k_splits, h, mparts, nm, small_list,
                                                               out);
   return cudaGetLastError();
@@ -445,9 +475,9 @@ cudaError_t launch_finalize2d(const double* q, int64_t n_q, const double2* parti
 cudaError_t launch_finalize3d(const double* q, int64_t n_q, int64_t nf, const double2* partial, int k_splits,
                               const WsHeader* h, const int32_t* small, const void* scratch, double* out,
                               cudaStream_t st) {
-  const int nt = finish_threads(n_q);
-  k_finalize3d<<<(unsigned)((n_q + nt - 1) / nt), nt, 0, st>>>(q, n_q, nf, partial, k_splits, h, small,
-                                                              static_cast<const char*>(scratch), out);
+  const int per = finish_points(n_q);
+  k_finalize3d<<<(unsigned)((n_q + per - 1) / per), kFinT, 0, st>>>(q, n_q, nf, partial, k_splits, h, small,
+                                                                   static_cast<const char*>(scratch), out, per);
   return cudaGetLastError();
 }
 

@@ -10,9 +10,9 @@
 //    of them) are summed over the faces once, and every small Q point evaluates the polynomial.
 // Line between them: a directly evaluated point costs about 70 FP64 operations a face and the moments
 // about 900 with lanes to spare, so they break even near 30 points (on 20,480 faces 32 points take
-// 75 us at the FP64 rate, the moments 60).  A curve of 2,928 points on
+// 75 us at the FP64 rate, the moments 102).  A curve of 2,928 points on
 // 20,480 faces, 1,220 of them small: the call took 5,267 us with one block per point and 17 terms,
-// 352 us with the moments.
+// 233 us with the moments (k_small3 102 us, the polynomials in k_finalize3d 25 us).
 // Both run in FP64, except that monomials of degree >= 8, which together stay below 1.1e-10 of
 // the result, are summed in compensated FP32 (an error below 2e-17 of it).
 #pragma once
@@ -57,64 +57,82 @@ __device__ __forceinline__ void tetra_series(const double (&x)[3], double& re, d
   simplex_series<3, 3, kMomK>(x, re, im);
 }
 
-// S0(Q) from the moments m (already holding (-1)^(k/2)/(k+3)! and the scale of the coordinates):
-// Horner in x for every y^b z^c, even and odd powers apart (the even degrees are the real part).
-// With GRAD also the derivatives in the scaled Q, g[d] = (re, im).
+// The summed moments' order: by b, then c downwards, then a upwards, so that an evaluation walks them.
+__host__ __device__ constexpr int mom_pos(int a, int b, int c) {
+  int n = 0;
+  for (int j = 0; j < b; ++j) n += (kMomK + 1 - j) * (kMomK + 2 - j) / 2;
+  const int r = kMomK - b - c;
+  return n + r * (r + 1) / 2 + a;
+}
+
+// S0(Q) from the summed moments m (already holding (-1)^(k/2)/(k+3)! and the scale of the coordinates), by
+// one warp (all lanes pass the same scaled Q and get the result): lane 2b + e takes the rows y^b z^c with
+// c of parity e, Horner in x and z^2, the even degrees (the real part) and the odd ones apart.  With GRAD
+// also the derivatives in the scaled Q, g[d] = (re, im).  One thread per point ran one long dependent
+// chain of FP64 operations: 95 us for 1,220 points, 149 us for 190 with GRAD.
 template <bool GRAD>
 __device__ __forceinline__ void mom_eval(const double* m, double x, double y, double z, double& re, double& im,
                                          double (&g)[3][2]) {
-  const double x2 = x * x;
-  double ev = 0.0, od = 0.0;
-  double gx[2] = {0.0, 0.0}, gy[2] = {0.0, 0.0}, gz[2] = {0.0, 0.0};   // [0] even degrees, [1] odd
-  double yp = 1.0;   // y^b over the outer loop, z^c over the inner one
-  double dyp = 0.0;  // b y^(b-1)
-  for (int b = 0; b <= kMomK; ++b) {
-    double w = yp, dwy = dyp, zc1 = 0.0, zp = 1.0;   // y^b z^c, its derivatives
-    for (int c = 0; b + c <= kMomK; ++c) {
-      const int s = b + c, row = s * (s + 1) / 2 + c;
-      // p[0] + x p[1] = sum_a M[a + s] x^a;  d[.] its derivative in x
-      double p0 = 0.0, p1 = 0.0, d0 = 0.0, d1 = 0.0;
-      for (int a = kMomK - s; a >= 0; --a) {
-        const int k = a + s;
-        const double M = m[k * (k + 1) * (k + 2) / 6 + row];
-        if (a & 1) {
-          p1 = fma(p1, x2, M);
-          if (GRAD) d1 = fma(d1, x2, (double)a * M);        // x^(a-1), a - 1 even
-        } else {
-          p0 = fma(p0, x2, M);
-          if (GRAD && a > 0) d0 = fma(d0, x2, (double)a * M);   // x^(a-1), a - 1 odd
+  const int lane = threadIdx.x & 31, b = lane >> 1, par = lane & 1;
+  const double x2 = x * x, z2 = z * z;
+  double v[2] = {0.0, 0.0}, vx[2] = {0.0, 0.0}, vz[2] = {0.0, 0.0};   // [0] even degrees, [1] odd
+  if (b <= kMomK) {
+    const int top = kMomK - b, first = top - ((top ^ par) & 1);   // the largest c of this parity
+    const double* row = m + mom_pos(0, b, top);
+    for (int c = first; c >= 0; c -= 2) {
+      const int n = top - c;                                  // the row's highest power of x
+      const double* w = row + n * (n + 1) / 2;
+      double p0 = 0.0, p1 = 0.0, d0 = 0.0, d1 = 0.0;   // sums over even a of M x^a; odd, less an x; a M x^(a-1)
+#pragma unroll 2
+      for (int a = n & ~1; a >= 0; a -= 2) {
+        const double M = w[a], N = a < n ? w[a + 1] : 0.0;
+        p1 = fma(p1, x2, N);
+        p0 = fma(p0, x2, M);
+        if (GRAD) {
+          d1 = fma(d1, x2, (double)(a + 1) * N);
+          if (a > 0) d0 = fma(d0, x2, (double)a * M);
         }
       }
-      // degree parity of p0 is that of s
-      const double e = (s & 1) ? x * p1 : p0, o = (s & 1) ? p0 : x * p1;
-      ev = fma(w, e, ev);
-      od = fma(w, o, od);
-      if (GRAD) {
-        // derivative in x: a odd -> d1 (even powers), a even -> x d0; they keep their terms' degrees
-        const double dxe = (s & 1) ? d1 : x * d0, dxo = (s & 1) ? x * d0 : d1;
-        gx[0] = fma(w, dxe, gx[0]);
-        gx[1] = fma(w, dxo, gx[1]);
-        const double dwz = yp * zc1;
-        gy[0] = fma(dwy, e, gy[0]);
-        gy[1] = fma(dwy, o, gy[1]);
-        gz[0] = fma(dwz, e, gz[0]);
-        gz[1] = fma(dwz, o, gz[1]);
-        zc1 = fma(zc1, z, zp);          // (c + 1) z^c from c z^(c-1) and z^c
-        zp *= z;
-        dwy = dyp * zp;
-        w = yp * zp;
-      } else {
-        w *= z;
+      const bool odd = (b + c) & 1;   // terms of degree parity e have a of parity e ^ (b + c)
+      p1 *= x;
+      d0 *= x;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const bool q = (e == 1) != odd;
+        if (GRAD) {   // d/dz of sum z^c: Horner in z^2 for c z^(c-1), less a z where c is odd (c = 0: nothing)
+          vz[e] = c > 1 || par ? fma(vz[e], z2, (double)c * (q ? p1 : p0)) : vz[e];
+          vx[e] = fma(vx[e], z2, q ? d1 : d0);
+        }
+        v[e] = fma(v[e], z2, q ? p1 : p0);
       }
     }
-    if (GRAD) dyp = fma(dyp, y, yp);
-    yp *= y;
   }
-  re = ev;
-  im = od;
-  if (GRAD) {
-    for (int t = 0; t < 2; ++t) { g[0][t] = gx[t]; g[1][t] = gy[t]; g[2][t] = gz[t]; }
+  // z^par, y^b and their derivatives; c z^(c-1) = z^(par - 1 + 2j): par odd needs no factor, even one z
+  double yb = 1.0, dy = 0.0;
+  for (int j = 0; j < b; ++j) {
+    dy = fma(dy, y, yb);
+    yb *= y;
   }
+  const double zp = par ? z : 1.0;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    g[0][e] = GRAD ? yb * zp * vx[e] : 0.0;
+    g[1][e] = GRAD ? dy * zp * v[e] : 0.0;
+    g[2][e] = GRAD ? yb * (par ? 1.0 : z) * vz[e] : 0.0;
+    v[e] *= yb * zp;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      v[e] += __shfl_xor_sync(0xffffffffu, v[e], o);
+      if (GRAD)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) g[d][e] += __shfl_xor_sync(0xffffffffu, g[d][e], o);
+    }
+  }
+  re = v[0];
+  im = v[1];
 }
 
 // Bytes by which the scratch exceeds the records of a pft3d_mesh call (part of its workspace size).
@@ -130,7 +148,7 @@ cudaError_t launch_small3(const float* v, int64_t nv, const int32_t* f, int64_t 
 // summed once into a polynomial in r - c (degree <= 12: the terms past it are below 1e-17), and every
 // face integrates that by Gauss quadrature of the order its size needs.
 constexpr int kSmallAdjoint = 24;
-constexpr int kPhiLo = 8;                  // degrees 0 .. 8 in FP64; 9 .. 12, below 1.1e-11, in FP32
+constexpr int kPhiLo = 7;                  // degrees 0 .. 7 in FP64; 8 .. 12, below 4e-10, in FP32
 constexpr int kPhiBlocks = 64;             // blocks that sum Phi's coefficients
 struct PhiPoly {
   double c64[mom_count(kPhiLo)];
