@@ -18,6 +18,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Opts {
   bool fp64;
+  bool shape_given;   // q_per_thread, block_threads or k_splits set by the caller
   int r, nt, k_splits;
   float tau;
   cudaEvent_t ev_start, ev_stop;
@@ -37,6 +38,7 @@ int resolve(const pft_options* o, int dim, Opts& out) {
   if (!r_ok || (out.nt != 128 && out.nt != 256)) return PFT_ERR_UNSUPPORTED;
   if (p.k_splits < 0) return PFT_ERR_INVALID_ARG;
   out.k_splits = p.k_splits;
+  out.shape_given = p.q_per_thread != 0 || p.block_threads != 0 || p.k_splits != 0;
   if (p.tile_items != 0) return PFT_ERR_UNSUPPORTED;
   float tau = p.face_series_tau;
   if (tau == 0.f) tau = 6.0f;
@@ -59,6 +61,12 @@ int device_sms() {
   return sms > 0 ? sms : 1;
 }
 
+// Padded pairs (groups of 128 Q points x tiles of 128 faces) below which a 3D FP32 launch runs
+// k_fwd_group.  Kernel times, k_fwd with up to one tile a chunk against k_fwd_group: 320 faces x 241 Q
+// 67 / 19 us, 5,120 x 520 35 / 17, 5,120 x 2,000 45 / 36, 20,480 x 520 49 / 36; past the line 5,120 x
+// 5,000 59 / 69, 20 x 200,000 30 / 52, 20,480 x 2,928 116 / 137.
+constexpr int64_t kGroupPairs = 24000000;
+
 // Split-K choice: the smallest number of chunks that fills the GPU in whole
 // waves (the last wave >= 97 % as full as the others), each chunk at least two
 // tiles long; then, for launches of fewer than 40 waves with chunks to spare,
@@ -69,13 +77,40 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, bool fi
   L.r = o.r;
   L.nt = o.nt;
   const int tile = fwd_tile(dim, o.fp64);
-  const int64_t q_per_block = (int64_t)o.r * o.nt;
+  if (fine && dim == 3 && !o.fp64 && !o.shape_given && o.face_pairs == 0 && n_items > 0 && n_q > 0) {
+    // k_fwd_group below kGroupPairs (padded) pairs
+    const int64_t tiles = (n_items + tile - 1) / tile, rest = n_q % 512;
+    const int64_t groups = 4 * (n_q / 512) + std::min<int64_t>(4, (rest + 31) / 32);
+    if (groups * 128 * tiles * tile < kGroupPairs && tiles <= 65535) {
+      L.group = true;
+      L.q_tiles = groups;
+      L.k_splits = (int)tiles;
+      L.per_split = tile;
+      return L;
+    }
+  }
+  if (fine && dim == 2 && !o.fp64 && !o.shape_given) {
+    // few Q points: fewer per thread and smaller blocks until the blocks cover the SMs (the sums of a Q
+    // point run over the same segments in the same order in any launch shape).  64 segments x 16,384 Q:
+    // 16 blocks of 256 x 4 took 15.6 us.
+    const int64_t chunks = std::max<int64_t>(1, n_items / (2 * tile));
+    const int shapes[4][2] = {{4, 256}, {4, 128}, {2, 128}, {1, 128}};
+    for (const auto& s : shapes) {
+      L.r = s[0];
+      L.nt = s[1];
+      if ((n_q + L.r * L.nt - 1) / (L.r * L.nt) * chunks >= device_sms()) break;
+    }
+  }
+  const int64_t q_per_block = (int64_t)L.r * L.nt;
   L.q_tiles = std::max<int64_t>(1, (n_q + q_per_block - 1) / q_per_block);
   const int64_t item_tiles = std::max<int64_t>(1, (n_items + tile - 1) / tile);
   int k = o.k_splits;
   if (k == 0) {
-    const int64_t slots = (int64_t)device_sms() * fwd_blocks_per_sm(dim, o.fp64, o.r, o.nt, o.face_pairs > 0);
-    const int kmax = (int)std::max<int64_t>(1, std::min<int64_t>(64, item_tiles / 2));
+    const int64_t slots = (int64_t)device_sms() * fwd_blocks_per_sm(dim, o.fp64, L.r, L.nt, o.face_pairs > 0);
+    int kmax = (int)std::max<int64_t>(1, std::min<int64_t>(64, item_tiles / 2));
+    // where that many chunks still leave resident blocks free: down to one tile each, up to 256
+    // (20,480 faces x 2,928 Q: 54 chunks 135 us, 80 chunks 116 us)
+    if (fine && !o.fp64 && L.q_tiles * kmax < slots) kmax = (int)std::min<int64_t>(256, item_tiles);
     double best_eff = -1.0;
     int best_k = 1;
     k = 0;

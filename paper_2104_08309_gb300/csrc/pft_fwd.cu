@@ -27,6 +27,25 @@ namespace {
 // bounded and every stop decision is warp-uniform; a wait that gives up sets
 // ST_TIMEOUT and the block stops early, after letting copies in flight land.
 // ---------------------------------------------------------------------------
+// 3D: whether Q point i (x: its coordinates as float) belongs to the small-|Q| pass (Q = 0 included),
+// and, if `list`, its entry in that pass's list.  Such points take no part in the pair sum (their place
+// in a warp's largest P is immaterial: it is the smallest).  The FP32 test settles all but those near
+// or below the bound.
+template <class QT>
+__device__ __forceinline__ bool list_small(const double* __restrict__ q, int64_t i, const QT (&x)[3], float rmax,
+                                           WsHeader* h, int32_t* __restrict__ small, bool list) {
+  const float fx = (float)x[0] * rmax, fy = (float)x[1] * rmax, fz = (float)x[2] * rmax;
+  if (fmaf(fx, fx, fmaf(fy, fy, fz * fz)) > 1.01f * (float)(kTauSmallQ * kTauSmallQ)) return false;
+  const double q2 = q_norm2(q[i * 3], q[i * 3 + 1], q[i * 3 + 2]);
+  const bool is_small = q2 == 0.0 || small_q(q2, rmax);
+  if (is_small && q2 != 0.0 && list) {
+    const uint32_t e = atomicAdd(&h->small_q_count, 1u);
+    small[i] = (int32_t)e;
+    if (e < (uint32_t)kSmallDirect) h->small_list[e] = (int32_t)i;
+  }
+  return is_small;
+}
+
 template <class Pol, int R, int NT>
 __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typename Pol::Item* __restrict__ items, int64_t n_items,
                                             int64_t per_split, const double* __restrict__ q, int64_t n_q,
@@ -61,23 +80,7 @@ __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typena
       const int64_t src = qperm ? (int64_t)qperm[iq] : iq;
 #pragma unroll
       for (int d = 0; d < D; ++d) qr[r][d] = (QT)q[src * D + d];
-      if constexpr (D == 3) {
-        // Points of the small-|Q| pass take no part in the pair sum (their place in a warp's largest
-        // P is immaterial: it is the smallest), and the first face chunk's blocks list them.  The
-        // FP32 test settles all but those near or below the bound.
-        const float fx = (float)qr[r][0] * rmax, fy = (float)qr[r][1] * rmax, fz = (float)qr[r][2] * rmax;
-        bool is_small = false;
-        if (!(fmaf(fx, fx, fmaf(fy, fy, fz * fz)) > 1.01f * (float)(kTauSmallQ * kTauSmallQ))) {
-          const double q2 = q_norm2(q[src * 3], q[src * 3 + 1], q[src * 3 + 2]);
-          is_small = q2 == 0.0 || small_q(q2, rmax);
-          if (is_small && q2 != 0.0 && blockIdx.y == 0) {
-            const uint32_t e = atomicAdd(&h->small_q_count, 1u);
-            small[src] = (int32_t)e;
-            if (e < (uint32_t)kSmallDirect) h->small_list[e] = (int32_t)src;
-          }
-        }
-        live = live || !is_small;
-      }
+      if constexpr (D == 3) live = !list_small(q, src, qr[r], rmax, h, small, blockIdx.y == 0) || live;
     }
   }
   live = __any_sync(0xffffffffu, live);
@@ -134,6 +137,106 @@ __global__ void __launch_bounds__(NT, kMinBlocks<Pol, R, NT>) k_fwd(const typena
   for (int r = 0; r < R; ++r) {
     const int64_t iq = qbase + (int64_t)r * NT;
     if (iq < n_q) partial[(int64_t)blockIdx.y * n_q + (qperm ? (int64_t)qperm[iq] : iq)] = acc.get(r);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Short launches of the 3D FP32 path (few faces x Q points: k_fwd would run a block or a few, each
+// walking its 128-face tiles alone, ~1,000 cycles a face).  A block takes one tile and one of k_fwd's
+// groups of 128 Q points (the 32 lanes x 4 points of a warp there, on which the branch of a face is
+// decided), and its 8 warps evaluate the tile's faces side by side, 4 faces at a time each.  The tile's
+// FP32 sums run in k_fwd's order all the same: every warp keeps its faces' terms in registers and
+// adds them to the sums that the warp before it passes on through shared memory, so the results are
+// those of k_fwd bit for bit.
+// ---------------------------------------------------------------------------
+constexpr int kGrpWarps = 8, kGrpFaces = 4;   // faces a warp holds at a time
+using GrpV = typename QPack<4>::V;
+
+// Hand-over between two warps: the giver arrives, the taker waits (named barrier of their 64 threads).
+__device__ __forceinline__ void give(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void take(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+
+__global__ void __launch_bounds__(kGrpWarps * 32, 2) k_fwd_group(const Face32* __restrict__ faces, int64_t n_faces,
+                                                                 const double* __restrict__ q, int64_t n_q, Thr th,
+                                                                 double2* __restrict__ partial, WsHeader* h,
+                                                                 int32_t* __restrict__ small) {
+  constexpr int R = 4, N = QPack<R>::N, TILE = Pol3F32::kTile;
+  __shared__ __align__(16) Face32 rec[TILE];
+  __shared__ GrpV sums[2][N][32];   // the running (re, im) sums of the 128 points
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i0 = (int64_t)blockIdx.y * TILE;
+  const int cnt = (int)min((int64_t)TILE, n_faces - i0);
+  // group g of k_fwd's block b: points b 512 + 128 r + 32 g + lane
+  const int64_t qbase = (int64_t)(blockIdx.x >> 2) * 512 + (blockIdx.x & 3) * 32 + lane;
+  float qr[R][3];
+  bool live = false;
+  const float rmax = __uint_as_float(h->rmax_bits);
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int64_t iq = qbase + (int64_t)r * 128;
+    float x[3] = {0.f, 0.f, 0.f};
+    if (iq < n_q) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) x[d] = (float)q[iq * 3 + d];
+      live = !list_small(q, iq, x, rmax, h, small, blockIdx.y == 0 && warp == 0) || live;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) qr[r][d] = x[d];
+  }
+  if (!__syncthreads_or(live)) return;   // (every warp holds the same points)
+  for (int t = threadIdx.x; t < cnt * 3; t += kGrpWarps * 32)
+    reinterpret_cast<float4*>(rec)[t] = reinterpret_cast<const float4*>(faces + i0)[t];
+  __syncthreads();
+  GrpV qv[N][3];
+  QPack<R>::pack<3>(qr, qv);
+  const int passes = (cnt + kGrpWarps * kGrpFaces - 1) / (kGrpWarps * kGrpFaces);
+  for (int p = 0; p < passes; ++p) {
+    GrpV c[kGrpFaces][N], d[kGrpFaces][N], zr[kGrpFaces][N], zi[kGrpFaces][N];
+    const int f0 = (p * kGrpWarps + warp) * kGrpFaces;
+#pragma unroll
+    for (int k = 0; k < kGrpFaces; ++k) {
+      if (f0 + k < cnt) {   // warp-uniform
+        const float4* t = reinterpret_cast<const float4*>(rec + f0 + k);
+        const float4 A = t[0], B = t[1], C = t[2];
+        FaceQ<R> f;
+        f.load(qv, A, B, C);
+        GrpV S0[N];
+        if (f.wmax < th.hi) f.series(th, zr[k], zi[k]);
+        else f.template edge<false>(th, qv, A, B, C, zr[k], zi[k], S0);
+#pragma unroll
+        for (int j = 0; j < N; ++j) face_weight(f.mu[j], f.s[j], c[k][j], d[k][j]);
+      }
+    }
+    GrpV tre[N], tim[N];
+    if (p + warp > 0) {
+      take(1 + warp);
+#pragma unroll
+      for (int j = 0; j < N; ++j) { tre[j] = sums[0][j][lane]; tim[j] = sums[1][j][lane]; }
+    } else {
+#pragma unroll
+      for (int j = 0; j < N; ++j) { tre[j] = vs<GrpV>(0.f); tim[j] = vs<GrpV>(0.f); }
+    }
+#pragma unroll
+    for (int k = 0; k < kGrpFaces; ++k)
+      if (f0 + k < cnt) {
+#pragma unroll
+        for (int j = 0; j < N; ++j) face_add(c[k][j], d[k][j], zr[k][j], zi[k][j], tre[j], tim[j]);
+      }
+    if (p + 1 < passes || warp + 1 < kGrpWarps) {
+#pragma unroll
+      for (int j = 0; j < N; ++j) { sums[0][j][lane] = tre[j]; sums[1][j][lane] = tim[j]; }
+      give(1 + (warp + 1) % kGrpWarps);
+    } else {
+      Acc32<R> acc;
+      acc.init();
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        acc.re[r].add(el(tre, r));
+        acc.im[r].add(el(tim, r));
+        const int64_t iq = qbase + (int64_t)r * 128;
+        if (iq < n_q) partial[(int64_t)blockIdx.y * n_q + iq] = acc.get(r);
+      }
+    }
   }
 }
 
@@ -204,6 +307,11 @@ cudaError_t launch_fwd(int dim, bool fp64, const FwdLaunch& L, const void* items
   const Thr th{0.25f * tau * tau, 0.25f * tau_lo * tau_lo, tau > 1.0f ? 1 : 0, tau > 3.0f ? 1 : 0,
                dim == 3 && !fp64 ? pair_faces : 0};
   LaunchF f{L, items, n_items, q, n_q, th, partial, h, small, st, qperm};
+  if (L.group) {
+    k_fwd_group<<<dim3((unsigned)L.q_tiles, (unsigned)L.k_splits), kGrpWarps * 32, 0, st>>>(
+        static_cast<const Face32*>(items), n_items, q, n_q, th, partial, h, small);
+    return cudaGetLastError();
+  }
   if (dim == 2) return fp64 ? dispatch<Pol2F64>(L.r, L.nt, f) : dispatch<Pol2F32>(L.r, L.nt, f);
   if (!fp64 && th.pair_end > 0) return dispatch_pairs(L.r, L.nt, f);
   return fp64 ? dispatch<Pol3F64>(L.r, L.nt, f) : dispatch<Pol3F32>(L.r, L.nt, f);

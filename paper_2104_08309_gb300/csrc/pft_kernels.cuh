@@ -79,6 +79,7 @@ struct FwdLaunch {
   int64_t q_tiles;    // blocks along x
   int k_splits;       // blocks along y (segment/face chunks)
   int64_t per_split;  // items per chunk (multiple of the tile)
+  bool group;         // k_fwd_group: q_tiles groups of 128 Q points x k_splits tiles (3D FP32)
 };
 
 // Host-side launchers (defined in pft_fwd.cu).  Each returns cudaSuccess or the launch error.

@@ -300,6 +300,20 @@ __device__ __forceinline__ void face_finish(V mu, V s, V zr, V zi, V& tre, V& ti
   tim = vfma(c, zi, vfma(d, zr, tim));
 }
 
+// The same in two halves, for terms that are evaluated in one place and added in another.
+template <class V>
+__device__ __forceinline__ void face_weight(V mu, V s, V& c, V& d) {
+  V sm, cm;
+  sincos_v(mu, sm, cm);
+  c = vmul(vneg(s), cm);
+  d = vmul(vneg(s), sm);
+}
+template <class V>
+__device__ __forceinline__ void face_add(V c, V d, V zr, V zi, V& tre, V& tim) {
+  tre = vfma(c, zr, vfma(vneg(d), zi, tre));
+  tim = vfma(c, zi, vfma(d, zr, tim));
+}
+
 // ---------------------------------------------------------------------------
 // Policies: record type, Q registers, accumulators and the per-tile loop.
 // ---------------------------------------------------------------------------
