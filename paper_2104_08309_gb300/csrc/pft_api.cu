@@ -54,13 +54,6 @@ int resolve(const pft_options* o, int dim, Opts& out) {
   return PFT_OK;
 }
 
-int device_sms() {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
-  return sms > 0 ? sms : 1;
-}
-
 // Padded pairs (groups of 128 Q points x tiles of 128 faces) below which a 3D FP32 launch runs
 // k_fwd_group.  Kernel times, k_fwd with up to one tile a chunk against k_fwd_group: 320 faces x 241 Q
 // 67 / 19 us, 5,120 x 520 35 / 17, 5,120 x 2,000 45 / 36, 20,480 x 520 49 / 36; past the line 5,120 x
@@ -157,7 +150,7 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, bool fi
 
 struct FwdLayout {
   size_t mparts, items, partial, small, qperm, qscratch, total;
-  size_t grown;   // bytes that the small-|Q| pass adds to the total
+  size_t grown;   // bytes of the total that the allocation-free call's limit does not count
   int nblk;
   bool tiled;   // the main kernel visits the Q points in the library's order (q_order option)
   FwdLaunch L;
@@ -166,15 +159,19 @@ struct FwdLayout {
 FwdLayout layout_plan(int dim, const Opts& o, int64_t n_items, int64_t n_prep, int64_t n_q, bool fine) {
   FwdLayout y{};
   y.L = plan_fwd(dim, o, n_items, n_q, fine);
-  y.nblk = std::max(1, prep_blocks(n_prep));
+  y.nblk = dim == 3 ? prep3_blocks(n_prep) : std::max(1, prep_blocks(n_prep));
   const size_t item_bytes = dim == 2 ? (o.fp64 ? sizeof(Seg64) : sizeof(Seg32)) : (o.fp64 ? sizeof(Face64) : sizeof(Face32));
   size_t off = align_up(sizeof(WsHeader));
   y.mparts = off;  off = align_up(off + sizeof(double) * (size_t)y.nblk);
+  // not counted by the allocation-free call's limit: what small prep blocks and the small-|Q| pass add
+  if (dim == 3) y.grown = off - y.mparts - align_up(sizeof(double) * (size_t)std::max(1, prep_blocks(n_prep)));
   y.items = off;   off = align_up(off + item_bytes * (size_t)std::max<int64_t>(n_items, 1));
   if (dim == 3) {   // the small-|Q| pass writes over the records once the pair sums are done
     const size_t end = align_up(y.items + small3_bytes(n_items, device_sms()));
-    y.grown = end > off ? end - off : 0;
-    off += y.grown;
+    if (end > off) {
+      y.grown += end - off;
+      off = end;
+    }
   }
   y.partial = off; off = align_up(off + sizeof(double2) * (size_t)y.L.k_splits * (size_t)std::max<int64_t>(n_q, 1));
   y.small = off;   off = align_up(off + sizeof(int32_t) * (size_t)std::max<int64_t>(n_q, 1));
@@ -263,14 +260,13 @@ int pft2d_polygons(const float* verts, int64_t n_verts, const int64_t* loop_off,
   if (bad_ws(ws, ws_bytes, y.total)) return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  PFT_LAUNCH(launch_init_header(h, st));
-  if (n_q == 0) return PFT_OK;
-  if (n_verts == 0) {
-    if (cudaMemsetAsync(out, 0, sizeof(double) * 2 * (size_t)n_q, st) != cudaSuccess) return PFT_ERR_CUDA;
+  if (n_q == 0 || n_verts == 0) {
+    PFT_LAUNCH(launch_init_header(h, st));
+    if (n_q > 0 && cudaMemsetAsync(out, 0, sizeof(double) * 2 * (size_t)n_q, st) != cudaSuccess) return PFT_ERR_CUDA;
     return PFT_OK;
   }
   double* mp = at<double>(ws, y.mparts);
-  PFT_LAUNCH(launch_bbox(verts, n_verts, 2, h, st));
+  if (launch_start(verts, n_verts, 2, h, st, &g_last_launches) != cudaSuccess) return PFT_ERR_CUDA;
   PFT_LAUNCH(launch_prep2d(verts, n_verts, loop_off, n_loops, h, at<void>(ws, y.items), o.fp64, mp, y.nblk, st));
   const int32_t* qperm;
   if (int e = fwd_qorder(2, y, q, n_q, ws, st, qperm)) return e;
@@ -298,14 +294,13 @@ int pft3d_mesh(const float* verts, int64_t n_verts, const int32_t* faces, int64_
   if (bad_ws(ws, ws_bytes, y.total)) return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  PFT_LAUNCH(launch_init_header(h, st));
-  if (n_q == 0) return PFT_OK;
-  if (n_faces == 0) {
-    if (cudaMemsetAsync(out, 0, sizeof(double) * 2 * (size_t)n_q, st) != cudaSuccess) return PFT_ERR_CUDA;
+  if (n_q == 0 || n_faces == 0) {
+    PFT_LAUNCH(launch_init_header(h, st));
+    if (n_q > 0 && cudaMemsetAsync(out, 0, sizeof(double) * 2 * (size_t)n_q, st) != cudaSuccess) return PFT_ERR_CUDA;
     return PFT_OK;
   }
   double* mp = at<double>(ws, y.mparts);
-  PFT_LAUNCH(launch_bbox(verts, n_verts, 3, h, st));
+  if (launch_start(verts, n_verts, 3, h, st, &g_last_launches) != cudaSuccess) return PFT_ERR_CUDA;
   PFT_LAUNCH(launch_prep3d(verts, n_verts, faces, n_faces, h, at<void>(ws, y.items), o.fp64, mp, y.nblk, st,
                            2 * o.face_pairs));
   const int32_t* qperm;
@@ -347,16 +342,15 @@ int pft3d_polymesh(const float* verts, int64_t n_verts, const int32_t* face_idx,
     return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  PFT_LAUNCH(launch_init_header(h, st));
-  if (n_q == 0) return PFT_OK;
-  if (n_faces == 0) {
-    if (cudaMemsetAsync(out, 0, sizeof(double) * 2 * (size_t)n_q, st) != cudaSuccess) return PFT_ERR_CUDA;
+  if (n_q == 0 || n_faces == 0) {
+    PFT_LAUNCH(launch_init_header(h, st));
+    if (n_q > 0 && cudaMemsetAsync(out, 0, sizeof(double) * 2 * (size_t)n_q, st) != cudaSuccess) return PFT_ERR_CUDA;
     return PFT_OK;
   }
   int32_t* tris = at<int32_t>(ws, tri_off);
   double* mp = at<double>(ws, y.mparts);
+  if (launch_start(verts, n_verts, 3, h, st, &g_last_launches) != cudaSuccess) return PFT_ERR_CUDA;
   PFT_LAUNCH(launch_fan3d(face_idx, n_idx, face_off, n_faces, tris, n_tris, h, st));
-  PFT_LAUNCH(launch_bbox(verts, n_verts, 3, h, st));
   PFT_LAUNCH(launch_prep3d(verts, n_verts, tris, n_tris, h, at<void>(ws, y.items), o.fp64, mp, y.nblk, st));
   const int32_t* qperm;
   if (int e = fwd_qorder(3, y, q, n_q, ws, st, qperm)) return e;

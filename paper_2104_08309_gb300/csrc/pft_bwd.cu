@@ -15,6 +15,7 @@
 //    series, then a fixed-order gather to the vertices (3D through a vertex ->
 //    face-corner CSR built on the device and sorted, so sums are reproducible).
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 
 #include "pft_pairs.cuh"
@@ -1294,7 +1295,7 @@ __global__ void k_bbvert(const float* __restrict__ v, int64_t nv, const int64_t*
 __global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, int64_t nv,
                                                   const int32_t* __restrict__ f, int64_t nf,
                                                   const int64_t* __restrict__ off, int64_t nm, Face32* recs,
-                                                  PolyC* mc, int32_t* nblk, WsHeader* h) {
+                                                  PolyC* mc, int32_t* nblk, int32_t* __restrict__ deg, WsHeader* h) {
   __shared__ float sh[kAux / 32];
   const int64_t i = blockIdx.x;
   const int64_t s0 = off[i], s1 = off[i + 1];
@@ -1305,6 +1306,10 @@ __global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, i
     const int32_t a = f[3 * m], b = f[3 * m + 1], c = f[3 * m + 2];
     return a >= 0 && b >= 0 && c >= 0 && a < nv && b < nv && c < nv;
   };
+  // corners at each vertex, for the gather: every face once, whatever the offsets say
+  for (int64_t m = i * kAux + threadIdx.x; m < nf; m += (int64_t)gridDim.x * kAux)
+    if (valid(m))
+      for (int k = 0; k < 3; ++k) atomicAdd(&deg[f[3 * m + k]], 1);
   float mn[3] = {3.4e38f, 3.4e38f, 3.4e38f}, mx[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
   bool bad_index = false, bad_value = false;
   for (int64_t j = threadIdx.x; j < n; j += kAux) {
@@ -1334,7 +1339,7 @@ __global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, i
       for (int k = 0; k < 3; ++k)
         for (int d = 0; d < 3; ++d) P[k][d] = (double)v[3 * (int64_t)f[3 * m + k] + d] - c[d];
       for (int d = 0; d < 3; ++d) {
-        g[d] = (P[0][d] + P[1][d] + P[2][d]) / 3.0;
+        g[d] = (P[0][d] + P[1][d] + P[2][d]) * (1.0 / 3.0);
         q0[d] = P[0][d] - g[d];
         q1[d] = P[1][d] - g[d];
       }
@@ -1344,8 +1349,10 @@ __global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, i
                            e1[0] * e2[1] - e1[1] * e2[0]};
       r = Face32{(float)g[0], (float)g[1], (float)g[2], (float)q0[0], (float)q0[1], (float)q0[2],
                  (float)q1[0], (float)q1[1], (float)q1[2], (float)N[0], (float)N[1], (float)N[2]};
-      for (int k = 0; k < 3; ++k)
-        rm = fmaxf(rm, __double2float_ru(sqrt(P[k][0] * P[k][0] + P[k][1] * P[k][1] + P[k][2] * P[k][2])));
+      // an upper bound of the radius: root in FP32, rounded up (squares beyond its range: FP64's root)
+      double r2 = 0.0;
+      for (int k = 0; k < 3; ++k) r2 = fmax(r2, P[k][0] * P[k][0] + P[k][1] * P[k][1] + P[k][2] * P[k][2]);
+      rm = fmaxf(rm, r2 < 1e38 && r2 > 1e-30 ? __fsqrt_ru(__double2float_ru(r2)) : __double2float_ru(sqrt(r2)));
     }
     recs[m] = r;
   }
@@ -1420,6 +1427,8 @@ __device__ void corner_adj(int64_t m, const float* __restrict__ v, int64_t nv, c
                            const int32_t* __restrict__ small, uint32_t ns, int64_t q_base, int64_t g_base,
                            const double* __restrict__ q, const double* __restrict__ g,
                            const double* __restrict__ face_phi, double* __restrict__ out);
+__device__ __forceinline__ void file_corners(int64_t m, const int32_t* __restrict__ f, int64_t nv,
+                                             const int64_t* __restrict__ start, int32_t* cursor, int32_t* list);
 
 // Per face: its mesh (bisection over the offsets), then the corner adjoints with that mesh's
 // centre and small-|Q| rows.
@@ -1428,6 +1437,7 @@ __global__ void k_bbcorner3(const float* __restrict__ v, int64_t nv, const int32
                             const PolyC* __restrict__ mc, const int32_t* __restrict__ small,
                             const int32_t* __restrict__ small_cnt, const double* __restrict__ q,
                             const int64_t* __restrict__ q_off, int64_t n_q, const double* __restrict__ g,
+                            const int64_t* __restrict__ start, int32_t* cursor, int32_t* list,
                             double* __restrict__ corner) {
   const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (m >= nf) return;
@@ -1441,6 +1451,7 @@ __global__ void k_bbcorner3(const float* __restrict__ v, int64_t nv, const int32
   const PolyC C = mc[lo];
   const double c[3] = {C.cx, C.cy, C.cz};
   const uint32_t ns = (uint32_t)max(0, min(small_cnt[lo], (int32_t)nqi));
+  file_corners(m, f, nv, start, cursor, list);
   corner_adj(m, v, nv, f, nf, partial, ks, c, small + gb, ns, qb, gb, q, g, nullptr, corner + 9 * m);
 }
 
@@ -1544,61 +1555,98 @@ __global__ void k_bcorner3d(const float* __restrict__ v, int64_t nv, const int32
                             const double* __restrict__ partial, int ks, const WsHeader* h,
                             const int32_t* __restrict__ small, const double* __restrict__ q,
                             const double* __restrict__ g, const double* __restrict__ face_phi,
+                            const int64_t* __restrict__ start, int32_t* cursor, int32_t* list,
                             double* __restrict__ corner) {
   const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (m >= nf) return;
   const double c[3] = {h->center[0], h->center[1], h->center[2]};
+  file_corners(m, f, nv, start, cursor, list);
   corner_adj(m, v, nv, f, nf, partial, ks, c, small, h->small_q_count, 0, 0, q, g, face_phi, corner + 9 * m);
 }
 
-// Vertex -> face-corner CSR: degrees, exclusive scan, fill, per-vertex sort.
-__global__ void k_deg(const int32_t* __restrict__ f, int64_t nf, int64_t nv, int32_t* deg) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= 3 * nf) return;
-  const int32_t vtx = f[i];
-  if (vtx >= 0 && vtx < nv) atomicAdd(&deg[vtx], 1);
-}
-
-// Exclusive scan in three steps: per-block scan with block totals, scan of the
-// totals (one block, sequential over chunks), add back.
-__global__ void k_scan_block(const int32_t* __restrict__ in, int64_t n, int64_t* out, int64_t* block_tot) {
-  __shared__ int64_t sh[kAux];
+// Vertex -> face-corner lists: the prep kernel counts the corners at each vertex, k_places gives each
+// vertex its stretch of the list, the corner kernel files its corners and k_gather3d sorts each
+// vertex's.  The stretches need no order among the vertices, so blocks take theirs with one atomic add
+// (scanning the counts in three kernels, one of them a single thread, took 18 us for 41,000).
+__global__ void __launch_bounds__(kAux) k_places(const int32_t* __restrict__ deg, int64_t n,
+                                                 int64_t* __restrict__ start, WsHeader* h) {
+  __shared__ uint32_t sh[kAux / 32];
+  __shared__ uint32_t base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t i = blockIdx.x * (int64_t)kAux + threadIdx.x;
-  int64_t x = (i < n) ? in[i] : 0;
-  sh[threadIdx.x] = x;
+  const uint32_t d = i < n ? (uint32_t)deg[i] : 0u;
+  uint32_t x = d;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) sh[warp] = x;
   __syncthreads();
-  for (int o = 1; o < kAux; o <<= 1) {
-    const int64_t y = (threadIdx.x >= (unsigned)o) ? sh[threadIdx.x - o] : 0;
+  if (threadIdx.x == 0) {
+    uint32_t t = 0;
+    for (int w = 0; w < kAux / 32; ++w) {
+      const uint32_t c = sh[w];
+      sh[w] = t;
+      t += c;
+    }
+    base = atomicAdd(&h->filed, t);
+  }
+  __syncthreads();
+  if (i < n) start[i] = (int64_t)base + sh[warp] + x - d;
+}
+
+// Exclusive scan in one block (8 values a thread and round), for the pair blocks of a batch's shapes.
+constexpr int kScanT = 1024, kScanV = 8;
+__global__ void __launch_bounds__(kScanT) k_scan(const int32_t* __restrict__ in, int64_t n, int64_t* __restrict__ out) {
+  __shared__ int64_t sh[kScanT / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t carry = 0;
+  for (int64_t b0 = 0; b0 < n; b0 += kScanT * kScanV) {   // uniform trip count over the block
+    const int64_t i = b0 + (int64_t)threadIdx.x * kScanV;
+    int32_t v[kScanV];
+    int64_t sum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanV; ++k) {
+      v[k] = i + k < n ? in[i + k] : 0;
+      sum += v[k];
+    }
+    int64_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) sh[warp] = x;
     __syncthreads();
-    sh[threadIdx.x] += y;
+    if (warp == 0) {
+      int64_t t = sh[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, t, o);
+        if (lane >= o) t += y;
+      }
+      sh[lane] = t;
+    }
+    __syncthreads();
+    int64_t run = carry + (warp > 0 ? sh[warp - 1] : 0) + x - sum;
+#pragma unroll
+    for (int k = 0; k < kScanV; ++k) {
+      if (i + k < n) out[i + k] = run;
+      run += v[k];
+    }
+    carry += sh[kScanT / 32 - 1];
     __syncthreads();
   }
-  if (i < n) out[i] = sh[threadIdx.x] - x;
-  if (threadIdx.x == kAux - 1) block_tot[blockIdx.x] = sh[kAux - 1];
 }
 
-__global__ void k_scan_totals(int64_t* block_tot, int64_t nb) {
-  if (threadIdx.x != 0) return;
-  int64_t run = 0;
-  for (int64_t b = 0; b < nb; ++b) {
-    const int64_t t = block_tot[b];
-    block_tot[b] = run;
-    run += t;
-  }
-}
-
-__global__ void k_scan_add(int64_t* out, int64_t n, const int64_t* block_tot) {
-  const int64_t i = blockIdx.x * (int64_t)kAux + threadIdx.x;
-  if (i < n) out[i] += block_tot[blockIdx.x];
-}
-
-__global__ void k_fill(const int32_t* __restrict__ f, int64_t nf, int64_t nv, const int64_t* __restrict__ start,
-                       int32_t* cursor, int32_t* list) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= 3 * nf) return;
-  const int32_t vtx = f[i];
-  if (vtx < 0 || vtx >= nv) return;
-  list[start[vtx] + atomicAdd(&cursor[vtx], 1)] = (int32_t)i;   // corner id 3m + k
+// Files the corners of a valid face m under its vertices (any order: k_gather3d sorts).
+__device__ __forceinline__ void file_corners(int64_t m, const int32_t* __restrict__ f, int64_t nv,
+                                             const int64_t* __restrict__ start, int32_t* cursor, int32_t* list) {
+  const int32_t id[3] = {f[3 * m], f[3 * m + 1], f[3 * m + 2]};
+  if (id[0] < 0 || id[1] < 0 || id[2] < 0 || id[0] >= nv || id[1] >= nv || id[2] >= nv) return;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) list[start[id[k]] + atomicAdd(&cursor[id[k]], 1)] = (int32_t)(3 * m + k);
 }
 
 __global__ void k_gather3d(int64_t nv, const int64_t* __restrict__ start, const int32_t* __restrict__ deg,
@@ -1622,11 +1670,6 @@ __global__ void k_gather3d(int64_t nv, const int64_t* __restrict__ start, const 
   for (int d = 0; d < 3; ++d) grad[3 * vtx + d] = (float)s[d];
 }
 
-__global__ void k_zero_i32(int32_t* p, int64_t n) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) p[i] = 0;
-}
-
 // ---------------------------------------------------------------------------
 // Host side.
 // ---------------------------------------------------------------------------
@@ -1636,10 +1679,18 @@ template <typename T>
 T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws) + off); }
 inline unsigned blocks(int64_t n, int t) { return (unsigned)std::max<int64_t>(1, (n + t - 1) / t); }
 
-int sm_count() {
-  int dev = 0, sms = 1;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return std::max(1, sms);
+int sm_count() { return device_sms(); }
+
+// Resident blocks per SM of a pair kernel of kBwdNT threads, asked once per device.
+template <class K>
+int resident_blocks(K kernel, std::atomic<int> (&known)[64]) {
+  int dev = 0, b = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  const bool keep = dev >= 0 && dev < 64;
+  if (keep && (b = known[dev].load(std::memory_order_relaxed)) > 0) return b;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kBwdNT, 0) != cudaSuccess || b < 1) return 1;
+  if (keep) known[dev].store(b, std::memory_order_relaxed);
+  return b;
 }
 
 // Q chunks so that the grid (item blocks x chunks) is 16 waves of 8 blocks per SM (about 25 waves at
@@ -1671,7 +1722,7 @@ int more_chunks(int k, int64_t q_blocks, int64_t slots, int64_t tiles) {
 }
 
 struct BwdLayout {
-  size_t mparts, items, qrec, small, partial, corner, deg, cursor, start, btot, list, phi, total;
+  size_t mparts, items, qrec, small, partial, corner, deg, cursor, start, list, phi, total;
   int nblk, ks;
   int64_t per_split;
 };
@@ -1682,7 +1733,7 @@ BwdLayout bwd_layout(int dim, int64_t n_verts, int64_t n_items, int64_t n_prep, 
   const int64_t q_tiles = std::max<int64_t>(1, (n_q + kQTile - 1) / kQTile);
   y.per_split = ((q_tiles + y.ks - 1) / y.ks) * kQTile;
   y.ks = (int)std::max<int64_t>(1, (n_q + y.per_split - 1) / y.per_split);
-  y.nblk = std::max(1, prep_blocks(n_prep));
+  y.nblk = dim == 3 ? prep3_blocks(n_prep) : std::max(1, prep_blocks(n_prep));
   const int nf = dim == 2 ? 4 : 12;
   size_t o = al(sizeof(WsHeader));
   y.mparts = o;  o = al(o + sizeof(double) * (size_t)y.nblk);
@@ -1692,10 +1743,9 @@ BwdLayout bwd_layout(int dim, int64_t n_verts, int64_t n_items, int64_t n_prep, 
   y.partial = o; o = al(o + sizeof(double) * nf * (size_t)y.ks * (size_t)std::max<int64_t>(n_items, 1));
   if (dim == 3) {
     y.corner = o; o = al(o + sizeof(double) * 9 * (size_t)std::max<int64_t>(n_items, 1));
-    y.deg = o;    o = al(o + sizeof(int32_t) * (size_t)std::max<int64_t>(n_verts, 1));
-    y.cursor = o; o = al(o + sizeof(int32_t) * (size_t)std::max<int64_t>(n_verts, 1));
+    y.deg = o;    y.cursor = o + sizeof(int32_t) * (size_t)n_verts;   // together: one range to zero
+    o = al(o + sizeof(int32_t) * 2 * (size_t)std::max<int64_t>(n_verts, 1));
     y.start = o;  o = al(o + sizeof(int64_t) * (size_t)std::max<int64_t>(n_verts, 1));
-    y.btot = o;   o = al(o + sizeof(int64_t) * (size_t)blocks(n_verts, kAux));
     y.list = o;   o = al(o + sizeof(int32_t) * 3 * (size_t)std::max<int64_t>(n_items, 1));
     y.phi = o;    o = al(o + small_adjoint_bytes(n_items));
   }
@@ -1725,8 +1775,8 @@ QgLayout qg_layout(int64_t n_faces, int64_t n_q, bool tiled) {
   QgLayout y{};
   const int64_t face_tiles = std::max<int64_t>(1, (n_faces + kFTile - 1) / kFTile);
   const int64_t q_blocks = std::max<int64_t>(1, (n_q + kBwdNT - 1) / kBwdNT);
-  int occ = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_qgrad, kBwdNT, 0) != cudaSuccess || occ < 1) occ = 1;
+  static std::atomic<int> known[64];
+  const int occ = resident_blocks(k_qgrad, known);
   const int64_t slots = (int64_t)sm_count() * occ;
   const int kmax = (int)std::max<int64_t>(1, std::min<int64_t>(64, face_tiles / 2));
   int k = 0, best_k = 1;
@@ -1742,7 +1792,7 @@ QgLayout qg_layout(int64_t n_faces, int64_t n_q, bool tiled) {
   const int64_t tiles_per = (face_tiles + k - 1) / k;
   y.per_split = tiles_per * kFTile;
   y.ks = (int)((face_tiles + tiles_per - 1) / tiles_per);
-  y.nblk = std::max(1, prep_blocks(n_faces));
+  y.nblk = prep3_blocks(n_faces);
   size_t o = al(sizeof(WsHeader));
   y.mparts = o;  o = al(o + sizeof(double) * (size_t)y.nblk);
   y.items = o;   o = al(o + sizeof(Face32) * (size_t)std::max<int64_t>(n_faces, 1));
@@ -1763,8 +1813,8 @@ QgLayout qg2_layout(int64_t n_segs, int64_t n_prep, int64_t n_q, bool tiled) {
   QgLayout y{};
   const int64_t seg_tiles = std::max<int64_t>(1, (n_segs + kSTile - 1) / kSTile);
   const int64_t q_blocks = std::max<int64_t>(1, (n_q + kBwdNT - 1) / kBwdNT);
-  int occ = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_qgrad2d, kBwdNT, 0) != cudaSuccess || occ < 1) occ = 1;
+  static std::atomic<int> known[64];
+  const int occ = resident_blocks(k_qgrad2d, known);
   const int64_t slots = (int64_t)sm_count() * occ;
   const int kmax = (int)std::max<int64_t>(1, std::min<int64_t>(64, seg_tiles / 2));
   int k = 0, best_k = 1;
@@ -1796,7 +1846,7 @@ QgLayout qg2_layout(int64_t n_segs, int64_t n_prep, int64_t n_q, bool tiled) {
 
 // Batched 2D adjoint workspace.
 struct BbLayout {
-  size_t segs, pc, nblk, bstart, btot, rec, small, scnt, partial, total;
+  size_t segs, pc, nblk, bstart, rec, small, scnt, partial, total;
   int ks;
   int64_t per_split, grid;
 };
@@ -1819,7 +1869,6 @@ BbLayout bb_layout(int64_t nv, int64_t np, int64_t n_q, bool per_poly_q) {
   y.pc = o;      o = al(o + sizeof(PolyC) * (size_t)std::max<int64_t>(np, 1));
   y.nblk = o;    o = al(o + sizeof(int32_t) * (size_t)std::max<int64_t>(np, 1));
   y.bstart = o;  o = al(o + sizeof(int64_t) * (size_t)std::max<int64_t>(np, 1));
-  y.btot = o;    o = al(o + sizeof(int64_t) * (size_t)blocks(np, kAux));
   y.rec = o;     o = al(o + sizeof(QRec) * (size_t)rows);
   y.small = o;   o = al(o + sizeof(int32_t) * (size_t)rows);
   y.scnt = o;    o = al(o + sizeof(int32_t) * (size_t)std::max<int64_t>(np, 1));
@@ -1832,7 +1881,7 @@ BbLayout bb_layout(int64_t nv, int64_t np, int64_t n_q, bool per_poly_q) {
 // Q records and small lists per (mesh, Q) row, FP64 partials per (Q chunk, face), corner adjoints
 // and the vertex -> face-corner CSR of the vertex gather.
 struct Bb3Layout {
-  size_t recs, mc, nblk, bstart, btot, rec, small, scnt, partial, corner, deg, cursor, start, vtot, list, total;
+  size_t recs, mc, nblk, bstart, rec, small, scnt, partial, corner, deg, cursor, start, list, total;
   int ks;
   int64_t per_split, grid;
 };
@@ -1855,16 +1904,14 @@ Bb3Layout bb3_layout(int64_t nv, int64_t nf, int64_t nm, int64_t n_q, bool per_m
   y.mc = o;      o = al(o + sizeof(PolyC) * nm1);
   y.nblk = o;    o = al(o + sizeof(int32_t) * nm1);
   y.bstart = o;  o = al(o + sizeof(int64_t) * nm1);
-  y.btot = o;    o = al(o + sizeof(int64_t) * (size_t)blocks(nm, kAux));
   y.rec = o;     o = al(o + sizeof(QRec) * (size_t)rows);
   y.small = o;   o = al(o + sizeof(int32_t) * (size_t)rows);
   y.scnt = o;    o = al(o + sizeof(int32_t) * nm1);
   y.partial = o; o = al(o + sizeof(double) * 12 * (size_t)y.ks * nf1);
   y.corner = o;  o = al(o + sizeof(double) * 9 * nf1);
-  y.deg = o;     o = al(o + sizeof(int32_t) * nv1);
-  y.cursor = o;  o = al(o + sizeof(int32_t) * nv1);
+  y.deg = o;     y.cursor = o + sizeof(int32_t) * (size_t)nv;   // together: one range to zero
+  o = al(o + sizeof(int32_t) * 2 * nv1);
   y.start = o;   o = al(o + sizeof(int64_t) * nv1);
-  y.vtot = o;    o = al(o + sizeof(int64_t) * (size_t)blocks(nv, kAux));
   y.list = o;    o = al(o + sizeof(int32_t) * 3 * nf1);
   y.total = o;
   return y;
@@ -1922,17 +1969,37 @@ using namespace pft;
 namespace pft {
 namespace {
 
-// The 3D adjoint after argument checks and the header reset: records, Q weights, the pair
-// kernel, corner adjoints, the vertex -> corner CSR and the fixed-order gather.
+// Header reset and, where there is work, the bounding box and zeroed corner counts.  Returns a status to
+// return at once (nothing to do, or an error), or -1 to go on.
+int start3d(const float* verts, int64_t n_verts, int64_t n_faces, int64_t n_q, float* grad_verts, void* ws,
+            const BwdLayout& y, WsHeader* h, cudaStream_t st) {
+  if (n_verts == 0 || n_faces == 0 || n_q == 0) {
+    if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
+    ++g_bwd_launches;
+    if (n_verts > 0 && cudaMemsetAsync(grad_verts, 0, sizeof(float) * 3 * (size_t)n_verts, st) != cudaSuccess)
+      return PFT_ERR_CUDA;
+    return PFT_OK;
+  }
+  return launch_start(verts, n_verts, 3, h, st, &g_bwd_launches, at<int32_t>(ws, y.deg), 2 * n_verts) == cudaSuccess
+             ? -1
+             : PFT_ERR_CUDA;
+}
+
+// The 3D adjoint after argument checks and launch_start (which zeroes deg and cursor): records, Q weights,
+// the pair kernel, corner adjoints and the fixed-order gather.
 int mesh3d_backward_body(const float* verts, int64_t n_verts, const int32_t* faces, int64_t n_faces,
                          const double* q, int64_t n_q, const double* grad_out, float* grad_verts, void* ws,
                          const BwdLayout& y, const Thr& th, WsHeader* h, cudaStream_t st) {
-  if (launch_bbox(verts, n_verts, 3, h, st) != cudaSuccess) return PFT_ERR_CUDA;
+  int32_t* deg = at<int32_t>(ws, y.deg);
+  int64_t* start = at<int64_t>(ws, y.start);
   if (launch_prep3d(verts, n_verts, faces, n_faces, h, at<void>(ws, y.items), false, at<double>(ws, y.mparts),
-                    y.nblk, st) != cudaSuccess)
+                    y.nblk, st, 0, deg) != cudaSuccess)
     return PFT_ERR_CUDA;
-  g_bwd_launches += 2;
-  k_bq<3><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
+  ++g_bwd_launches;
+  k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
+  PFT_BWD_LAUNCH();
+  const int bt = n_q >= 65536 ? kAux : 64;   // few points (faces below): smaller blocks, so that all SMs take part
+  k_bq<3><<<blocks(n_q, bt), bt, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_faces, kBwdNT), (unsigned)y.ks);
   PFT_MARK(g_ev_start);
@@ -1944,32 +2011,16 @@ int mesh3d_backward_body(const float* verts, int64_t n_verts, const int32_t* fac
       cudaSuccess)
     return PFT_ERR_CUDA;
   g_bwd_launches += 2;
-  const int nt = n_faces >= 65536 ? kAux : 64;   // few faces: smaller blocks, so that all SMs take part
+  const int nt = n_faces >= 65536 ? kAux : 64;
   k_bcorner3d<<<blocks(n_faces, nt), nt, 0, st>>>(verts, n_verts, faces, n_faces, at<double>(ws, y.partial), y.ks, h,
                                                   at<int32_t>(ws, y.small), q, grad_out,
-                                                  small_adjoint_faces(at<void>(ws, y.phi)), at<double>(ws, y.corner));
+                                                  small_adjoint_faces(at<void>(ws, y.phi)), start,
+                                                  at<int32_t>(ws, y.cursor), at<int32_t>(ws, y.list),
+                                                  at<double>(ws, y.corner));
   PFT_BWD_LAUNCH();
-  int32_t* deg = at<int32_t>(ws, y.deg);
-  int32_t* cursor = at<int32_t>(ws, y.cursor);
-  int64_t* start = at<int64_t>(ws, y.start);
-  int64_t* btot = at<int64_t>(ws, y.btot);
-  k_zero_i32<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts);
-  PFT_BWD_LAUNCH();
-  k_zero_i32<<<blocks(n_verts, kAux), kAux, 0, st>>>(cursor, n_verts);
-  PFT_BWD_LAUNCH();
-  k_deg<<<blocks(3 * n_faces, kAux), kAux, 0, st>>>(faces, n_faces, n_verts, deg);
-  PFT_BWD_LAUNCH();
-  const unsigned nb = blocks(n_verts, kAux);
-  k_scan_block<<<nb, kAux, 0, st>>>(deg, n_verts, start, btot);
-  PFT_BWD_LAUNCH();
-  k_scan_totals<<<1, 32, 0, st>>>(btot, nb);
-  PFT_BWD_LAUNCH();
-  k_scan_add<<<nb, kAux, 0, st>>>(start, n_verts, btot);
-  PFT_BWD_LAUNCH();
-  k_fill<<<blocks(3 * n_faces, kAux), kAux, 0, st>>>(faces, n_faces, n_verts, start, cursor, at<int32_t>(ws, y.list));
-  PFT_BWD_LAUNCH();
-  k_gather3d<<<blocks(n_verts, kAux), kAux, 0, st>>>(n_verts, start, deg, at<int32_t>(ws, y.list),
-                                                     at<double>(ws, y.corner), grad_verts);
+  const int gt = n_verts >= 65536 ? kAux : 64;
+  k_gather3d<<<blocks(n_verts, gt), gt, 0, st>>>(n_verts, start, deg, at<int32_t>(ws, y.list),
+                                                 at<double>(ws, y.corner), grad_verts);
   PFT_BWD_LAUNCH();
   return PFT_OK;
 }
@@ -2006,18 +2057,18 @@ int pft2d_polygons_backward(const float* verts, int64_t n_verts, const int64_t* 
   if (ws == nullptr || reinterpret_cast<uintptr_t>(ws) % 256 != 0 || ws_bytes < y.total) return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
-  ++g_bwd_launches;
-  if (n_verts == 0) return PFT_OK;
-  if (n_q == 0) {
-    return cudaMemsetAsync(grad_verts, 0, sizeof(float) * 2 * (size_t)n_verts, st) == cudaSuccess ? PFT_OK
-                                                                                                  : PFT_ERR_CUDA;
+  if (n_verts == 0 || n_q == 0) {
+    if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
+    ++g_bwd_launches;
+    if (n_verts > 0 && cudaMemsetAsync(grad_verts, 0, sizeof(float) * 2 * (size_t)n_verts, st) != cudaSuccess)
+      return PFT_ERR_CUDA;
+    return PFT_OK;
   }
-  if (launch_bbox(verts, n_verts, 2, h, st) != cudaSuccess) return PFT_ERR_CUDA;
+  if (launch_start(verts, n_verts, 2, h, st, &g_bwd_launches) != cudaSuccess) return PFT_ERR_CUDA;
   if (launch_prep2d(verts, n_verts, loop_off, n_loops, h, at<void>(ws, y.items), false, at<double>(ws, y.mparts),
                     y.nblk, st) != cudaSuccess)
     return PFT_ERR_CUDA;
-  g_bwd_launches += 2;
+  ++g_bwd_launches;
   k_bq<2><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_verts, kBwdNT), (unsigned)y.ks);
@@ -2047,13 +2098,7 @@ int pft3d_mesh_backward(const float* verts, int64_t n_verts, const int32_t* face
   if (ws == nullptr || reinterpret_cast<uintptr_t>(ws) % 256 != 0 || ws_bytes < y.total) return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
-  ++g_bwd_launches;
-  if (n_verts == 0) return PFT_OK;
-  if (n_faces == 0 || n_q == 0) {
-    return cudaMemsetAsync(grad_verts, 0, sizeof(float) * 3 * (size_t)n_verts, st) == cudaSuccess ? PFT_OK
-                                                                                                  : PFT_ERR_CUDA;
-  }
+  if (int e = start3d(verts, n_verts, n_faces, n_q, grad_verts, ws, y, h, st); e >= 0) return e;
   return mesh3d_backward_body(verts, n_verts, faces, n_faces, q, n_q, grad_out, grad_verts, ws, y, th, h, st);
 }
 
@@ -2085,13 +2130,7 @@ int pft3d_polymesh_backward(const float* verts, int64_t n_verts, const int32_t* 
   if (ws == nullptr || reinterpret_cast<uintptr_t>(ws) % 256 != 0 || ws_bytes < need) return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
-  ++g_bwd_launches;
-  if (n_verts == 0) return PFT_OK;
-  if (n_faces == 0 || n_q == 0) {
-    return cudaMemsetAsync(grad_verts, 0, sizeof(float) * 3 * (size_t)n_verts, st) == cudaSuccess ? PFT_OK
-                                                                                                  : PFT_ERR_CUDA;
-  }
+  if (int e = start3d(verts, n_verts, n_faces, n_q, grad_verts, ws, y, h, st); e >= 0) return e;
   int32_t* tris = at<int32_t>(ws, y.total);
   if (launch_fan3d(face_idx, n_idx, face_off, n_faces, tris, n_tris, h, st) != cudaSuccess) return PFT_ERR_CUDA;
   ++g_bwd_launches;
@@ -2120,16 +2159,18 @@ int pft3d_mesh_qgrad(const float* verts, int64_t n_verts, const int32_t* faces, 
   if (ws == nullptr || reinterpret_cast<uintptr_t>(ws) % 256 != 0 || ws_bytes < y.total) return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
-  ++g_bwd_launches;
-  if (n_q == 0) return PFT_OK;
-  if (n_faces == 0)
-    return cudaMemsetAsync(grad_q, 0, sizeof(double) * 3 * (size_t)n_q, st) == cudaSuccess ? PFT_OK : PFT_ERR_CUDA;
-  if (launch_bbox(verts, n_verts, 3, h, st) != cudaSuccess) return PFT_ERR_CUDA;
+  if (n_q == 0 || n_faces == 0) {
+    if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
+    ++g_bwd_launches;
+    if (n_q > 0 && cudaMemsetAsync(grad_q, 0, sizeof(double) * 3 * (size_t)n_q, st) != cudaSuccess)
+      return PFT_ERR_CUDA;
+    return PFT_OK;
+  }
+  if (launch_start(verts, n_verts, 3, h, st, &g_bwd_launches) != cudaSuccess) return PFT_ERR_CUDA;
   if (launch_prep3d(verts, n_verts, faces, n_faces, h, at<void>(ws, y.items), false, at<double>(ws, y.mparts),
                     y.nblk, st) != cudaSuccess)
     return PFT_ERR_CUDA;
-  g_bwd_launches += 2;
+  ++g_bwd_launches;
   const int32_t* perm = nullptr;
   if (int e = qg_order(3, y, q, n_q, ws, st, perm)) return e;
   k_bq<3><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
@@ -2179,16 +2220,18 @@ int pft2d_polygons_qgrad(const float* verts, int64_t n_verts, const int64_t* loo
   if (ws == nullptr || reinterpret_cast<uintptr_t>(ws) % 256 != 0 || ws_bytes < y.total) return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
-  ++g_bwd_launches;
-  if (n_q == 0) return PFT_OK;
-  if (n_verts == 0)
-    return cudaMemsetAsync(grad_q, 0, sizeof(double) * 2 * (size_t)n_q, st) == cudaSuccess ? PFT_OK : PFT_ERR_CUDA;
-  if (launch_bbox(verts, n_verts, 2, h, st) != cudaSuccess) return PFT_ERR_CUDA;
+  if (n_q == 0 || n_verts == 0) {
+    if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
+    ++g_bwd_launches;
+    if (n_q > 0 && cudaMemsetAsync(grad_q, 0, sizeof(double) * 2 * (size_t)n_q, st) != cudaSuccess)
+      return PFT_ERR_CUDA;
+    return PFT_OK;
+  }
+  if (launch_start(verts, n_verts, 2, h, st, &g_bwd_launches) != cudaSuccess) return PFT_ERR_CUDA;
   if (launch_prep2d(verts, n_verts, loop_off, n_loops, h, at<void>(ws, y.items), false, at<double>(ws, y.mparts),
                     y.nblk, st) != cudaSuccess)
     return PFT_ERR_CUDA;
-  g_bwd_launches += 2;
+  ++g_bwd_launches;
   const int32_t* perm = nullptr;
   if (int e = qg_order(2, y, q, n_q, ws, st, perm)) return e;
   k_bq<2><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
@@ -2246,15 +2289,9 @@ int pft2d_polygons_batched_backward(const float* verts, int64_t n_verts, const i
   PolyC* pc = at<PolyC>(ws, y.pc);
   int32_t* nblk = at<int32_t>(ws, y.nblk);
   int64_t* bstart = at<int64_t>(ws, y.bstart);
-  int64_t* btot = at<int64_t>(ws, y.btot);
   k_bbprep<<<(unsigned)n_polys, kAux, 0, st>>>(verts, n_verts, poly_off, n_polys, segs, pc, nblk, h);
   PFT_BWD_LAUNCH();
-  const unsigned nb = blocks(n_polys, kAux);
-  k_scan_block<<<nb, kAux, 0, st>>>(nblk, n_polys, bstart, btot);
-  PFT_BWD_LAUNCH();
-  k_scan_totals<<<1, 32, 0, st>>>(btot, nb);
-  PFT_BWD_LAUNCH();
-  k_scan_add<<<nb, kAux, 0, st>>>(bstart, n_polys, btot);
+  k_scan<<<1, kScanT, 0, st>>>(nblk, n_polys, bstart);
   PFT_BWD_LAUNCH();
   k_bbq<2><<<(unsigned)n_polys, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
                                             at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
@@ -2301,8 +2338,9 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   if (y.grid > INT32_MAX) return PFT_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   WsHeader* h = at<WsHeader>(ws, 0);
-  if (launch_init_header(h, st) != cudaSuccess) return PFT_ERR_CUDA;
-  ++g_bwd_launches;
+  int32_t* deg = at<int32_t>(ws, y.deg);
+  // no common bounding box (each mesh has its own): the header reset and the zeroed corner counts only
+  if (launch_start(nullptr, 0, 3, h, st, &g_bwd_launches, deg, 2 * n_verts) != cudaSuccess) return PFT_ERR_CUDA;
   if (n_verts == 0) return PFT_OK;
   if (n_q == 0 || n_faces == 0)
     return cudaMemsetAsync(grad_verts, 0, sizeof(float) * 3 * (size_t)n_verts, st) == cudaSuccess ? PFT_OK
@@ -2311,16 +2349,13 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   PolyC* mc = at<PolyC>(ws, y.mc);
   int32_t* nblk = at<int32_t>(ws, y.nblk);
   int64_t* bstart = at<int64_t>(ws, y.bstart);
-  int64_t* btot = at<int64_t>(ws, y.btot);
   k_bbprep3<<<(unsigned)n_meshes, kAux, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes, recs, mc, nblk,
-                                                 h);
+                                                 deg, h);
   PFT_BWD_LAUNCH();
-  const unsigned nb = blocks(n_meshes, kAux);
-  k_scan_block<<<nb, kAux, 0, st>>>(nblk, n_meshes, bstart, btot);
+  k_scan<<<1, kScanT, 0, st>>>(nblk, n_meshes, bstart);
   PFT_BWD_LAUNCH();
-  k_scan_totals<<<1, 32, 0, st>>>(btot, nb);
-  PFT_BWD_LAUNCH();
-  k_scan_add<<<nb, kAux, 0, st>>>(bstart, n_meshes, btot);
+  int64_t* start = at<int64_t>(ws, y.start);
+  k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
   PFT_BWD_LAUNCH();
   k_bbq<3><<<(unsigned)n_meshes, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
                                                 at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
@@ -2333,27 +2368,9 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   PFT_MARK(g_ev_stop);
   k_bbcorner3<<<blocks(n_faces, kAux), kAux, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes,
                                                       at<double>(ws, y.partial), y.ks, mc, at<int32_t>(ws, y.small),
-                                                      at<int32_t>(ws, y.scnt), q, q_off, n_q, grad_out,
+                                                      at<int32_t>(ws, y.scnt), q, q_off, n_q, grad_out, start,
+                                                      at<int32_t>(ws, y.cursor), at<int32_t>(ws, y.list),
                                                       at<double>(ws, y.corner));
-  PFT_BWD_LAUNCH();
-  int32_t* deg = at<int32_t>(ws, y.deg);
-  int32_t* cursor = at<int32_t>(ws, y.cursor);
-  int64_t* start = at<int64_t>(ws, y.start);
-  int64_t* vtot = at<int64_t>(ws, y.vtot);
-  k_zero_i32<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts);
-  PFT_BWD_LAUNCH();
-  k_zero_i32<<<blocks(n_verts, kAux), kAux, 0, st>>>(cursor, n_verts);
-  PFT_BWD_LAUNCH();
-  k_deg<<<blocks(3 * n_faces, kAux), kAux, 0, st>>>(faces, n_faces, n_verts, deg);
-  PFT_BWD_LAUNCH();
-  const unsigned nbv = blocks(n_verts, kAux);
-  k_scan_block<<<nbv, kAux, 0, st>>>(deg, n_verts, start, vtot);
-  PFT_BWD_LAUNCH();
-  k_scan_totals<<<1, 32, 0, st>>>(vtot, nbv);
-  PFT_BWD_LAUNCH();
-  k_scan_add<<<nbv, kAux, 0, st>>>(start, n_verts, vtot);
-  PFT_BWD_LAUNCH();
-  k_fill<<<blocks(3 * n_faces, kAux), kAux, 0, st>>>(faces, n_faces, n_verts, start, cursor, at<int32_t>(ws, y.list));
   PFT_BWD_LAUNCH();
   k_gather3d<<<blocks(n_verts, kAux), kAux, 0, st>>>(n_verts, start, deg, at<int32_t>(ws, y.list),
                                                      at<double>(ws, y.corner), grad_verts);

@@ -42,7 +42,8 @@ struct WsHeader {
   double center[3];         // bounding-box midpoint c (all coordinates are taken relative to c)
   double measure;           // volume (3D forward), FP64, fixed-order sum
   int32_t small_list[kSmallDirect];   // the first listed small Q points (3D forward)
-  uint8_t pad[256 - 4 * 10 - 8 * 4 - 4 * kSmallDirect];
+  uint32_t filed;           // corner entries handed out so far (3D adjoint)
+  uint8_t pad[256 - 4 * 11 - 8 * 4 - 4 * kSmallDirect];
 };
 static_assert(sizeof(WsHeader) == 256, "header must stay 256 bytes");
 

@@ -9,6 +9,8 @@
 // per thread and in a fixed order: FP32 within a tile, error-free (TwoSum)
 // compensation across tiles; the per-chunk partials are added in FP64 by the
 // finalize kernel.  No atomics on data, so results are deterministic.
+#include <atomic>
+
 #include "pft_pairs.cuh"
 
 namespace pft {
@@ -317,14 +319,37 @@ cudaError_t launch_fwd(int dim, bool fp64, const FwdLaunch& L, const void* items
   return fp64 ? dispatch<Pol3F64>(L.r, L.nt, f) : dispatch<Pol3F32>(L.r, L.nt, f);
 }
 
+constexpr int kDevices = 64;   // devices whose properties are remembered
+
+int device_sms() {
+  static std::atomic<int> known[kDevices];   // 0: not asked yet
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  if (dev >= 0 && dev < kDevices && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 1;
+  if (dev >= 0 && dev < kDevices) known[dev].store(sms, std::memory_order_relaxed);
+  return sms;
+}
+
 int fwd_blocks_per_sm(int dim, bool fp64, int r, int nt, bool pairs) {
+  static std::atomic<int> known[kDevices][64];   // 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  std::atomic<int>* slot = nullptr;
+  if (dev >= 0 && dev < kDevices) {
+    const int lr = r == 1 ? 0 : (r == 2 ? 1 : (r == 4 ? 2 : 3));
+    slot = &known[dev][((((dim - 2) * 2 + fp64) * 2 + pairs) * 2 + (nt == 256)) * 4 + lr];
+    if (const int b = slot->load(std::memory_order_relaxed)) return b;
+  }
   int b = 1;
   OccF f{&b};
   cudaError_t e;
   if (dim == 2) e = fp64 ? dispatch<Pol2F64>(r, nt, f) : dispatch<Pol2F32>(r, nt, f);
   else if (!fp64 && pairs) e = dispatch_pairs(r, nt, f);
   else e = fp64 ? dispatch<Pol3F64>(r, nt, f) : dispatch<Pol3F32>(r, nt, f);
-  return e == cudaSuccess ? b : 1;
+  if (e != cudaSuccess) return 1;
+  if (slot) slot->store(b, std::memory_order_relaxed);
+  return b;
 }
 
 int fwd_tile(int dim, bool fp64) {

@@ -84,14 +84,16 @@ struct FwdLaunch {
 
 // Host-side launchers (defined in pft_fwd.cu).  Each returns cudaSuccess or the launch error.
 cudaError_t launch_init_header(WsHeader* h, cudaStream_t st);
-cudaError_t launch_bbox(const float* v, int64_t n, int dim, WsHeader* h, cudaStream_t st);
+// Header reset, bounding box and (zero != NULL) n_zero words set to 0; adds its launches to *launches.
+cudaError_t launch_start(const float* v, int64_t n, int dim, WsHeader* h, cudaStream_t st, int* launches,
+                         int32_t* zero = nullptr, int64_t n_zero = 0);
 cudaError_t launch_prep2d(const float* v, int64_t nv, const int64_t* off, int64_t nl, WsHeader* h,
                           void* segs, bool fp64, double* partials, int nblk, cudaStream_t st);
 // pair_faces: the faces [0, pair_faces) come in pairs (2k, 2k+1) that share their first edge in
 // opposite directions (face_pairs option); k_prep3d checks them, k_fwd shares the edge's sinc.
 cudaError_t launch_prep3d(const float* v, int64_t nv, const int32_t* f, int64_t nf, WsHeader* h,
                           void* faces, bool fp64, double* partials, int nblk, cudaStream_t st,
-                          int64_t pair_faces = 0);
+                          int64_t pair_faces = 0, int32_t* deg = nullptr);
 // qperm: NULL, or the slot -> Q index map of launch_qorder (the kernel reads Q point qperm[slot]
 // and writes its partial sums at that index).  In 3D the kernel also counts and lists the small-|Q|
 // points: small[i] is point i's place among them.
@@ -113,6 +115,8 @@ cudaError_t launch_finalize3d(const double* q, int64_t n_q, int64_t nf, const do
 // Prep blocks used for the per-block FP64 area/volume partial sums.
 constexpr int kPrepThreads = 256;
 inline int prep_blocks(int64_t n) { return (int)((n + kPrepThreads - 1) / kPrepThreads); }
+constexpr int kPrep3Threads = 64;   // 3D (see k_prep3d)
+inline int prep3_blocks(int64_t n) { return n > 0 ? (int)((n + kPrep3Threads - 1) / kPrep3Threads) : 1; }
 
 // Q order (pft_qorder.cu): a slot -> Q index map that puts Q points close together in Q space
 // into the same group of 32 threads of a pair kernel with r Q points per thread and nt threads
@@ -127,6 +131,10 @@ bool qorder_wanted(int64_t n_q, int64_t n_items, int r, int nt);
 // perm[n_q] <- the map; q is [n_q x dim] FP64 on the device; adds its launches to *launches.
 cudaError_t launch_qorder(int dim, const double* q, int64_t n_q, int r, int nt, void* scratch, int32_t* perm,
                           cudaStream_t st, int* launches);
+
+// SMs of the current device (1 if it cannot be asked), looked up once per device: a property that does
+// not change, read several times by every call's planning.
+int device_sms();
 
 // Occupancy query for the main kernel of a configuration (blocks per SM).
 int fwd_blocks_per_sm(int dim, bool fp64, int r, int nt, bool pairs = false);

@@ -83,6 +83,63 @@ __global__ void k_bbox(const float* __restrict__ v, int64_t n, WsHeader* h) {
   }
 }
 
+// Few vertices: the header reset and the bounding box in one block, the rest of the grid zeroing an
+// optional array (one launch instead of two to four; a launch costs a small call more than the work).
+constexpr int kStartT = 1024;
+constexpr int64_t kStartVerts = 16384;   // 16 rounds of the block
+template <int D>
+__global__ void __launch_bounds__(kStartT) k_start(const float* __restrict__ v, int64_t n, WsHeader* h,
+                                                   int32_t* __restrict__ zero, int64_t n_zero) {
+  __shared__ float red[2][D][kStartT / 32];
+  if (blockIdx.x > 0) {
+    for (int64_t i = (int64_t)(blockIdx.x - 1) * kStartT + threadIdx.x; i < n_zero; i += (int64_t)(gridDim.x - 1) * kStartT)
+      zero[i] = 0;
+    return;
+  }
+  float mn[D], mx[D];
+#pragma unroll
+  for (int c = 0; c < D; ++c) { mn[c] = __int_as_float(0x7f800000); mx[c] = -mn[c]; }
+  bool bad = false;
+  for (int64_t i = threadIdx.x; i < n; i += kStartT) {
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+      const float x = v[i * D + c];
+      if (!isfinite(x)) { bad = true; continue; }
+      mn[c] = fminf(mn[c], x);
+      mx[c] = fmaxf(mx[c], x);
+    }
+  }
+  if (threadIdx.x < (int)(sizeof(WsHeader) / 4)) reinterpret_cast<uint32_t*>(h)[threadIdx.x] = 0u;
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    mn[c] = -warp_max(-mn[c]);
+    mx[c] = warp_max(mx[c]);
+    if ((threadIdx.x & 31) == 0) { red[0][c][threadIdx.x >> 5] = mn[c]; red[1][c][threadIdx.x >> 5] = mx[c]; }
+  }
+  const bool any_bad = __syncthreads_or(bad);
+  if (threadIdx.x < 32) {
+    if (threadIdx.x < 3) {   // above every code, as for an axis without a finite coordinate
+      h->bbox_enc[threadIdx.x] = 0xffffffffu;
+      h->bbox_enc[3 + threadIdx.x] = 0u;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+      const float lo = -warp_max(-red[0][c][threadIdx.x]), hi = warp_max(red[1][c][threadIdx.x]);
+      if (threadIdx.x == 0 && lo <= hi) {
+        h->bbox_enc[c] = f2ord(lo);
+        h->bbox_enc[3 + c] = f2ord(hi);
+      }
+    }
+    if (threadIdx.x == 0 && any_bad) h->status = ST_NONFINITE;
+  }
+}
+
+__global__ void k_zero_i32(int32_t* p, int64_t n) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) p[i] = 0;
+}
+
 // 2D: one thread per vertex j builds the segment j -> next(j) of its loop.
 template <bool FP64>
 __global__ void __launch_bounds__(kPrepThreads) k_prep2d(const float* __restrict__ v, int64_t nv,
@@ -133,13 +190,17 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep2d(const float* __restrict
   if (blockIdx.x == 0 && threadIdx.x == 0) { h->center[0] = c[0]; h->center[1] = c[1]; h->center[2] = 0.0; }
 }
 
-// 3D: one thread per face.
+// 3D: one thread per face.  Bound: FP64 arithmetic (about 80 operations a face), so the blocks are small
+// (kPrep3Threads) and the faces spread over all SMs: 256 threads a block, with three FP64 divisions and a
+// square root a face, took 13 us for 320 faces as for 20,480.  deg != NULL: counts the corners at each
+// vertex (for the vertex adjoint's gather).
 template <bool FP64>
-__global__ void __launch_bounds__(kPrepThreads) k_prep3d(const float* __restrict__ v, int64_t nv,
-                                                         const int32_t* __restrict__ f, int64_t nf, WsHeader* h,
-                                                         void* items, double* partials, int64_t pair_faces) {
-  __shared__ double sh[kPrepThreads / 32];
-  const int64_t m = blockIdx.x * (int64_t)kPrepThreads + threadIdx.x;
+__global__ void __launch_bounds__(kPrep3Threads) k_prep3d(const float* __restrict__ v, int64_t nv,
+                                                          const int32_t* __restrict__ f, int64_t nf, WsHeader* h,
+                                                          void* items, double* partials, int64_t pair_faces,
+                                                          int32_t* __restrict__ deg) {
+  __shared__ double sh[kPrep3Threads / 32];
+  const int64_t m = blockIdx.x * (int64_t)kPrep3Threads + threadIdx.x;
   double c[3];
   load_center(h, 3, c);
   double vol = 0.0;
@@ -159,10 +220,15 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep3d(const float* __restrict
     } else {
       double P[3][3];
       const int32_t id[3] = {i0, i1, i2};
-      for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (deg != nullptr) atomicAdd(&deg[id[k]], 1);
+#pragma unroll
         for (int d = 0; d < 3; ++d) P[k][d] = (double)v[3 * (int64_t)id[k] + d] - c[d];
+      }
+#pragma unroll
       for (int d = 0; d < 3; ++d) {
-        g[d] = (P[0][d] + P[1][d] + P[2][d]) / 3.0;
+        g[d] = (P[0][d] + P[1][d] + P[2][d]) * (1.0 / 3.0);
         q0[d] = P[0][d] - g[d];
         q1[d] = P[1][d] - g[d];
       }
@@ -172,10 +238,13 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep3d(const float* __restrict
       N[1] = e1[2] * e2[0] - e1[0] * e2[2];
       N[2] = e1[0] * e2[1] - e1[1] * e2[0];
       vol = (P[0][0] * (P[1][1] * P[2][2] - P[1][2] * P[2][1]) + P[0][1] * (P[1][2] * P[2][0] - P[1][0] * P[2][2]) +
-             P[0][2] * (P[1][0] * P[2][1] - P[1][1] * P[2][0])) / 6.0;
+             P[0][2] * (P[1][0] * P[2][1] - P[1][1] * P[2][0])) * (1.0 / 6.0);
       double r2 = 0.0;
+#pragma unroll
       for (int k = 0; k < 3; ++k) r2 = fmax(r2, P[k][0] * P[k][0] + P[k][1] * P[k][1] + P[k][2] * P[k][2]);
-      rm = __double2float_ru(sqrt(r2));
+      // an upper bound of the radius: square root in FP32, both steps rounded up (a square beyond the
+      // FP32 range keeps FP64's root)
+      rm = r2 < 1e38 && r2 > 1e-30 ? __fsqrt_ru(__double2float_ru(r2)) : __double2float_ru(sqrt(r2));
     }
     if (FP64) {
       reinterpret_cast<Face64*>(items)[m] = Face64{g[0], g[1], g[2], q0[0], q0[1], q0[2], q1[0], q1[1], q1[2],
@@ -187,7 +256,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep3d(const float* __restrict
                  (float)N[0], (float)N[1], (float)N[2]};
     }
   }
-  double s = block_sum<kPrepThreads>(vol, sh);
+  double s = block_sum<kPrep3Threads>(vol, sh);
   float mm = warp_max(rm);
   if ((threadIdx.x & 31) == 0) atomicMax(&h->rmax_bits, __float_as_uint(mm));
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
@@ -422,11 +491,24 @@ cudaError_t launch_init_header(WsHeader* h, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_bbox(const float* v, int64_t n, int dim, WsHeader* h, cudaStream_t st) {
-  int blocks = (int)std::min<int64_t>(1024, (n + 255) / 256);
-  if (blocks < 1) blocks = 1;
+cudaError_t launch_start(const float* v, int64_t n, int dim, WsHeader* h, cudaStream_t st, int* launches,
+                         int32_t* zero, int64_t n_zero) {
+  if (n <= kStartVerts) {
+    const unsigned grid = 1 + (unsigned)std::min<int64_t>(256, (n_zero + kStartT - 1) / kStartT);
+    if (dim == 2) k_start<2><<<grid, kStartT, 0, st>>>(v, n, h, zero, n_zero);
+    else k_start<3><<<grid, kStartT, 0, st>>>(v, n, h, zero, n_zero);
+    ++*launches;
+    return cudaGetLastError();
+  }
+  if (cudaError_t e = launch_init_header(h, st)) return e;
+  const int blocks = (int)std::min<int64_t>(1024, (n + 255) / 256);
   if (dim == 2) k_bbox<2><<<blocks, 256, 0, st>>>(v, n, h);
   else k_bbox<3><<<blocks, 256, 0, st>>>(v, n, h);
+  *launches += 2;
+  if (n_zero > 0) {
+    k_zero_i32<<<(unsigned)((n_zero + 255) / 256), 256, 0, st>>>(zero, n_zero);
+    ++*launches;
+  }
   return cudaGetLastError();
 }
 
@@ -441,9 +523,10 @@ cudaError_t launch_prep2d(const float* v, int64_t nv, const int64_t* off, int64_
 }
 
 cudaError_t launch_prep3d(const float* v, int64_t nv, const int32_t* f, int64_t nf, WsHeader* h, void* faces,
-                          bool fp64, double* partials, int nblk, cudaStream_t st, int64_t pair_faces) {
-  if (fp64) k_prep3d<true><<<nblk, kPrepThreads, 0, st>>>(v, nv, f, nf, h, faces, partials, pair_faces);
-  else k_prep3d<false><<<nblk, kPrepThreads, 0, st>>>(v, nv, f, nf, h, faces, partials, pair_faces);
+                          bool fp64, double* partials, int nblk, cudaStream_t st, int64_t pair_faces, int32_t* deg) {
+  if (nblk != prep3_blocks(nf)) return cudaErrorInvalidValue;
+  if (fp64) k_prep3d<true><<<nblk, kPrep3Threads, 0, st>>>(v, nv, f, nf, h, faces, partials, pair_faces, deg);
+  else k_prep3d<false><<<nblk, kPrep3Threads, 0, st>>>(v, nv, f, nf, h, faces, partials, pair_faces, deg);
   return cudaGetLastError();
 }
 
@@ -460,7 +543,7 @@ cudaError_t launch_fan3d(const int32_t* idx, int64_t n_idx, const int64_t* off, 
 // sincos, the small-|Q| polynomial) spreads over all SMs.
 static int finish_points(int64_t n_q) {
   int n = 256;
-  while (n > 8 && n_q < (int64_t)n * 512) n /= 2;
+  while (n > 8 && n_q < (int64_t)n * 256) n /= 2;
   return n;
 }
 
@@ -481,16 +564,9 @@ cudaError_t launch_finalize3d(const double* q, int64_t n_q, int64_t nf, const do
   return cudaGetLastError();
 }
 
-static int small_grid() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms > 0 ? sms : 1;
-}
-
 cudaError_t launch_smallq2d(const float* v, int64_t nv, const int64_t* off, int64_t nl, const double* q,
                             const WsHeader* h, const int32_t* list, double* out, cudaStream_t st) {
-  k_smallq2d<<<small_grid(), kSmallThreads, 0, st>>>(v, nv, off, nl, q, h, list, out);
+  k_smallq2d<<<device_sms(), kSmallThreads, 0, st>>>(v, nv, off, nl, q, h, list, out);
   return cudaGetLastError();
 }
 

@@ -609,9 +609,7 @@ cudaError_t launch_small_adjoint3(const float* v, int64_t nv, const int32_t* f, 
 
 cudaError_t launch_small3(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q, WsHeader* h,
                           const double* mparts, int n_measure, void* scratch, cudaStream_t st) {
-  int dev = 0, sms = 1;
-  if (cudaError_t e = cudaGetDevice(&dev)) return e;
-  if (cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) return e;
+  const int sms = device_sms();
   if (cudaError_t e = cudaFuncSetAttribute(k_small3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShared)) return e;
   k_small3<<<(unsigned)small3_blocks(nf, sms), kNT, kShared, st>>>(v, nv, f, nf, q, h, mparts, n_measure,
                                                                   static_cast<char*>(scratch));
