@@ -18,6 +18,7 @@
 #include <atomic>
 #include <cstring>
 
+#include "pft_adj3.cuh"
 #include "pft_pairs.cuh"
 #include "pft_small.cuh"
 
@@ -100,6 +101,15 @@ struct Ring {
     }
   }
 };
+
+// Q records from their values: the scalar kernels' and the paired 3D adjoint's.
+__device__ __forceinline__ void put_rec(QRec& r, float qx, float qy, float qz, float gr, float gi) {
+  r = QRec{qx, qy, qz, gr, gi, 0.f, 0.f, 0.f};
+}
+__device__ __forceinline__ void put_rec(QDup& r, float qx, float qy, float qz, float gr, float gi) {
+  r = QDup{make_float2(qx, qx), make_float2(qy, qy), make_float2(qz, qz),
+           make_float2(gr, gr), make_float2(gi, gi), make_float2(-gi, -gi)};
+}
 
 // sinc(u) and its derivative: the Chebyshev polynomial and its derivative on
 // |u| <= pi, sin and cos of the turn-reduced argument beyond.  V = float2 takes two
@@ -464,9 +474,9 @@ struct QAdj {
 
 // Q records: Q rounded to FP32 (as the forward uses it) and gt; Q = 0 and small
 // |Q| go to the FP64 list with a zero weight here.
-template <int D>
+template <int D, class Rec>
 __global__ void k_bq(const double* __restrict__ q, const double* __restrict__ g, int64_t n_q, WsHeader* h,
-                     double scale, QRec* rec, int32_t* small, const int32_t* __restrict__ perm = nullptr) {
+                     double scale, Rec* rec, int32_t* small, const int32_t* __restrict__ perm = nullptr) {
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // record slot
   if (s >= n_q) return;
   const int64_t i = perm ? (int64_t)perm[s] : s;                      // its Q point (caller's index)
@@ -479,17 +489,17 @@ __global__ void k_bq(const double* __restrict__ q, const double* __restrict__ g,
     qf[d] = (float)Q[d];
   }
   const double q2 = q_norm2(Q[0], Q[1], Q[2]);
-  QRec r{qf[0], qf[1], qf[2], 0.f, 0.f, 0.f, 0.f, 0.f};
+  float wr = 0.f, wi = 0.f;
   if (q2 == 0.0 || small_q(q2, __uint_as_float(h->rmax_bits))) {
     small[atomicAdd(&h->small_q_count, 1u)] = (int32_t)i;
   } else {
     double sp, cp;
     sincos(-(Q[0] * h->center[0] + Q[1] * h->center[1] + Q[2] * h->center[2]), &sp, &cp);
     const double gr = g[2 * i], gi = g[2 * i + 1], k = scale / q2;
-    r.gr = (float)(k * (gr * cp - gi * sp));
-    r.gi = (float)(k * (gr * sp + gi * cp));
+    wr = (float)(k * (gr * cp - gi * sp));
+    wi = (float)(k * (gr * sp + gi * cp));
   }
-  rec[s] = r;
+  put_rec(rec[s], qf[0], qf[1], qf[2], wr, wi);
 }
 
 // Thread <-> item (segment or face); Q chunk blockIdx.y; FP64 partial per (chunk, item, field).
@@ -874,51 +884,173 @@ __global__ void k_qsmall2d_fin(int64_t nv, const double* __restrict__ q, const d
   }
 }
 
-template <int D, int NF>
-__global__ void __launch_bounds__(kBwdNT) k_bwd(const void* __restrict__ items, int64_t n_items,
-                                                const QRec* __restrict__ rec, int64_t n_q, int64_t per_split,
-                                                Thr th, double* __restrict__ partial, uint32_t* status) {
+// 2D: thread <-> segment, Q chunk blockIdx.y.
+__global__ void __launch_bounds__(kBwdNT) k_bwd2(const Seg32* __restrict__ segs, int64_t n_items,
+                                                 const QRec* __restrict__ rec, int64_t n_q, int64_t per_split,
+                                                 double* __restrict__ partial, uint32_t* status) {
   __shared__ __align__(128) QRec slots[kStages * kQTile];
   __shared__ __align__(8) uint64_t full[kStages];
   __shared__ int done[kStages];
   __shared__ int issued;
   const int64_t m = blockIdx.x * (int64_t)kBwdNT + threadIdx.x;
-  float4 F[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-  if (m < n_items) {
-    if constexpr (D == 2) F[0] = reinterpret_cast<const float4*>(items)[m];
-    else for (int k = 0; k < 3; ++k) F[k] = reinterpret_cast<const float4*>(items)[3 * m + k];
-  }
+  float4 F = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (m < n_items) F = reinterpret_cast<const float4*>(segs)[m];
   const int64_t q0 = (int64_t)blockIdx.y * per_split;
   const int64_t nq = max((int64_t)0, min(per_split, n_q - q0));
   Ring<QRec, kQTile, kBwdNT> ring{slots, full, done, &issued, rec + q0, nq, (int)((nq + kQTile - 1) / kQTile)};
   ring.start();
-  CAcc acc[NF];
+  CAcc acc[4];
 #pragma unroll
-  for (int f = 0; f < NF; ++f) acc[f].init();
+  for (int f = 0; f < 4; ++f) acc[f].init();
   bool ok = true;
   for (int t = 0; t < ring.ntiles; ++t) {
     if (!ring.wait(t)) { ok = false; break; }
     const QRec* tq = ring.tile(t);
     const int cnt = ring.count(t);
-    float a[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) a[f] = 0.f;
+    const float sv[4] = {F.x, F.y, F.z, F.w};
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-    for (int j = 0; j < cnt; ++j) {
-      const QRec Q = tq[j];
-      if constexpr (D == 2) seg_adj(Q, *reinterpret_cast<const float(*)[4]>(&F[0]), *reinterpret_cast<float(*)[4]>(a));
-      else face_adj(Q, F[0], F[1], F[2], th, *reinterpret_cast<float(*)[12]>(a));
-    }
+    for (int j = 0; j < cnt; ++j) seg_adj(tq[j], sv, a);
 #pragma unroll
-    for (int f = 0; f < NF; ++f) acc[f].add(a[f]);
+    for (int f = 0; f < 4; ++f) acc[f].add(a[f]);
     ring.release(t);
   }
   if (!ok) set_status(status, ST_TIMEOUT);
   ring.finish();
   if (!ok || m >= n_items) return;
-  double* dst = partial + ((int64_t)blockIdx.y * n_items + m) * NF;
+  double* dst = partial + ((int64_t)blockIdx.y * n_items + m) * 4;
 #pragma unroll
-  for (int f = 0; f < NF; ++f) dst[f] = (double)acc[f].hi + (double)acc[f].lo;
+  for (int f = 0; f < 4; ++f) dst[f] = (double)acc[f].hi + (double)acc[f].lo;
+}
+
+// 3D: a thread's two faces (2t, 2t + 1 of the block's kPairFaces) against a stream of Q records.  The
+// state of a block; `run` walks the ring and leaves the sums in acc (shared memory, [field][face of the
+// pair][thread]).
+constexpr int kPairFaces = 2 * kBwdNT;
+struct PairShared {
+  QDup slots[kStages * kQTile];
+  float2 acc[24][kBwdNT];   // compensated sums (hi, lo) of 12 fields x 2 faces
+  uint64_t full[kStages];
+  int done[kStages];
+  int issued;
+};
+constexpr int kPairBlocks = 4;   // resident blocks per SM the registers are held to (128 each)
+
+__device__ __forceinline__ void scalar_adj(const QDup& Q, const float2 (&F)[12], Thr th, float2 (&a)[12], bool second) {
+  const QRec q{Q.qx.x, Q.qy.x, Q.qz.x, Q.gr.x, Q.gi.x, 0.f, 0.f, 0.f};
+  float f[12], d[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    f[k] = second ? F[k].y : F[k].x;
+    d[k] = 0.f;
+  }
+  face_adj(q, make_float4(f[0], f[1], f[2], f[3]), make_float4(f[4], f[5], f[6], f[7]),
+           make_float4(f[8], f[9], f[10], f[11]), th, d);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    if (second) a[k].y = fmaf(adj_sign(k), d[k], a[k].y);
+    else a[k].x = fmaf(adj_sign(k), d[k], a[k].x);
+  }
+}
+
+// live: the warp holds a face.  Returns false when a wait gave up.
+__device__ __forceinline__ bool pair_run(PairShared& sh, const QDup* rec, int64_t nq, const float2 (&F)[12], bool live,
+                                         Thr th) {
+  using V = float2;
+  Ring<QDup, kQTile, kBwdNT> ring{sh.slots, sh.full, sh.done, &sh.issued, rec, nq, (int)((nq + kQTile - 1) / kQTile)};
+  ring.start();
+#pragma unroll
+  for (int k = 0; k < 24; ++k) sh.acc[k][threadIdx.x] = make_float2(0.f, 0.f);
+  bool ok = true;
+  for (int t = 0; t < ring.ntiles; ++t) {
+    if (!ring.wait(t)) { ok = false; break; }
+    if (live) {
+      const QDup* tq = ring.tile(t);
+      const int cnt = ring.count(t);
+      V a[12];
+#pragma unroll
+      for (int k = 0; k < 12; ++k) a[k] = vs<V>(0.f);
+#pragma unroll 1
+      for (int j = 0; j < cnt; ++j) {
+        const QDup Q = tq[j];
+        const V a0 = vfma(Q.qx, F[3], vfma(Q.qy, F[4], vmul(Q.qz, F[5])));
+        const V a1 = vfma(Q.qx, F[6], vfma(Q.qy, F[7], vmul(Q.qz, F[8])));
+        const V s1 = vadd(a0, a1), m = vmul(a1, s1), P = vfma(a0, a0, m);
+        // the largest |P| of the warp's faces decides, as in face_adj_t (the sign bit is cleared there
+        // for the same reason)
+        const float wmax = __uint_as_float(
+            __reduce_max_sync(0xffffffffu, max(__float_as_uint(P.x) & 0x7fffffffu, __float_as_uint(P.y) & 0x7fffffffu)));
+        if (wmax < th.hi) {
+          const V mu = vfma(Q.qx, F[0], vfma(Q.qy, F[1], vmul(Q.qz, F[2])));
+          const V s = vfma(Q.qx, F[9], vfma(Q.qy, F[10], vmul(Q.qz, F[11])));
+          if (wmax < kPShort) series_adj<0>(Q, mu, a0, a1, s1, m, s, a);
+          else if (wmax < kP9) series_adj<1>(Q, mu, a0, a1, s1, m, s, a);
+          else if (wmax < kPLong) series_adj<2>(Q, mu, a0, a1, s1, m, s, a);
+          else series_adj<3>(Q, mu, a0, a1, s1, m, s, a);
+        } else {
+          scalar_adj(Q, F, th, a, false);
+          scalar_adj(Q, F, th, a, true);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float2 c = sh.acc[2 * k + e][threadIdx.x];
+          CAcc v{c.x, c.y};
+          v.add(e ? a[k].y : a[k].x);
+          sh.acc[2 * k + e][threadIdx.x] = make_float2(v.hi, v.lo);
+        }
+      }
+    }
+    ring.release(t);
+  }
+  ring.finish();
+  return ok;
+}
+__device__ __forceinline__ void pair_load(const Face32* faces, int64_t m, int64_t end, float2 (&F)[12]) {
+  float f[2][12];
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (m + e < end) x = reinterpret_cast<const float4*>(faces + m + e)[k];
+      f[e][4 * k] = x.x;
+      f[e][4 * k + 1] = x.y;
+      f[e][4 * k + 2] = x.z;
+      f[e][4 * k + 3] = x.w;
+    }
+#pragma unroll
+  for (int k = 0; k < 12; ++k) F[k] = make_float2(f[0][k], f[1][k]);
+}
+// dst: partial sums of the thread's first face (12 doubles a face)
+__device__ __forceinline__ void pair_store(const PairShared& sh, int64_t m, int64_t end, double* dst) {
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    if (m + e < end)
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        const float2 c = sh.acc[2 * k + e][threadIdx.x];
+        const double v = (double)c.x + (double)c.y;
+        dst[12 * e + k] = adj_sign(k) > 0.f ? v : -v;
+      }
+}
+
+__global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bwd3(const Face32* __restrict__ faces, int64_t n_faces,
+                                                             const QDup* __restrict__ rec, int64_t n_q,
+                                                             int64_t per_split, Thr th, double* __restrict__ partial,
+                                                             uint32_t* status) {
+  extern __shared__ __align__(128) unsigned char raw[];
+  PairShared& sh = *reinterpret_cast<PairShared*>(raw);
+  const int64_t m = blockIdx.x * (int64_t)kPairFaces + 2 * threadIdx.x;
+  float2 F[12];
+  pair_load(faces, m, n_faces, F);
+  const int64_t q0 = (int64_t)blockIdx.y * per_split;
+  const int64_t nq = max((int64_t)0, min(per_split, n_q - q0));
+  const bool ok = pair_run(sh, rec + q0, nq, F, __any_sync(0xffffffffu, m < n_faces), th);
+  if (!ok) set_status(status, ST_TIMEOUT);
+  if (ok) pair_store(sh, m, n_faces, partial + ((int64_t)blockIdx.y * n_faces + m) * 12);
 }
 
 // 2D vertex gradients: record adjoints of segment j (start) and of the segment
@@ -1092,10 +1224,10 @@ __device__ __forceinline__ void bb_rows(const int64_t* q_off, int64_t i, int64_t
 }
 
 // D = 2: weight 2 g e^{-iQ.c}/|Q|^2 (records hold half segment vectors); D = 3: g e^{-iQ.c}/|Q|^2.
-template <int D>
+template <int D, class Rec>
 __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, const int64_t* __restrict__ q_off,
                                               const double* __restrict__ g, int64_t n_q, int64_t np,
-                                              const PolyC* __restrict__ pc, QRec* rec, int32_t* small,
+                                              const PolyC* __restrict__ pc, Rec* rec, int32_t* small,
                                               int32_t* small_cnt, WsHeader* h) {
   __shared__ int wcount[kAux / 32];
   __shared__ int base;
@@ -1117,7 +1249,7 @@ __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, cons
       const double Qx = q[D * (qb + l)], Qy = q[D * (qb + l) + 1], Qz = D == 3 ? q[D * (qb + l) + D - 1] : 0.0;
       const float qx = (float)Qx, qy = (float)Qy, qz = (float)Qz;
       const double q2 = Qx * Qx + Qy * Qy + Qz * Qz;
-      QRec r{qx, qy, qz, 0.f, 0.f, 0.f, 0.f, 0.f};
+      float wr = 0.f, wi = 0.f;
       if (q2 == 0.0 || q2 * ((double)P.rmax * (double)P.rmax) < kTauSmallQ * kTauSmallQ) {
         is_small = true;
       } else {
@@ -1129,10 +1261,10 @@ __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, cons
         sincosf(pr, &sp, &cp);
         const float gr = (float)g[2 * (gb + l)], gi = (float)g[2 * (gb + l) + 1];
         const float k = (D == 2 ? 2.0f : 1.0f) / (float)q2;
-        r.gr = k * fmaf(gr, cp, -gi * sp);
-        r.gi = k * fmaf(gr, sp, gi * cp);
+        wr = k * fmaf(gr, cp, -gi * sp);
+        wi = k * fmaf(gr, sp, gi * cp);
       }
-      rec[gb + l] = r;
+      put_rec(rec[gb + l], qx, qy, qz, wr, wi);
     }
     const unsigned m = __ballot_sync(0xffffffffu, is_small);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1359,23 +1491,23 @@ __global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, i
   rm = block_minmax_f(rm, true, sh);
   if (threadIdx.x == 0) {
     mc[i] = PolyC{c[0], c[1], c[2], rm, 0};
-    nblk[i] = (int32_t)((n + kBwdNT - 1) / kBwdNT);
+    nblk[i] = (int32_t)((n + kPairFaces - 1) / kPairFaces);
   }
 }
 
-// Pair blocks: block b is pair block b - bstart[i] of mesh i; thread t <-> face t of that block;
-// the mesh's Q records stream through the ring (Q chunk blockIdx.y).  Warps with no face only wait
-// for and release the tiles.  Blocks past the last mesh leave at once.
-__global__ void __launch_bounds__(kBwdNT) k_bbwd3(const Face32* __restrict__ recs, int64_t nf,
-                                                  const int64_t* __restrict__ off, int64_t nm,
-                                                  const int64_t* __restrict__ bstart, const int32_t* __restrict__ nblk,
-                                                  const QRec* __restrict__ rec, const int64_t* __restrict__ q_off,
-                                                  int64_t n_q, int64_t per_split, Thr th,
-                                                  double* __restrict__ partial, uint32_t* status) {
-  __shared__ __align__(128) QRec slots[kStages * kQTile];
-  __shared__ __align__(8) uint64_t full[kStages];
-  __shared__ int done[kStages];
-  __shared__ int issued;
+// Pair blocks: block b is pair block b - bstart[i] of mesh i (kPairFaces faces, two a thread); the mesh's Q
+// records stream through the ring (Q chunk blockIdx.y).  Warps with no face only wait for and release
+// the tiles.  Blocks past the last mesh leave at once.
+__global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bbwd3(const Face32* __restrict__ recs, int64_t nf,
+                                                              const int64_t* __restrict__ off, int64_t nm,
+                                                              const int64_t* __restrict__ bstart,
+                                                              const int32_t* __restrict__ nblk,
+                                                              const QDup* __restrict__ rec,
+                                                              const int64_t* __restrict__ q_off, int64_t n_q,
+                                                              int64_t per_split, Thr th,
+                                                              double* __restrict__ partial, uint32_t* status) {
+  extern __shared__ __align__(128) unsigned char raw[];
+  PairShared& sh = *reinterpret_cast<PairShared*>(raw);
   const int64_t b = blockIdx.x;
   if (b >= bstart[nm - 1] + nblk[nm - 1]) return;   // uniform over the block
   int64_t lo = 0, hi = nm - 1;                      // the last mesh whose blocks start at or before b
@@ -1385,41 +1517,16 @@ __global__ void __launch_bounds__(kBwdNT) k_bbwd3(const Face32* __restrict__ rec
     else hi = mid - 1;
   }
   const int64_t s0 = max((int64_t)0, min(off[lo], nf)), s1 = max(s0, min(off[lo + 1], nf));
-  const int64_t m = s0 + (b - bstart[lo]) * kBwdNT + threadIdx.x;
-  const bool mine = m < s1;
-  float4 F[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-  if (mine)
-    for (int k = 0; k < 3; ++k) F[k] = reinterpret_cast<const float4*>(recs)[3 * m + k];
-  const bool live = __any_sync(0xffffffffu, mine);
+  const int64_t m = s0 + (b - bstart[lo]) * kPairFaces + 2 * threadIdx.x;
+  float2 F[12];
+  pair_load(recs, m, s1, F);
   int64_t qb, gb, nqi;
   bb_rows(q_off, lo, n_q, qb, gb, nqi);
   const int64_t q0 = (int64_t)blockIdx.y * per_split;
   const int64_t nq = max((int64_t)0, min(per_split, nqi - q0));
-  Ring<QRec, kQTile, kBwdNT> ring{slots, full, done, &issued, rec + gb + q0, nq, (int)((nq + kQTile - 1) / kQTile)};
-  ring.start();
-  CAcc acc[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k].init();
-  bool ok = true;
-  for (int t = 0; t < ring.ntiles; ++t) {
-    if (!ring.wait(t)) { ok = false; break; }
-    const QRec* tq = ring.tile(t);
-    const int cnt = ring.count(t);
-    float a[12] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (live) {
-#pragma unroll 1
-      for (int j = 0; j < cnt; ++j) face_adj(tq[j], F[0], F[1], F[2], th, a);
-    }
-#pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k].add(a[k]);
-    ring.release(t);
-  }
+  const bool ok = pair_run(sh, rec + gb + q0, nq, F, __any_sync(0xffffffffu, m < s1), th);
   if (!ok) set_status(status, ST_TIMEOUT);
-  ring.finish();
-  if (!ok || !mine) return;
-  double* dst = partial + ((int64_t)blockIdx.y * nf + m) * 12;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) dst[k] = (double)acc[k].hi + (double)acc[k].lo;
+  if (ok) pair_store(sh, m, s1, partial + ((int64_t)blockIdx.y * nf + m) * 12);
 }
 
 __device__ void corner_adj(int64_t m, const float* __restrict__ v, int64_t nv, const int32_t* __restrict__ f,
@@ -1705,6 +1812,17 @@ int q_splits(int64_t n_items, int64_t n_q) {
   return (int)std::min<int64_t>({k, q_tiles, 256});
 }
 
+// The same for the paired 3D adjoints' blocks (kPairBlocks resident ones per SM): 12 waves for one mesh
+// (81,920 faces x 32,768 Q: 6.03 / 5.91 / 5.89 ms for 6 / 12 / 25 waves, and the corner kernel, which
+// adds the chunks, 0.08 / 0.10 / 0.16 ms), 24 for a batch, whose blocks are uneven (96 meshes x 13,824
+// Q: 8.4 / 7.2 / 6.9 ms, corners 0.09 / 0.12 / 0.15 ms).
+int pair_splits(int64_t item_blocks, int64_t n_q, int waves) {
+  const int64_t slots = (int64_t)sm_count() * kPairBlocks;
+  const int64_t q_tiles = std::max<int64_t>(1, (n_q + kQTile - 1) / kQTile);
+  const int64_t k = std::max<int64_t>(1, (waves * slots + item_blocks - 1) / item_blocks);
+  return (int)std::min<int64_t>({k, q_tiles, 256});
+}
+
 // Chunks of a Q-gradient launch: k (the fewest that fill whole waves, the last >= 97 % full) raised,
 // for a launch of fewer than 40 waves, as far as chunks of at least 16 tiles and 64 chunks allow,
 // the last wave still >= 97 % full (the tail of the last blocks, as above).  The 3D Q-gradient on
@@ -1729,7 +1847,8 @@ struct BwdLayout {
 
 BwdLayout bwd_layout(int dim, int64_t n_verts, int64_t n_items, int64_t n_prep, int64_t n_q) {
   BwdLayout y{};
-  y.ks = q_splits(n_items, n_q);
+  y.ks = dim == 3 ? pair_splits(std::max<int64_t>(1, (n_items + kPairFaces - 1) / kPairFaces), n_q, 12)
+                  : q_splits(n_items, n_q);
   const int64_t q_tiles = std::max<int64_t>(1, (n_q + kQTile - 1) / kQTile);
   y.per_split = ((q_tiles + y.ks - 1) / y.ks) * kQTile;
   y.ks = (int)std::max<int64_t>(1, (n_q + y.per_split - 1) / y.per_split);
@@ -1738,7 +1857,7 @@ BwdLayout bwd_layout(int dim, int64_t n_verts, int64_t n_items, int64_t n_prep, 
   size_t o = al(sizeof(WsHeader));
   y.mparts = o;  o = al(o + sizeof(double) * (size_t)y.nblk);
   y.items = o;   o = al(o + (dim == 2 ? sizeof(Seg32) : sizeof(Face32)) * (size_t)std::max<int64_t>(n_items, 1));
-  y.qrec = o;    o = al(o + sizeof(QRec) * (size_t)std::max<int64_t>(n_q, 1));
+  y.qrec = o;    o = al(o + (dim == 2 ? sizeof(QRec) : sizeof(QDup)) * (size_t)std::max<int64_t>(n_q, 1));
   y.small = o;   o = al(o + sizeof(int32_t) * (size_t)std::max<int64_t>(n_q, 1));
   y.partial = o; o = al(o + sizeof(double) * nf * (size_t)y.ks * (size_t)std::max<int64_t>(n_items, 1));
   if (dim == 3) {
@@ -1888,12 +2007,9 @@ struct Bb3Layout {
 
 Bb3Layout bb3_layout(int64_t nv, int64_t nf, int64_t nm, int64_t n_q, bool per_mesh_q) {
   Bb3Layout y{};
-  y.grid = std::max<int64_t>(1, nm + (nf + kBwdNT - 1) / kBwdNT);   // at least the pair blocks needed
-  const int64_t slots = (int64_t)sm_count() * 8;
+  y.grid = std::max<int64_t>(1, nm + (nf + kPairFaces - 1) / kPairFaces);   // at least the pair blocks needed
   const int64_t q_tiles = std::max<int64_t>(1, (n_q + kQTile - 1) / kQTile);
-  // Q chunks for 16 waves of 8 blocks per SM, as q_splits (the tail of the last blocks to start):
-  // 4,096 polygons x 64^2 Q 17.32 -> 17.04 ms, 1,024 meshes x 32^3 Q 218.5 -> 212.6 ms against 4 waves
-  const int64_t k = std::min<int64_t>({std::max<int64_t>(1, (16 * slots + y.grid - 1) / y.grid), q_tiles, 256});
+  const int64_t k = pair_splits(y.grid, n_q, 24);
   y.per_split = ((q_tiles + k - 1) / k) * kQTile;
   y.ks = (int)std::max<int64_t>(1, (n_q + y.per_split - 1) / y.per_split);
   const int64_t rows = std::max<int64_t>(per_mesh_q ? n_q : nm * n_q, 1);
@@ -1904,7 +2020,7 @@ Bb3Layout bb3_layout(int64_t nv, int64_t nf, int64_t nm, int64_t n_q, bool per_m
   y.mc = o;      o = al(o + sizeof(PolyC) * nm1);
   y.nblk = o;    o = al(o + sizeof(int32_t) * nm1);
   y.bstart = o;  o = al(o + sizeof(int64_t) * nm1);
-  y.rec = o;     o = al(o + sizeof(QRec) * (size_t)rows);
+  y.rec = o;     o = al(o + sizeof(QDup) * (size_t)rows);
   y.small = o;   o = al(o + sizeof(int32_t) * (size_t)rows);
   y.scnt = o;    o = al(o + sizeof(int32_t) * nm1);
   y.partial = o; o = al(o + sizeof(double) * 12 * (size_t)y.ks * nf1);
@@ -1936,6 +2052,12 @@ int check_opts(const pft_options* o, Thr& th, bool* tiled = nullptr) {
   const float lo = std::min(tau, 0.05f);
   th = Thr{0.25f * tau * tau, 0.25f * lo * lo, tau > 1.f ? 1 : 0, tau > 3.f ? 1 : 0};
   return PFT_OK;
+}
+
+// The paired 3D adjoints' shared memory is beyond the default limit.
+template <class K>
+bool allow_shared(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PairShared)) == cudaSuccess;
 }
 
 #define PFT_MARK(ev)                                                                        \
@@ -1999,12 +2121,14 @@ int mesh3d_backward_body(const float* verts, int64_t n_verts, const int32_t* fac
   k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
   PFT_BWD_LAUNCH();
   const int bt = n_q >= 65536 ? kAux : 64;   // few points (faces below): smaller blocks, so that all SMs take part
-  k_bq<3><<<blocks(n_q, bt), bt, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
+  k_bq<3, QDup><<<blocks(n_q, bt), bt, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QDup>(ws, y.qrec),
+                                               at<int32_t>(ws, y.small));
   PFT_BWD_LAUNCH();
-  dim3 grid(blocks(n_faces, kBwdNT), (unsigned)y.ks);
+  dim3 grid(blocks(n_faces, kPairFaces), (unsigned)y.ks);
+  if (!allow_shared(k_bwd3)) return PFT_ERR_CUDA;
   PFT_MARK(g_ev_start);
-  k_bwd<3, 12><<<grid, kBwdNT, 0, st>>>(at<void>(ws, y.items), n_faces, at<QRec>(ws, y.qrec), n_q, y.per_split, th,
-                                        at<double>(ws, y.partial), &h->status);
+  k_bwd3<<<grid, kBwdNT, sizeof(PairShared), st>>>(at<Face32>(ws, y.items), n_faces, at<QDup>(ws, y.qrec), n_q,
+                                                   y.per_split, th, at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
   if (launch_small_adjoint3(verts, n_verts, faces, n_faces, q, grad_out, n_q, h, at<void>(ws, y.phi), st) !=
@@ -2069,12 +2193,12 @@ int pft2d_polygons_backward(const float* verts, int64_t n_verts, const int64_t* 
                     y.nblk, st) != cudaSuccess)
     return PFT_ERR_CUDA;
   ++g_bwd_launches;
-  k_bq<2><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
+  k_bq<2, QRec><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_verts, kBwdNT), (unsigned)y.ks);
   PFT_MARK(g_ev_start);
-  k_bwd<2, 4><<<grid, kBwdNT, 0, st>>>(at<void>(ws, y.items), n_verts, at<QRec>(ws, y.qrec), n_q, y.per_split, th,
-                                       at<double>(ws, y.partial), &h->status);
+  k_bwd2<<<grid, kBwdNT, 0, st>>>(at<Seg32>(ws, y.items), n_verts, at<QRec>(ws, y.qrec), n_q, y.per_split,
+                                  at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
   k_bvert2d<<<blocks(n_verts, kAux), kAux, 0, st>>>(verts, n_verts, loop_off, n_loops, at<double>(ws, y.partial),
@@ -2173,7 +2297,7 @@ int pft3d_mesh_qgrad(const float* verts, int64_t n_verts, const int32_t* faces, 
   ++g_bwd_launches;
   const int32_t* perm = nullptr;
   if (int e = qg_order(3, y, q, n_q, ws, st, perm)) return e;
-  k_bq<3><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
+  k_bq<3, QRec><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
                                               perm);
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_q, kBwdNT), (unsigned)y.ks);
@@ -2234,7 +2358,7 @@ int pft2d_polygons_qgrad(const float* verts, int64_t n_verts, const int64_t* loo
   ++g_bwd_launches;
   const int32_t* perm = nullptr;
   if (int e = qg_order(2, y, q, n_q, ws, st, perm)) return e;
-  k_bq<2><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
+  k_bq<2, QRec><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
                                               perm);
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_q, kBwdNT), (unsigned)y.ks);
@@ -2293,7 +2417,7 @@ int pft2d_polygons_batched_backward(const float* verts, int64_t n_verts, const i
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_polys, bstart);
   PFT_BWD_LAUNCH();
-  k_bbq<2><<<(unsigned)n_polys, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
+  k_bbq<2, QRec><<<(unsigned)n_polys, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
                                             at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
   PFT_BWD_LAUNCH();
   if (y.grid > INT32_MAX) return PFT_ERR_UNSUPPORTED;
@@ -2357,13 +2481,14 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   int64_t* start = at<int64_t>(ws, y.start);
   k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
   PFT_BWD_LAUNCH();
-  k_bbq<3><<<(unsigned)n_meshes, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
+  k_bbq<3, QDup><<<(unsigned)n_meshes, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_meshes, mc, at<QDup>(ws, y.rec),
                                                 at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
   PFT_BWD_LAUNCH();
   dim3 grid((unsigned)y.grid, (unsigned)y.ks);
+  if (!allow_shared(k_bbwd3)) return PFT_ERR_CUDA;
   PFT_MARK(g_ev_start);
-  k_bbwd3<<<grid, kBwdNT, 0, st>>>(recs, n_faces, mesh_off, n_meshes, bstart, nblk, at<QRec>(ws, y.rec), q_off, n_q,
-                                   y.per_split, th, at<double>(ws, y.partial), &h->status);
+  k_bbwd3<<<grid, kBwdNT, sizeof(PairShared), st>>>(recs, n_faces, mesh_off, n_meshes, bstart, nblk,
+                                   at<QDup>(ws, y.rec), q_off, n_q, y.per_split, th, at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
   k_bbcorner3<<<blocks(n_faces, kAux), kAux, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes,
