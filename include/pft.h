@@ -349,7 +349,7 @@ int pft2d_polygons_batched_backward(const float* verts, int64_t n_verts, const i
  * adjoint is that of pft3d_mesh_backward (Eq. 14 and its series differentiated in
  * reverse mode, FP32 with compensated sums; |Q| r_max < 0.25 in FP64 from the corner
  * series), the vertex sums in a fixed order.  Options and errors as for
- * pft3d_mesh_backward; the workspace holds one 52-byte Q record per (mesh, Q) row
+ * pft3d_mesh_backward; the workspace holds one 36-byte Q record per (mesh, Q) row
  * (n_meshes x n_q rows shared, n_q rows with q_off) plus 204 bytes per face.
  * per_mesh_q tells the size function which (0: shared, 1: q_off). */
 size_t pft3d_batched_backward_workspace_size(int64_t n_verts, int64_t n_faces, int64_t n_meshes, int64_t n_q,

@@ -4,10 +4,10 @@
 // The face term J = -s exp(i mu) Z of a (Q, face) pair (pft_pairs.cuh), weight gt, differentiated in
 // reverse mode into the 12 record fields.  Bound: the FP32 lanes (65 / 74 / 83 / 115 operations a pair in
 // the four series forms below), two of them per issue slot.  A thread holds faces 2t and 2t + 1 of its
-// block, field by field as float2, and one Q point at a time, whose fields lie twice in shared memory
-// (QDup), so no operand is assembled.  (Two Q points of one face per thread instead need the face's fields
-// doubled in registers: 168-182 of them, and ran slower than scalar code.)  The compensated sums, touched
-// once per tile, live in shared memory.  Faces whose phases need the edge sum take the scalar pair
+// block, field by field as float2, and takes one Q point at a time, its fields broadcast (doubling them in
+// shared memory, 48 B a record, ran 2-3 % slower: 5.82 against 5.69 ms on 81,920 faces x 32,768 Q; two Q
+// points of one face per thread took 168-182 registers and ran slower than scalar code: 11.7 against 9.3
+// ms).  The compensated sums, touched once per tile, live in shared memory.  Faces whose phases need the edge sum take the scalar pair
 // adjoint one after the other.
 #pragma once
 
@@ -15,11 +15,11 @@
 
 namespace pft {
 
-// Q record of the 3D vertex adjoints: every value twice; ngi = -gi.
-struct __align__(16) QDup {
-  float2 qx, qy, qz, gr, gi, ngi;
+// Q record of the adjoints: Q in FP32, the weight gt and -Im gt.
+struct __align__(16) QRec {
+  float qx, qy, qz, gr, gi, ngi, pad0, pad1;
 };
-static_assert(sizeof(QDup) == 48, "Q record is three float4");
+static_assert(sizeof(QRec) == 32, "Q record is two float4");
 
 // Z = zr + i zi (zi = G_re, zr = -G_im = t r) and its derivatives in P and in t = a0 a1 (a0 + a1) = -T, for the
 // series k <= 7 (FORM 0), k <= 9 (1), k <= 11 (2) and k <= 17 (3): the coefficients of face_series,
@@ -143,14 +143,14 @@ __device__ __forceinline__ void series_grad(V t, V P, V& zr, V& zi, V& zr_P, V& 
 __device__ __forceinline__ constexpr float adj_sign(int k) { return k < 3 ? 1.f : -1.f; }
 
 template <int FORM, class V>
-__device__ __forceinline__ void series_adj(const QDup& Q, V mu, V a0, V a1, V s1, V m, V s, V (&a)[12]) {
+__device__ __forceinline__ void series_adj(const QRec& Q, V mu, V a0, V a1, V s1, V m, V s, V (&a)[12]) {
   const V P = vfma(a0, a0, m), t = vmul(a0, m);   // m = a1 (a0 + a1)
   V zr, zi, zr_P, zr_t, zi_P, zi_t;
   series_grad<FORM>(t, P, zr, zi, zr_P, zr_t, zi_P, zi_t);
   V sm, cm;
   sincos_v(mu, sm, cm);
-  const V p = vfma(Q.gr, cm, vmul(Q.gi, sm));     // conj(gt) exp(i mu) = p + i q
-  const V q = vfma(Q.gr, sm, vmul(Q.ngi, cm));
+  const V p = vfma(vs<V>(Q.gr), cm, vmul(vs<V>(Q.gi), sm));     // conj(gt) exp(i mu) = p + i q
+  const V q = vfma(vs<V>(Q.gr), sm, vmul(vs<V>(Q.ngi), cm));
   const V nq = vmul(q, vs<V>(-1.0f));
   const V nsb = vfma(p, zr, vmul(nq, zi));        // -dc/ds = Re((p + i q) Z), c = Re(conj(gt) J)
   const V mub = vmul(s, vfma(p, zi, vmul(q, zr)));   // dc/dmu = s Im((p + i q) Z)
@@ -158,18 +158,19 @@ __device__ __forceinline__ void series_adj(const QDup& Q, V mu, V a0, V a1, V s1
   const V nP = vfma(ps, zr_P, vmul(ns, zi_P)), nT = vfma(ps, zr_t, vmul(ns, zi_t));
   // dP = e0 da0 + e1 da1, dt = a1 e0 da0 + a0 e1 da1, e0 = 2 a0 + a1, e1 = 2 a1 + a0
   const V n0 = vmul(vadd(a0, s1), vfma(nT, a1, nP)), n1 = vmul(vadd(a1, s1), vfma(nT, a0, nP));
-  a[0] = vfma(mub, Q.qx, a[0]);
-  a[1] = vfma(mub, Q.qy, a[1]);
-  a[2] = vfma(mub, Q.qz, a[2]);
-  a[3] = vfma(n0, Q.qx, a[3]);
-  a[4] = vfma(n0, Q.qy, a[4]);
-  a[5] = vfma(n0, Q.qz, a[5]);
-  a[6] = vfma(n1, Q.qx, a[6]);
-  a[7] = vfma(n1, Q.qy, a[7]);
-  a[8] = vfma(n1, Q.qz, a[8]);
-  a[9] = vfma(nsb, Q.qx, a[9]);
-  a[10] = vfma(nsb, Q.qy, a[10]);
-  a[11] = vfma(nsb, Q.qz, a[11]);
+  const V qx = vs<V>(Q.qx), qy = vs<V>(Q.qy), qz = vs<V>(Q.qz);
+  a[0] = vfma(mub, qx, a[0]);
+  a[1] = vfma(mub, qy, a[1]);
+  a[2] = vfma(mub, qz, a[2]);
+  a[3] = vfma(n0, qx, a[3]);
+  a[4] = vfma(n0, qy, a[4]);
+  a[5] = vfma(n0, qz, a[5]);
+  a[6] = vfma(n1, qx, a[6]);
+  a[7] = vfma(n1, qy, a[7]);
+  a[8] = vfma(n1, qz, a[8]);
+  a[9] = vfma(nsb, qx, a[9]);
+  a[10] = vfma(nsb, qy, a[10]);
+  a[11] = vfma(nsb, qz, a[11]);
 }
 
 }  // namespace pft

@@ -32,11 +32,6 @@ constexpr int kAux = 256;          // threads per block of the auxiliary kernels
 constexpr double kTwoPiD = 6.283185307179586477;      // 2 pi (FP64)
 constexpr double kInvTwoPiD = 0.1591549430918953358;  // 1 / (2 pi) (FP64)
 
-struct __align__(16) QRec {
-  float qx, qy, qz, gr, gi, pad0, pad1, pad2;
-};
-static_assert(sizeof(QRec) == 32, "Q record is two float4");
-
 // ---------------------------------------------------------------------------
 // Generic bulk-copy ring over an array of records (same protocol as k_fwd: the
 // last warp out of a slot issues the tile kStages further on).
@@ -101,15 +96,6 @@ struct Ring {
     }
   }
 };
-
-// Q records from their values: the scalar kernels' and the paired 3D adjoint's.
-__device__ __forceinline__ void put_rec(QRec& r, float qx, float qy, float qz, float gr, float gi) {
-  r = QRec{qx, qy, qz, gr, gi, 0.f, 0.f, 0.f};
-}
-__device__ __forceinline__ void put_rec(QDup& r, float qx, float qy, float qz, float gr, float gi) {
-  r = QDup{make_float2(qx, qx), make_float2(qy, qy), make_float2(qz, qz),
-           make_float2(gr, gr), make_float2(gi, gi), make_float2(-gi, -gi)};
-}
 
 // sinc(u) and its derivative: the Chebyshev polynomial and its derivative on
 // |u| <= pi, sin and cos of the turn-reduced argument beyond.  V = float2 takes two
@@ -474,9 +460,9 @@ struct QAdj {
 
 // Q records: Q rounded to FP32 (as the forward uses it) and gt; Q = 0 and small
 // |Q| go to the FP64 list with a zero weight here.
-template <int D, class Rec>
+template <int D>
 __global__ void k_bq(const double* __restrict__ q, const double* __restrict__ g, int64_t n_q, WsHeader* h,
-                     double scale, Rec* rec, int32_t* small, const int32_t* __restrict__ perm = nullptr) {
+                     double scale, QRec* rec, int32_t* small, const int32_t* __restrict__ perm = nullptr) {
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // record slot
   if (s >= n_q) return;
   const int64_t i = perm ? (int64_t)perm[s] : s;                      // its Q point (caller's index)
@@ -499,7 +485,7 @@ __global__ void k_bq(const double* __restrict__ q, const double* __restrict__ g,
     wr = (float)(k * (gr * cp - gi * sp));
     wi = (float)(k * (gr * sp + gi * cp));
   }
-  put_rec(rec[s], qf[0], qf[1], qf[2], wr, wi);
+  rec[s] = QRec{qf[0], qf[1], qf[2], wr, wi, -wi, 0.f, 0.f};
 }
 
 // Thread <-> item (segment or face); Q chunk blockIdx.y; FP64 partial per (chunk, item, field).
@@ -928,7 +914,7 @@ __global__ void __launch_bounds__(kBwdNT) k_bwd2(const Seg32* __restrict__ segs,
 // pair][thread]).
 constexpr int kPairFaces = 2 * kBwdNT;
 struct PairShared {
-  QDup slots[kStages * kQTile];
+  __align__(128) QRec slots[kStages * kQTile];
   float2 acc[24][kBwdNT];   // compensated sums (hi, lo) of 12 fields x 2 faces
   uint64_t full[kStages];
   int done[kStages];
@@ -936,15 +922,14 @@ struct PairShared {
 };
 constexpr int kPairBlocks = 4;   // resident blocks per SM the registers are held to (128 each)
 
-__device__ __forceinline__ void scalar_adj(const QDup& Q, const float2 (&F)[12], Thr th, float2 (&a)[12], bool second) {
-  const QRec q{Q.qx.x, Q.qy.x, Q.qz.x, Q.gr.x, Q.gi.x, 0.f, 0.f, 0.f};
-  float f[12], d[12];
+__device__ __forceinline__ void scalar_adj(const QRec& Q, const float2 (&F)[12], Thr th, float2 (&a)[12], bool second) {
+    float f[12], d[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
     f[k] = second ? F[k].y : F[k].x;
     d[k] = 0.f;
   }
-  face_adj(q, make_float4(f[0], f[1], f[2], f[3]), make_float4(f[4], f[5], f[6], f[7]),
+  face_adj(Q, make_float4(f[0], f[1], f[2], f[3]), make_float4(f[4], f[5], f[6], f[7]),
            make_float4(f[8], f[9], f[10], f[11]), th, d);
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
@@ -954,10 +939,10 @@ __device__ __forceinline__ void scalar_adj(const QDup& Q, const float2 (&F)[12],
 }
 
 // live: the warp holds a face.  Returns false when a wait gave up.
-__device__ __forceinline__ bool pair_run(PairShared& sh, const QDup* rec, int64_t nq, const float2 (&F)[12], bool live,
+__device__ __forceinline__ bool pair_run(PairShared& sh, const QRec* rec, int64_t nq, const float2 (&F)[12], bool live,
                                          Thr th) {
   using V = float2;
-  Ring<QDup, kQTile, kBwdNT> ring{sh.slots, sh.full, sh.done, &sh.issued, rec, nq, (int)((nq + kQTile - 1) / kQTile)};
+  Ring<QRec, kQTile, kBwdNT> ring{sh.slots, sh.full, sh.done, &sh.issued, rec, nq, (int)((nq + kQTile - 1) / kQTile)};
   ring.start();
 #pragma unroll
   for (int k = 0; k < 24; ++k) sh.acc[k][threadIdx.x] = make_float2(0.f, 0.f);
@@ -965,24 +950,25 @@ __device__ __forceinline__ bool pair_run(PairShared& sh, const QDup* rec, int64_
   for (int t = 0; t < ring.ntiles; ++t) {
     if (!ring.wait(t)) { ok = false; break; }
     if (live) {
-      const QDup* tq = ring.tile(t);
+      const QRec* tq = ring.tile(t);
       const int cnt = ring.count(t);
       V a[12];
 #pragma unroll
       for (int k = 0; k < 12; ++k) a[k] = vs<V>(0.f);
 #pragma unroll 1
       for (int j = 0; j < cnt; ++j) {
-        const QDup Q = tq[j];
-        const V a0 = vfma(Q.qx, F[3], vfma(Q.qy, F[4], vmul(Q.qz, F[5])));
-        const V a1 = vfma(Q.qx, F[6], vfma(Q.qy, F[7], vmul(Q.qz, F[8])));
+        const QRec Q = tq[j];
+        const V qx = vs<V>(Q.qx), qy = vs<V>(Q.qy), qz = vs<V>(Q.qz);
+        const V a0 = vfma(qx, F[3], vfma(qy, F[4], vmul(qz, F[5])));
+        const V a1 = vfma(qx, F[6], vfma(qy, F[7], vmul(qz, F[8])));
         const V s1 = vadd(a0, a1), m = vmul(a1, s1), P = vfma(a0, a0, m);
         // the largest |P| of the warp's faces decides, as in face_adj_t (the sign bit is cleared there
         // for the same reason)
         const float wmax = __uint_as_float(
             __reduce_max_sync(0xffffffffu, max(__float_as_uint(P.x) & 0x7fffffffu, __float_as_uint(P.y) & 0x7fffffffu)));
         if (wmax < th.hi) {
-          const V mu = vfma(Q.qx, F[0], vfma(Q.qy, F[1], vmul(Q.qz, F[2])));
-          const V s = vfma(Q.qx, F[9], vfma(Q.qy, F[10], vmul(Q.qz, F[11])));
+          const V mu = vfma(qx, F[0], vfma(qy, F[1], vmul(qz, F[2])));
+          const V s = vfma(qx, F[9], vfma(qy, F[10], vmul(qz, F[11])));
           if (wmax < kPShort) series_adj<0>(Q, mu, a0, a1, s1, m, s, a);
           else if (wmax < kP9) series_adj<1>(Q, mu, a0, a1, s1, m, s, a);
           else if (wmax < kPLong) series_adj<2>(Q, mu, a0, a1, s1, m, s, a);
@@ -1038,7 +1024,7 @@ __device__ __forceinline__ void pair_store(const PairShared& sh, int64_t m, int6
 }
 
 __global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bwd3(const Face32* __restrict__ faces, int64_t n_faces,
-                                                             const QDup* __restrict__ rec, int64_t n_q,
+                                                             const QRec* __restrict__ rec, int64_t n_q,
                                                              int64_t per_split, Thr th, double* __restrict__ partial,
                                                              uint32_t* status) {
   extern __shared__ __align__(128) unsigned char raw[];
@@ -1224,10 +1210,10 @@ __device__ __forceinline__ void bb_rows(const int64_t* q_off, int64_t i, int64_t
 }
 
 // D = 2: weight 2 g e^{-iQ.c}/|Q|^2 (records hold half segment vectors); D = 3: g e^{-iQ.c}/|Q|^2.
-template <int D, class Rec>
+template <int D>
 __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, const int64_t* __restrict__ q_off,
                                               const double* __restrict__ g, int64_t n_q, int64_t np,
-                                              const PolyC* __restrict__ pc, Rec* rec, int32_t* small,
+                                              const PolyC* __restrict__ pc, QRec* rec, int32_t* small,
                                               int32_t* small_cnt, WsHeader* h) {
   __shared__ int wcount[kAux / 32];
   __shared__ int base;
@@ -1264,7 +1250,7 @@ __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, cons
         wr = k * fmaf(gr, cp, -gi * sp);
         wi = k * fmaf(gr, sp, gi * cp);
       }
-      put_rec(rec[gb + l], qx, qy, qz, wr, wi);
+      rec[gb + l] = QRec{qx, qy, qz, wr, wi, -wi, 0.f, 0.f};
     }
     const unsigned m = __ballot_sync(0xffffffffu, is_small);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1502,7 +1488,7 @@ __global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bbwd3(const Face32* __r
                                                               const int64_t* __restrict__ off, int64_t nm,
                                                               const int64_t* __restrict__ bstart,
                                                               const int32_t* __restrict__ nblk,
-                                                              const QDup* __restrict__ rec,
+                                                              const QRec* __restrict__ rec,
                                                               const int64_t* __restrict__ q_off, int64_t n_q,
                                                               int64_t per_split, Thr th,
                                                               double* __restrict__ partial, uint32_t* status) {
@@ -1813,7 +1799,7 @@ int q_splits(int64_t n_items, int64_t n_q) {
 }
 
 // The same for the paired 3D adjoints' blocks (kPairBlocks resident ones per SM): 12 waves for one mesh
-// (81,920 faces x 32,768 Q: 6.03 / 5.91 / 5.89 ms for 6 / 12 / 25 waves, and the corner kernel, which
+// (81,920 faces x 32,768 Q, at an earlier stage: 6.03 / 5.91 / 5.89 ms for 6 / 12 / 25 waves, and the corner kernel, which
 // adds the chunks, 0.08 / 0.10 / 0.16 ms), 24 for a batch, whose blocks are uneven (96 meshes x 13,824
 // Q: 8.4 / 7.2 / 6.9 ms, corners 0.09 / 0.12 / 0.15 ms).
 int pair_splits(int64_t item_blocks, int64_t n_q, int waves) {
@@ -1857,7 +1843,7 @@ BwdLayout bwd_layout(int dim, int64_t n_verts, int64_t n_items, int64_t n_prep, 
   size_t o = al(sizeof(WsHeader));
   y.mparts = o;  o = al(o + sizeof(double) * (size_t)y.nblk);
   y.items = o;   o = al(o + (dim == 2 ? sizeof(Seg32) : sizeof(Face32)) * (size_t)std::max<int64_t>(n_items, 1));
-  y.qrec = o;    o = al(o + (dim == 2 ? sizeof(QRec) : sizeof(QDup)) * (size_t)std::max<int64_t>(n_q, 1));
+  y.qrec = o;    o = al(o + sizeof(QRec) * (size_t)std::max<int64_t>(n_q, 1));
   y.small = o;   o = al(o + sizeof(int32_t) * (size_t)std::max<int64_t>(n_q, 1));
   y.partial = o; o = al(o + sizeof(double) * nf * (size_t)y.ks * (size_t)std::max<int64_t>(n_items, 1));
   if (dim == 3) {
@@ -2020,7 +2006,7 @@ Bb3Layout bb3_layout(int64_t nv, int64_t nf, int64_t nm, int64_t n_q, bool per_m
   y.mc = o;      o = al(o + sizeof(PolyC) * nm1);
   y.nblk = o;    o = al(o + sizeof(int32_t) * nm1);
   y.bstart = o;  o = al(o + sizeof(int64_t) * nm1);
-  y.rec = o;     o = al(o + sizeof(QDup) * (size_t)rows);
+  y.rec = o;     o = al(o + sizeof(QRec) * (size_t)rows);
   y.small = o;   o = al(o + sizeof(int32_t) * (size_t)rows);
   y.scnt = o;    o = al(o + sizeof(int32_t) * nm1);
   y.partial = o; o = al(o + sizeof(double) * 12 * (size_t)y.ks * nf1);
@@ -2121,13 +2107,12 @@ int mesh3d_backward_body(const float* verts, int64_t n_verts, const int32_t* fac
   k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
   PFT_BWD_LAUNCH();
   const int bt = n_q >= 65536 ? kAux : 64;   // few points (faces below): smaller blocks, so that all SMs take part
-  k_bq<3, QDup><<<blocks(n_q, bt), bt, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QDup>(ws, y.qrec),
-                                               at<int32_t>(ws, y.small));
+  k_bq<3><<<blocks(n_q, bt), bt, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_faces, kPairFaces), (unsigned)y.ks);
   if (!allow_shared(k_bwd3)) return PFT_ERR_CUDA;
   PFT_MARK(g_ev_start);
-  k_bwd3<<<grid, kBwdNT, sizeof(PairShared), st>>>(at<Face32>(ws, y.items), n_faces, at<QDup>(ws, y.qrec), n_q,
+  k_bwd3<<<grid, kBwdNT, sizeof(PairShared), st>>>(at<Face32>(ws, y.items), n_faces, at<QRec>(ws, y.qrec), n_q,
                                                    y.per_split, th, at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
@@ -2193,7 +2178,7 @@ int pft2d_polygons_backward(const float* verts, int64_t n_verts, const int64_t* 
                     y.nblk, st) != cudaSuccess)
     return PFT_ERR_CUDA;
   ++g_bwd_launches;
-  k_bq<2, QRec><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
+  k_bq<2><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_verts, kBwdNT), (unsigned)y.ks);
   PFT_MARK(g_ev_start);
@@ -2297,7 +2282,7 @@ int pft3d_mesh_qgrad(const float* verts, int64_t n_verts, const int32_t* faces, 
   ++g_bwd_launches;
   const int32_t* perm = nullptr;
   if (int e = qg_order(3, y, q, n_q, ws, st, perm)) return e;
-  k_bq<3, QRec><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
+  k_bq<3><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
                                               perm);
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_q, kBwdNT), (unsigned)y.ks);
@@ -2358,7 +2343,7 @@ int pft2d_polygons_qgrad(const float* verts, int64_t n_verts, const int64_t* loo
   ++g_bwd_launches;
   const int32_t* perm = nullptr;
   if (int e = qg_order(2, y, q, n_q, ws, st, perm)) return e;
-  k_bq<2, QRec><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
+  k_bq<2><<<blocks(n_q, kAux), kAux, 0, st>>>(q, grad_out, n_q, h, 2.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small),
                                               perm);
   PFT_BWD_LAUNCH();
   dim3 grid(blocks(n_q, kBwdNT), (unsigned)y.ks);
@@ -2417,7 +2402,7 @@ int pft2d_polygons_batched_backward(const float* verts, int64_t n_verts, const i
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_polys, bstart);
   PFT_BWD_LAUNCH();
-  k_bbq<2, QRec><<<(unsigned)n_polys, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
+  k_bbq<2><<<(unsigned)n_polys, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
                                             at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
   PFT_BWD_LAUNCH();
   if (y.grid > INT32_MAX) return PFT_ERR_UNSUPPORTED;
@@ -2481,14 +2466,14 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   int64_t* start = at<int64_t>(ws, y.start);
   k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
   PFT_BWD_LAUNCH();
-  k_bbq<3, QDup><<<(unsigned)n_meshes, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_meshes, mc, at<QDup>(ws, y.rec),
+  k_bbq<3><<<(unsigned)n_meshes, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
                                                 at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
   PFT_BWD_LAUNCH();
   dim3 grid((unsigned)y.grid, (unsigned)y.ks);
   if (!allow_shared(k_bbwd3)) return PFT_ERR_CUDA;
   PFT_MARK(g_ev_start);
   k_bbwd3<<<grid, kBwdNT, sizeof(PairShared), st>>>(recs, n_faces, mesh_off, n_meshes, bstart, nblk,
-                                   at<QDup>(ws, y.rec), q_off, n_q, y.per_split, th, at<double>(ws, y.partial), &h->status);
+                                   at<QRec>(ws, y.rec), q_off, n_q, y.per_split, th, at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
   k_bbcorner3<<<blocks(n_faces, kAux), kAux, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes,
