@@ -132,8 +132,9 @@ int resolve_batched(int dim, const pft_options* o, bool shared_q, int64_t n_q, b
 
 int batched_blocks_per_sm(int dim, bool fp64, int r, int nt);
 
+// schedule = false: only the header (sizes), for the workspace size; no items are made or dealt.
 int build_plan(int dim, const int64_t* poly_off, int64_t n_polys, const int64_t* q_off, int64_t n_q,
-               const pft_options* opts, HostPlan& P) {
+               const pft_options* opts, HostPlan& P, bool schedule = true) {
   bool fp64;
   int r, nt, q_order;
   float tau;
@@ -156,25 +157,27 @@ int build_plan(int dim, const int64_t* poly_off, int64_t n_polys, const int64_t*
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t G = std::max(1, sms) * (int64_t)batched_blocks_per_sm(dim, fp64, r, nt);
 
-  P.pplan.resize((size_t)n_polys);
+  if (schedule) P.pplan.resize((size_t)n_polys);
   std::vector<int64_t> cost;
-  int64_t part_rows = 0;
+  int64_t part_rows = 0, n_items = 0, n_mc = 0;
   for (int64_t i = 0; i < n_polys; ++i) {
-    PolyPlan& pp = P.pplan[(size_t)i];
+    PolyPlan pp{};
     pp.seg_begin = poly_off[i];
     pp.n_seg = (int32_t)(poly_off[i + 1] - poly_off[i]);
     pp.q_begin = q_off ? q_off[i] : 0;
     pp.n_q = (int32_t)(q_off ? q_off[i + 1] - q_off[i] : n_q);
     pp.out_base = q_off ? q_off[i] : i * n_q;
     pp.n_chunks = pp.n_seg > 0 ? (int32_t)((pp.n_seg + kChunk - 1) / kChunk) : 1;
-    pp.part_base = 0;
-    pp.pad = 0;
     if (pp.n_chunks > 1) {
       pp.part_base = part_rows;
       part_rows += (int64_t)pp.n_chunks * pp.n_q;
-      P.mc.push_back((int32_t)i);
+      ++n_mc;
+      if (schedule) P.mc.push_back((int32_t)i);
     }
     const int64_t n_qt = (pp.n_q + qt - 1) / qt;
+    n_items += (int64_t)pp.n_chunks * n_qt;
+    if (!schedule) continue;
+    P.pplan[(size_t)i] = pp;
     for (int32_t c = 0; c < pp.n_chunks; ++c) {
       const int64_t segs = std::min<int64_t>(kChunk, std::max<int64_t>(0, pp.n_seg - (int64_t)c * kChunk));
       for (int64_t t = 0; t < n_qt; ++t) {
@@ -184,29 +187,30 @@ int build_plan(int dim, const int64_t* poly_off, int64_t n_polys, const int64_t*
       }
     }
   }
-  // longest processing time first onto the least loaded block (ties: lowest index)
-  const int64_t n_items = (int64_t)P.items.size();
-  std::vector<int64_t> order((size_t)n_items);
-  std::iota(order.begin(), order.end(), 0);
-  std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) { return cost[a] > cost[b]; });
-  using Slot = std::pair<int64_t, int64_t>;   // (load, block)
-  std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
-  for (int64_t b = 0; b < G; ++b) heap.push({0, b});
-  std::vector<std::vector<int64_t>> lists((size_t)G);
-  for (int64_t k : order) {
-    Slot s = heap.top();
-    heap.pop();
-    lists[(size_t)s.second].push_back(k);
-    heap.push({s.first + cost[k], s.second});
+  if (schedule) {
+    // longest processing time first onto the least loaded block (ties: lowest index)
+    std::vector<int64_t> order((size_t)n_items);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) { return cost[a] > cost[b]; });
+    using Slot = std::pair<int64_t, int64_t>;   // (load, block)
+    std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
+    for (int64_t b = 0; b < G; ++b) heap.push({0, b});
+    std::vector<int32_t> block((size_t)n_items);   // of the k-th item in that order
+    P.cta_off.assign((size_t)G + 1, 0);
+    for (int64_t k = 0; k < n_items; ++k) {
+      const Slot s = heap.top();
+      heap.pop();
+      block[(size_t)k] = (int32_t)s.second;
+      ++P.cta_off[(size_t)s.second + 1];
+      heap.push({s.first + cost[(size_t)order[(size_t)k]], s.second});
+    }
+    std::partial_sum(P.cta_off.begin(), P.cta_off.end(), P.cta_off.begin());
+    std::vector<int32_t> next(P.cta_off.begin(), P.cta_off.end() - 1);
+    std::vector<BItem> sorted((size_t)n_items);
+    for (int64_t k = 0; k < n_items; ++k)
+      sorted[(size_t)next[(size_t)block[(size_t)k]]++] = P.items[(size_t)order[(size_t)k]];
+    P.items.swap(sorted);
   }
-  std::vector<BItem> sorted;
-  sorted.reserve((size_t)n_items);
-  P.cta_off.assign((size_t)G + 1, 0);
-  for (int64_t b = 0; b < G; ++b) {
-    for (int64_t k : lists[(size_t)b]) sorted.push_back(P.items[(size_t)k]);
-    P.cta_off[(size_t)b + 1] = (int32_t)sorted.size();
-  }
-  P.items.swap(sorted);
   std::memset(&P.h, 0, sizeof(P.h));
   P.h.magic = kPlanMagic;
   P.h.n_polys = n_polys;
@@ -214,7 +218,7 @@ int build_plan(int dim, const int64_t* poly_off, int64_t n_polys, const int64_t*
   P.h.n_q = n_q;
   P.h.n_items = n_items;
   P.h.n_cta = G;
-  P.h.n_mc = (int64_t)P.mc.size();
+  P.h.n_mc = n_mc;
   P.h.part_rows = part_rows;
   P.h.n_out = n_out;
   P.h.r = r;
@@ -1059,7 +1063,7 @@ static_assert(sizeof(PlanHandle) <= sizeof(pft_batched_plan), "plan handle fits 
 size_t workspace_impl(int dim, int64_t n_items, const int64_t* off_host, int64_t n_shapes, const int64_t* q_off_host,
                       int64_t n_q, const pft_options* opts) {
   HostPlan P;
-  if (n_items < 0 || build_plan(dim, off_host, n_shapes, q_off_host, n_q, opts, P) != PFT_OK) return 0;
+  if (n_items < 0 || build_plan(dim, off_host, n_shapes, q_off_host, n_q, opts, P, false) != PFT_OK) return 0;
   if (P.h.n_verts != n_items) return 0;
   return layout_of(P.h).total;
 }
@@ -1073,14 +1077,17 @@ int prepare_impl(int dim, const int64_t* off_host, int64_t n_shapes, const int64
   const BLayout y = layout_of(P.h);
   if (ws == nullptr || reinterpret_cast<uintptr_t>(ws) % 256 != 0 || ws_bytes < y.total) return PFT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // the plan's regions follow one another: one copy
+  std::vector<char> stage(y.info - y.plan_hdr);
   auto put = [&](size_t off, const void* src, size_t bytes) {
-    return bytes == 0 || cudaMemcpyAsync(at<char>(ws, off), src, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    if (bytes > 0) std::memcpy(stage.data() + (off - y.plan_hdr), src, bytes);
   };
-  bool ok = put(y.plan_hdr, &P.h, sizeof(P.h)) &&
-            put(y.cta_off, P.cta_off.data(), sizeof(int32_t) * P.cta_off.size()) &&
-            put(y.items, P.items.data(), sizeof(BItem) * P.items.size()) &&
-            put(y.pplan, P.pplan.data(), sizeof(PolyPlan) * P.pplan.size()) &&
-            put(y.mc, P.mc.data(), sizeof(int32_t) * P.mc.size());
+  put(y.plan_hdr, &P.h, sizeof(P.h));
+  put(y.cta_off, P.cta_off.data(), sizeof(int32_t) * P.cta_off.size());
+  put(y.items, P.items.data(), sizeof(BItem) * P.items.size());
+  put(y.pplan, P.pplan.data(), sizeof(PolyPlan) * P.pplan.size());
+  put(y.mc, P.mc.data(), sizeof(int32_t) * P.mc.size());
+  bool ok = cudaMemcpyAsync(at<char>(ws, y.plan_hdr), stage.data(), stage.size(), cudaMemcpyHostToDevice, st) == cudaSuccess;
   ok = ok && cudaStreamSynchronize(st) == cudaSuccess;   // the host vectors die on return
   if (!ok) return PFT_ERR_CUDA;
   PlanHandle ph{};
