@@ -1149,12 +1149,24 @@ __device__ __forceinline__ float block_minmax_f(float x, bool is_max, float* sh)
   return r;
 }
 
+// Q coordinates as float pairs (q rounded to float, and the rest), for k_bbq: converted once here, spread
+// over the prep kernel's grid.
+__device__ __forceinline__ void split_q(const double* __restrict__ q, int64_t n, float2* __restrict__ qs) {
+  for (int64_t i = blockIdx.x * (int64_t)kAux + threadIdx.x; i < n; i += (int64_t)gridDim.x * kAux) {
+    const double x = q[i];
+    const float hi = (float)x;
+    qs[i] = make_float2(hi, (float)(x - (double)hi));
+  }
+}
+
 // One block per polygon: offset checks, bounding-box centre, segment records relative to it,
 // max radius, and the number of pair blocks (kBbSegs segments each) the polygon needs.
 __global__ void __launch_bounds__(kAux) k_bbprep(const float* __restrict__ v, int64_t nv,
                                                  const int64_t* __restrict__ off, int64_t np, Seg32* segs,
-                                                 PolyC* pc, int32_t* nblk, WsHeader* h) {
+                                                 PolyC* pc, int32_t* nblk, const double* __restrict__ q, int64_t n_q,
+                                                 float2* __restrict__ qs, WsHeader* h) {
   __shared__ float sh[kAux / 32];
+  split_q(q, 2 * n_q, qs);
   const int64_t i = blockIdx.x;
   const int64_t s0 = off[i], s1 = off[i + 1];
   if (threadIdx.x == 0 && (s1 < s0 || s0 < 0 || s1 > nv || (i == 0 && s0 != 0) || (i == np - 1 && s1 != nv)))
@@ -1209,9 +1221,16 @@ __device__ __forceinline__ void bb_rows(const int64_t* q_off, int64_t i, int64_t
   }
 }
 
-// D = 2: weight 2 g e^{-iQ.c}/|Q|^2 (records hold half segment vectors); D = 3: g e^{-iQ.c}/|Q|^2.
+// D = 2: weight 2 g e^{-iQ.c}/|Q|^2 (records hold half segment vectors); D = 3: g e^{-iQ.c}/|Q|^2.  Bound: the
+// FP64 pipe if the phase runs in FP64 (16 operations a row: 140 us for 1,000 polygons x 4,095 Q), so the
+// phase and |Q|^2 are carried as float pairs (the scheme of the batched forward's finish: the phase less
+// its nearest multiple of 2 pi within 1.2e-7 rad, the factor rounded once), the caller's Q coming in split
+// (qs); rows near the small-|Q| bound and phases beyond 2^20 rad take FP64.
+constexpr float kTwoPiHi32 = 6.28318548202514648438f;    // 2 pi rounded to FP32
+constexpr float kTwoPiLo32 = -1.7484555314695172e-07f;   // 2 pi - kTwoPiHi32, rounded to FP32
 template <int D>
-__global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, const int64_t* __restrict__ q_off,
+__global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, const float2* __restrict__ qs,
+                                              const int64_t* __restrict__ q_off,
                                               const double* __restrict__ g, int64_t n_q, int64_t np,
                                               const PolyC* __restrict__ pc, QRec* rec, int32_t* small,
                                               int32_t* small_cnt, WsHeader* h) {
@@ -1225,6 +1244,13 @@ __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, cons
     set_status(&h->status, ST_OFFSETS);
   int64_t qb, gb, nqi;
   bb_rows(q_off, i, n_q, qb, gb, nqi);
+  const double c[3] = {P.cx, P.cy, P.cz};
+  float chi[3], clo[3];   // the centre as float pairs
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    chi[d] = (float)c[d];
+    clo[d] = (float)(c[d] - (double)chi[d]);
+  }
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
   for (int64_t l0 = 0; l0 < nqi; l0 += kAux) {
@@ -1232,25 +1258,46 @@ __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, cons
     bool is_small = false;
     if (l < nqi) {
       // the record holds Q rounded to float; the weight's phase and factor take the caller's Q
-      const double Qx = q[D * (qb + l)], Qy = q[D * (qb + l) + 1], Qz = D == 3 ? q[D * (qb + l) + D - 1] : 0.0;
-      const float qx = (float)Qx, qy = (float)Qy, qz = (float)Qz;
-      const double q2 = Qx * Qx + Qy * Qy + Qz * Qz;
+      float2 Q[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+      for (int d = 0; d < D; ++d) Q[d] = qs[D * (qb + l) + d];
+      // |Q|^2 = n + nt and Q.c = s + t
+      float n = 0.f, nt = 0.f, s = 0.f, t = 0.f;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        const float a = Q[d].x * Q[d].x, b = Q[d].x * chi[d];
+        float e, f;
+        two_sum(n, a, n, e);
+        nt += e + fmaf(2.f * Q[d].x, Q[d].y, fmaf(Q[d].x, Q[d].x, -a));
+        two_sum(s, b, s, f);
+        t += f + fmaf(Q[d].x, chi[d], -b);
+      }
+#pragma unroll
+      for (int d = 0; d < D; ++d) t = fmaf(Q[d].y, chi[d], fmaf(Q[d].x, clo[d], t));
+      if (!(n * P.rmax * P.rmax > 1.01f * (float)(kTauSmallQ * kTauSmallQ))) {
+        const double Qx = q[D * (qb + l)], Qy = q[D * (qb + l) + 1], Qz = D == 3 ? q[D * (qb + l) + D - 1] : 0.0;
+        const double q2 = q_norm2(Qx, Qy, Qz);
+        is_small = q2 == 0.0 || q2 * ((double)P.rmax * (double)P.rmax) < kTauSmallQ * kTauSmallQ;
+      }
       float wr = 0.f, wi = 0.f;
-      if (q2 == 0.0 || q2 * ((double)P.rmax * (double)P.rmax) < kTauSmallQ * kTauSmallQ) {
-        is_small = true;
-      } else {
-        // e^{-iQ.c}: the phase in FP64, less its nearest multiple of 2 pi (FP64), then an FP32
-        // sincos on [-pi, pi]; the record holds FP32 weights, so this loses nothing further
-        const double ph = -(Qx * P.cx + Qy * P.cy + Qz * P.cz);
-        const float pr = (float)fma(-rint(ph * kInvTwoPiD), kTwoPiD, ph);
+      if (!is_small) {
+        float pr;   // Q.c less its nearest multiple of 2 pi
+        if (fabsf(s) < 1048576.f) {
+          const float k = rintf(s * kInvTwoPi);
+          pr = fmaf(-k, kTwoPiHi32, s) + fmaf(-k, kTwoPiLo32, t);
+        } else {
+          double ph = 0.0;
+          for (int d = 0; d < D; ++d) ph = fma(q[D * (qb + l) + d], d == 0 ? P.cx : (d == 1 ? P.cy : P.cz), ph);
+          pr = (float)fma(-rint(ph * kInvTwoPiD), kTwoPiD, ph);
+        }
         float sp, cp;
-        sincosf(pr, &sp, &cp);
+        sincosf(-pr, &sp, &cp);
         const float gr = (float)g[2 * (gb + l)], gi = (float)g[2 * (gb + l) + 1];
-        const float k = (D == 2 ? 2.0f : 1.0f) / (float)q2;
+        const float k = n > 3e38f ? 0.f : (D == 2 ? 2.0f : 1.0f) / (n + nt);   // |Q|^2 beyond FP32: 0
         wr = k * fmaf(gr, cp, -gi * sp);
         wi = k * fmaf(gr, sp, gi * cp);
       }
-      rec[gb + l] = QRec{qx, qy, qz, wr, wi, -wi, 0.f, 0.f};
+      rec[gb + l] = QRec{Q[0].x, Q[1].x, Q[2].x, wr, wi, -wi, 0.f, 0.f};
     }
     const unsigned m = __ballot_sync(0xffffffffu, is_small);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1413,8 +1460,11 @@ __global__ void k_bbvert(const float* __restrict__ v, int64_t nv, const int64_t*
 __global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, int64_t nv,
                                                   const int32_t* __restrict__ f, int64_t nf,
                                                   const int64_t* __restrict__ off, int64_t nm, Face32* recs,
-                                                  PolyC* mc, int32_t* nblk, int32_t* __restrict__ deg, WsHeader* h) {
+                                                  PolyC* mc, int32_t* nblk, int32_t* __restrict__ deg,
+                                                  const double* __restrict__ q, int64_t n_q, float2* __restrict__ qs,
+                                                  WsHeader* h) {
   __shared__ float sh[kAux / 32];
+  split_q(q, 3 * n_q, qs);
   const int64_t i = blockIdx.x;
   const int64_t s0 = off[i], s1 = off[i + 1];
   if (threadIdx.x == 0 && (s1 < s0 || s0 < 0 || s1 > nf || (i == 0 && s0 != 0) || (i == nm - 1 && s1 != nf)))
@@ -1951,7 +2001,7 @@ QgLayout qg2_layout(int64_t n_segs, int64_t n_prep, int64_t n_q, bool tiled) {
 
 // Batched 2D adjoint workspace.
 struct BbLayout {
-  size_t segs, pc, nblk, bstart, rec, small, scnt, partial, total;
+  size_t segs, pc, nblk, bstart, qsplit, rec, small, scnt, partial, total;
   int ks;
   int64_t per_split, grid;
 };
@@ -1974,6 +2024,7 @@ BbLayout bb_layout(int64_t nv, int64_t np, int64_t n_q, bool per_poly_q) {
   y.pc = o;      o = al(o + sizeof(PolyC) * (size_t)std::max<int64_t>(np, 1));
   y.nblk = o;    o = al(o + sizeof(int32_t) * (size_t)std::max<int64_t>(np, 1));
   y.bstart = o;  o = al(o + sizeof(int64_t) * (size_t)std::max<int64_t>(np, 1));
+  y.qsplit = o;  o = al(o + sizeof(float2) * 2 * (size_t)std::max<int64_t>(n_q, 1));
   y.rec = o;     o = al(o + sizeof(QRec) * (size_t)rows);
   y.small = o;   o = al(o + sizeof(int32_t) * (size_t)rows);
   y.scnt = o;    o = al(o + sizeof(int32_t) * (size_t)std::max<int64_t>(np, 1));
@@ -1986,7 +2037,7 @@ BbLayout bb_layout(int64_t nv, int64_t np, int64_t n_q, bool per_poly_q) {
 // Q records and small lists per (mesh, Q) row, FP64 partials per (Q chunk, face), corner adjoints
 // and the vertex -> face-corner CSR of the vertex gather.
 struct Bb3Layout {
-  size_t recs, mc, nblk, bstart, rec, small, scnt, partial, corner, deg, cursor, start, list, total;
+  size_t recs, mc, nblk, bstart, qsplit, rec, small, scnt, partial, corner, deg, cursor, start, list, total;
   int ks;
   int64_t per_split, grid;
 };
@@ -2006,6 +2057,7 @@ Bb3Layout bb3_layout(int64_t nv, int64_t nf, int64_t nm, int64_t n_q, bool per_m
   y.mc = o;      o = al(o + sizeof(PolyC) * nm1);
   y.nblk = o;    o = al(o + sizeof(int32_t) * nm1);
   y.bstart = o;  o = al(o + sizeof(int64_t) * nm1);
+  y.qsplit = o;  o = al(o + sizeof(float2) * 3 * (size_t)std::max<int64_t>(n_q, 1));
   y.rec = o;     o = al(o + sizeof(QRec) * (size_t)rows);
   y.small = o;   o = al(o + sizeof(int32_t) * (size_t)rows);
   y.scnt = o;    o = al(o + sizeof(int32_t) * nm1);
@@ -2398,11 +2450,12 @@ int pft2d_polygons_batched_backward(const float* verts, int64_t n_verts, const i
   PolyC* pc = at<PolyC>(ws, y.pc);
   int32_t* nblk = at<int32_t>(ws, y.nblk);
   int64_t* bstart = at<int64_t>(ws, y.bstart);
-  k_bbprep<<<(unsigned)n_polys, kAux, 0, st>>>(verts, n_verts, poly_off, n_polys, segs, pc, nblk, h);
+  k_bbprep<<<(unsigned)n_polys, kAux, 0, st>>>(verts, n_verts, poly_off, n_polys, segs, pc, nblk, q, n_q,
+                                               at<float2>(ws, y.qsplit), h);
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_polys, bstart);
   PFT_BWD_LAUNCH();
-  k_bbq<2><<<(unsigned)n_polys, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
+  k_bbq<2><<<(unsigned)n_polys, kAux, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
                                             at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
   PFT_BWD_LAUNCH();
   if (y.grid > INT32_MAX) return PFT_ERR_UNSUPPORTED;
@@ -2459,14 +2512,14 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   int32_t* nblk = at<int32_t>(ws, y.nblk);
   int64_t* bstart = at<int64_t>(ws, y.bstart);
   k_bbprep3<<<(unsigned)n_meshes, kAux, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes, recs, mc, nblk,
-                                                 deg, h);
+                                                 deg, q, n_q, at<float2>(ws, y.qsplit), h);
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_meshes, bstart);
   PFT_BWD_LAUNCH();
   int64_t* start = at<int64_t>(ws, y.start);
   k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
   PFT_BWD_LAUNCH();
-  k_bbq<3><<<(unsigned)n_meshes, kAux, 0, st>>>(q, q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
+  k_bbq<3><<<(unsigned)n_meshes, kAux, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
                                                 at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
   PFT_BWD_LAUNCH();
   dim3 grid((unsigned)y.grid, (unsigned)y.ks);
