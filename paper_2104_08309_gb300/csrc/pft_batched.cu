@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "pft_pairs.cuh"
+#include "pft_records.cuh"
 
 namespace pft {
 namespace {
@@ -439,71 +440,40 @@ __global__ void __launch_bounds__(kBThreads) k_bprep3(const float* __restrict__ 
                                                   N[0], N[1], N[2]};
     }
   } else {
-    // FP32 records without FP64 arithmetic, as k_bprep: each centred corner is a float pair
-    // s + t (TwoSum of the vertex and the centre's high part, less its low part); the centroid is
-    // rounded once from the pair sum over 3 (the remainder of the rounded quotient is exact through
-    // its FMA), q0, q1 and the edges from TwoSum differences, N = e1 x e2 with Kahan's FMA form of
-    // each 2 x 2 determinant.  The volume is the records' own: det(P0, P1, P2) = g . N for the
-    // centroid g and N = (P1 - P0) x (P2 - P0), so it is the compensated sum of g . N over 6, each
-    // product split exactly by its FMA.  Radius bound as in 2D.
+    // FP32 records without FP64 arithmetic (face_record32).  The volume is the records' own: det(P0, P1, P2)
+    // = g . N for the centroid g and N = (P1 - P0) x (P2 - P0), so it is the compensated sum of g . N over
+    // 6, each product split exactly by its FMA.
     float chi[3], clo[3];
     for (int d = 0; d < 3; ++d) {
       chi[d] = __double2float_rn(c[d]);
       clo[d] = __double2float_rn(c[d] - (double)chi[d]);
     }
-    auto det2 = [](float a, float b, float cc, float dd) {   // a b - cc dd
-      const float w = cc * dd;
-      return fmaf(a, b, -w) + fmaf(-cc, dd, w);
-    };
     CAcc va;
     va.init();
     for (int64_t j = threadIdx.x; j < n; j += kBThreads) {
       const int64_t m = pp.seg_begin + j;
-      float G[3] = {0.f, 0.f, 0.f}, Q0[3] = {0.f, 0.f, 0.f}, Q1[3] = {0.f, 0.f, 0.f}, Nn[3] = {0.f, 0.f, 0.f};
+      Face32 r{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       if (corner_ok(m)) {
-        float sp[3][3], tp[3][3];
+        float x[3][3];
         bool fin = true;
         for (int k = 0; k < 3; ++k)
           for (int d = 0; d < 3; ++d) {
-            const float x = v[3 * (int64_t)f[3 * m + k] + d];
-            fin = fin && isfinite(x);
-            float e;
-            two_sum(x, -chi[d], sp[k][d], e);
-            tp[k][d] = e - clo[d];
+            x[k][d] = v[3 * (int64_t)f[3 * m + k] + d];
+            fin = fin && isfinite(x[k][d]);
           }
         if (fin) {
-          float e1[3], e2[3];
-          for (int d = 0; d < 3; ++d) {
-            float a, ea, b, eb;
-            two_sum(sp[0][d], sp[1][d], a, ea);
-            two_sum(a, sp[2][d], b, eb);
-            const float lo = (ea + eb) + (tp[0][d] + tp[1][d] + tp[2][d]);
-            const float gh = b / 3.0f;
-            G[d] = gh + (fmaf(-gh, 3.0f, b) + lo) / 3.0f;
-            float x, ex;
-            two_sum(sp[0][d], -G[d], x, ex);
-            Q0[d] = x + (ex + tp[0][d]);
-            two_sum(sp[1][d], -G[d], x, ex);
-            Q1[d] = x + (ex + tp[1][d]);
-            two_sum(sp[1][d], -sp[0][d], x, ex);
-            e1[d] = x + (ex + (tp[1][d] - tp[0][d]));
-            two_sum(sp[2][d], -sp[0][d], x, ex);
-            e2[d] = x + (ex + (tp[2][d] - tp[0][d]));
-          }
-          Nn[0] = det2(e1[1], e2[2], e1[2], e2[1]);
-          Nn[1] = det2(e1[2], e2[0], e1[0], e2[2]);
-          Nn[2] = det2(e1[0], e2[1], e1[1], e2[0]);
+          float far;
+          r = face_record32<false>(x, chi, clo, far);
+          const float G[3] = {r.gx, r.gy, r.gz}, Nn[3] = {r.nx, r.ny, r.nz};
           for (int d = 0; d < 3; ++d) {
             const float pr = G[d] * Nn[d];
             va.add(pr);
             va.add(fmaf(G[d], Nn[d], -pr));
           }
-          for (int k = 0; k < 3; ++k)
-            rm = fmaxf(rm, sqrtf(fmaf(sp[k][0], sp[k][0], fmaf(sp[k][1], sp[k][1], sp[k][2] * sp[k][2]))) * 1.000001f);
+          rm = fmaxf(rm, far);
         }
       }
-      reinterpret_cast<Face32*>(recs)[m] = Face32{G[0], G[1], G[2], Q0[0], Q0[1], Q0[2], Q1[0], Q1[1], Q1[2],
-                                                  Nn[0], Nn[1], Nn[2]};
+      reinterpret_cast<Face32*>(recs)[m] = r;
     }
     vol = ((double)va.hi + (double)va.lo) / 6.0;
   }
@@ -833,7 +803,7 @@ __global__ void __launch_bounds__(kBThreads) k_bfinal(const BPlanHeader* ph, con
   if (!fp64) {
     const CenterF cf = center_f(pi);
     const float4* pf = reinterpret_cast<const float4*>(partial);
-    for (int64_t l = threadIdx.x; l < pp.n_q; l += kBThreads) {
+    for (int64_t l = blockIdx.y * (int64_t)kBThreads + threadIdx.x; l < pp.n_q; l += (int64_t)gridDim.y * kBThreads) {
       CAcc re, im;
       re.init();
       im.init();
@@ -856,7 +826,7 @@ __global__ void __launch_bounds__(kBThreads) k_bfinal(const BPlanHeader* ph, con
     }
     return;
   }
-  for (int64_t l = threadIdx.x; l < pp.n_q; l += kBThreads) {
+  for (int64_t l = blockIdx.y * (int64_t)kBThreads + threadIdx.x; l < pp.n_q; l += (int64_t)gridDim.y * kBThreads) {
     double re = 0.0, im = 0.0;
     for (int c = 0; c < pp.n_chunks; ++c) {
       const double2 p = partial[pp.part_base + (int64_t)c * pp.n_q + l];
@@ -1164,7 +1134,10 @@ int run_rest(const PlanHandle& p, void* ws, const double* q, double* out, WsHead
     return PFT_ERR_CUDA;
   ++g_batched_launches;
   if (p.n_mc > 0) {
-    k_bfinal<<<(unsigned)p.n_mc, kBThreads, 0, st>>>(phd, at<int32_t>(ws, (size_t)p.mc), pplan, info, q, partial,
+    // a few multi-chunk shapes: their Q points spread over blocks (24 meshes x 13,824 Q: 77 us at one each)
+    const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>((p.n_q + kBThreads - 1) / kBThreads,
+                                                                        4096 / std::min<int64_t>(p.n_mc, 4096)));
+    k_bfinal<<<dim3((unsigned)p.n_mc, gy), kBThreads, 0, st>>>(phd, at<int32_t>(ws, (size_t)p.mc), pplan, info, q, partial,
                                                       out, small, h, qlo);
     if (cudaGetLastError() != cudaSuccess) return PFT_ERR_CUDA;
     ++g_batched_launches;

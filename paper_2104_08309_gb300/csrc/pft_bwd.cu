@@ -20,6 +20,7 @@
 
 #include "pft_adj3.cuh"
 #include "pft_pairs.cuh"
+#include "pft_records.cuh"
 #include "pft_small.cuh"
 
 namespace pft {
@@ -1134,6 +1135,7 @@ struct PolyC {
   int32_t pad;
 };
 
+template <int NT = kAux>
 __device__ __forceinline__ float block_minmax_f(float x, bool is_max, float* sh) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -1144,7 +1146,7 @@ __device__ __forceinline__ float block_minmax_f(float x, bool is_max, float* sh)
   if (lane == 0) sh[wid] = x;
   __syncthreads();
   float r = sh[0];
-  for (int w = 1; w < kAux / 32; ++w) r = is_max ? fmaxf(r, sh[w]) : fminf(r, sh[w]);
+  for (int w = 1; w < NT / 32; ++w) r = is_max ? fmaxf(r, sh[w]) : fminf(r, sh[w]);
   __syncthreads();
   return r;
 }
@@ -1152,7 +1154,7 @@ __device__ __forceinline__ float block_minmax_f(float x, bool is_max, float* sh)
 // Q coordinates as float pairs (q rounded to float, and the rest), for k_bbq: converted once here, spread
 // over the prep kernel's grid.
 __device__ __forceinline__ void split_q(const double* __restrict__ q, int64_t n, float2* __restrict__ qs) {
-  for (int64_t i = blockIdx.x * (int64_t)kAux + threadIdx.x; i < n; i += (int64_t)gridDim.x * kAux) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double x = q[i];
     const float hi = (float)x;
     qs[i] = make_float2(hi, (float)(x - (double)hi));
@@ -1228,13 +1230,13 @@ __device__ __forceinline__ void bb_rows(const int64_t* q_off, int64_t i, int64_t
 // (qs); rows near the small-|Q| bound and phases beyond 2^20 rad take FP64.
 constexpr float kTwoPiHi32 = 6.28318548202514648438f;    // 2 pi rounded to FP32
 constexpr float kTwoPiLo32 = -1.7484555314695172e-07f;   // 2 pi - kTwoPiHi32, rounded to FP32
-template <int D>
-__global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, const float2* __restrict__ qs,
+template <int D, int NT>
+__global__ void __launch_bounds__(NT) k_bbq(const double* __restrict__ q, const float2* __restrict__ qs,
                                               const int64_t* __restrict__ q_off,
                                               const double* __restrict__ g, int64_t n_q, int64_t np,
                                               const PolyC* __restrict__ pc, QRec* rec, int32_t* small,
                                               int32_t* small_cnt, WsHeader* h) {
-  __shared__ int wcount[kAux / 32];
+  __shared__ int wcount[NT / 32];
   __shared__ int base;
   const int64_t i = blockIdx.x;
   const PolyC P = pc[i];
@@ -1253,7 +1255,7 @@ __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, cons
   }
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
-  for (int64_t l0 = 0; l0 < nqi; l0 += kAux) {
+  for (int64_t l0 = 0; l0 < nqi; l0 += NT) {
     const int64_t l = l0 + threadIdx.x;
     bool is_small = false;
     if (l < nqi) {
@@ -1304,7 +1306,7 @@ __global__ void __launch_bounds__(kAux) k_bbq(const double* __restrict__ q, cons
     if (lane == 0) wcount[wid] = __popc(m);
     __syncthreads();
     int before = 0, total = 0;
-    for (int w = 0; w < kAux / 32; ++w) {
+    for (int w = 0; w < NT / 32; ++w) {
       if (w < wid) before += wcount[w];
       total += wcount[w];
     }
@@ -1457,13 +1459,16 @@ __global__ void k_bbvert(const float* __restrict__ v, int64_t nv, const int64_t*
 // k_bbcorner3 (corner adjoints with the mesh's small-|Q| rows), and the vertex gather of the
 // single-mesh adjoint over all faces.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, int64_t nv,
+// One block per mesh; with FP64 records the largest mesh's block took 124 us (5,120 faces at 2 FP64
+// operations a clock).
+constexpr int kMeshT = 1024;
+__global__ void __launch_bounds__(kMeshT) k_bbprep3(const float* __restrict__ v, int64_t nv,
                                                   const int32_t* __restrict__ f, int64_t nf,
                                                   const int64_t* __restrict__ off, int64_t nm, Face32* recs,
                                                   PolyC* mc, int32_t* nblk, int32_t* __restrict__ deg,
                                                   const double* __restrict__ q, int64_t n_q, float2* __restrict__ qs,
                                                   WsHeader* h) {
-  __shared__ float sh[kAux / 32];
+  __shared__ float sh[kMeshT / 32];
   split_q(q, 3 * n_q, qs);
   const int64_t i = blockIdx.x;
   const int64_t s0 = off[i], s1 = off[i + 1];
@@ -1475,12 +1480,12 @@ __global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, i
     return a >= 0 && b >= 0 && c >= 0 && a < nv && b < nv && c < nv;
   };
   // corners at each vertex, for the gather: every face once, whatever the offsets say
-  for (int64_t m = i * kAux + threadIdx.x; m < nf; m += (int64_t)gridDim.x * kAux)
+  for (int64_t m = i * kMeshT + threadIdx.x; m < nf; m += (int64_t)gridDim.x * kMeshT)
     if (valid(m))
       for (int k = 0; k < 3; ++k) atomicAdd(&deg[f[3 * m + k]], 1);
   float mn[3] = {3.4e38f, 3.4e38f, 3.4e38f}, mx[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
   bool bad_index = false, bad_value = false;
-  for (int64_t j = threadIdx.x; j < n; j += kAux) {
+  for (int64_t j = threadIdx.x; j < n; j += kMeshT) {
     const int64_t m = b0 + j;
     if (!valid(m)) { bad_index = true; continue; }
     for (int k = 0; k < 3; ++k)
@@ -1495,36 +1500,27 @@ __global__ void __launch_bounds__(kAux) k_bbprep3(const float* __restrict__ v, i
   if (bad_value) set_status(&h->status, ST_NONFINITE);
   double c[3];
   for (int d = 0; d < 3; ++d) {
-    const float lo = block_minmax_f(mn[d], false, sh), hi = block_minmax_f(mx[d], true, sh);
+    const float lo = block_minmax_f<kMeshT>(mn[d], false, sh), hi = block_minmax_f<kMeshT>(mx[d], true, sh);
     c[d] = (n > 0 && lo <= hi) ? 0.5 * ((double)lo + (double)hi) : 0.0;
   }
-  float rm = 0.f;
-  for (int64_t j = threadIdx.x; j < n; j += kAux) {
+  float rm = 0.f, chi[3], clo[3];
+  for (int d = 0; d < 3; ++d) {
+    chi[d] = (float)c[d];
+    clo[d] = (float)(c[d] - (double)chi[d]);
+  }
+  for (int64_t j = threadIdx.x; j < n; j += kMeshT) {
     const int64_t m = b0 + j;
     Face32 r{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // skipped faces contribute 0
     if (valid(m)) {
-      double P[3][3], g[3], q0[3], q1[3];
+      float x[3][3], far;
       for (int k = 0; k < 3; ++k)
-        for (int d = 0; d < 3; ++d) P[k][d] = (double)v[3 * (int64_t)f[3 * m + k] + d] - c[d];
-      for (int d = 0; d < 3; ++d) {
-        g[d] = (P[0][d] + P[1][d] + P[2][d]) * (1.0 / 3.0);
-        q0[d] = P[0][d] - g[d];
-        q1[d] = P[1][d] - g[d];
-      }
-      const double e1[3] = {P[1][0] - P[0][0], P[1][1] - P[0][1], P[1][2] - P[0][2]};
-      const double e2[3] = {P[2][0] - P[0][0], P[2][1] - P[0][1], P[2][2] - P[0][2]};
-      const double N[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2],
-                           e1[0] * e2[1] - e1[1] * e2[0]};
-      r = Face32{(float)g[0], (float)g[1], (float)g[2], (float)q0[0], (float)q0[1], (float)q0[2],
-                 (float)q1[0], (float)q1[1], (float)q1[2], (float)N[0], (float)N[1], (float)N[2]};
-      // an upper bound of the radius: root in FP32, rounded up (squares beyond its range: FP64's root)
-      double r2 = 0.0;
-      for (int k = 0; k < 3; ++k) r2 = fmax(r2, P[k][0] * P[k][0] + P[k][1] * P[k][1] + P[k][2] * P[k][2]);
-      rm = fmaxf(rm, r2 < 1e38 && r2 > 1e-30 ? __fsqrt_ru(__double2float_ru(r2)) : __double2float_ru(sqrt(r2)));
+        for (int d = 0; d < 3; ++d) x[k][d] = v[3 * (int64_t)f[3 * m + k] + d];
+      r = face_record32<true>(x, chi, clo, far);
+      rm = fmaxf(rm, far);
     }
     recs[m] = r;
   }
-  rm = block_minmax_f(rm, true, sh);
+  rm = block_minmax_f<kMeshT>(rm, true, sh);
   if (threadIdx.x == 0) {
     mc[i] = PolyC{c[0], c[1], c[2], rm, 0};
     nblk[i] = (int32_t)((n + kPairFaces - 1) / kPairFaces);
@@ -2455,7 +2451,10 @@ int pft2d_polygons_batched_backward(const float* verts, int64_t n_verts, const i
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_polys, bstart);
   PFT_BWD_LAUNCH();
-  k_bbq<2><<<(unsigned)n_polys, kAux, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
+  // one block per shape, bound by latency where there are few
+  if (n_polys < 4 * sm_count()) k_bbq<2, 1024><<<(unsigned)n_polys, 1024, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
+                                            at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
+  else k_bbq<2, kAux><<<(unsigned)n_polys, kAux, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
                                             at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
   PFT_BWD_LAUNCH();
   if (y.grid > INT32_MAX) return PFT_ERR_UNSUPPORTED;
@@ -2511,7 +2510,7 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   PolyC* mc = at<PolyC>(ws, y.mc);
   int32_t* nblk = at<int32_t>(ws, y.nblk);
   int64_t* bstart = at<int64_t>(ws, y.bstart);
-  k_bbprep3<<<(unsigned)n_meshes, kAux, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes, recs, mc, nblk,
+  k_bbprep3<<<(unsigned)n_meshes, kMeshT, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes, recs, mc, nblk,
                                                  deg, q, n_q, at<float2>(ws, y.qsplit), h);
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_meshes, bstart);
@@ -2519,7 +2518,10 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   int64_t* start = at<int64_t>(ws, y.start);
   k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
   PFT_BWD_LAUNCH();
-  k_bbq<3><<<(unsigned)n_meshes, kAux, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
+  // one block per shape, bound by latency where there are few
+  if (n_meshes < 4 * sm_count()) k_bbq<3, 1024><<<(unsigned)n_meshes, 1024, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
+                                                at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
+  else k_bbq<3, kAux><<<(unsigned)n_meshes, kAux, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
                                                 at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
   PFT_BWD_LAUNCH();
   dim3 grid((unsigned)y.grid, (unsigned)y.ks);
