@@ -121,17 +121,16 @@ __device__ __forceinline__ void sinc_d(V u, V& S, V& dS) {
 #pragma unroll
   for (int e = 0; e < kE; ++e) big = big || (el(&v, e) > kPi2);
   if (__any_sync(__activemask(), big)) {   // warp-uniform: the SFU work only where some lane needs it
+    V s, c, r;
+    sincos_v(turn_rest(vmul(u, vs<V>(kInvTwoPi))), s, c);
+#pragma unroll
+    for (int e = 0; e < kE; ++e) el(&r, e) = rcp_approx(el(&u, e));
+    const V L = vmul(s, r), dL = vmul(vadd(c, vneg(L)), r);
 #pragma unroll
     for (int e = 0; e < kE; ++e) {
-      if (el(&v, e) > kPi2) {
-        const float ue = el(&u, e);
-        float s, c;
-        sincos_turns(ue * kInvTwoPi, &s, &c);
-        const float r = rcp_approx(ue);
-        const float Se = s * r;
-        el(&S, e) = Se;
-        el(&dS, e) = (c - Se) * r;
-      }
+      const bool b = el(&v, e) > kPi2;
+      el(&S, e) = b ? el(&L, e) : el(&S, e);
+      el(&dS, e) = b ? el(&dL, e) : el(&dS, e);
     }
   }
 }

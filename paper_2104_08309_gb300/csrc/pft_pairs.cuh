@@ -261,19 +261,22 @@ __device__ __forceinline__ void face_edge(V qx, V qy, V qz, const float4 A, cons
     u2[l] = vmul(u[l], u[l]);
     S[l] = sinc_poly_v(u2[l]);
   }
-  // rare: an edge with |Q.d_l| > 2 pi somewhere in the warp (face_edge runs warp-converged)
+  // an edge with |Q.d_l| > 2 pi somewhere in the warp (face_edge runs warp-converged): that edge's sincs on
+  // the SFU, both elements in paired code and selected by lane
   constexpr int kE = sizeof(V) / sizeof(float);
-  bool big = false;
+  bool big[3] = {false, false, false};
 #pragma unroll
   for (int l = kShared ? 1 : 0; l < 3; ++l)
 #pragma unroll
-    for (int e = 0; e < kE; ++e) big = big || (el(&u2[l], e) > kPi2);
-  if (__any_sync(0xffffffffu, big)) {
+    for (int e = 0; e < kE; ++e) big[l] = big[l] || (el(&u2[l], e) > kPi2);
+  if (__any_sync(0xffffffffu, big[0] || big[1] || big[2])) {
 #pragma unroll
     for (int l = kShared ? 1 : 0; l < 3; ++l)
+      if (__any_sync(0xffffffffu, big[l])) {
+        const V L = sinc_large(u[l]);
 #pragma unroll
-      for (int e = 0; e < kE; ++e)
-        if (el(&u2[l], e) > kPi2) el(&S[l], e) = sinc_large(el(&u[l], e));
+        for (int e = 0; e < kE; ++e) el(&S[l], e) = el(&u2[l], e) > kPi2 ? el(&L, e) : el(&S[l], e);
+      }
   }
   if (kShared) S[0] = S0;
   else S0 = S[0];
@@ -392,9 +395,11 @@ struct Pol2F32 {
       for (int r = 0; r < R; ++r) big = big || (el(u2, r) > kPi2);
       // segments long against 1/|Q|: the SFU sinc, only in warps where some lane needs it
       if (__any_sync(0xffffffffu, big)) {
+        V L[N];
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-          if (el(u2, r) > kPi2) el(S, r) = sinc_large(el(u, r));
+        for (int j = 0; j < N; ++j) L[j] = sinc_large(u[j]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) el(S, r) = el(u2, r) > kPi2 ? el(L, r) : el(S, r);
       }
 #pragma unroll
       for (int j = 0; j < N; ++j) {
