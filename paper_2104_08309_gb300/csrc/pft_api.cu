@@ -64,8 +64,8 @@ constexpr int64_t kGroupPairs = 24000000;
 // waves (the last wave >= 97 % as full as the others), each chunk at least two
 // tiles long; then, for launches of fewer than 40 waves with chunks to spare,
 // more chunks (below).
-// fine: more chunks than that where it pays (see layout_fwd for when it is not asked for).
-FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, bool fine) {
+// fine > 0: more chunks than that where it pays, up to `fine` of them (see layout_fwd for the values).
+FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, int fine) {
   FwdLaunch L{};
   L.r = o.r;
   L.nt = o.nt;
@@ -101,9 +101,10 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, bool fi
   if (k == 0) {
     const int64_t slots = (int64_t)device_sms() * fwd_blocks_per_sm(dim, o.fp64, L.r, L.nt, o.face_pairs > 0);
     int kmax = (int)std::max<int64_t>(1, std::min<int64_t>(64, item_tiles / 2));
-    // where that many chunks still leave resident blocks free: down to one tile each, up to 256
-    // (20,480 faces x 2,928 Q: 54 chunks 135 us, 80 chunks 116 us)
-    if (fine && !o.fp64 && L.q_tiles * kmax < slots) kmax = (int)std::min<int64_t>(256, item_tiles);
+    // where that many chunks still leave resident blocks free: down to one tile each, up to 256 chunks in 2D
+    // and more in 3D, whose finishing kernel adds them side by side
+    const bool under = fine && !o.fp64 && L.q_tiles * kmax < slots;
+    if (under) kmax = (int)std::min<int64_t>(dim == 3 ? fine : std::min(fine, 256), item_tiles);
     double best_eff = -1.0;
     int best_k = 1;
     k = 0;
@@ -114,6 +115,21 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, bool fi
       if (eff > best_eff + 1e-9) { best_eff = eff; best_k = c; }
     }
     if (k == 0) k = best_k;
+    if (under && dim == 3) {
+      // An SM takes about n + 1 times 9 us for a tile of n blocks (the one: a lone block's latency), so the
+      // chunks of t tiles that keep t (n + 1) smallest, n = blocks of the fullest SM.  Calls at 1, 2, 3 and
+      // 4 tiles a chunk: 20,480 faces x 2,925 Q 132, 149, 169, 171 us; x 4,913 Q 181, 199, 206, 214 us;
+      // 81,920 x 1,000 Q 166, 184, 177, 216 us; 327,680 x 1,000 Q 580, 578, 604, 611 us.  Whole waves, as
+      // below, and 256 chunks at most gave 155, 209, 199 and 743 us; 79,996 sliver faces x 512 and x 2,197 Q 420 -> 238 and
+      // 957 -> 645 us.
+      int64_t best = INT64_MAX;
+      for (int64_t t = (item_tiles + kmax - 1) / kmax; t <= std::max<int64_t>(1, item_tiles / 2) && 2 * t < best; ++t) {
+        const int64_t c = (item_tiles + t - 1) / t, n = (L.q_tiles * c + device_sms() - 1) / device_sms();
+        if (t * (n + 1) >= best) continue;
+        best = t * (n + 1);
+        k = (int)c;
+      }
+    }
     // Long launches: more chunks, up to about 40 waves (chunks of at least 4,096 faces or 8,192
     // segments, the last wave still >= 97 % full).  Blocks do not finish in waves: the resident
     // blocks of an SM share it unevenly, and the last blocks to start leave SMs partly idle for about
@@ -156,7 +172,7 @@ struct FwdLayout {
   FwdLaunch L;
 };
 
-FwdLayout layout_plan(int dim, const Opts& o, int64_t n_items, int64_t n_prep, int64_t n_q, bool fine) {
+FwdLayout layout_plan(int dim, const Opts& o, int64_t n_items, int64_t n_prep, int64_t n_q, int fine) {
   FwdLayout y{};
   y.L = plan_fwd(dim, o, n_items, n_q, fine);
   y.nblk = dim == 3 ? prep3_blocks(n_prep) : std::max(1, prep_blocks(n_prep));
@@ -185,12 +201,14 @@ FwdLayout layout_plan(int dim, const Opts& o, int64_t n_items, int64_t n_prep, i
 }
 
 // A finer plan's partial sums must not push a problem out of the allocation-free call's scratch: one
-// that fits it with the coarser plan keeps that.
+// that fits it with a coarser plan takes that (327,680 faces x 1,000 Q: 854 chunks; with the coarsest plan the
+// call took 1,151 us instead of 605).
 FwdLayout layout_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_prep, int64_t n_q) {
-  const FwdLayout y = layout_plan(dim, o, n_items, n_prep, n_q, true);
-  if (y.total - y.grown <= kScratchLimit) return y;
-  const FwdLayout z = layout_plan(dim, o, n_items, n_prep, n_q, false);
-  return z.total - z.grown <= kScratchLimit ? z : y;
+  for (const int fine : {2048, 1024, 512, 256, 128, 0}) {
+    const FwdLayout y = layout_plan(dim, o, n_items, n_prep, n_q, fine);
+    if (y.total - y.grown <= kScratchLimit) return y;
+  }
+  return layout_plan(dim, o, n_items, n_prep, n_q, 2048);
 }
 
 template <typename T>
