@@ -89,6 +89,13 @@ OPS_ADJ = {"common": {"fp32": 53, "sfu": 2},
 OPS_QADJ = {"common": {"fp32": 57, "sfu": 2},
             "short": {"fp32": 27, "sfu": 0}, "k9": {"fp32": 36, "sfu": 0}, "long": {"fp32": 44, "sfu": 0},
             "xlong": {"fp32": 80, "sfu": 0}, "edge": {"fp32": 155, "sfu": 5}}
+# The vertex adjoint (pair_run / series_adj in pft_bwd.cu and pft_adj3.cuh: two faces a thread in paired
+# instructions), whole cost per pair by series form (the k <= 7 form: projections and P 15, t 1, the form and
+# its derivatives 14, sincos scaling 1, weights and adjoints 21, range test 1, 12 updates); the edge sum runs
+# the scalar code above.
+OPS_PADJ = {"short": {"fp32": 65, "sfu": 2}, "k9": {"fp32": 74, "sfu": 2}, "long": {"fp32": 83, "sfu": 2},
+            "xlong": {"fp32": 115, "sfu": 2},
+            "edge": {k: OPS_ADJ["common"][k] + OPS_ADJ["edge"][k] for k in ("fp32", "sfu")}}
 FP32_LANES, SFU_LANES = 128, 16       # per SM per clock
 # A fixed per-pair count of the triangle term taken as the edge sum of Eq. 14 with a polynomial sinc
 # (projections, three edges' phase/sinc/term, face factor): the basis of frac_vs_survey_count.
@@ -259,10 +266,10 @@ def kernel_order(pft, q, qd, r, nt, n_items):
     return q
 
 
-def adjoint_branch_mix(v, f, q, tau=6.0, lanes="faces", n_warps=4096, seed=0):
+def adjoint_branch_mix(v, f, q, tau=6.0, lanes="faces", n_warps=4096, seed=0, width=32):
     """The pair adjoint's branch rule on a seeded sample of warps, and the per-pair cost it implies.
 
-    lanes="faces" (k_bwd: a warp holds 32 consecutive faces and takes one Q record at a time) or
+    lanes="faces" (a warp holds `width` consecutive faces, 64 in k_bwd3, and takes one Q record at a time) or
     "q" (k_qgrad: 32 consecutive Q points, one face at a time).  Per lane, with P in float32 and
     wmax the warp's largest P: short when every P < 1/4 (tau > 1; else every P < tau^2/4) or its
     own P < tau_lo^2/4; the k <= 9 form when not short and every P < 1 (and < tau^2/4); long when
@@ -273,9 +280,9 @@ def adjoint_branch_mix(v, f, q, tau=6.0, lanes="faces", n_warps=4096, seed=0):
     rng = np.random.default_rng(seed)
     v64 = v.astype(np.float64)
     if lanes == "faces":
-        fi = 32 * rng.integers(0, max(1, f.shape[0] // 32), n_warps)[:, None] + np.arange(32)[None, :]
+        fi = width * rng.integers(0, max(1, f.shape[0] // width), n_warps)[:, None] + np.arange(width)[None, :]
         fi = np.minimum(fi, f.shape[0] - 1)
-        qq = np.broadcast_to(q[rng.integers(0, q.shape[0], n_warps)][:, None, :], (n_warps, 32, 3))
+        qq = np.broadcast_to(q[rng.integers(0, q.shape[0], n_warps)][:, None, :], (n_warps, width, 3))
     else:
         qi = 32 * rng.integers(0, max(1, q.shape[0] // 32), n_warps)[:, None] + np.arange(32)[None, :]
         qq = q[np.minimum(qi, q.shape[0] - 1)]
@@ -797,18 +804,20 @@ def bench_adjoint(dev, warmup, steps):
     def rl(kernel, ms_k, lanes, table):
         # k_qgrad holds one Q point per thread, in the library's order (q_order's default)
         qm = kernel_order(pft, w.q, qd, 1, 128, w.faces.shape[0]) if lanes == "q" else w.q
-        lane, warp = adjoint_branch_mix(w.verts, w.faces, qm, lanes=lanes)
-        ops = adjoint_ops(warp, table)
-        issue = ops["fp32"] + ops["sfu"]
-        cyc = max(issue / FP32_LANES, ops["sfu"] / SFU_LANES)
+        paired = table is OPS_PADJ   # bound by the FP32 lanes; scalar code by the issue slots
+        lane, warp = adjoint_branch_mix(w.verts, w.faces, qm, lanes=lanes, width=64 if paired else 32)
+        ops = ({k: sum(warp[b] * table[b][k] for b in warp) for k in ("fp32", "sfu")} if paired
+               else adjoint_ops(warp, table))
+        cyc, issue = bound_cycles(ops, paired)
         peak = n_sm * clk * 1e6 * issue / cyc
         return {"bound": "alu", "kernel": kernel, "kernel_ms": ms_k, "achieved": issue * pairs / (ms_k / 1e3) / 1e12,
                 "peak": peak / 1e12, "unit": "Tops/s", "frac": issue * pairs / (ms_k / 1e3) / peak,
                 "ops_per_pair": ops, "branch_lanes": lane, "branch_warps": warp,
-                "peak_basis": f"{n_sm} SMs x 128 issue slots x {clk:.0f} MHz ({pk_kind} max SM clock)"}
+                "peak_basis": f"{n_sm} SMs x 128 {'FP32 lanes' if paired else 'issue slots'} x {clk:.0f} MHz "
+                              f"({pk_kind} max SM clock)"}
 
     return {"value": pairs / (ms_b / 1e3) / 1e9, "unit": UNIT + " (adjoint call)", "ms_adjoint": ms_b,
-            "roofline": rl("k_bwd<3,12>", ms_kbwd, "faces", OPS_ADJ),
+            "roofline": rl("k_bwd3", ms_kbwd, "faces", OPS_PADJ),
             "qgrad": {"value": pairs / (ms_q / 1e3) / 1e9, "unit": UNIT + " (Q-gradient call)", "ms": ms_q,
                       "launches": launches_q, "roofline": rl("k_qgrad", ms_kq, "q", OPS_QADJ)},
             "ms_forward_plus_adjoint": ms, "pairs_per_call": pairs, "faces": int(w.faces.shape[0]),
