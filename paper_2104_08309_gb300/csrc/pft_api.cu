@@ -105,23 +105,13 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, int fin
     // and more in 3D, whose finishing kernel adds them side by side
     const bool under = fine && !o.fp64 && L.q_tiles * kmax < slots;
     if (under) kmax = (int)std::min<int64_t>(dim == 3 ? fine : std::min(fine, 256), item_tiles);
-    double best_eff = -1.0;
-    int best_k = 1;
-    k = 0;
-    for (int c = 1; c <= kmax; ++c) {
-      const double waves = (double)(L.q_tiles * c) / (double)slots;
-      const double eff = waves / std::ceil(waves);
-      if (L.q_tiles * c >= slots && eff >= 0.97) { k = c; break; }
-      if (eff > best_eff + 1e-9) { best_eff = eff; best_k = c; }
-    }
-    if (k == 0) k = best_k;
     if (under && dim == 3) {
       // An SM takes about n + 1 times 9 us for a tile of n blocks (the one: a lone block's latency), so the
       // chunks of t tiles that keep t (n + 1) smallest, n = blocks of the fullest SM.  Calls at 1, 2, 3 and
       // 4 tiles a chunk: 20,480 faces x 2,925 Q 132, 149, 169, 171 us; x 4,913 Q 181, 199, 206, 214 us;
       // 81,920 x 1,000 Q 166, 184, 177, 216 us; 327,680 x 1,000 Q 580, 578, 604, 611 us.  Whole waves, as
-      // below, and 256 chunks at most gave 155, 209, 199 and 743 us; 79,996 sliver faces x 512 and x 2,197 Q 420 -> 238 and
-      // 957 -> 645 us.
+      // below, and 256 chunks at most gave 155, 209, 199 and 743 us; 79,996 sliver faces x 512 and x 2,197 Q
+      // 420 -> 238 and 957 -> 645 us.
       int64_t best = INT64_MAX;
       for (int64_t t = (item_tiles + kmax - 1) / kmax; t <= std::max<int64_t>(1, item_tiles / 2) && 2 * t < best; ++t) {
         const int64_t c = (item_tiles + t - 1) / t, n = (L.q_tiles * c + device_sms() - 1) / device_sms();
@@ -129,6 +119,16 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, int fin
         best = t * (n + 1);
         k = (int)c;
       }
+    } else {
+      double best_eff = -1.0;
+      int best_k = 1;
+      for (int c = 1; c <= kmax; ++c) {
+        const double waves = (double)(L.q_tiles * c) / (double)slots;
+        const double eff = waves / std::ceil(waves);
+        if (L.q_tiles * c >= slots && eff >= 0.97) { k = c; break; }
+        if (eff > best_eff + 1e-9) { best_eff = eff; best_k = c; }
+      }
+      if (k == 0) k = best_k;
     }
     // Long launches: more chunks, up to about 40 waves (chunks of at least 4,096 faces or 8,192
     // segments, the last wave still >= 97 % full).  Blocks do not finish in waves: the resident
