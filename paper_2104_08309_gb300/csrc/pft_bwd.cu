@@ -120,17 +120,20 @@ __device__ __forceinline__ void sinc_d(V u, V& S, V& dS) {
   bool big = false;
 #pragma unroll
   for (int e = 0; e < kE; ++e) big = big || (el(&v, e) > kPi2);
-  if (__any_sync(__activemask(), big)) {   // warp-uniform: the SFU work only where some lane needs it
-    V s, c, r;
-    sincos_v(turn_rest(vmul(u, vs<V>(kInvTwoPi))), s, c);
-#pragma unroll
-    for (int e = 0; e < kE; ++e) el(&r, e) = rcp_approx(el(&u, e));
-    const V L = vmul(s, r), dL = vmul(vadd(c, vneg(L)), r);
+  // warp-uniform: the SFU work only where some lane needs it (both elements evaluated and selected, as in the
+  // forward: k_bbwd on 2.7e6 segments x 4,096 Q 15.79 instead of 15.37 ms)
+  if (__any_sync(__activemask(), big)) {
 #pragma unroll
     for (int e = 0; e < kE; ++e) {
-      const bool b = el(&v, e) > kPi2;
-      el(&S, e) = b ? el(&L, e) : el(&S, e);
-      el(&dS, e) = b ? el(&dL, e) : el(&dS, e);
+      if (el(&v, e) > kPi2) {
+        const float ue = el(&u, e);
+        float s, c;
+        __sincosf(turn_rest(ue * kInvTwoPi), &s, &c);
+        const float r = rcp_approx(ue);
+        const float Se = s * r;
+        el(&S, e) = Se;
+        el(&dS, e) = (c - Se) * r;
+      }
     }
   }
 }

@@ -109,9 +109,9 @@ constexpr float kPi2 = 9.86960440108935861883f;   // pi^2
 
 // 2 pi (t - rint(t)) for a phase t in turns (the difference is exact).  Paired: rint by adding and subtracting
 // 1.5 * 2^23 (|t| < 2^22), two elements an instruction, where rintf is a conversion per element on the
-// SFU's pipe; the same bits.  With it, callers evaluate both elements and select, where each element had a
-// divergent block of its own: 32,760 sliver faces x 131,072 Q 11.21 -> 10.26 ms, 2.7e6 segments x 4,096 Q
-// 7.64 -> 7.34 ms.
+// SFU's pipe; the same bits.  With it, the forward kernels evaluate both elements and select, where each
+// element had a divergent block of its own: 32,760 sliver faces x 131,072 Q 11.21 -> 10.63 ms, 2.7e6 segments x
+// 4,096 Q 7.64 -> 7.34 ms.  The adjoint's sinc_d, with sin and cos, keeps a block per element.
 __device__ __forceinline__ float turn_rest(float t) { return kTwoPi * (t - rintf(t)); }
 __device__ __forceinline__ float2 turn_rest(float2 t) {
   constexpr float kM = 12582912.0f;

@@ -261,22 +261,23 @@ __device__ __forceinline__ void face_edge(V qx, V qy, V qz, const float4 A, cons
     u2[l] = vmul(u[l], u[l]);
     S[l] = sinc_poly_v(u2[l]);
   }
-  // an edge with |Q.d_l| > 2 pi somewhere in the warp (face_edge runs warp-converged): that edge's sincs on
-  // the SFU, both elements in paired code and selected by lane
+  // an edge with |Q.d_l| > 2 pi somewhere in the warp (face_edge runs warp-converged): the sincs on the SFU,
+  // both elements in paired code and selected by lane.  All edges at once: a vote for each (most slivers have
+  // a short one) ran the prism at 10.24 instead of 10.63 ms, but 327,680 faces x 881,730 Q, which has few edge
+  // sums, at 318.9 instead of 315.2 ms.
   constexpr int kE = sizeof(V) / sizeof(float);
-  bool big[3] = {false, false, false};
+  bool big = false;
 #pragma unroll
   for (int l = kShared ? 1 : 0; l < 3; ++l)
 #pragma unroll
-    for (int e = 0; e < kE; ++e) big[l] = big[l] || (el(&u2[l], e) > kPi2);
-  if (__any_sync(0xffffffffu, big[0] || big[1] || big[2])) {
+    for (int e = 0; e < kE; ++e) big = big || (el(&u2[l], e) > kPi2);
+  if (__any_sync(0xffffffffu, big)) {
 #pragma unroll
-    for (int l = kShared ? 1 : 0; l < 3; ++l)
-      if (__any_sync(0xffffffffu, big[l])) {
-        const V L = sinc_large(u[l]);
+    for (int l = kShared ? 1 : 0; l < 3; ++l) {
+      const V L = sinc_large(u[l]);
 #pragma unroll
-        for (int e = 0; e < kE; ++e) el(&S[l], e) = el(&u2[l], e) > kPi2 ? el(&L, e) : el(&S[l], e);
-      }
+      for (int e = 0; e < kE; ++e) el(&S[l], e) = el(&u2[l], e) > kPi2 ? el(&L, e) : el(&S[l], e);
+    }
   }
   if (kShared) S[0] = S0;
   else S0 = S[0];
