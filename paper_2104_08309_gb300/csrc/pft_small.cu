@@ -73,6 +73,9 @@ struct Sum32 {
 };
 // Barrier of one half of the block (id 1: the FP64 warps, 2: the FP32 warps).
 __device__ __forceinline__ void half_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kGW * 32) : "memory"); }
+// Barrier of the whole block for code where the halves are in different branches: __syncthreads() there would be
+// two barriers of the source, reached on a condition that is not the same for the block.
+__device__ __forceinline__ void both_sync() { asm volatile("bar.sync 3, %0;" ::"n"(kNT) : "memory"); }
 
 // One batch of 32 faces, one per lane, over kGW warps: the coefficients of h_k(x0, x1, x2) as
 // polynomials in Q, x_j = Q.p_j, degree by degree.  The complete homogeneous polynomials obey
@@ -299,7 +302,7 @@ __global__ void __launch_bounds__(kNT) k_small3(const float* __restrict__ v, int
 #pragma unroll
       for (int k = 0; k < 9; ++k) P[k / 3][k % 3] = face64[slot][k][lane];
       batch<double, Sum64, 0, kMomLo>(P, face64[slot][9][lane], buf, a64, lane, warp, 1);
-      __syncthreads();
+      both_sync();
     }
     // lanes -> one sum per monomial through shared memory (33 doubles a row: no bank conflicts)
 #pragma unroll
@@ -327,7 +330,7 @@ __global__ void __launch_bounds__(kNT) k_small3(const float* __restrict__ v, int
 #pragma unroll
       for (int k = 0; k < 9; ++k) P[k / 3][k % 3] = face32[slot][k][lane];
       batch<float, Sum32, kMomLo + 1, kMomK>(P, face32[slot][9][lane], buf, a32, lane, warp - kGW, 2);
-      __syncthreads();
+      both_sync();
     }
 #pragma unroll
     for (int k = kMomLo + 1; k <= kMomK; ++k)
