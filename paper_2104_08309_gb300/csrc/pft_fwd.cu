@@ -32,12 +32,14 @@ namespace {
 // 3D: whether Q point i (x: its coordinates as float) belongs to the small-|Q| pass (Q = 0 included),
 // and, if `list`, its entry in that pass's list.  Such points take no part in the pair sum (their place
 // in a warp's largest P is immaterial: it is the smallest).  The FP32 test settles all but those near
-// or below the bound.
+// or below the bound and those that leave the FP32 range on the way: the finishing kernel asks in FP64 alone,
+// and reads a place in the list for every point that it finds small.
 template <class QT>
 __device__ __forceinline__ bool list_small(const double* __restrict__ q, int64_t i, const QT (&x)[3], float rmax,
                                            WsHeader* h, int32_t* __restrict__ small, bool list) {
   const float fx = (float)x[0] * rmax, fy = (float)x[1] * rmax, fz = (float)x[2] * rmax;
-  if (fmaf(fx, fx, fmaf(fy, fy, fz * fz)) > 1.01f * (float)(kTauSmallQ * kTauSmallQ)) return false;
+  const float x2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+  if (x2 > 1.01f * (float)(kTauSmallQ * kTauSmallQ) && x2 <= 3.402823466e38f) return false;
   const double q2 = q_norm2(q[i * 3], q[i * 3 + 1], q[i * 3 + 2]);
   const bool is_small = q2 == 0.0 || small_q(q2, rmax);
   if (is_small && q2 != 0.0 && list) {
