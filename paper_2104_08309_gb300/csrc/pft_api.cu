@@ -328,8 +328,8 @@ int pft3d_mesh(const float* verts, int64_t n_verts, const int32_t* faces, int64_
                         h, at<int32_t>(ws, y.small), st, 2 * o.face_pairs, qperm));
   if (mark(o.ev_stop, st) != cudaSuccess) return PFT_ERR_CUDA;
   PFT_LAUNCH(launch_small3(verts, n_verts, faces, n_faces, q, h, mp, y.nblk, at<void>(ws, y.items), st));
-  PFT_LAUNCH(launch_finalize3d(q, n_q, n_faces, at<double2>(ws, y.partial), y.L.k_splits, h, at<int32_t>(ws, y.small),
-                               at<void>(ws, y.items), out, st));
+  PFT_LAUNCH(launch_finalize3d(verts, n_verts, faces, n_faces, q, n_q, at<double2>(ws, y.partial), y.L.k_splits, h,
+                               at<int32_t>(ws, y.small), at<void>(ws, y.items), out, st));
   return PFT_OK;
 }
 
@@ -377,8 +377,8 @@ int pft3d_polymesh(const float* verts, int64_t n_verts, const int32_t* face_idx,
                         h, at<int32_t>(ws, y.small), st, 0, qperm));
   if (mark(o.ev_stop, st) != cudaSuccess) return PFT_ERR_CUDA;
   PFT_LAUNCH(launch_small3(verts, n_verts, tris, n_tris, q, h, mp, y.nblk, at<void>(ws, y.items), st));
-  PFT_LAUNCH(launch_finalize3d(q, n_q, n_tris, at<double2>(ws, y.partial), y.L.k_splits, h, at<int32_t>(ws, y.small),
-                               at<void>(ws, y.items), out, st));
+  PFT_LAUNCH(launch_finalize3d(verts, n_verts, tris, n_tris, q, n_q, at<double2>(ws, y.partial), y.L.k_splits, h,
+                               at<int32_t>(ws, y.small), at<void>(ws, y.items), out, st));
   return PFT_OK;
 }
 

@@ -613,7 +613,7 @@ __global__ void __launch_bounds__(kAux) k_qsmall_part(const float* __restrict__ 
                                                       double* __restrict__ part) {
   __shared__ double sh[kAux / 32];
   const uint32_t count = h->small_q_count;   // <= n_q <= slots
-  if (count > (uint32_t)kSmallDirect) return;   // from the moments
+  if (!qsmall_direct(count, nf)) return;   // from the moments
   const int64_t nch = qsmall_chunks(count, nf, slots);
   const int64_t per = (nf + nch - 1) / nch;
   const double c[3] = {h->center[0], h->center[1], h->center[2]};
@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(kAux) k_qsmall_part(const float* __restrict__ 
   }
 }
 
-// With more than kSmallDirect listed points, S0 and dS0/dQ are the polynomial of the shape's moments
+// Where qsmall_direct does not hold, S0 and dS0/dQ are the polynomial of the shape's moments
 // (pft_small.cuh) and its gradient.
 // One warp per listed point (lane 0 finishes it).
 __global__ void k_qsmall_fin(int64_t nf, const double* __restrict__ q, const double* __restrict__ g,
@@ -666,7 +666,7 @@ __global__ void k_qsmall_fin(int64_t nf, const double* __restrict__ q, const dou
   const uint32_t count = h->small_q_count;
   const int64_t per = blockDim.x / 32;
   if (blockIdx.x * per >= count) return;
-  const bool direct = count <= (uint32_t)kSmallDirect;
+  const bool direct = qsmall_direct(count, nf);
   if (!direct) {
     for (int t = threadIdx.x; t < kMomN; t += blockDim.x) mom[t] = moments[t];
     __syncthreads();

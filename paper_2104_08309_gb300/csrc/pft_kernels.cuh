@@ -108,9 +108,9 @@ cudaError_t launch_finalize2d(const double* q, int64_t n_q, const double2* parti
 cudaError_t launch_smallq2d(const float* v, int64_t nv, const int64_t* off, int64_t nl, const double* q,
                             const WsHeader* h, const int32_t* small_list, double* out, cudaStream_t st);
 // scratch: what launch_small3 wrote.
-cudaError_t launch_finalize3d(const double* q, int64_t n_q, int64_t nf, const double2* partial, int k_splits,
-                              const WsHeader* h, const int32_t* small, const void* scratch, double* out,
-                              cudaStream_t st);
+cudaError_t launch_finalize3d(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q, int64_t n_q,
+                              const double2* partial, int k_splits, const WsHeader* h, const int32_t* small,
+                              const void* scratch, double* out, cudaStream_t st);
 
 // Prep blocks used for the per-block FP64 area/volume partial sums.
 constexpr int kPrepThreads = 256;

@@ -370,20 +370,24 @@ __global__ void k_finalize2d(const double* __restrict__ q, int64_t n_q, const do
   finish(Q, re, im, h, out + 2 * i);
 }
 
-// 3D: small-|Q| points (as k_fwd listed them) take their sum from k_small3's results.  A block finishes
-// per_block = 8 .. 256 points (a power of two), one per thread; those that need the moments' polynomial are
-// dealt to its warps.  With fewer points than threads, 256 / per_block lanes of a warp add a point's chunk
+// 3D: small-|Q| points (as k_fwd listed them) take their sum from k_small3's results, or over the faces of a
+// small mesh.  A block finishes per_block = 2 .. 256 points (a power of two), one per thread; those that need
+// the moments' polynomial, or the (point, 32 faces) of a direct sum, are dealt to its warps.  With fewer points than threads, 256 / per_block lanes of a warp add a point's chunk
 // sums side by side (in a fixed order): one thread per point walked 640 chunks in 50 us for 1,000 points
 // (81,920 faces x 1,000 Q at 640 chunks: the call 237 us, 166 us so).
 constexpr int kFinT = 256;
-__global__ void __launch_bounds__(kFinT) k_finalize3d(const double* __restrict__ q, int64_t n_q, int64_t nf,
+constexpr int kFewPts = 32;   // points of one round of the direct sums
+__global__ void __launch_bounds__(kFinT) k_finalize3d(const float* __restrict__ v, int64_t nv,
+                                                      const int32_t* __restrict__ f, int64_t nf,
+                                                      const double* __restrict__ q, int64_t n_q,
                                                       const double2* __restrict__ partial, int ks,
                                                       const WsHeader* __restrict__ h,
                                                       const int32_t* __restrict__ small,
                                                       const char* __restrict__ scratch, double* __restrict__ out,
                                                       int per_block) {
   __shared__ double mom[kMomN];
-  __shared__ double at[kFinT][3];   // a point's scaled Q, then its result
+  __shared__ double at[kFinT][3];   // a point's Q (scaled, for the moments), then its result
+  __shared__ double few_sums[kFewPts * (kFewFaces / 32)][2];
   __shared__ int list[kFinT];
   __shared__ int n_list;
   __shared__ double sums[kFinT / 2][2];
@@ -392,7 +396,7 @@ __global__ void __launch_bounds__(kFinT) k_finalize3d(const double* __restrict__
   const int64_t i = blockIdx.x * (int64_t)per_block + t;
   const bool mine = t < per_block && i < n_q;
   const float rmax = __uint_as_float(h->rmax_bits);
-  const bool direct = h->small_q_count <= (uint32_t)kSmallDirect;
+  const bool few = small_few(h->small_q_count, nf), direct = !few && h->small_q_count <= (uint32_t)kSmallDirect;
   double Q[3] = {0.0, 0.0, 0.0}, q2 = 0.0;
   bool is_small = false;
   if (mine) {
@@ -403,23 +407,58 @@ __global__ void __launch_bounds__(kFinT) k_finalize3d(const double* __restrict__
   if (!direct) {   // uniform
     if (t == 0) n_list = 0;
     if (__syncthreads_or(is_small)) {
+      const double unit = few ? 1.0 : (double)rmax;
       if (is_small) {
-        for (int d = 0; d < 3; ++d) at[t][d] = Q[d] * (double)rmax;
+        for (int d = 0; d < 3; ++d) at[t][d] = Q[d] * unit;
         list[atomicAdd(&n_list, 1)] = t;   // their order is immaterial
       }
-      for (int j = t; j < kMomN; j += kFinT) mom[j] = reinterpret_cast<const double*>(scratch)[j];
+      if (!few)
+        for (int j = t; j < kMomN; j += kFinT) mom[j] = reinterpret_cast<const double*>(scratch)[j];
       __syncthreads();
-      for (int e = t >> 5; e < n_list; e += kFinT / 32) {
-        const int l = list[e];
-        double re, im, g[3][2];
-        mom_eval<false>(mom, at[l][0], at[l][1], at[l][2], re, im, g);
-        __syncwarp();
-        if ((t & 31) == 0) {
-          at[l][0] = re;
-          at[l][1] = im;
+      if (few) {
+        const double c[3] = {h->center[0], h->center[1], h->center[2]};
+        const int ng = (int)((nf + 31) / 32);
+        for (int e0 = 0; e0 < n_list; e0 += kFewPts) {   // uniform
+          const int cnt = min(kFewPts, n_list - e0);
+          for (int u = t >> 5; u < cnt * ng; u += kFinT / 32) {
+            const int l = list[e0 + u / ng], m = (u % ng) * 32 + (t & 31);
+            double P[3][3], re = 0.0, im = 0.0;
+            if (m < nf && corners(v, nv, f, m, c, P)) {
+              double x[3];
+              for (int k = 0; k < 3; ++k) x[k] = at[l][0] * P[k][0] + at[l][1] * P[k][1] + at[l][2] * P[k][2];
+              const double det = det3(P);
+              tetra_series(x, re, im);
+              re *= det;
+              im *= det;
+            }
+            re = warp_sum(re);
+            im = warp_sum(im);
+            if ((t & 31) == 0) {
+              few_sums[u][0] = re;
+              few_sums[u][1] = im;
+            }
+          }
+          __syncthreads();
+          if (t < 2 * cnt) {
+            double s = 0.0;
+            for (int k = 0; k < ng; ++k) s += few_sums[(t >> 1) * ng + k][t & 1];
+            at[list[e0 + (t >> 1)]][t & 1] = s;
+          }
+          __syncthreads();
         }
+      } else {
+        for (int e = t >> 5; e < n_list; e += kFinT / 32) {
+          const int l = list[e];
+          double re, im, g[3][2];
+          mom_eval<false>(mom, at[l][0], at[l][1], at[l][2], re, im, g);
+          __syncwarp();
+          if ((t & 31) == 0) {
+            at[l][0] = re;
+            at[l][1] = im;
+          }
+        }
+        __syncthreads();
       }
-      __syncthreads();
     }
   }
   const int lanes = ks > 16 ? kFinT / per_block : 1;   // uniform; up to 16 chunks are two rounds of loads anyway
@@ -575,25 +614,26 @@ cudaError_t launch_fan3d(const int32_t* idx, int64_t n_idx, const int64_t* off, 
 
 // Points per block of the finishing kernels: few enough that a small call's FP64 arithmetic (the phase's
 // sincos, the small-|Q| polynomial) spreads over all SMs.
-static int finish_points(int64_t n_q) {
+static int finish_points(int64_t n_q, int least) {
   int n = 256;
-  while (n > 8 && n_q < (int64_t)n * 256) n /= 2;
+  while (n > least && n_q < (int64_t)n * 256) n /= 2;
   return n;
 }
 
 cudaError_t launch_finalize2d(const double* q, int64_t n_q, const double2* partial, int k_splits, WsHeader* h,
                               const double* mparts, int nm, int32_t* small_list, double* out, cudaStream_t st) {
-  const int nt = std::max(32, finish_points(n_q));
+  const int nt = finish_points(n_q, 32);
   k_finalize2d<<<(unsigned)((n_q + nt - 1) / nt), nt, 0, st>>>(q, n_q, partial, k_splits, h, mparts, nm, small_list,
                                                               out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize3d(const double* q, int64_t n_q, int64_t nf, const double2* partial, int k_splits,
-                              const WsHeader* h, const int32_t* small, const void* scratch, double* out,
-                              cudaStream_t st) {
-  const int per = finish_points(n_q);
-  k_finalize3d<<<(unsigned)((n_q + per - 1) / per), kFinT, 0, st>>>(q, n_q, nf, partial, k_splits, h, small,
+cudaError_t launch_finalize3d(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q, int64_t n_q,
+                              const double2* partial, int k_splits, const WsHeader* h, const int32_t* small,
+                              const void* scratch, double* out, cudaStream_t st) {
+  // side-by-side chunk sums take a warp's lanes a point at most, so 8 points or more
+  const int per = finish_points(n_q, nf <= kFewFaces && k_splits <= 16 ? 2 : 8);
+  k_finalize3d<<<(unsigned)((n_q + per - 1) / per), kFinT, 0, st>>>(v, nv, f, nf, q, n_q, partial, k_splits, h, small,
                                                                    static_cast<const char*>(scratch), out, per);
   return cudaGetLastError();
 }

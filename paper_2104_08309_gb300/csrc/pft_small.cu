@@ -133,22 +133,6 @@ __device__ __forceinline__ double wsum(double x) {
   return x;
 }
 
-// Corners of face m relative to c; false (and zeros) for an index out of range.
-__device__ __forceinline__ bool corners(const float* v, int64_t nv, const int32_t* f, int64_t m, const double* c,
-                                        double (&P)[3][3]) {
-  const int32_t id[3] = {f[3 * m], f[3 * m + 1], f[3 * m + 2]};
-  const bool ok = id[0] >= 0 && id[1] >= 0 && id[2] >= 0 && id[0] < nv && id[1] < nv && id[2] < nv;
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int d = 0; d < 3; ++d) P[k][d] = ok ? (double)v[3 * (int64_t)id[k] + d] - c[d] : 0.0;
-  return ok;
-}
-__device__ __forceinline__ double det3(const double (&P)[3][3]) {
-  return P[0][0] * (P[1][1] * P[2][2] - P[1][2] * P[2][1]) + P[0][1] * (P[1][2] * P[2][0] - P[1][0] * P[2][2]) +
-         P[0][2] * (P[1][0] * P[2][1] - P[1][1] * P[2][0]);
-}
-
 // dynamic shared memory: two levels of three nodes' coefficients in FP64 (then the lanes' sums) and FP32
 constexpr size_t kBuf64 = 2 * 3 * (size_t)rows_of(kMomLo - 1) * 32 * sizeof(double);
 constexpr size_t kBuf32 = 2 * 3 * (size_t)rows_of(kMomK - 1) * 32 * sizeof(float);
@@ -224,11 +208,10 @@ __global__ void __launch_bounds__(kNT) k_small3(const float* __restrict__ v, int
     __syncthreads();
   }
   const uint32_t count = h->small_q_count;
-  if (count == 0) return;
+  if (count == 0 || (q != nullptr ? small_few(count, nf) : qsmall_direct(count, nf))) return;
   const double c[3] = {h->center[0], h->center[1], h->center[2]};
   char* parts = scratch + kMomHead;
-  if (count <= (uint32_t)kSmallDirect) {
-    if (q == nullptr) return;
+  if (q != nullptr && count <= (uint32_t)kSmallDirect) {
     const int64_t nch = small3_chunks(nf), per = (nf + nch - 1) / nch;
     for (int64_t u = blockIdx.x; u < (int64_t)count * nch; u += gridDim.x) {
       const int64_t i = h->small_list[u / nch], m0 = (u % nch) * per, m1 = min(nf, m0 + per);

@@ -8,6 +8,7 @@
 //    units spread over the grid, the chunk sums added in order by the finishing kernel;
 //  * more: the series' coefficients (moments of the shape, one per monomial of degree <= 12, 455
 //    of them) are summed over the faces once, and every small Q point evaluates the polynomial.
+// Of a shape of few faces the finishing kernel sums each point over the faces itself (small_few).
 // Line between them: a directly evaluated point costs about 70 FP64 operations a face and the moments
 // about 900 with lanes to spare, so they break even near 30 points (on 20,480 faces 32 points take
 // 75 us at the FP64 rate, the moments 102).  A curve of 2,928 points on
@@ -38,6 +39,24 @@ constexpr int kMomFaces = 32;             // faces of one batch (one per lane)
 constexpr int kDirectChunks = 64;         // face chunks of a directly evaluated Q point at most
 static_assert(kMomN * 8 <= kMomHead && kMomN64 * 8 + kMomN32 * 8 <= kMomPart, "moment scratch");
 
+// Up to kFewFaces faces, k_finalize3d's warps take a small point's faces 32 at a time and k_small3 has only
+// the volume to do: 120 FP64 instructions a point and 32 faces, 6.6 ns of the chip, against 25 us and more for
+// the moments (a batch, its block's sums and their hand-over) and a block for only 32 faces where k_small3
+// sums directly.  Calls with all points small, through k_small3 / so: 12 faces x 20 Q 131 / 30 us, x 300 68 / 34,
+// x 3,000 86 / 53; 80 faces x 40 Q 64 / 35 us, x 300 67 / 37; past the line 80 x 3,000 84.
+constexpr int64_t kFewFaces = 256;
+__host__ __device__ inline bool small_few(uint32_t count, int64_t nf) {
+  return nf <= kFewFaces && (int64_t)count * ((nf + 31) / 32) <= 3000;
+}
+
+// The Q-gradient: points evaluated one by one in blocks of their own (k_qsmall_part; 22 ns of the chip a point
+// and 32 faces, 30 ns a point besides), where that is less than the 30 us that the moments add.  Calls with all
+// points small, moments / direct: 12 faces x 40 Q 85 / 56 us, 80 x 300 95 / 74, 320 x 40 114 / 86; past the line 320
+// x 300 112 / 148 (with 17 terms), 1,280 x 40 105 / 111.
+__host__ __device__ inline bool qsmall_direct(uint32_t count, int64_t nf) {
+  return count <= (uint32_t)kSmallDirect || (int64_t)count * (nf + 48) <= 40000;
+}
+
 inline int64_t small3_blocks(int64_t nf, int sms) {
   return std::max<int64_t>(1, std::min<int64_t>(sms, (nf + kMomFaces - 1) / kMomFaces));
 }
@@ -49,6 +68,22 @@ __host__ __device__ inline int64_t small3_chunks(int64_t nf) {   // face chunks 
 inline size_t small3_bytes(int64_t nf, int sms) {
   return kMomHead + std::max((size_t)small3_blocks(nf, sms) * kMomPart,
                              (size_t)(kSmallDirect * small3_chunks(nf)) * 8 * sizeof(double));
+}
+
+// Corners of face m relative to c; false (and zeros) for an index out of range.
+__device__ __forceinline__ bool corners(const float* v, int64_t nv, const int32_t* f, int64_t m, const double* c,
+                                        double (&P)[3][3]) {
+  const int32_t id[3] = {f[3 * m], f[3 * m + 1], f[3 * m + 2]};
+  const bool ok = id[0] >= 0 && id[1] >= 0 && id[2] >= 0 && id[0] < nv && id[1] < nv && id[2] < nv;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) P[k][d] = ok ? (double)v[3 * (int64_t)id[k] + d] - c[d] : 0.0;
+  return ok;
+}
+__device__ __forceinline__ double det3(const double (&P)[3][3]) {
+  return P[0][0] * (P[1][1] * P[2][2] - P[1][2] * P[2][1]) + P[0][1] * (P[1][2] * P[2][0] - P[1][0] * P[2][2]) +
+         P[0][2] * (P[1][0] * P[2][1] - P[1][1] * P[2][0]);
 }
 
 // The direct series of one tetrahedron (c, p0, p1, p2): its corner phases x and the monomials'
@@ -138,7 +173,7 @@ __device__ __forceinline__ void mom_eval(const double* m, double x, double y, do
 // Bytes by which the scratch exceeds the records of a pft3d_mesh call (part of its workspace size).
 size_t small3_growth(int64_t n_faces, int64_t n_q, const pft_options* opts);
 
-// pft_small.cu.  q = NULL: only the moments (nothing for h->small_q_count <= kSmallDirect).
+// pft_small.cu.  q = NULL: the moments for the Q-gradient, where qsmall_direct does not hold.
 cudaError_t launch_small3(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q, WsHeader* h,
                           const double* mparts, int n_measure, void* scratch, cudaStream_t st);
 
