@@ -1461,16 +1461,18 @@ __global__ void k_bbvert(const float* __restrict__ v, int64_t nv, const int64_t*
 // k_bbcorner3 (corner adjoints with the mesh's small-|Q| rows), and the vertex gather of the
 // single-mesh adjoint over all faces.
 // ---------------------------------------------------------------------------
-// One block per mesh; with FP64 records the largest mesh's block took 124 us (5,120 faces at 2 FP64
-// operations a clock).
-constexpr int kMeshT = 1024;
-__global__ void __launch_bounds__(kMeshT) k_bbprep3(const float* __restrict__ v, int64_t nv,
+// One block per mesh, of 1,024 threads for meshes of more than 512 faces on average (the largest mesh's block is
+// what the launch waits for; with FP64 records and 256 threads 5,120 faces took 124 us), else of 256: a
+// block of 1,024 costs its five block reductions and two blocks an SM whatever the mesh.  Adjoint of 10,000
+// meshes of 20 faces at 16 Q each, 1,024 / 256 threads: 1,148 / 762 us; at 64 shared Q 1,884 / 1,499 us.
+template <int NT>
+__global__ void __launch_bounds__(NT) k_bbprep3(const float* __restrict__ v, int64_t nv,
                                                   const int32_t* __restrict__ f, int64_t nf,
                                                   const int64_t* __restrict__ off, int64_t nm, Face32* recs,
                                                   PolyC* mc, int32_t* nblk, int32_t* __restrict__ deg,
                                                   const double* __restrict__ q, int64_t n_q, float2* __restrict__ qs,
                                                   WsHeader* h) {
-  __shared__ float sh[kMeshT / 32];
+  __shared__ float sh[NT / 32];
   split_q(q, 3 * n_q, qs);
   const int64_t i = blockIdx.x;
   const int64_t s0 = off[i], s1 = off[i + 1];
@@ -1482,12 +1484,12 @@ __global__ void __launch_bounds__(kMeshT) k_bbprep3(const float* __restrict__ v,
     return a >= 0 && b >= 0 && c >= 0 && a < nv && b < nv && c < nv;
   };
   // corners at each vertex, for the gather: every face once, whatever the offsets say
-  for (int64_t m = i * kMeshT + threadIdx.x; m < nf; m += (int64_t)gridDim.x * kMeshT)
+  for (int64_t m = i * NT + threadIdx.x; m < nf; m += (int64_t)gridDim.x * NT)
     if (valid(m))
       for (int k = 0; k < 3; ++k) atomicAdd(&deg[f[3 * m + k]], 1);
   float mn[3] = {3.4e38f, 3.4e38f, 3.4e38f}, mx[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
   bool bad_index = false, bad_value = false;
-  for (int64_t j = threadIdx.x; j < n; j += kMeshT) {
+  for (int64_t j = threadIdx.x; j < n; j += NT) {
     const int64_t m = b0 + j;
     if (!valid(m)) { bad_index = true; continue; }
     for (int k = 0; k < 3; ++k)
@@ -1502,7 +1504,7 @@ __global__ void __launch_bounds__(kMeshT) k_bbprep3(const float* __restrict__ v,
   if (bad_value) set_status(&h->status, ST_NONFINITE);
   double c[3];
   for (int d = 0; d < 3; ++d) {
-    const float lo = block_minmax_f<kMeshT>(mn[d], false, sh), hi = block_minmax_f<kMeshT>(mx[d], true, sh);
+    const float lo = block_minmax_f<NT>(mn[d], false, sh), hi = block_minmax_f<NT>(mx[d], true, sh);
     c[d] = (n > 0 && lo <= hi) ? 0.5 * ((double)lo + (double)hi) : 0.0;
   }
   float rm = 0.f, chi[3], clo[3];
@@ -1510,7 +1512,7 @@ __global__ void __launch_bounds__(kMeshT) k_bbprep3(const float* __restrict__ v,
     chi[d] = (float)c[d];
     clo[d] = (float)(c[d] - (double)chi[d]);
   }
-  for (int64_t j = threadIdx.x; j < n; j += kMeshT) {
+  for (int64_t j = threadIdx.x; j < n; j += NT) {
     const int64_t m = b0 + j;
     Face32 r{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // skipped faces contribute 0
     if (valid(m)) {
@@ -1522,7 +1524,7 @@ __global__ void __launch_bounds__(kMeshT) k_bbprep3(const float* __restrict__ v,
     }
     recs[m] = r;
   }
-  rm = block_minmax_f<kMeshT>(rm, true, sh);
+  rm = block_minmax_f<NT>(rm, true, sh);
   if (threadIdx.x == 0) {
     mc[i] = PolyC{c[0], c[1], c[2], rm, 0};
     nblk[i] = (int32_t)((n + kPairFaces - 1) / kPairFaces);
@@ -2512,8 +2514,12 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   PolyC* mc = at<PolyC>(ws, y.mc);
   int32_t* nblk = at<int32_t>(ws, y.nblk);
   int64_t* bstart = at<int64_t>(ws, y.bstart);
-  k_bbprep3<<<(unsigned)n_meshes, kMeshT, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes, recs, mc, nblk,
-                                                 deg, q, n_q, at<float2>(ws, y.qsplit), h);
+  auto prep = [&](auto kernel, int nt) {
+    kernel<<<(unsigned)n_meshes, nt, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes, recs, mc, nblk, deg, q,
+                                              n_q, at<float2>(ws, y.qsplit), h);
+  };
+  if (n_faces > 512 * n_meshes) prep(k_bbprep3<1024>, 1024);
+  else prep(k_bbprep3<kAux>, kAux);
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_meshes, bstart);
   PFT_BWD_LAUNCH();
