@@ -171,7 +171,8 @@ __device__ __forceinline__ void seg_adj(const QRec& Q, const V (&s)[4], V (&a)[4
 // s = Q.N (and, in the edge branch, of X = N x Q and b_k = q_k.X) go to `out`,
 // which turns them into record adjoints (RecAdj) or Q adjoints (QAdj): the
 // projections are bilinear in Q and the record, so the two are mirror images.
-template <class Out>
+// kEdge: the caller knows that the warp takes the edge sum.
+template <bool kEdge = false, class Out>
 __device__ __forceinline__ void face_adj_t(const QRec& Q, const float4 A, const float4 B, const float4 C, Thr th,
                                            Out& out) {
   const float qx = Q.qx, qy = Q.qy, qz = Q.qz;
@@ -187,10 +188,10 @@ __device__ __forceinline__ void face_adj_t(const QRec& Q, const float4 A, const 
   // the sign bit is cleared: the bits of |P| (and of NaN, above +inf) order as
   // unsigned integers, and one reduction serves all three tests.
   const float wmax =
-      __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(P) & 0x7fffffffu));
-  const bool all_hi = wmax < th.hi;
-  const bool all_short = wmax < kPShort;
-  const bool all_long = wmax < kPLong;
+      kEdge ? 0.f : __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(P) & 0x7fffffffu));
+  const bool all_hi = !kEdge && wmax < th.hi;
+  const bool all_short = !kEdge && wmax < kPShort;
+  const bool all_long = !kEdge && wmax < kPLong;
   const bool shorts = (th.longs ? all_short : all_hi) || (P < th.lo);
   const bool k9s = !shorts && all_hi && wmax < kP9;   // tau > 1 here (else every series lane is short)
   const bool longs = !shorts && !k9s && all_hi && (!th.xlongs || all_long);
@@ -397,43 +398,47 @@ __device__ __forceinline__ void face_adj_t(const QRec& Q, const float4 A, const 
 }
 
 // Record adjoints of one (Q, face) pair: g += mub Q, q0 += a0b Q (+ b0b X), q1 += a1b Q (+ b1b X),
-// N += sb Q (+ Q x Xbar), in the order of Face32's 12 fields.
+// N += sb Q (+ Q x Xbar), in the order of Face32's 12 fields; those of q0, q1 and N are kept negated (adj_sign).
+// Acc: a float& for each field.
+template <class Acc>
 struct RecAdj {
-  float (&a)[12];
+  Acc a;
   float qx, qy, qz;
   __device__ __forceinline__ void value(float, float) {}
   __device__ __forceinline__ void edge(float b0b, float b1b, float Xx, float Xy, float Xz, float Xbx, float Xby,
                                        float Xbz) {
-    a[3] = fmaf(b0b, Xx, a[3]);
-    a[4] = fmaf(b0b, Xy, a[4]);
-    a[5] = fmaf(b0b, Xz, a[5]);
-    a[6] = fmaf(b1b, Xx, a[6]);
-    a[7] = fmaf(b1b, Xy, a[7]);
-    a[8] = fmaf(b1b, Xz, a[8]);
-    a[9] = fmaf(qy, Xbz, fmaf(-qz, Xby, a[9]));    // N += Q x Xbar
-    a[10] = fmaf(qz, Xbx, fmaf(-qx, Xbz, a[10]));
-    a[11] = fmaf(qx, Xby, fmaf(-qy, Xbx, a[11]));
+    a(3) = fmaf(-b0b, Xx, a(3));
+    a(4) = fmaf(-b0b, Xy, a(4));
+    a(5) = fmaf(-b0b, Xz, a(5));
+    a(6) = fmaf(-b1b, Xx, a(6));
+    a(7) = fmaf(-b1b, Xy, a(7));
+    a(8) = fmaf(-b1b, Xz, a(8));
+    a(9) = fmaf(-qy, Xbz, fmaf(qz, Xby, a(9)));    // N += Q x Xbar
+    a(10) = fmaf(-qz, Xbx, fmaf(qx, Xbz, a(10)));
+    a(11) = fmaf(-qx, Xby, fmaf(qy, Xbx, a(11)));
   }
   __device__ __forceinline__ void common(float mub, float a0b, float a1b, float sb) {
-    a[0] = fmaf(mub, qx, a[0]);
-    a[1] = fmaf(mub, qy, a[1]);
-    a[2] = fmaf(mub, qz, a[2]);
-    a[3] = fmaf(a0b, qx, a[3]);
-    a[4] = fmaf(a0b, qy, a[4]);
-    a[5] = fmaf(a0b, qz, a[5]);
-    a[6] = fmaf(a1b, qx, a[6]);
-    a[7] = fmaf(a1b, qy, a[7]);
-    a[8] = fmaf(a1b, qz, a[8]);
-    a[9] = fmaf(sb, qx, a[9]);
-    a[10] = fmaf(sb, qy, a[10]);
-    a[11] = fmaf(sb, qz, a[11]);
+    a(0) = fmaf(mub, qx, a(0));
+    a(1) = fmaf(mub, qy, a(1));
+    a(2) = fmaf(mub, qz, a(2));
+    a(3) = fmaf(-a0b, qx, a(3));
+    a(4) = fmaf(-a0b, qy, a(4));
+    a(5) = fmaf(-a0b, qz, a(5));
+    a(6) = fmaf(-a1b, qx, a(6));
+    a(7) = fmaf(-a1b, qy, a(7));
+    a(8) = fmaf(-a1b, qz, a(8));
+    a(9) = fmaf(-sb, qx, a(9));
+    a(10) = fmaf(-sb, qy, a(10));
+    a(11) = fmaf(-sb, qz, a(11));
   }
 };
 
-__device__ __forceinline__ void face_adj(const QRec& Q, const float4 A, const float4 B, const float4 C, Thr th,
-                                         float (&a)[12]) {
-  RecAdj o{a, Q.qx, Q.qy, Q.qz};
-  face_adj_t(Q, A, B, C, th, o);
+// Adds the record adjoints of one Q and one face f (12 fields) to a.
+template <bool kEdge, class Acc>
+__device__ __forceinline__ void face_adj(const QRec& Q, const float (&f)[12], Thr th, Acc a) {
+  RecAdj<Acc> o{a, Q.qx, Q.qy, Q.qz};
+  face_adj_t<kEdge>(Q, make_float4(f[0], f[1], f[2], f[3]), make_float4(f[4], f[5], f[6], f[7]),
+                    make_float4(f[8], f[9], f[10], f[11]), th, o);
 }
 
 // Q adjoint of one (Q, face) pair, and the pair's term J itself (tile sums):
@@ -912,9 +917,8 @@ __global__ void __launch_bounds__(kBwdNT) k_bwd2(const Seg32* __restrict__ segs,
   for (int f = 0; f < 4; ++f) dst[f] = (double)acc[f].hi + (double)acc[f].lo;
 }
 
-// 3D: a thread's two faces (2t, 2t + 1 of the block's kPairFaces) against a stream of Q records.  The
-// state of a block; `run` walks the ring and leaves the sums in acc (shared memory, [field][face of the
-// pair][thread]).
+// 3D: a thread's faces against a stream of Q records.  The state of a block; pair_run walks the ring and leaves the
+// sums in acc (shared memory, [field][face of the thread][thread]).
 constexpr int kPairFaces = 2 * kBwdNT;
 struct PairShared {
   __align__(128) QRec slots[kStages * kQTile];
@@ -925,70 +929,140 @@ struct PairShared {
 };
 constexpr int kPairBlocks = 4;   // resident blocks per SM the registers are held to (128 each)
 
-__device__ __forceinline__ void scalar_adj(const QRec& Q, const float2 (&F)[12], Thr th, float2 (&a)[12], bool second) {
-    float f[12], d[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    f[k] = second ? F[k].y : F[k].x;
-    d[k] = 0.f;
-  }
-  face_adj(Q, make_float4(f[0], f[1], f[2], f[3]), make_float4(f[4], f[5], f[6], f[7]),
-           make_float4(f[8], f[9], f[10], f[11]), th, d);
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    if (second) a[k].y = fmaf(adj_sign(k), d[k], a[k].y);
-    else a[k].x = fmaf(adj_sign(k), d[k], a[k].x);
-  }
+// The faces of a thread: m and, if n == 2, m + 1 (n == 0: none).  A block with more than kBwdNT faces gives each
+// thread two, 2t and 2t + 1 of its warp's 64, for the paired series.  Fewer go one a thread (`single`), and where
+// they take one or two of the four warps only, the others hold copies and take their part of every tile's
+// records: two a thread leave the edge sums twice as long and most warps idle.
+// Adjoint call, two a thread / so: 20 faces a mesh, 1,024 meshes x 4,096 Q 7.87 / 1.81 ms, 96 meshes x 64 Q 126 / 70 us;
+// one mesh of 12 faces x 241 Q 188 / 67 us, of 80 x 4,096 217 / 135 us.
+struct PairSpan {
+  int64_t m;
+  int n, copy, copies;
+  bool single;
+};
+// fpb: faces of a block (kPairFaces, or kBwdNT); b0: the block's first, end: the shape's last + 1.
+__device__ __forceinline__ PairSpan pair_span(int64_t b0, int64_t end, int fpb) {
+  static_assert(kBwdNT == 128, "the faces of one warp, two or four");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nb = (int)min(end - b0, (int64_t)fpb);
+  const bool single = nb <= kBwdNT;
+  const int parts = !single || nb > 64 ? 4 : (nb > 32 ? 2 : 1);   // warps with different faces
+  const int64_t m = b0 + (single ? (warp % parts) * 32 + lane : warp * 64 + 2 * lane);
+  return PairSpan{m, (int)max((int64_t)0, min(end - m, (int64_t)(single ? 1 : 2))), warp / parts, 4 / parts, single};
 }
 
-// live: the warp holds a face.  Returns false when a wait gave up.
-__device__ __forceinline__ bool pair_run(PairShared& sh, const QRec* rec, int64_t nq, const float2 (&F)[12], bool live,
-                                         Thr th) {
-  using V = float2;
+// Accumulators of a thread: the fields of one of its two faces, or of its only one.
+struct HalfAcc {
+  float2 (&a)[12];
+  bool second;
+  __device__ __forceinline__ float& operator()(int k) const { return second ? a[k].y : a[k].x; }
+};
+struct OneAcc {
+  float (&a)[12];
+  __device__ __forceinline__ float& operator()(int k) const { return a[k]; }
+};
+
+// The pair adjoint of one of a thread's two faces.
+__device__ __forceinline__ void scalar_adj(const QRec& Q, const float2 (&F)[12], Thr th, float2 (&a)[12], bool second) {
+  float f[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) f[k] = second ? F[k].y : F[k].x;
+  face_adj<true>(Q, f, th, HalfAcc{a, second});
+}
+
+__device__ __forceinline__ void acc_add(float2& c, float x) {
+  CAcc v{c.x, c.y};
+  v.add(x);
+  c = make_float2(v.hi, v.lo);
+}
+
+// Projections of Q on a record, and the warp's largest |P| from them (the sign bit cleared as in face_adj_t).
+template <class V>
+struct AdjCommon {
+  V a0, a1, s1, m, P;
+  __device__ __forceinline__ AdjCommon(const QRec& Q, const V (&F)[12]) {
+    const V qx = vs<V>(Q.qx), qy = vs<V>(Q.qy), qz = vs<V>(Q.qz);
+    a0 = vfma(qx, F[3], vfma(qy, F[4], vmul(qz, F[5])));
+    a1 = vfma(qx, F[6], vfma(qy, F[7], vmul(qz, F[8])));
+    s1 = vadd(a0, a1);
+    m = vmul(a1, s1);
+    P = vfma(a0, a0, m);
+  }
+  __device__ __forceinline__ float wmax() const {
+    uint32_t u = __float_as_uint(el(&P, 0)) & 0x7fffffffu;
+    if (sizeof(V) == 8) u = max(u, __float_as_uint(el(&P, sizeof(V) / 8)) & 0x7fffffffu);
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, u));
+  }
+  // the series of the form that wmax < th.hi allows
+  __device__ __forceinline__ void series(const QRec& Q, const V (&F)[12], float wmax, V (&a)[12]) const {
+    const V qx = vs<V>(Q.qx), qy = vs<V>(Q.qy), qz = vs<V>(Q.qz);
+    const V mu = vfma(qx, F[0], vfma(qy, F[1], vmul(qz, F[2])));
+    const V s = vfma(qx, F[9], vfma(qy, F[10], vmul(qz, F[11])));
+    if (wmax < kPShort) series_adj<0>(Q, mu, a0, a1, s1, m, s, a);
+    else if (wmax < kP9) series_adj<1>(Q, mu, a0, a1, s1, m, s, a);
+    else if (wmax < kPLong) series_adj<2>(Q, mu, a0, a1, s1, m, s, a);
+    else series_adj<3>(Q, mu, a0, a1, s1, m, s, a);
+  }
+};
+
+// Returns false when a wait gave up.
+__device__ __forceinline__ bool pair_run(PairShared& sh, const QRec* rec, int64_t nq, const float2 (&F)[12],
+                                         const PairSpan& sp, Thr th) {
   Ring<QRec, kQTile, kBwdNT> ring{sh.slots, sh.full, sh.done, &sh.issued, rec, nq, (int)((nq + kQTile - 1) / kQTile)};
   ring.start();
 #pragma unroll
   for (int k = 0; k < 24; ++k) sh.acc[k][threadIdx.x] = make_float2(0.f, 0.f);
+  const bool live = __any_sync(0xffffffffu, sp.n > 0);   // the warp holds a face
   bool ok = true;
   for (int t = 0; t < ring.ntiles; ++t) {
     if (!ring.wait(t)) { ok = false; break; }
     if (live) {
       const QRec* tq = ring.tile(t);
       const int cnt = ring.count(t);
-      V a[12];
+      // Two faces side by side, unless the record in the tile's middle asks for the edge sum, which takes one face
+      // at a time anyway: slivers (32,760 faces x 10,000 Q, nearly all edge sums) 2.95 / 2.86 ms.  Asking costs
+      // 0.3 % of a tile.
+      if (!sp.single && !(AdjCommon<float2>(tq[cnt / 2], F).wmax() >= th.hi)) {
+        float2 a[12];
 #pragma unroll
-      for (int k = 0; k < 12; ++k) a[k] = vs<V>(0.f);
+        for (int k = 0; k < 12; ++k) a[k] = vs<float2>(0.f);
 #pragma unroll 1
-      for (int j = 0; j < cnt; ++j) {
-        const QRec Q = tq[j];
-        const V qx = vs<V>(Q.qx), qy = vs<V>(Q.qy), qz = vs<V>(Q.qz);
-        const V a0 = vfma(qx, F[3], vfma(qy, F[4], vmul(qz, F[5])));
-        const V a1 = vfma(qx, F[6], vfma(qy, F[7], vmul(qz, F[8])));
-        const V s1 = vadd(a0, a1), m = vmul(a1, s1), P = vfma(a0, a0, m);
-        // the largest |P| of the warp's faces decides, as in face_adj_t (the sign bit is cleared there
-        // for the same reason)
-        const float wmax = __uint_as_float(
-            __reduce_max_sync(0xffffffffu, max(__float_as_uint(P.x) & 0x7fffffffu, __float_as_uint(P.y) & 0x7fffffffu)));
-        if (wmax < th.hi) {
-          const V mu = vfma(qx, F[0], vfma(qy, F[1], vmul(qz, F[2])));
-          const V s = vfma(qx, F[9], vfma(qy, F[10], vmul(qz, F[11])));
-          if (wmax < kPShort) series_adj<0>(Q, mu, a0, a1, s1, m, s, a);
-          else if (wmax < kP9) series_adj<1>(Q, mu, a0, a1, s1, m, s, a);
-          else if (wmax < kPLong) series_adj<2>(Q, mu, a0, a1, s1, m, s, a);
-          else series_adj<3>(Q, mu, a0, a1, s1, m, s, a);
-        } else {
-          scalar_adj(Q, F, th, a, false);
-          scalar_adj(Q, F, th, a, true);
+        for (int j = 0; j < cnt; ++j) {
+          const QRec Q = tq[j];
+          const AdjCommon<float2> c(Q, F);
+          const float wmax = c.wmax();
+          if (wmax < th.hi) {
+            c.series(Q, F, wmax, a);
+          } else {
+            scalar_adj(Q, F, th, a, false);
+            scalar_adj(Q, F, th, a, true);
+          }
         }
-      }
 #pragma unroll
-      for (int k = 0; k < 12; ++k) {
+        for (int k = 0; k < 12; ++k) {
+          acc_add(sh.acc[2 * k][threadIdx.x], a[k].x);
+          acc_add(sh.acc[2 * k + 1][threadIdx.x], a[k].y);
+        }
+      } else {
+        const int j0 = cnt * sp.copy / sp.copies, j1 = cnt * (sp.copy + 1) / sp.copies;
+#pragma unroll 1
+        for (int e = 0; e < (sp.single ? 1 : 2); ++e) {
+          float f[12], a[12];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float2 c = sh.acc[2 * k + e][threadIdx.x];
-          CAcc v{c.x, c.y};
-          v.add(e ? a[k].y : a[k].x);
-          sh.acc[2 * k + e][threadIdx.x] = make_float2(v.hi, v.lo);
+          for (int k = 0; k < 12; ++k) {
+            f[k] = e ? F[k].y : F[k].x;
+            a[k] = 0.f;
+          }
+#pragma unroll 1
+          for (int j = j0; j < j1; ++j) {
+            const QRec Q = tq[j];
+            const AdjCommon<float> c(Q, f);
+            const float wmax = c.wmax();
+            if (wmax < th.hi) c.series(Q, f, wmax, a);
+            else face_adj<true>(Q, f, th, OneAcc{a});
+          }
+#pragma unroll
+          for (int k = 0; k < 12; ++k) acc_add(sh.acc[2 * k + e][threadIdx.x], a[k]);
         }
       }
     }
@@ -997,14 +1071,14 @@ __device__ __forceinline__ bool pair_run(PairShared& sh, const QRec* rec, int64_
   ring.finish();
   return ok;
 }
-__device__ __forceinline__ void pair_load(const Face32* faces, int64_t m, int64_t end, float2 (&F)[12]) {
+__device__ __forceinline__ void pair_load(const Face32* faces, const PairSpan& sp, float2 (&F)[12]) {
   float f[2][12];
 #pragma unroll
   for (int e = 0; e < 2; ++e)
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (m + e < end) x = reinterpret_cast<const float4*>(faces + m + e)[k];
+      if (e < sp.n) x = reinterpret_cast<const float4*>(faces + sp.m + e)[k];
       f[e][4 * k] = x.x;
       f[e][4 * k + 1] = x.y;
       f[e][4 * k + 2] = x.z;
@@ -1013,33 +1087,39 @@ __device__ __forceinline__ void pair_load(const Face32* faces, int64_t m, int64_
 #pragma unroll
   for (int k = 0; k < 12; ++k) F[k] = make_float2(f[0][k], f[1][k]);
 }
-// dst: partial sums of the thread's first face (12 doubles a face)
-__device__ __forceinline__ void pair_store(const PairShared& sh, int64_t m, int64_t end, double* dst) {
+// dst: partial sums of the thread's first face (12 doubles a face); the first copy's threads add the others'.
+__device__ __forceinline__ void pair_store(const PairShared& sh, const PairSpan& sp, double* dst) {
+  if (sp.copy > 0) return;
 #pragma unroll
   for (int e = 0; e < 2; ++e)
-    if (m + e < end)
+    if (e < sp.n)
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
         const float2 c = sh.acc[2 * k + e][threadIdx.x];
-        const double v = (double)c.x + (double)c.y;
+        double v = (double)c.x + (double)c.y;
+        if (sp.copies > 1)
+          for (int o = kBwdNT / sp.copies; o < kBwdNT; o += kBwdNT / sp.copies) {
+            const float2 x = sh.acc[2 * k + e][threadIdx.x + o];
+            v += (double)x.x + (double)x.y;
+          }
         dst[12 * e + k] = adj_sign(k) > 0.f ? v : -v;
       }
 }
 
 __global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bwd3(const Face32* __restrict__ faces, int64_t n_faces,
                                                              const QRec* __restrict__ rec, int64_t n_q,
-                                                             int64_t per_split, Thr th, double* __restrict__ partial,
-                                                             uint32_t* status) {
+                                                             int64_t per_split, Thr th, int fpb,
+                                                             double* __restrict__ partial, uint32_t* status) {
   extern __shared__ __align__(128) unsigned char raw[];
   PairShared& sh = *reinterpret_cast<PairShared*>(raw);
-  const int64_t m = blockIdx.x * (int64_t)kPairFaces + 2 * threadIdx.x;
+  const PairSpan sp = pair_span(blockIdx.x * (int64_t)fpb, n_faces, fpb);
   float2 F[12];
-  pair_load(faces, m, n_faces, F);
+  pair_load(faces, sp, F);
   const int64_t q0 = (int64_t)blockIdx.y * per_split;
   const int64_t nq = max((int64_t)0, min(per_split, n_q - q0));
-  const bool ok = pair_run(sh, rec + q0, nq, F, __any_sync(0xffffffffu, m < n_faces), th);
+  const bool ok = pair_run(sh, rec + q0, nq, F, sp, th);
   if (!ok) set_status(status, ST_TIMEOUT);
-  if (ok) pair_store(sh, m, n_faces, partial + ((int64_t)blockIdx.y * n_faces + m) * 12);
+  if (ok) pair_store(sh, sp, partial + ((int64_t)blockIdx.y * n_faces + sp.m) * 12);
 }
 
 // 2D vertex gradients: record adjoints of segment j (start) and of the segment
@@ -1471,7 +1551,7 @@ __global__ void __launch_bounds__(NT) k_bbprep3(const float* __restrict__ v, int
                                                   const int64_t* __restrict__ off, int64_t nm, Face32* recs,
                                                   PolyC* mc, int32_t* nblk, int32_t* __restrict__ deg,
                                                   const double* __restrict__ q, int64_t n_q, float2* __restrict__ qs,
-                                                  WsHeader* h) {
+                                                  int fpb, WsHeader* h) {
   __shared__ float sh[NT / 32];
   split_q(q, 3 * n_q, qs);
   const int64_t i = blockIdx.x;
@@ -1527,12 +1607,11 @@ __global__ void __launch_bounds__(NT) k_bbprep3(const float* __restrict__ v, int
   rm = block_minmax_f<NT>(rm, true, sh);
   if (threadIdx.x == 0) {
     mc[i] = PolyC{c[0], c[1], c[2], rm, 0};
-    nblk[i] = (int32_t)((n + kPairFaces - 1) / kPairFaces);
+    nblk[i] = (int32_t)((n + fpb - 1) / fpb);
   }
 }
 
-// Pair blocks: block b is pair block b - bstart[i] of mesh i (kPairFaces faces, two a thread); the mesh's Q
-// records stream through the ring (Q chunk blockIdx.y).  Warps with no face only wait for and release
+// Pair blocks: block b is pair block b - bstart[i] of mesh i (fpb faces); the mesh's Q records stream through the ring (Q chunk blockIdx.y).  Warps with no face only wait for and release
 // the tiles.  Blocks past the last mesh leave at once.
 __global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bbwd3(const Face32* __restrict__ recs, int64_t nf,
                                                               const int64_t* __restrict__ off, int64_t nm,
@@ -1540,7 +1619,7 @@ __global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bbwd3(const Face32* __r
                                                               const int32_t* __restrict__ nblk,
                                                               const QRec* __restrict__ rec,
                                                               const int64_t* __restrict__ q_off, int64_t n_q,
-                                                              int64_t per_split, Thr th,
+                                                              int64_t per_split, Thr th, int fpb,
                                                               double* __restrict__ partial, uint32_t* status) {
   extern __shared__ __align__(128) unsigned char raw[];
   PairShared& sh = *reinterpret_cast<PairShared*>(raw);
@@ -1553,16 +1632,16 @@ __global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bbwd3(const Face32* __r
     else hi = mid - 1;
   }
   const int64_t s0 = max((int64_t)0, min(off[lo], nf)), s1 = max(s0, min(off[lo + 1], nf));
-  const int64_t m = s0 + (b - bstart[lo]) * kPairFaces + 2 * threadIdx.x;
+  const PairSpan sp = pair_span(s0 + (b - bstart[lo]) * fpb, s1, fpb);
   float2 F[12];
-  pair_load(recs, m, s1, F);
+  pair_load(recs, sp, F);
   int64_t qb, gb, nqi;
   bb_rows(q_off, lo, n_q, qb, gb, nqi);
   const int64_t q0 = (int64_t)blockIdx.y * per_split;
   const int64_t nq = max((int64_t)0, min(per_split, nqi - q0));
-  const bool ok = pair_run(sh, rec + gb + q0, nq, F, __any_sync(0xffffffffu, m < s1), th);
+  const bool ok = pair_run(sh, rec + gb + q0, nq, F, sp, th);
   if (!ok) set_status(status, ST_TIMEOUT);
-  if (ok) pair_store(sh, m, s1, partial + ((int64_t)blockIdx.y * nf + m) * 12);
+  if (ok) pair_store(sh, sp, partial + ((int64_t)blockIdx.y * nf + sp.m) * 12);
 }
 
 __device__ void corner_adj(int64_t m, const float* __restrict__ v, int64_t nv, const int32_t* __restrict__ f,
@@ -1875,17 +1954,24 @@ int more_chunks(int k, int64_t q_blocks, int64_t slots, int64_t tiles) {
   return k;
 }
 
+// Faces of a pair block: two a thread, or one where the blocks of pairs, each with a tile of Q records, would not
+// fill the GPU.  Adjoint call, two a thread / one: 320 faces x 241 Q 169 / 107 us, x 4,096 200 / 128 us; 24 meshes of
+// 1,280 faces with 500 Q each 431 / 296 us.
+int pair_faces(int64_t pair_blocks, int64_t q_tiles) {
+  return pair_blocks * std::min<int64_t>(q_tiles, 256) < (int64_t)sm_count() * kPairBlocks ? kBwdNT : kPairFaces;
+}
+
 struct BwdLayout {
   size_t mparts, items, qrec, small, partial, corner, deg, cursor, start, list, phi, total;
-  int nblk, ks;
+  int nblk, ks, fpb;
   int64_t per_split;
 };
 
 BwdLayout bwd_layout(int dim, int64_t n_verts, int64_t n_items, int64_t n_prep, int64_t n_q) {
   BwdLayout y{};
-  y.ks = dim == 3 ? pair_splits(std::max<int64_t>(1, (n_items + kPairFaces - 1) / kPairFaces), n_q, 12)
-                  : q_splits(n_items, n_q);
   const int64_t q_tiles = std::max<int64_t>(1, (n_q + kQTile - 1) / kQTile);
+  y.fpb = pair_faces(blocks(n_items, kPairFaces), q_tiles);
+  y.ks = dim == 3 ? pair_splits(blocks(n_items, y.fpb), n_q, 12) : q_splits(n_items, n_q);
   y.per_split = ((q_tiles + y.ks - 1) / y.ks) * kQTile;
   y.ks = (int)std::max<int64_t>(1, (n_q + y.per_split - 1) / y.per_split);
   y.nblk = dim == 3 ? prep3_blocks(n_prep) : std::max(1, prep_blocks(n_prep));
@@ -2038,14 +2124,17 @@ BbLayout bb_layout(int64_t nv, int64_t np, int64_t n_q, bool per_poly_q) {
 // and the vertex -> face-corner CSR of the vertex gather.
 struct Bb3Layout {
   size_t recs, mc, nblk, bstart, qsplit, rec, small, scnt, partial, corner, deg, cursor, start, list, total;
-  int ks;
+  int ks, fpb;
   int64_t per_split, grid;
 };
 
 Bb3Layout bb3_layout(int64_t nv, int64_t nf, int64_t nm, int64_t n_q, bool per_mesh_q) {
   Bb3Layout y{};
-  y.grid = std::max<int64_t>(1, nm + (nf + kPairFaces - 1) / kPairFaces);   // at least the pair blocks needed
   const int64_t q_tiles = std::max<int64_t>(1, (n_q + kQTile - 1) / kQTile);
+  // per-mesh lists: the tiles of a list of average length
+  const int64_t own = per_mesh_q && nm > 0 ? (n_q / nm + kQTile - 1) / kQTile : q_tiles;
+  y.fpb = pair_faces(nm + (nf + kPairFaces - 1) / kPairFaces, std::max<int64_t>(1, own));
+  y.grid = std::max<int64_t>(1, nm + (nf + y.fpb - 1) / y.fpb);   // at least the pair blocks needed
   const int64_t k = pair_splits(y.grid, n_q, 24);
   y.per_split = ((q_tiles + k - 1) / k) * kQTile;
   y.ks = (int)std::max<int64_t>(1, (n_q + y.per_split - 1) / y.per_split);
@@ -2161,11 +2250,11 @@ int mesh3d_backward_body(const float* verts, int64_t n_verts, const int32_t* fac
   const int bt = n_q >= 65536 ? kAux : 64;   // few points (faces below): smaller blocks, so that all SMs take part
   k_bq<3><<<blocks(n_q, bt), bt, 0, st>>>(q, grad_out, n_q, h, 1.0, at<QRec>(ws, y.qrec), at<int32_t>(ws, y.small));
   PFT_BWD_LAUNCH();
-  dim3 grid(blocks(n_faces, kPairFaces), (unsigned)y.ks);
+  dim3 grid(blocks(n_faces, y.fpb), (unsigned)y.ks);
   if (!allow_shared(k_bwd3)) return PFT_ERR_CUDA;
   PFT_MARK(g_ev_start);
   k_bwd3<<<grid, kBwdNT, sizeof(PairShared), st>>>(at<Face32>(ws, y.items), n_faces, at<QRec>(ws, y.qrec), n_q,
-                                                   y.per_split, th, at<double>(ws, y.partial), &h->status);
+                                                   y.per_split, th, y.fpb, at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
   if (launch_small_adjoint3(verts, n_verts, faces, n_faces, q, grad_out, n_q, h, at<void>(ws, y.phi), st) !=
@@ -2516,7 +2605,7 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   int64_t* bstart = at<int64_t>(ws, y.bstart);
   auto prep = [&](auto kernel, int nt) {
     kernel<<<(unsigned)n_meshes, nt, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes, recs, mc, nblk, deg, q,
-                                              n_q, at<float2>(ws, y.qsplit), h);
+                                              n_q, at<float2>(ws, y.qsplit), y.fpb, h);
   };
   if (n_faces > 512 * n_meshes) prep(k_bbprep3<1024>, 1024);
   else prep(k_bbprep3<kAux>, kAux);
@@ -2536,7 +2625,8 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   if (!allow_shared(k_bbwd3)) return PFT_ERR_CUDA;
   PFT_MARK(g_ev_start);
   k_bbwd3<<<grid, kBwdNT, sizeof(PairShared), st>>>(recs, n_faces, mesh_off, n_meshes, bstart, nblk,
-                                   at<QRec>(ws, y.rec), q_off, n_q, y.per_split, th, at<double>(ws, y.partial), &h->status);
+                                                     at<QRec>(ws, y.rec), q_off, n_q, y.per_split, th, y.fpb,
+                                                     at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
   k_bbcorner3<<<blocks(n_faces, kAux), kAux, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes,
