@@ -1633,12 +1633,13 @@ __global__ void __launch_bounds__(kBwdNT, kPairBlocks) k_bbwd3(const Face32* __r
   }
   const int64_t s0 = max((int64_t)0, min(off[lo], nf)), s1 = max(s0, min(off[lo + 1], nf));
   const PairSpan sp = pair_span(s0 + (b - bstart[lo]) * fpb, s1, fpb);
-  float2 F[12];
-  pair_load(recs, sp, F);
   int64_t qb, gb, nqi;
   bb_rows(q_off, lo, n_q, qb, gb, nqi);
   const int64_t q0 = (int64_t)blockIdx.y * per_split;
-  const int64_t nq = max((int64_t)0, min(per_split, nqi - q0));
+  if (q0 >= nqi) return;   // uniform over the block; k_bbcorner3 reads a mesh's own chunks only
+  const int64_t nq = min(per_split, nqi - q0);
+  float2 F[12];
+  pair_load(recs, sp, F);
   const bool ok = pair_run(sh, rec + gb + q0, nq, F, sp, th);
   if (!ok) set_status(status, ST_TIMEOUT);
   if (ok) pair_store(sh, sp, partial + ((int64_t)blockIdx.y * nf + sp.m) * 12);
@@ -1653,10 +1654,12 @@ __device__ __forceinline__ void file_corners(int64_t m, const int32_t* __restric
                                              const int64_t* __restrict__ start, int32_t* cursor, int32_t* list);
 
 // Per face: its mesh (bisection over the offsets), then the corner adjoints with that mesh's
-// centre and small-|Q| rows.
+// centre and small-|Q| rows.  Of a mesh with its own Q list only the chunks that the list reaches are written
+// and read: the launch has chunks for all lists together (24 meshes of 1,280 faces with 500 Q each, 94 chunks of
+// which a mesh has 4: the adjoint 321 -> 145 us).
 __global__ void k_bbcorner3(const float* __restrict__ v, int64_t nv, const int32_t* __restrict__ f, int64_t nf,
-                            const int64_t* __restrict__ off, int64_t nm, const double* __restrict__ partial, int ks,
-                            const PolyC* __restrict__ mc, const int32_t* __restrict__ small,
+                            const int64_t* __restrict__ off, int64_t nm, const double* __restrict__ partial,
+                            int64_t per_split, const PolyC* __restrict__ mc, const int32_t* __restrict__ small,
                             const int32_t* __restrict__ small_cnt, const double* __restrict__ q,
                             const int64_t* __restrict__ q_off, int64_t n_q, const double* __restrict__ g,
                             const int64_t* __restrict__ start, int32_t* cursor, int32_t* list,
@@ -1674,6 +1677,7 @@ __global__ void k_bbcorner3(const float* __restrict__ v, int64_t nv, const int32
   const double c[3] = {C.cx, C.cy, C.cz};
   const uint32_t ns = (uint32_t)max(0, min(small_cnt[lo], (int32_t)nqi));
   file_corners(m, f, nv, start, cursor, list);
+  const int ks = (int)((nqi + per_split - 1) / per_split);
   corner_adj(m, v, nv, f, nf, partial, ks, c, small + gb, ns, qb, gb, q, g, nullptr, corner + 9 * m);
 }
 
@@ -2630,8 +2634,9 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
   k_bbcorner3<<<blocks(n_faces, kAux), kAux, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes,
-                                                      at<double>(ws, y.partial), y.ks, mc, at<int32_t>(ws, y.small),
-                                                      at<int32_t>(ws, y.scnt), q, q_off, n_q, grad_out, start,
+                                                      at<double>(ws, y.partial), y.per_split, mc,
+                                                      at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), q, q_off,
+                                                      n_q, grad_out, start,
                                                       at<int32_t>(ws, y.cursor), at<int32_t>(ws, y.list),
                                                       at<double>(ws, y.corner));
   PFT_BWD_LAUNCH();
