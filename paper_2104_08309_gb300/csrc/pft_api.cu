@@ -57,7 +57,11 @@ int resolve(const pft_options* o, int dim, Opts& out) {
 // Padded pairs (groups of 128 Q points x tiles of 128 faces) below which a 3D FP32 launch runs
 // k_fwd_group.  Kernel times, k_fwd with up to one tile a chunk against k_fwd_group: 320 faces x 241 Q
 // 67 / 19 us, 5,120 x 520 35 / 17, 5,120 x 2,000 45 / 36, 20,480 x 520 49 / 36; past the line 5,120 x
-// 5,000 59 / 69, 20 x 200,000 30 / 52, 20,480 x 2,928 116 / 137.
+// 5,000 59 / 69, 20,480 x 2,928 116 / 137.
+// Of a single tile with few faces, k_fwd_group's time hardly falls (its warps hand their sums on one after the
+// other), while k_fwd's blocks of 512 Q points walk just these faces: past 6 blocks a face and 20 more, k_fwd.
+// Calls, k_fwd / k_fwd_group: 1 face x 20,000 Q 31 / 33 us, x 180,000 52 / 67; 12 faces x 30,000 38 / 36, x 50,000 40 / 43,
+// x 180,000 60 / 77; 20 x 50,000 44 / 44, x 180,000 69 / 81; 32 x 78,000 62 / 57, x 140,000 66 / 72; 128 x 180,000 177 / 155.
 constexpr int64_t kGroupPairs = 24000000;
 
 // Split-K choice: the smallest number of chunks that fills the GPU in whole
@@ -74,7 +78,8 @@ FwdLaunch plan_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_q, int fin
     // k_fwd_group below kGroupPairs (padded) pairs
     const int64_t tiles = (n_items + tile - 1) / tile, rest = n_q % 512;
     const int64_t groups = 4 * (n_q / 512) + std::min<int64_t>(4, (rest + 31) / 32);
-    if (groups * 128 * tiles * tile < kGroupPairs && tiles <= 65535) {
+    const bool few = tiles == 1 && (n_q + 511) / 512 > 6 * n_items + 20;
+    if (groups * 128 * tiles * tile < kGroupPairs && tiles <= 65535 && !few) {
       L.group = true;
       L.q_tiles = groups;
       L.k_splits = (int)tiles;
