@@ -412,10 +412,11 @@ int pft_backward_last_launch_count(void);
  * counterpart; this is a calling convenience.)
  *  - Same arguments, result and options as pft3d_mesh, minus ws / ws_bytes.
  *    It allocates nothing and calls no allocating routine.
- *  - Scratch is a file-scope device array of 33 MiB, which every GPU that loads
- *    the library keeps until the process exits.  Problems whose
- *    pft3d_workspace_size() exceeds 32 MiB, not counting the up to 0.6 MiB that the
- *    small-|Q| pass adds to it, return PFT_ERR_SCRATCH_LIMIT at once.
+ *  - Scratch is a file-scope device array of 65 MiB, which every GPU that loads
+ *    the library keeps until the process exits.  Problems that need more than 32 MiB
+ *    of workspace, not counting up to 0.6 MiB that the small-|Q| pass adds and what
+ *    finer launch plans add, return PFT_ERR_SCRATCH_LIMIT at once (pft3d_workspace_size()
+ *    up to 32 MiB is always taken; up to 65 MiB may be).
  *  - All calls on a device share that array and it keeps the last call's
  *    contents; calls whose GPU work overlaps (several streams or host threads)
  *    race on it, so serialise them.

@@ -205,15 +205,24 @@ FwdLayout layout_plan(int dim, const Opts& o, int64_t n_items, int64_t n_prep, i
   return y;
 }
 
-// A finer plan's partial sums must not push a problem out of the allocation-free call's scratch: one
-// that fits it with a coarser plan takes that (327,680 faces x 1,000 Q: 854 chunks; with the coarsest plan the
-// call took 1,151 us instead of 605).
+// The finest plan, but for problems that the allocation-free call takes (its limit asks for some plan that fits it)
+// the finest that fits kFineBytes more: that call has them, and so runs with the plan, and to the bit the result,
+// of the call with a workspace.  (With the finer plans held to the limit itself, 650,000 faces x 1,000 Q took 1,264 us
+// and 690,000, which fit it with no plan of these, 948; now 912.  690,000 x 241 Q 1,899 us, now 586.)
 FwdLayout layout_fwd(int dim, const Opts& o, int64_t n_items, int64_t n_prep, int64_t n_q) {
-  for (const int fine : {2048, 1024, 512, 256, 128, 0}) {
-    const FwdLayout y = layout_plan(dim, o, n_items, n_prep, n_q, fine);
-    if (y.total - y.grown <= kScratchLimit) return y;
+  constexpr int kPlans = 6, kFine[kPlans] = {2048, 1024, 512, 256, 128, 0};
+  FwdLayout y[kPlans];
+  size_t least = SIZE_MAX;
+  for (int i = 0; i < kPlans; ++i) {
+    y[i] = layout_plan(dim, o, n_items, n_prep, n_q, kFine[i]);
+    least = std::min(least, y[i].total - y[i].grown);
+    if (i == 0 && least <= kScratchLimit) return y[0];
   }
-  return layout_plan(dim, o, n_items, n_prep, n_q, 2048);
+  int i = 0;
+  if (least <= kScratchLimit)
+    while (y[i].total - y[i].grown > kScratchLimit + kFineBytes) ++i;
+  y[i].grown = y[i].total - least;
+  return y[i];
 }
 
 template <typename T>
@@ -246,7 +255,7 @@ inline cudaError_t mark(cudaEvent_t ev, cudaStream_t st) { return ev ? cudaEvent
 
 }  // namespace
 
-size_t small3_growth(int64_t n_faces, int64_t n_q, const pft_options* opts) {
+size_t uncounted_bytes(int64_t n_faces, int64_t n_q, const pft_options* opts) {
   Opts o;
   if (resolve(opts, 3, o) != PFT_OK) return 0;
   return layout_fwd(3, o, n_faces, n_faces, n_q).grown;

@@ -69,8 +69,10 @@ __device__ __forceinline__ void simplex_series(const double* x, double& re, doub
   }
 }
 
-// Largest workspace, without what the small-|Q| pass adds to it, that pft3d_mesh_noalloc takes.
+// Largest workspace, with the plan that needs least and without what the small-|Q| pass adds to it, that
+// pft3d_mesh_noalloc takes; and what a finer plan of such a problem may need beyond that.
 constexpr size_t kScratchLimit = size_t(32) << 20;   // 32 MiB
+constexpr size_t kFineBytes = size_t(32) << 20;
 
 // Launch description computed on the host.
 struct FwdLaunch {

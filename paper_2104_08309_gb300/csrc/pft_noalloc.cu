@@ -28,9 +28,9 @@
 namespace pft {
 namespace {
 
-// 33 MiB per device: the limit on a problem's workspace without what the small-|Q| pass adds to it,
-// and room for that (at most 0.6 MiB).
-constexpr size_t kScratchBytes = kScratchLimit + (size_t(1) << 20);
+// 65 MiB per device: the limit on a problem's workspace with the plan that needs least and without what the
+// small-|Q| pass adds to it, and room for a finer plan and for that (at most 0.6 MiB).
+constexpr size_t kScratchBytes = kScratchLimit + kFineBytes + (size_t(1) << 20);
 constexpr int kMaxDevices = 64;
 
 // The scratch array.  In host code this name is only a stand-in for the device
@@ -71,7 +71,8 @@ extern "C" int pft3d_mesh_noalloc(const float* verts, int64_t n_verts, const int
   // Sizes or options that pft3d_workspace_size rejects: pft3d_mesh refuses them
   // before it looks at the workspace, with the code it would give any caller.
   if (need == 0) return pft3d_mesh(verts, n_verts, faces, n_faces, q, n_q, out, nullptr, 0, opts, stream);
-  if (need - pft::small3_growth(n_faces, n_q, opts) > pft::kScratchLimit || need > pft::kScratchBytes) return PFT_ERR_SCRATCH_LIMIT;
+  if (need - pft::uncounted_bytes(n_faces, n_q, opts) > pft::kScratchLimit || need > pft::kScratchBytes)
+    return PFT_ERR_SCRATCH_LIMIT;
   void* scratch = nullptr;
   if (int e = pft::scratch_address(static_cast<cudaStream_t>(stream), &scratch)) return e;
   // The header at the start of the scratch (status word, counters, bounding box)

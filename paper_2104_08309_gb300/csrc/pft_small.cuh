@@ -170,8 +170,8 @@ __device__ __forceinline__ void mom_eval(const double* m, double x, double y, do
   im = v[1];
 }
 
-// Bytes by which the scratch exceeds the records of a pft3d_mesh call (part of its workspace size).
-size_t small3_growth(int64_t n_faces, int64_t n_q, const pft_options* opts);
+// Bytes of a pft3d_mesh workspace that pft3d_mesh_noalloc's limit does not count.
+size_t uncounted_bytes(int64_t n_faces, int64_t n_q, const pft_options* opts);
 
 // pft_small.cu.  q = NULL: the moments for the Q-gradient, where qsmall_direct does not hold.
 cudaError_t launch_small3(const float* v, int64_t nv, const int32_t* f, int64_t nf, const double* q, WsHeader* h,
