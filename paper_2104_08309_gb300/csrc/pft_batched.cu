@@ -607,7 +607,9 @@ __device__ __forceinline__ void finish_out_f32(const float* Q, const float* Qlo,
 // warp to finish a slot issues the tile kStages further on (as in k_fwd).
 // Register budget: as the single-shape kernel, except that the 3D FP32 shapes with 128 threads
 // keep one block per SM fewer here (4 at 4 Q points, 5 at 2), where the item loop and the
-// in-place finish would otherwise spill, and that 512 threads are one block per SM (up to 128
+// in-place finish would otherwise spill, that the 2D one with 4 Q points keeps five (it fits 92 registers, but
+// takes 102 by itself: 4,096 8-gons with 2,000 Q points each 407 us with four, 376 with five), that 2D with
+// 8 Q points is left free (155 and more), and that 512 threads are one block per SM (up to 128
 // registers: 16 warps, as 2 x 256 or 4 x 128).
 // Records per tile of the batched kernel's ring.  With one block of 16 warps per SM walking it (the
 // 512-thread shapes), 256 segments ran faster than 128 (4,096 polygons: 7.63 against 7.70 ms) and
@@ -619,6 +621,8 @@ constexpr int kBTile = NT >= 512 ? (Pol::kDim == 2 ? 256 : 128) : Pol::kTile;
 template <class Pol, int R, int NT>
 constexpr int kBatchedMinBlocks = NT >= 512 ? 1
                                   : (Pol::kDim == 3 && R == 4 && NT == 128) ? 4
+                                  : (Pol::kDim == 2 && R == 4 && NT == 128 && sizeof(typename Pol::QT) == 4) ? 5
+                                  : (Pol::kDim == 2 && R == 8) ? (NT == 256 ? 1 : 2)
                                   : (Pol::kDim == 3 && R == 2 && NT == 128 && sizeof(typename Pol::QT) == 4)
                                       ? 5
                                       : kMinBlocks<Pol, R, NT>;
