@@ -987,8 +987,8 @@ cudaError_t launch_batched_one(int grid, const BPlanHeader* ph, const int32_t* c
 #define PFT_BATCHED_CASES(X)                                                                          \
   X(Pol2F32, 1, 128) X(Pol2F32, 2, 128) X(Pol2F32, 4, 128) X(Pol2F32, 8, 128) X(Pol2F32, 1, 256)      \
   X(Pol2F32, 2, 256) X(Pol2F32, 4, 256) X(Pol2F32, 8, 256) X(Pol2F64, 1, 128) X(Pol2F64, 2, 128)      \
-  X(Pol2F64, 1, 256) X(Pol2F64, 2, 256) X(Pol3F32, 2, 128) X(Pol3F32, 4, 128) X(Pol3F64, 1, 128)      \
-  X(Pol2F32, 4, 512) X(Pol3F32, 4, 512)
+  X(Pol2F64, 1, 256) X(Pol2F64, 2, 256) X(Pol3F32Batch, 2, 128) X(Pol3F32Batch, 4, 128) X(Pol3F64, 1, 128)      \
+  X(Pol2F32, 4, 512) X(Pol3F32Batch, 4, 512)
 
 #define PFT_BATCHED_MATCH(P, RR, NN) \
   (P::kDim == dim && (sizeof(P::QT) == 8) == fp64 && r == RR && nt == NN)

@@ -237,7 +237,8 @@ __device__ __forceinline__ void sincos_v(float2 x, float2& sn, float2& cs) {
 __device__ __forceinline__ float rcp_or0(float x2) { return x2 > 0.f ? rcp_approx(x2) : 0.f; }
 __device__ __forceinline__ float2 rcp_or0(float2 x2) { return make_float2(rcp_or0(x2.x), rcp_or0(x2.y)); }
 
-template <bool kShared, class V>
+// kEach: the large-argument sinc of each element in a branch of its own (below).
+template <bool kShared, bool kEach, class V>
 __device__ __forceinline__ void face_edge(V qx, V qy, V qz, const float4 A, const float4 B, const float4 C,
                                           V a0, V a1, V& zr, V& zi, V& S0) {
   const float nx = C.y, ny = C.z, nz = C.w;
@@ -267,7 +268,9 @@ __device__ __forceinline__ void face_edge(V qx, V qy, V qz, const float4 A, cons
   // an edge with |Q.d_l| > 2 pi somewhere in the warp (face_edge runs warp-converged): the sincs on the SFU,
   // both elements in paired code and selected by lane.  All edges at once: a vote for each (most slivers have
   // a short one) ran the prism at 10.24 instead of 10.63 ms, but 327,680 faces x 881,730 Q, which has few edge
-  // sums, at 318.9 instead of 315.2 ms.
+  // sums, at 318.9 instead of 315.2 ms.  In the batched kernel even that costs more than it gives, but for meshes
+  // of a few faces (1,024 meshes of 5,120 faces x 4,096 Q 26.48 ms, with a branch for each element 25.88; of 320 and
+  // 1,280 faces 0.5 and 1.5 %; of 20 faces 0.40 against 0.43 ms): kEach.
   constexpr int kE = sizeof(V) / sizeof(float);
   bool big = false;
 #pragma unroll
@@ -277,9 +280,15 @@ __device__ __forceinline__ void face_edge(V qx, V qy, V qz, const float4 A, cons
   if (__any_sync(0xffffffffu, big)) {
 #pragma unroll
     for (int l = kShared ? 1 : 0; l < 3; ++l) {
-      const V L = sinc_large(u[l]);
+      if constexpr (kEach) {
 #pragma unroll
-      for (int e = 0; e < kE; ++e) el(&S[l], e) = el(&u2[l], e) > kPi2 ? el(&L, e) : el(&S[l], e);
+        for (int e = 0; e < kE; ++e)
+          if (el(&u2[l], e) > kPi2) el(&S[l], e) = sinc_large(el(&u[l], e));
+      } else {
+        const V L = sinc_large(u[l]);
+#pragma unroll
+        for (int e = 0; e < kE; ++e) el(&S[l], e) = el(&u2[l], e) > kPi2 ? el(&L, e) : el(&S[l], e);
+      }
     }
   }
   if (kShared) S[0] = S0;
@@ -481,12 +490,12 @@ struct FaceQ {
     }
   }
   // the edge sum (per Q point), with the few Q points below tau_lo^2/4 redone by the short series
-  template <bool kShared>
+  template <bool kShared, bool kEach = false>
   __device__ __forceinline__ void edge(const Thr& th, const V (&qv)[N][3], const float4 A, const float4 B,
                                        const float4 C, V (&zr)[N], V (&zi)[N], V (&S0)[N]) const {
 #pragma unroll
     for (int j = 0; j < N; ++j)
-      face_edge<kShared>(qv[j][0], qv[j][1], qv[j][2], A, B, C, a0[j], a1[j], zr[j], zi[j], S0[j]);
+      face_edge<kShared, kEach>(qv[j][0], qv[j][1], qv[j][2], A, B, C, a0[j], a1[j], zr[j], zi[j], S0[j]);
     if (pmin < th.lo) {
 #pragma unroll
       for (int r = 0; r < R; ++r)
@@ -502,8 +511,8 @@ struct FaceQ {
 // kPairs: faces [0, th.pair_end) come in pairs that share their first edge (face_pairs option): when
 // both faces of a pair take the edge sum in a warp, the second takes the shared edge's sinc from the
 // first (carried in registers from one face to the next).  A separate instantiation, so that the
-// single-face kernel is unchanged.
-template <bool kPairs>
+// single-face kernel is unchanged.  kEach: see face_edge (the batched kernel's policy).
+template <bool kPairs, bool kEach = false>
 struct Pol3F32T {
   using Item = Face32;
   // 128 faces (6 KB) per tile: on the 1.31M-face mesh x 128^3 Q, 3262 against 3283 ms at 64
@@ -539,10 +548,10 @@ struct Pol3F32T {
       } else if (kPairs && held && first + i < th.pair_end) {
         // the second face of a pair whose first face took the edge sum in this warp: the shared
         // edge's sinc comes from it
-        f.template edge<true>(th, qv, A, B, C, zr, zi, S0);
+        f.template edge<true, kEach>(th, qv, A, B, C, zr, zi, S0);
         held = false;
       } else {
-        f.template edge<false>(th, qv, A, B, C, zr, zi, S0);
+        f.template edge<false, kEach>(th, qv, A, B, C, zr, zi, S0);
         held = kPairs && ((first + i) & 1) == 0 && first + i < th.pair_end;   // the first face of a pair
       }
       f.finish(zr, zi, tre, tim);
@@ -553,6 +562,7 @@ struct Pol3F32T {
 };
 using Pol3F32 = Pol3F32T<false>;
 using Pol3F32Pair = Pol3F32T<true>;
+using Pol3F32Batch = Pol3F32T<false, true>;
 
 struct Pol3F64 {
   using Item = Face64;
