@@ -1358,7 +1358,8 @@ __global__ void __launch_bounds__(NT) k_bbq(const double* __restrict__ q, const 
       }
 #pragma unroll
       for (int d = 0; d < D; ++d) t = fmaf(Q[d].y, chi[d], fmaf(Q[d].x, clo[d], t));
-      if (!(n * P.rmax * P.rmax > 1.01f * (float)(kTauSmallQ * kTauSmallQ))) {
+      // FP32 settles what is clear of the small-|Q| bound; |Q|^2 beyond its range, as for a shape of 1e-20, asks FP64
+      if (!(n * P.rmax * P.rmax > 1.01f * (float)(kTauSmallQ * kTauSmallQ) && n <= 3.402823466e38f)) {
         const double Qx = q[D * (qb + l)], Qy = q[D * (qb + l) + 1], Qz = D == 3 ? q[D * (qb + l) + D - 1] : 0.0;
         const double q2 = q_norm2(Qx, Qy, Qz);
         is_small = q2 == 0.0 || q2 * ((double)P.rmax * (double)P.rmax) < kTauSmallQ * kTauSmallQ;
@@ -1377,7 +1378,7 @@ __global__ void __launch_bounds__(NT) k_bbq(const double* __restrict__ q, const 
         float sp, cp;
         sincosf(-pr, &sp, &cp);
         const float gr = (float)g[2 * (gb + l)], gi = (float)g[2 * (gb + l) + 1];
-        const float k = n > 3e38f ? 0.f : (D == 2 ? 2.0f : 1.0f) / (n + nt);   // |Q|^2 beyond FP32: 0
+        const float k = n <= 3.402823466e38f ? (D == 2 ? 2.0f : 1.0f) / (n + nt) : 0.f;   // |Q|^2 beyond FP32: 0
         wr = k * fmaf(gr, cp, -gi * sp);
         wi = k * fmaf(gr, sp, gi * cp);
       }
