@@ -1245,11 +1245,12 @@ __device__ __forceinline__ void split_q(const double* __restrict__ q, int64_t n,
 
 // One block per polygon: offset checks, bounding-box centre, segment records relative to it,
 // max radius, and the number of pair blocks (kBbSegs segments each) the polygon needs.
-__global__ void __launch_bounds__(kAux) k_bbprep(const float* __restrict__ v, int64_t nv,
+template <int NT>
+__global__ void __launch_bounds__(NT) k_bbprep(const float* __restrict__ v, int64_t nv,
                                                  const int64_t* __restrict__ off, int64_t np, Seg32* segs,
                                                  PolyC* pc, int32_t* nblk, const double* __restrict__ q, int64_t n_q,
                                                  float2* __restrict__ qs, WsHeader* h) {
-  __shared__ float sh[kAux / 32];
+  __shared__ float sh[NT / 32];
   split_q(q, 2 * n_q, qs);
   const int64_t i = blockIdx.x;
   const int64_t s0 = off[i], s1 = off[i + 1];
@@ -1258,7 +1259,7 @@ __global__ void __launch_bounds__(kAux) k_bbprep(const float* __restrict__ v, in
   const int64_t b0 = max((int64_t)0, min(s0, nv)), n = max((int64_t)0, min(s1, nv) - b0);
   float mn[2] = {3.4e38f, 3.4e38f}, mx[2] = {-3.4e38f, -3.4e38f};
   bool bad = false;
-  for (int64_t j = threadIdx.x; j < n; j += kAux)
+  for (int64_t j = threadIdx.x; j < n; j += NT)
     for (int d = 0; d < 2; ++d) {
       const float x = v[2 * (b0 + j) + d];
       if (!isfinite(x)) { bad = true; continue; }
@@ -1268,11 +1269,11 @@ __global__ void __launch_bounds__(kAux) k_bbprep(const float* __restrict__ v, in
   if (bad) set_status(&h->status, ST_NONFINITE);
   double c[2];
   for (int d = 0; d < 2; ++d) {
-    const float lo = block_minmax_f(mn[d], false, sh), hi = block_minmax_f(mx[d], true, sh);
+    const float lo = block_minmax_f<NT>(mn[d], false, sh), hi = block_minmax_f<NT>(mx[d], true, sh);
     c[d] = (n > 0 && lo <= hi) ? 0.5 * ((double)lo + (double)hi) : 0.0;
   }
   float rm = 0.f;
-  for (int64_t j = threadIdx.x; j < n; j += kAux) {
+  for (int64_t j = threadIdx.x; j < n; j += NT) {
     const int64_t a = b0 + j, b = b0 + (j + 1 < n ? j + 1 : 0);
     const double x0 = (double)v[2 * a] - c[0], y0 = (double)v[2 * a + 1] - c[1];
     const double x1 = (double)v[2 * b] - c[0], y1 = (double)v[2 * b + 1] - c[1];
@@ -1280,7 +1281,7 @@ __global__ void __launch_bounds__(kAux) k_bbprep(const float* __restrict__ v, in
                     (float)(0.5 * (y1 - y0))};
     rm = fmaxf(rm, __double2float_ru(sqrt(x0 * x0 + y0 * y0)));
   }
-  rm = block_minmax_f(rm, true, sh);
+  rm = block_minmax_f<NT>(rm, true, sh);
   if (threadIdx.x == 0) {
     pc[i] = PolyC{c[0], c[1], 0.0, rm, 0};
     nblk[i] = (int32_t)((n + kBbSegs - 1) / kBbSegs);
@@ -2223,6 +2224,23 @@ using namespace pft;
 namespace pft {
 namespace {
 
+// The batched adjoints' kernels with a block per shape: of kFewItems threads where shapes (or lists) have no more
+// segments (or rows) on average.  20,000 polygons of 8 segments, 256 / 64 threads: k_bbprep 134 / 63 us, k_bbq 80 / 26 us for
+// 16 rows each and 84 / 29 us for 64.  k_bbq takes 1,024 where the shapes are few: it is bound by latency there.
+constexpr int kFewItems = 64;
+// Whether so few blocks of nt threads would take more than four rounds of split_q (few shapes, many Q points).
+bool splits_long(int64_t n, int64_t blocks, int nt) { return blocks < 4 * sm_count() && n > 4 * nt * blocks; }
+template <int D>
+void launch_bbq(const double* q, const float2* qs, const int64_t* q_off, const double* g, int64_t n_q, int64_t n,
+                const PolyC* pc, QRec* rec, int32_t* small, int32_t* small_cnt, WsHeader* h, cudaStream_t st) {
+  auto go = [&](auto kernel, int nt) {
+    kernel<<<(unsigned)n, nt, 0, st>>>(q, qs, q_off, g, n_q, n, pc, rec, small, small_cnt, h);
+  };
+  if (n_q <= kFewItems * (q_off != nullptr ? n : 1)) go(k_bbq<D, kFewItems>, kFewItems);
+  else if (n < 4 * sm_count()) go(k_bbq<D, 1024>, 1024);
+  else go(k_bbq<D, kAux>, kAux);
+}
+
 // Header reset and, where there is work, the bounding box and zeroed corner counts.  Returns a status to
 // return at once (nothing to do, or an error), or -1 to go on.
 int start3d(const float* verts, int64_t n_verts, int64_t n_faces, int64_t n_q, float* grad_verts, void* ws,
@@ -2544,16 +2562,17 @@ int pft2d_polygons_batched_backward(const float* verts, int64_t n_verts, const i
   PolyC* pc = at<PolyC>(ws, y.pc);
   int32_t* nblk = at<int32_t>(ws, y.nblk);
   int64_t* bstart = at<int64_t>(ws, y.bstart);
-  k_bbprep<<<(unsigned)n_polys, kAux, 0, st>>>(verts, n_verts, poly_off, n_polys, segs, pc, nblk, q, n_q,
-                                               at<float2>(ws, y.qsplit), h);
+  auto prep = [&](auto kernel, int nt) {
+    kernel<<<(unsigned)n_polys, nt, 0, st>>>(verts, n_verts, poly_off, n_polys, segs, pc, nblk, q, n_q,
+                                             at<float2>(ws, y.qsplit), h);
+  };
+  if (n_verts > kFewItems * n_polys || splits_long(2 * n_q, n_polys, kFewItems)) prep(k_bbprep<kAux>, kAux);
+  else prep(k_bbprep<kFewItems>, kFewItems);
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_polys, bstart);
   PFT_BWD_LAUNCH();
-  // one block per shape, bound by latency where there are few
-  if (n_polys < 4 * sm_count()) k_bbq<2, 1024><<<(unsigned)n_polys, 1024, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
-                                            at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
-  else k_bbq<2, kAux><<<(unsigned)n_polys, kAux, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
-                                            at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
+  launch_bbq<2>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_polys, pc, at<QRec>(ws, y.rec),
+                at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h, st);
   PFT_BWD_LAUNCH();
   if (y.grid > INT32_MAX) return PFT_ERR_UNSUPPORTED;
   dim3 grid((unsigned)y.grid, (unsigned)y.ks);
@@ -2612,7 +2631,7 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
     kernel<<<(unsigned)n_meshes, nt, 0, st>>>(verts, n_verts, faces, n_faces, mesh_off, n_meshes, recs, mc, nblk, deg, q,
                                               n_q, at<float2>(ws, y.qsplit), y.fpb, h);
   };
-  if (n_faces > 512 * n_meshes) prep(k_bbprep3<1024>, 1024);
+  if (n_faces > 512 * n_meshes || splits_long(3 * n_q, n_meshes, kAux)) prep(k_bbprep3<1024>, 1024);
   else prep(k_bbprep3<kAux>, kAux);
   PFT_BWD_LAUNCH();
   k_scan<<<1, kScanT, 0, st>>>(nblk, n_meshes, bstart);
@@ -2620,11 +2639,8 @@ int pft3d_meshes_batched_backward(const float* verts, int64_t n_verts, const int
   int64_t* start = at<int64_t>(ws, y.start);
   k_places<<<blocks(n_verts, kAux), kAux, 0, st>>>(deg, n_verts, start, h);
   PFT_BWD_LAUNCH();
-  // one block per shape, bound by latency where there are few
-  if (n_meshes < 4 * sm_count()) k_bbq<3, 1024><<<(unsigned)n_meshes, 1024, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
-                                                at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
-  else k_bbq<3, kAux><<<(unsigned)n_meshes, kAux, 0, st>>>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
-                                                at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h);
+  launch_bbq<3>(q, at<float2>(ws, y.qsplit), q_off, grad_out, n_q, n_meshes, mc, at<QRec>(ws, y.rec),
+                at<int32_t>(ws, y.small), at<int32_t>(ws, y.scnt), h, st);
   PFT_BWD_LAUNCH();
   dim3 grid((unsigned)y.grid, (unsigned)y.ks);
   if (!allow_shared(k_bbwd3)) return PFT_ERR_CUDA;
