@@ -8,8 +8,8 @@
 //  * k_bq: per Q, the weight gt = g exp(-iQ.c) * scale / |Q|^2 that carries the
 //    finalize factors onto each pair (scale 2 in 2D for the half vectors), and
 //    the list of Q = 0 / small-|Q| points, which take an FP64 path instead;
-//  * k_bwd2d / k_bwd3d: thread <-> segment or face, Q records streamed through
-//    shared memory by the same bulk-copy ring as the forward kernels, adjoints
+//  * k_bwd2 / k_bwd3: thread <-> segment, or one or two faces, Q records streamed
+//    through shared memory by the same bulk-copy ring as the forward kernels, adjoints
 //    of the record fields accumulated per thread, FP64 partials per Q chunk;
 //  * FP64 small-|Q| contributions from the boundary-flux (shape derivative)
 //    series, then a fixed-order gather to the vertices (3D through a vertex ->
@@ -120,8 +120,8 @@ __device__ __forceinline__ void sinc_d(V u, V& S, V& dS) {
   bool big = false;
 #pragma unroll
   for (int e = 0; e < kE; ++e) big = big || (el(&v, e) > kPi2);
-  // warp-uniform: the SFU work only where some lane needs it (both elements evaluated and selected, as in the
-  // forward: k_bbwd on 2.7e6 segments x 4,096 Q 15.79 instead of 15.37 ms)
+  // warp-uniform: the SFU work only where some lane needs it, a branch for each element (both evaluated and
+  // selected, as in the forward, ran k_bbwd on 2.7e6 segments x 4,096 Q at 15.79 instead of 15.37 ms)
   if (__any_sync(__activemask(), big)) {
 #pragma unroll
     for (int e = 0; e < kE; ++e) {

@@ -38,7 +38,7 @@ struct WsHeader {
   uint32_t small_q_count;   // number of Q points routed to the FP64 small-|Q| pass
   uint32_t bbox_enc[6];     // order-preserving encodings: min x,y,z then max x,y,z
   uint32_t rmax_bits;       // max |v - c| as float bits (non-negative floats order as ints)
-  uint32_t ticket;          // blocks of k_small3 that have written their part
+  uint32_t ticket;          // blocks of k_small3 (or, in the vertex adjoint, k_phi) that have written their part
   double center[3];         // bounding-box midpoint c (all coordinates are taken relative to c)
   double measure;           // volume (3D forward), FP64, fixed-order sum
   int32_t small_list[kSmallDirect];   // the first listed small Q points (3D forward)
@@ -111,7 +111,10 @@ constexpr float kPi2 = 9.86960440108935861883f;   // pi^2
 // 1.5 * 2^23 (|t| < 2^22), two elements an instruction, where rintf is a conversion per element on the
 // SFU's pipe; the same bits.  With it, the forward kernels evaluate both elements and select, where each
 // element had a divergent block of its own: 32,760 sliver faces x 131,072 Q 11.21 -> 10.63 ms, 2.7e6 segments x
-// 4,096 Q 7.64 -> 7.34 ms.  The adjoint's sinc_d, with sin and cos, keeps a block per element.
+// 4,096 Q 7.64 -> 7.34 ms, 1,000 long segments x 1e6 Q 1.23 -> 1.10 ms; where few lanes need it, it costs (a noisy outline
+// of 100,000 short segments x 16,384 Q 1.20 -> 1.24 ms).  A vote, or a branch, for each pair of elements in 2D ran the
+// 2.7e6 segments at 8.45 and 7.94 ms.  The adjoint's sinc_d, with sin and cos, and the batched 3D kernel keep a
+// block per element.
 __device__ __forceinline__ float turn_rest(float t) { return kTwoPi * (t - rintf(t)); }
 __device__ __forceinline__ float2 turn_rest(float2 t) {
   constexpr float kM = 12582912.0f;

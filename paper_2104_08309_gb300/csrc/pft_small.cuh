@@ -3,19 +3,20 @@
 //
 // There S0(Q) = sum over the signed tetrahedra (c, p0, p1, p2) of det sum_k i^k h_k(x)/(k+3)!,
 // x_j = Q.(p_j - c), is a power series in Q: with |x_j| < 1/4 the terms past k = 12 are below
-// 5e-19 of sum |det|/6.  Two ways to it:
+// 5e-19 of sum |det|/6.  Three ways to it:
 //  * kSmallDirect listed Q points or fewer: each evaluated over the faces, (Q point, face chunk)
 //    units spread over the grid, the chunk sums added in order by the finishing kernel;
 //  * more: the series' coefficients (moments of the shape, one per monomial of degree <= 12, 455
 //    of them) are summed over the faces once, and every small Q point evaluates the polynomial.
-// Of a shape of few faces the finishing kernel sums each point over the faces itself (small_few).
-// Line between them: a directly evaluated point costs about 70 FP64 operations a face and the moments
+//  * of a shape of few faces the finishing kernel sums each point over the faces itself (small_few).
+// Line between the first two: a directly evaluated point costs about 70 FP64 operations a face and the moments
 // about 900 with lanes to spare, so they break even near 30 points (on 20,480 faces 32 points take
 // 75 us at the FP64 rate, the moments 102).  A curve of 2,928 points on
 // 20,480 faces, 1,220 of them small: the call took 5,267 us with one block per point and 17 terms,
 // 233 us with the moments (k_small3 102 us, the polynomials in k_finalize3d 25 us).
-// Both run in FP64, except that monomials of degree >= 8, which together stay below 1.1e-10 of
-// the result, are summed in compensated FP32 (an error below 2e-17 of it).
+// Both run in FP64, except that monomials of degree >= 8, which together stay below 1.1e-10 of sum |det|/6,
+// are evaluated in FP32 and summed there in compensated pairs (some 16 roundings of 2^-24 on that: about
+// 1e-16 of sum |det|/6, what FP64 roundings of the other terms amount to).
 #pragma once
 
 #include "pft_kernels.cuh"
