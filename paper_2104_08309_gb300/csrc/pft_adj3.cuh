@@ -7,8 +7,8 @@
 // block, field by field as float2, and takes one Q point at a time, its fields broadcast (doubling them in
 // shared memory, 48 B a record, ran 2-3 % slower: 5.82 against 5.69 ms on 81,920 faces x 32,768 Q; two Q
 // points of one face per thread took 168-182 registers and ran slower than scalar code: 11.7 against 9.3
-// ms).  The compensated sums, touched once per tile, live in shared memory.  Faces whose phases need the edge sum take the scalar pair
-// adjoint one after the other.
+// ms).  The compensated sums, touched once per tile, live in shared memory.  Where a warp's phases need the edge sum, a
+// thread's faces take it in scalar code, one after the other.  Blocks of few faces hold one a thread (pair_span).
 #pragma once
 
 #include "pft_pairs.cuh"

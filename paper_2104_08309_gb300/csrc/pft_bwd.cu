@@ -433,11 +433,11 @@ struct RecAdj {
   }
 };
 
-// Adds the record adjoints of one Q and one face f (12 fields) to a.
-template <bool kEdge, class Acc>
+// Adds the record adjoints of one Q and one face f (12 fields), by the edge sum, to a.
+template <class Acc>
 __device__ __forceinline__ void face_adj(const QRec& Q, const float (&f)[12], Thr th, Acc a) {
   RecAdj<Acc> o{a, Q.qx, Q.qy, Q.qz};
-  face_adj_t<kEdge>(Q, make_float4(f[0], f[1], f[2], f[3]), make_float4(f[4], f[5], f[6], f[7]),
+  face_adj_t<true>(Q, make_float4(f[0], f[1], f[2], f[3]), make_float4(f[4], f[5], f[6], f[7]),
                     make_float4(f[8], f[9], f[10], f[11]), th, o);
 }
 
@@ -933,7 +933,7 @@ constexpr int kPairBlocks = 4;   // resident blocks per SM the registers are hel
 // thread two, 2t and 2t + 1 of its warp's 64, for the paired series.  Fewer go one a thread (`single`), and where
 // they take one or two of the four warps only, the others hold copies and take their part of every tile's
 // records: two a thread leave the edge sums twice as long and most warps idle.
-// Adjoint call, two a thread / so: 20 faces a mesh, 1,024 meshes x 4,096 Q 7.87 / 1.81 ms, 96 meshes x 64 Q 126 / 70 us;
+// Adjoint call, two a thread / so: 20 faces a mesh, 1,024 meshes x 4,096 Q 7.87 / 1.72 ms, 96 meshes x 64 Q 126 / 62 us;
 // one mesh of 12 faces x 241 Q 188 / 67 us, of 80 x 4,096 217 / 135 us.
 struct PairSpan {
   int64_t m;
@@ -962,12 +962,14 @@ struct OneAcc {
   __device__ __forceinline__ float& operator()(int k) const { return a[k]; }
 };
 
-// The pair adjoint of one of a thread's two faces.
+// The edge sums of a thread's two faces, one after the other.  Both take it where one of them has to: deciding again
+// for each half, with the scalar series beside the edge sum, ran slivers (32,760 faces x 10,000 Q, nearly all edge
+// sums) at 2.95 instead of 2.69 ms.
 __device__ __forceinline__ void scalar_adj(const QRec& Q, const float2 (&F)[12], Thr th, float2 (&a)[12], bool second) {
   float f[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) f[k] = second ? F[k].y : F[k].x;
-  face_adj<true>(Q, f, th, HalfAcc{a, second});
+  face_adj(Q, f, th, HalfAcc{a, second});
 }
 
 __device__ __forceinline__ void acc_add(float2& c, float x) {
@@ -1019,10 +1021,7 @@ __device__ __forceinline__ bool pair_run(PairShared& sh, const QRec* rec, int64_
     if (live) {
       const QRec* tq = ring.tile(t);
       const int cnt = ring.count(t);
-      // Two faces side by side, unless the record in the tile's middle asks for the edge sum, which takes one face
-      // at a time anyway: slivers (32,760 faces x 10,000 Q, nearly all edge sums) 2.95 / 2.86 ms.  Asking costs
-      // 0.3 % of a tile.
-      if (!sp.single && !(AdjCommon<float2>(tq[cnt / 2], F).wmax() >= th.hi)) {
+      if (!sp.single) {
         float2 a[12];
 #pragma unroll
         for (int k = 0; k < 12; ++k) a[k] = vs<float2>(0.f);
@@ -1044,26 +1043,23 @@ __device__ __forceinline__ bool pair_run(PairShared& sh, const QRec* rec, int64_
           acc_add(sh.acc[2 * k + 1][threadIdx.x], a[k].y);
         }
       } else {
-        const int j0 = cnt * sp.copy / sp.copies, j1 = cnt * (sp.copy + 1) / sp.copies;
-#pragma unroll 1
-        for (int e = 0; e < (sp.single ? 1 : 2); ++e) {
-          float f[12], a[12];
+        const int j1 = cnt * (sp.copy + 1) / sp.copies;
+        float f[12], a[12];
 #pragma unroll
-          for (int k = 0; k < 12; ++k) {
-            f[k] = e ? F[k].y : F[k].x;
-            a[k] = 0.f;
-          }
-#pragma unroll 1
-          for (int j = j0; j < j1; ++j) {
-            const QRec Q = tq[j];
-            const AdjCommon<float> c(Q, f);
-            const float wmax = c.wmax();
-            if (wmax < th.hi) c.series(Q, f, wmax, a);
-            else face_adj<true>(Q, f, th, OneAcc{a});
-          }
-#pragma unroll
-          for (int k = 0; k < 12; ++k) acc_add(sh.acc[2 * k + e][threadIdx.x], a[k]);
+        for (int k = 0; k < 12; ++k) {
+          f[k] = F[k].x;
+          a[k] = 0.f;
         }
+#pragma unroll 1
+        for (int j = cnt * sp.copy / sp.copies; j < j1; ++j) {
+          const QRec Q = tq[j];
+          const AdjCommon<float> c(Q, f);
+          const float wmax = c.wmax();
+          if (wmax < th.hi) c.series(Q, f, wmax, a);
+          else face_adj(Q, f, th, OneAcc{a});
+        }
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc_add(sh.acc[2 * k][threadIdx.x], a[k]);
       }
     }
     ring.release(t);
