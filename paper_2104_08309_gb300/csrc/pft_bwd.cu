@@ -2276,10 +2276,12 @@ int mesh3d_backward_body(const float* verts, int64_t n_verts, const int32_t* fac
                                                    y.per_split, th, y.fpb, at<double>(ws, y.partial), &h->status);
   PFT_BWD_LAUNCH();
   PFT_MARK(g_ev_stop);
-  if (launch_small_adjoint3(verts, n_verts, faces, n_faces, q, grad_out, n_q, h, at<void>(ws, y.phi), st) !=
-      cudaSuccess)
-    return PFT_ERR_CUDA;
-  g_bwd_launches += 2;
+  if (n_q > kSmallAdjoint) {   // fewer are never enough for Phi
+    if (launch_small_adjoint3(verts, n_verts, faces, n_faces, q, grad_out, n_q, h, at<void>(ws, y.phi), st) !=
+        cudaSuccess)
+      return PFT_ERR_CUDA;
+    g_bwd_launches += 2;
+  }
   const int nt = n_faces >= 65536 ? kAux : 64;
   k_bcorner3d<<<blocks(n_faces, nt), nt, 0, st>>>(verts, n_verts, faces, n_faces, at<double>(ws, y.partial), y.ks, h,
                                                   at<int32_t>(ws, y.small), q, grad_out,
@@ -2458,9 +2460,11 @@ int pft3d_mesh_qgrad(const float* verts, int64_t n_verts, const int32_t* faces, 
                                                              at<int32_t>(ws, y.small), y.slots,
                                                              at<double>(ws, y.spart));
   PFT_BWD_LAUNCH();
-  if (launch_small3(verts, n_verts, faces, n_faces, nullptr, h, nullptr, 0, at<void>(ws, y.mom), st) != cudaSuccess)
-    return PFT_ERR_CUDA;
-  ++g_bwd_launches;
+  if (!qsmall_direct((uint32_t)n_q, n_faces)) {   // so many small points that the moments may be asked for
+    if (launch_small3(verts, n_verts, faces, n_faces, nullptr, h, nullptr, 0, at<void>(ws, y.mom), st) != cudaSuccess)
+      return PFT_ERR_CUDA;
+    ++g_bwd_launches;
+  }
   k_qsmall_fin<<<std::min(blocks(n_q, 2), 4096u), 64, 0, st>>>(n_faces, q, grad_out, h, at<int32_t>(ws, y.small), y.slots,
                                                at<double>(ws, y.spart), at<double>(ws, y.mom), grad_q);
   PFT_BWD_LAUNCH();
