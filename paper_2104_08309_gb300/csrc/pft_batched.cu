@@ -131,7 +131,8 @@ int resolve_batched(int dim, const pft_options* o, bool shared_q, int64_t n_q, b
   return PFT_OK;
 }
 
-int batched_blocks_per_sm(int dim, bool fp64, int r, int nt);
+bool few_items(int dim, bool fp64, int r, int nt, int64_t n_items, int64_t n_shapes);
+int batched_blocks_per_sm(int dim, bool fp64, int r, int nt, bool few);
 
 // schedule = false: only the header (sizes), for the workspace size; no items are made or dealt.
 int build_plan(int dim, const int64_t* poly_off, int64_t n_polys, const int64_t* q_off, int64_t n_q,
@@ -156,7 +157,8 @@ int build_plan(int dim, const int64_t* poly_off, int64_t n_polys, const int64_t*
   const int64_t qt = (int64_t)r * nt;
   int dev = 0, sms = 1;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t G = std::max(1, sms) * (int64_t)batched_blocks_per_sm(dim, fp64, r, nt);
+  const int64_t G = std::max(1, sms) * (int64_t)batched_blocks_per_sm(
+      dim, fp64, r, nt, few_items(dim, fp64, r, nt, n_polys > 0 ? poly_off[n_polys] : 0, n_polys));
 
   if (schedule) P.pplan.resize((size_t)n_polys);
   std::vector<int64_t> cost;
@@ -607,10 +609,20 @@ __device__ __forceinline__ void finish_out_f32(const float* Q, const float* Qlo,
 // warp to finish a slot issues the tile kStages further on (as in k_fwd).
 // Register budget: as the single-shape kernel, except that the 3D FP32 shapes with 128 threads
 // keep one block per SM fewer here (4 at 4 Q points, 5 at 2), where the item loop and the
-// in-place finish would otherwise spill, that the 2D one with 4 Q points keeps five (it fits 92 registers, but
-// takes 102 by itself: 4,096 8-gons with 2,000 Q points each 407 us with four, 376 with five), that 2D with
-// 8 Q points is left free (155 and more), and that 512 threads are one block per SM (up to 128
-// registers: 16 warps, as 2 x 256 or 4 x 128).
+// in-place finish would otherwise spill, that 2D with 8 Q points is left free (155 and more), and that 512
+// threads are one block per SM (up to 128 registers: 16 warps, as 2 x 256 or 4 x 128).
+//
+// Batches of tiny shapes have policies of their own (few_items), the same arithmetic to the bit:
+//  * Pol2F32Few, 4 Q points and 128 threads, up to 16 segments a polygon on average: five blocks an SM (92 registers;
+//    102 by itself), which hide the items' ends.  4,096 8-gons with 2,000 Q points each 408 us with four, 378 with
+//    five; from 32 segments on the shorter schedule of the 92 registers costs more: 2,048 polygons of 128 segments with
+//    16 Q points each 156 / 173 us.
+//  * Pol3F32, up to 32 faces a mesh: the large-argument sinc paired (see face_edge), 1,024 meshes of 20 faces x 4,096 Q
+//    0.43 ms with a branch for each element, 0.40 so.
+struct Pol2F32Few : Pol2F32 {};
+template <class Pol> constexpr bool kFew = false;
+template <> constexpr bool kFew<Pol2F32Few> = true;
+template <> constexpr bool kFew<Pol3F32> = true;
 // Records per tile of the batched kernel's ring.  With one block of 16 warps per SM walking it (the
 // 512-thread shapes), 256 segments ran faster than 128 (4,096 polygons: 7.63 against 7.70 ms) and
 // 128 faces faster than 64 (1,024 meshes: 67.2 against 68.2 ms): a 16 KB or 24 KB ring.  The other
@@ -621,7 +633,7 @@ constexpr int kBTile = NT >= 512 ? (Pol::kDim == 2 ? 256 : 128) : Pol::kTile;
 template <class Pol, int R, int NT>
 constexpr int kBatchedMinBlocks = NT >= 512 ? 1
                                   : (Pol::kDim == 3 && R == 4 && NT == 128) ? 4
-                                  : (Pol::kDim == 2 && R == 4 && NT == 128 && sizeof(typename Pol::QT) == 4) ? 5
+                                  : std::is_same<Pol, Pol2F32Few>::value ? 5
                                   : (Pol::kDim == 2 && R == 8) ? (NT == 256 ? 1 : 2)
                                   : (Pol::kDim == 3 && R == 2 && NT == 128 && sizeof(typename Pol::QT) == 4)
                                       ? 5
@@ -988,12 +1000,19 @@ cudaError_t launch_batched_one(int grid, const BPlanHeader* ph, const int32_t* c
   X(Pol2F32, 1, 128) X(Pol2F32, 2, 128) X(Pol2F32, 4, 128) X(Pol2F32, 8, 128) X(Pol2F32, 1, 256)      \
   X(Pol2F32, 2, 256) X(Pol2F32, 4, 256) X(Pol2F32, 8, 256) X(Pol2F64, 1, 128) X(Pol2F64, 2, 128)      \
   X(Pol2F64, 1, 256) X(Pol2F64, 2, 256) X(Pol3F32Batch, 2, 128) X(Pol3F32Batch, 4, 128) X(Pol3F64, 1, 128)      \
-  X(Pol2F32, 4, 512) X(Pol3F32Batch, 4, 512)
+  X(Pol2F32, 4, 512) X(Pol3F32Batch, 4, 512) X(Pol2F32Few, 4, 128) X(Pol3F32, 2, 128) X(Pol3F32, 4, 128)           \
+  X(Pol3F32, 4, 512)
 
 #define PFT_BATCHED_MATCH(P, RR, NN) \
-  (P::kDim == dim && (sizeof(P::QT) == 8) == fp64 && r == RR && nt == NN)
+  (P::kDim == dim && (sizeof(P::QT) == 8) == fp64 && r == RR && nt == NN && kFew<P> == few)
+
+// Whether a batch of n_items segments or faces takes the policies for tiny shapes.
+bool few_items(int dim, bool fp64, int r, int nt, int64_t n_items, int64_t n_shapes) {
+  return !fp64 && (dim == 2 ? r == 4 && nt == 128 && n_items <= 16 * n_shapes : n_items <= 32 * n_shapes);
+}
 
 bool batched_config(int dim, bool fp64, int r, int nt) {
+  constexpr bool few = false;   // the tiny shapes' launch shapes are among the others'
 #define X(P, RR, NN) \
   if (PFT_BATCHED_MATCH(P, RR, NN)) return true;
   PFT_BATCHED_CASES(X)
@@ -1001,7 +1020,7 @@ bool batched_config(int dim, bool fp64, int r, int nt) {
   return false;
 }
 
-int batched_blocks_per_sm(int dim, bool fp64, int r, int nt) {
+int batched_blocks_per_sm(int dim, bool fp64, int r, int nt, bool few) {
 #define X(P, RR, NN) \
   if (PFT_BATCHED_MATCH(P, RR, NN)) return occ_batched<P, RR, NN>();
   PFT_BATCHED_CASES(X)
@@ -1009,7 +1028,8 @@ int batched_blocks_per_sm(int dim, bool fp64, int r, int nt) {
   return 1;
 }
 
-cudaError_t launch_batched(int dim, bool fp64, int r, int nt, int grid, const BPlanHeader* ph, const int32_t* cta_off,
+cudaError_t launch_batched(int dim, bool fp64, int r, int nt, bool few, int grid, const BPlanHeader* ph,
+                           const int32_t* cta_off,
                            const BItem* items, const PolyPlan* pplan, const PolyInfo* info, const void* segs,
                            const double* q, double2* partial, double* out, uint32_t* small, WsHeader* h, Thr th,
                            cudaStream_t st, const int32_t* qperm, const float* qlo) {
@@ -1131,7 +1151,8 @@ int run_rest(const PlanHandle& p, void* ws, const double* q, double* out, WsHead
       ++g_batched_launches;
     }
   }
-  if (launch_batched((int)p.dim, p.fp64 != 0, (int)p.r, (int)p.nt, (int)p.grid, phd,
+  const bool few = few_items((int)p.dim, p.fp64 != 0, (int)p.r, (int)p.nt, p.n_verts, p.n_polys);
+  if (launch_batched((int)p.dim, p.fp64 != 0, (int)p.r, (int)p.nt, few, (int)p.grid, phd,
                      at<int32_t>(ws, (size_t)p.cta_off), at<BItem>(ws, (size_t)p.items), pplan, info,
                      at<void>(ws, (size_t)p.segs), q, partial, out, small, h, plan_thr(p), st, qperm,
                      qlo) != cudaSuccess)

@@ -270,7 +270,7 @@ __device__ __forceinline__ void face_edge(V qx, V qy, V qz, const float4 A, cons
   // a short one) ran the prism at 10.24 instead of 10.63 ms, but 327,680 faces x 881,730 Q, which has few edge
   // sums, at 318.9 instead of 315.2 ms.  In the batched kernel even that costs more than it gives, but for meshes
   // of a few faces (1,024 meshes of 5,120 faces x 4,096 Q 26.48 ms, with a branch for each element 25.88; of 320 and
-  // 1,280 faces 0.5 and 1.5 %; of 20 faces 0.40 against 0.43 ms): kEach.
+  // 1,280 faces 0.5 and 1.5 %): kEach.
   constexpr int kE = sizeof(V) / sizeof(float);
   bool big = false;
 #pragma unroll
